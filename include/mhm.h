@@ -209,8 +209,8 @@ mhm_status mhm_mesh_query(const mhm_mesh* mesh, int32_t what, void* host_out, si
 
 /* Bytes of device scratch memory mhm_local_solve_batch needs for `precision`: a
  * region per refinement level of the mesh, one after the other.  MHM_FP64 levels
- * whose level window fits in shared memory need none (0 for a mesh of those
- * only); wider windows (P1 r = 7, P2 r = 5) live in one slot per SM of
+ * eliminated in registers need none (0 for a mesh of those only); the others
+ * (P2 r = 7) keep a level window in one slot per SM of
  * rows x (rows + N_I + 1) doubles.  MHM_MIXED adds its per-level buffers. */
 mhm_status mhm_local_workspace_size(const mhm_mesh* mesh, int32_t precision, size_t* bytes);
 

@@ -1,0 +1,303 @@
+// Frontal elimination of the local problems in FP64.
+//
+// What it computes.  The pinned matrix A_p of a local problem bordered by its R load columns,
+//     [ 0  G^T ]
+//     [ G  A_p ],
+// is eliminated node by node; after all nodes the leading block holds -G^T A_p^{-1} G, the
+// face integrals of Eq. "mat_global".  A node enters when the elimination first touches it
+// (front_plan.h), so the matrix at hand is the R loads and the nodes in the front, at most
+// M = R + slots rows: 33 slots for P1 at N = 32, 35 for P2 at N = 16 (an elimination level by
+// level works on windows of two levels, 64 and 127 rows).
+//
+// How.  This GPU has two FP64 multiply-adds per clock and SM: one warp instruction takes 16
+// clocks of the whole SM, however many of its lanes work, and about 60 other instructions
+// per scheduler fit beside it.  So the layout is made for full FP64 instructions: the lower
+// triangle lives in registers in tiles of 4 x 8 entries, one entry per lane, and a step is one
+// multiply-add per tile of the rows in use, a_ij -= (w_i / d) w_j with w the pivot's column in
+// shared memory.  The step's other FP64 work is the reciprocal (3), the scaling of w and the
+// entering node's couplings and loads (about 6).  The entering node usually takes the pivot's
+// slot in the same step.
+// One warp per element while the triangle fits its registers (M <= 64).  Larger fronts take
+// WR x WC warps: warp (r, c) owns rows 4 r .. 4 r + 3 and columns 8 c .. 8 c + 7 of every
+// 4 WR x 8 WC block, so which of its registers hold a row or a column is known at compile
+// time up to the block's index; a further warp prepares the entering rows.
+#pragma once
+
+#include <utility>
+
+#include "front_plan.h"
+#include "local_common.cuh"
+
+namespace mhm {
+
+// fn(integral_constant<int, 0>) .. fn(integral_constant<int, N - 1>): loops whose index must
+// be a constant (entries of a register array).
+template <class F, int... I>
+__device__ __forceinline__ void static_for_seq(F&& fn, std::integer_sequence<int, I...>) {
+    (fn(std::integral_constant<int, I>{}), ...);
+}
+template <int N, class F> __device__ __forceinline__ void static_for(F&& fn) {
+    static_for_seq(fn, std::make_integer_sequence<int, N>{});
+}
+
+// fn(integral_constant<int, i>) for a run-time i in [LO, HI), by halving.
+template <int LO, int HI, class F> __device__ __forceinline__ void static_select(int i, F&& fn) {
+    if constexpr (HI - LO == 1) {
+        fn(std::integral_constant<int, LO>{});
+    } else {
+        constexpr int M = (LO + HI) / 2;
+        if (i < M) static_select<LO, M>(i, fn);
+        else static_select<M, HI>(i, fn);
+    }
+}
+// fn(0), fn(1), .. fn(n - 1) for a run-time n <= N, each index a constant.  The rest of the
+// range hangs in one branch: under a loop of conditions the compiler issues every
+// instruction with a predicate, and a switched-off FP64 instruction takes its 16 clocks too.
+template <int I, int N, class F> __device__ __forceinline__ void static_upto(int n, F&& fn) {
+    if constexpr (I < N) {
+        if (n > I) {
+            fn(std::integral_constant<int, I>{});
+            static_upto<I + 1, N>(n, fn);
+        }
+    }
+}
+
+// The distribution of the triangle: AR rows of blocks of 4 WR x 8 WC entries.
+template <int WR_, int WC_, int AR_>
+struct FrontTiles {
+    static constexpr int WR = WR_, WC = WC_, AR = AR_, NW = WR * WC;
+    static constexpr int cols(int a) { return (4 * WR * a + 4 * WR - 1) / (8 * WC) + 1; }   // blocks of row a
+    static constexpr int at(int a) { return a == 0 ? 0 : at(a - 1) + cols(a - 1); }
+    static constexpr int NT = at(AR);        // entries per lane
+    static constexpr int NB = cols(AR - 1);  // block columns
+    static constexpr int rows = 4 * WR * AR;
+    static constexpr int vec = (rows + 31) / 32 * 32;   // entries of a vector over the rows
+    static constexpr int threads = NW == 1 ? 32 : 32 * (NW + 1);
+    // first block row that holds entries of block column b
+    static constexpr int first(int b) { return (8 * WC * b) / (4 * WR); }
+};
+// Shared memory of one element: pivot column, scaled pivot column and entering row (two of
+// each, used in turn), a row of zeros, the inverse pivots and the pivots' couplings.
+struct FrontShared {
+    double *w[2], *s[2], *nb[2], *zero, *piv;
+};
+__host__ __device__ constexpr size_t front_shared_doubles(int vec) { return 7 * (size_t)vec + 4; }
+__device__ __forceinline__ FrontShared front_shared(double* base, int v) {
+    FrontShared f;
+    for (int k = 0; k < 2; ++k) f.w[k] = base + k * v, f.s[k] = base + (2 + k) * v, f.nb[k] = base + (4 + k) * v;
+    f.zero = base + 6 * v;
+    f.piv = base + 7 * v;   // inverse pivot per parity; then the pivot's coupling with the entering node
+    return f;
+}
+
+// 1 / d for a normal d by one third-order step y (1 + e + e^2), e = 1 - d y, from the
+// hardware's estimate (relative error below 2^-20): truncation below 2^-60.
+__device__ __forceinline__ double front_rcp(double d) {
+    double y;
+    asm("rcp.approx.ftz.f64 %0, %1;" : "=d"(y) : "d"(d));
+    const double e = fma(-d, y, 1.0), t = fma(e, e, e);
+    return fma(t, y, y);
+}
+
+template <int NW> __device__ __forceinline__ void front_sync() {
+    if (NW == 1) __syncwarp();
+    else __syncthreads();
+}
+
+// The elimination.  T: FrontTiles.  ev: the step table (front_plan.h).
+// prob.prep(e, ev[e], nb, wnew) is called by one warp for every step in order: it fills nb
+// (T::vec entries) with the row of step e's entering node against the loads and the front
+// as the step leaves it, zero elsewhere, and *wnew with its coupling to the pivot.  keep (NULL: none) gets the scaled
+// pivot column of every step, `stride` doubles apart.  *bad: 1 if a pivot was not positive.
+// A: the entries; the result is read with front_result.  All warps of the element call it;
+// starts and ends with a barrier.
+template <class T, class Prob>
+__device__ __forceinline__ void front_eliminate(Prob& prob, const int4* __restrict__ ev, int steps, int R,
+                                                const FrontShared& sh, double (&A)[T::NT], int* bad, double* keep,
+                                                int stride) {
+    constexpr int WR = T::WR, WC = T::WC, NW = T::NW, AR = T::AR;
+    const int tid = NW == 1 ? (int)(threadIdx.x & 31) : (int)threadIdx.x;
+    const int warp = NW == 1 ? 0 : __shfl_sync(0xffffffffu, tid >> 5, 0), lane = tid & 31;
+    const int row = 4 * (warp / WC) + (lane >> 3), col = 8 * (warp % WC) + (lane & 7);   // inside a block
+#pragma unroll
+    for (int q = 0; q < T::NT; ++q) A[q] = 0.0;
+    for (int t = tid; t < 7 * T::vec; t += T::threads) sh.w[0][t] = 0.0;
+    front_sync<NW>();
+    int4 v = ev[0];
+    if (NW > 1 && warp == NW) {
+        int4 vn = ev[steps > 1];
+        prob.prep(0, v, sh.nb[0], sh.piv + 2);
+        __syncthreads();
+        for (int e = 0; e < steps; ++e) {
+            const bool pivot = (v.x & 255) != kNoSlot;
+            v = vn;
+            if (e + 2 < steps) vn = ev[e + 2];
+            if (e + 1 < steps) prob.prep(e + 1, v, sh.nb[(e + 1) & 1], sh.piv + 2 + ((e + 1) & 1));
+            __syncthreads();
+            if (pivot) __syncthreads();
+        }
+        __syncthreads();
+        return;
+    }
+    if (NW == 1) prob.prep(0, v, sh.nb[0], sh.piv + 2);
+    front_sync<NW>();
+    for (int e = 0; e < steps; ++e) {
+        const int par = e & 1;
+        const int ps = v.x & 255, zs = (v.x >> 8) & 255, mm = R + ((v.x >> 16) & 255);
+        if (e + 1 < steps) v = ev[e + 1];
+        const int P = ps == kNoSlot ? -1 : R + ps, Z = zs == kNoSlot ? -1 : R + zs;
+        double* w = sh.w[par];
+        double* s = sh.s[par];
+        const double* nb = sh.nb[par];
+        // the pivot's row and column to w, then those of the entering node from nb (a slot
+        // left free goes to zero and stays there)
+        auto cross = [&](int X, auto&& fn) {   // fn(entry, other index) on row and column X
+            static_select<0, AR>(X / (4 * WR), [&](auto ca) {
+                constexpr int a = ca;
+                if (X - row == 4 * WR * a)
+                    static_for<T::cols(a)>([&](auto cb) {
+                        constexpr int b = cb;
+                        if (8 * WC * b + col <= X) fn(A[T::at(a) + b], 8 * WC * b + col);
+                    });
+            });
+            static_select<0, T::NB>(X / (8 * WC), [&](auto cb) {
+                constexpr int b = cb;
+                if (X - col == 8 * WC * b)
+                    static_for<AR - T::first(b)>([&](auto ca) {
+                        constexpr int a = ca + T::first(b);
+                        const int i = 4 * WR * a + row;
+                        if (a > T::first(b) + 2 * WC / WR || i > X) fn(A[T::at(a) + b], i);
+                    });
+            });
+        };
+        if (P >= 0) {
+            const double* in = Z == P ? nb : sh.zero;
+            cross(P, [&](double& x, int k) {
+                w[k] = x;
+                if (NW > 1 && k == P) {
+                    if (!(x > 0.0)) *bad = 1;
+                    sh.piv[par] = front_rcp(x);
+                }
+                x = in[k];
+            });
+        }
+        if (Z >= 0 && Z != P) cross(Z, [&](double& x, int k) { x = nb[k]; });
+        front_sync<NW>();
+        double inv = 0.0;
+        if (NW == 1 && P >= 0) {   // (read by all lanes before w[P] changes)
+            const double d = w[P];
+            if (!(d > 0.0)) *bad = 1;
+            inv = front_rcp(d);
+        }
+        if (NW == 1 && e + 1 < steps) prob.prep(e + 1, v, sh.nb[par ^ 1], sh.piv + 2 + (par ^ 1));
+        if (NW == 1) __syncwarp();
+        if (P >= 0) {
+            const double wnew = sh.piv[2 + par];
+            if (NW > 1) inv = sh.piv[par];
+            // whole blocks: rows past the ones in use get zeros
+            const int top = (mm + 8 * WC - 1) / (8 * WC) * (8 * WC);
+            for (int q = tid; q < top; q += 32 * NW) {
+                double x = q == Z ? wnew : (q == P || q >= mm) ? 0.0 : w[q];
+                if (q == Z || q == P || q >= mm) w[q] = x;
+                x *= inv;
+                s[q] = x;
+                if (keep && q < mm) keep[(size_t)e * stride + q] = x;
+            }
+        }
+        if (NW == 1 || P >= 0) front_sync<NW>();
+        if (P >= 0) {
+            double wb[T::NB];
+            static_for<T::NB>([&](auto b) { wb[b] = 8 * WC * b < mm ? w[8 * WC * b + col] : 0.0; });
+            // rows of blocks with this warp's rows in use
+            static_upto<0, AR>((mm - 4 * (warp / WC) + 4 * WR - 1) / (4 * WR), [&](auto ca) {
+                constexpr int a = ca;
+                const double sa = s[4 * WR * a + row];
+                static_for<T::cols(a)>([&](auto cb) {
+                    constexpr int b = cb;
+                    A[T::at(a) + b] = fma(-sa, wb[b], A[T::at(a) + b]);
+                });
+            });
+        }
+    }
+    front_sync<NW>();
+}
+
+// Calls fn(i, j, value) for this thread's entries i >= j of the leading R x R block.
+template <class T, class F>
+__device__ __forceinline__ void front_result(int R, const double (&A)[T::NT], F&& fn) {
+    const int tid = T::NW == 1 ? (int)(threadIdx.x & 31) : (int)threadIdx.x, warp = tid >> 5, lane = tid & 31;
+    if (warp >= T::NW) return;
+    const int row = 4 * (warp / T::WC) + (lane >> 3), col = 8 * (warp % T::WC) + (lane & 7);
+    static_for<T::AR>([&](auto ca) {
+        constexpr int a = ca;
+        if (4 * T::WR * a < R)
+            static_for<T::cols(a)>([&](auto cb) {
+                constexpr int b = cb;
+                const int i = 4 * T::WR * a + row, j = 8 * T::WC * b + col;
+                if (i < R && j <= i) fn(i, j, A[T::at(a) + b]);
+            });
+    });
+}
+
+// Entering rows of the 2-D local problems (FrontPlan's tables): couplings from kappa and the
+// two element matrices, ahead of their use by one batch of 32 / ncp steps (loads of the batch
+// after it in flight).  load(x, y, mass count | faces << 8, column) gives the node's load.  The pinned
+// node is kept as a node coupled to nothing, with a unit pivot and no loads.
+template <int NCP, class Load>
+struct FrontRows2D {
+    static constexpr int B = 32 / NCP;
+    const uint2* cp;
+    const double* kap;
+    const double* Ke;
+    int steps, R, vec, pin;   // vec: entries of a row; pin: lattice point x | y << 16
+    Load load;
+    int pin_slot = -1;
+    uint2 cur, nxt, far;
+    double val = 0.0, diag = 0.0, k0 = 0.0, k1 = 0.0;
+
+    __device__ __forceinline__ uint2 entry(int batch) const {
+        const int lane = threadIdx.x & 31, e = batch * B + lane / NCP;
+        return e < steps ? cp[(size_t)e * NCP + lane % NCP] : make_uint2(kNoSlot, 0xffff0000u);
+    }
+    __device__ __forceinline__ void fetch(uint2 q) {
+        const uint32_t t1 = q.y >> 16;
+        const bool any = (q.x & 255) != kNoSlot;
+        k0 = any ? kap[q.y & 0xffff] : 0.0;
+        k1 = any && t1 != 0xffff ? kap[t1] : 0.0;
+    }
+    __device__ __forceinline__ void start() {
+        nxt = entry(0);
+        fetch(nxt);
+        far = entry(1);
+    }
+    __device__ __forceinline__ void prep(int e, const int4& v, double* nb, double* wnew) {
+        const int lane = threadIdx.x & 31, sub = lane % NCP;
+        if (e % B == 0) {
+            cur = nxt;
+            val = fma(k1, Ke[(cur.x >> 16) & 255], k0 * Ke[(cur.x >> 8) & 255]);
+            diag = val + __shfl_down_sync(0xffffffffu, val, 1) + __shfl_down_sync(0xffffffffu, val, 2);
+            nxt = far;
+            fetch(nxt);
+            far = entry(e / B + 2);
+        }
+        const int ps = v.x & 255, zs = (v.x >> 8) & 255;
+        if (zs != kNoSlot) {
+            const bool pinned = v.y == pin;
+            for (int q = lane; q < vec; q += 32) nb[q] = q < R && !pinned ? load(v.y & 0xffff, v.y >> 16, v.z, q) : 0.0;
+            if (lane == 0) *wnew = 0.0;
+            __syncwarp();
+            if (lane / NCP == e % B) {
+                const int sl = cur.x & 255;
+                if (sub == NCP - 3) nb[R + zs] = pinned ? 1.0 : diag;
+                else if (sl < kDiagSlot && !pinned && sl != pin_slot) nb[R + sl] = val;
+                else if (sl == kPivotSlot && !pinned && ps != pin_slot) *wnew = val;
+            }
+            if (ps == pin_slot && ps != kNoSlot) pin_slot = -1;
+            if (pinned) pin_slot = zs;
+        } else if (ps == pin_slot && ps != kNoSlot) {
+            pin_slot = -1;
+        }
+    }
+};
+
+}  // namespace mhm

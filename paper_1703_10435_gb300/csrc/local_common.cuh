@@ -96,6 +96,43 @@ __device__ inline void element_stiffness(int P, const double X[3][2], double* S 
     }
 }
 
+// Element matrices of the up and the down fine triangles of the coarse triangle X (N
+// segments per face) as element_stiffness, an entry per thread: Ke[36 down + nb a + b].
+__device__ inline void element_stiffness_pair(int P, int N, const double X[3][2], double* Ke, int tid, int nthr) {
+    const double e1[2] = {(X[1][0] - X[0][0]) / N, (X[1][1] - X[0][1]) / N};
+    const double e2[2] = {(X[2][0] - X[0][0]) / N, (X[2][1] - X[0][1]) / N};
+    const int nb = P == 1 ? 3 : 6;
+    for (int t = tid; t < 2 * nb * nb; t += nthr) {
+        const int dn = t >= nb * nb, ab = t - dn * nb * nb, a = ab / nb, b = ab - a * nb;
+        // edge vectors B - A and C - A: (e1, e2) up, (e2, e2 - e1) down
+        const double j00 = dn ? e2[0] : e1[0], j10 = dn ? e2[1] : e1[1];
+        const double j01 = dn ? e2[0] - e1[0] : e2[0], j11 = dn ? e2[1] - e1[1] : e2[1];
+        const double det = j00 * j11 - j01 * j10, adet = fabs(det), id = 1.0 / det;
+        const double i00 = j11 * id, i01 = -j01 * id, i10 = -j10 * id, i11 = j00 * id;
+        const double g00 = i00 * i00 + i01 * i01, g01 = i00 * i10 + i01 * i11, g11 = i10 * i10 + i11 * i11;
+        double s = 0.0;
+        for (int q = 0; q < (P == 1 ? 1 : 3); ++q) {   // P2: the edge midpoints (exact)
+            const double l1 = q < 2 ? 0.5 : 0.0, l2 = q > 0 ? 0.5 : 0.0, l0 = 1.0 - l1 - l2;
+            double gr[2][2];
+            for (int k = 0; k < 2; ++k) {
+                const int n = k ? b : a;
+                double gx, gy;
+                if (P == 1) gx = n == 0 ? -1.0 : (n == 1), gy = n == 0 ? -1.0 : (n == 2);
+                else if (n == 0) gx = gy = 1.0 - 4.0 * l0;
+                else if (n == 1) gx = 4.0 * l1 - 1.0, gy = 0.0;
+                else if (n == 2) gx = 0.0, gy = 4.0 * l2 - 1.0;
+                else if (n == 3) gx = 4.0 * l2, gy = 4.0 * l1;
+                else if (n == 4) gx = -4.0 * l2, gy = 4.0 * (l0 - l2);
+                else gx = 4.0 * (l0 - l1), gy = -4.0 * l1;
+                gr[k][0] = gx, gr[k][1] = gy;
+            }
+            s += adet * (P == 1 ? 0.5 : 1.0 / 6.0) *
+                 (gr[0][0] * (g00 * gr[1][0] + g01 * gr[1][1]) + gr[0][1] * (g01 * gr[1][0] + g11 * gr[1][1]));
+        }
+        Ke[36 * dn + ab] = s;
+    }
+}
+
 // Lattice coordinates (P-lattice) of the element nodes of fine triangle
 // (type up/down, column i, fine row j).
 __device__ __forceinline__ void element_nodes(int P, bool up, int i, int j, int nx[6], int ny[6]) {

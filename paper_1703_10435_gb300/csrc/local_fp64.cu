@@ -1,5 +1,5 @@
 // solveLocalProblem in FP64 (Alg. 1; Sec. 3, Eqs. "etaf", "etai", "etaf_comb";
-// Sec. 4.2, Eq. "source_term"), one thread block per coarse triangle K.
+// Sec. 4.2, Eq. "source_term").
 //
 // What is computed.  With A the stiffness matrix of a(.,.)_K on the submesh,
 // m_w = int_K phi_w, and the loads N_i = -(s psi_i, phi_w)_{dK}, F = (f, phi_w)_K,
@@ -7,36 +7,31 @@
 // system pinned at one DOF (choose_pin: inside the stiffest region touching the
 // first two levels) with the compatible loads g~ = g - (1^T g / |K|) m.
 // The face integrals of Eq. "mat_global" then reduce to a Gram matrix:
-//     A_K = -N~^T A_p^{-1} N~ = -Y^T Y,   E_K = Y^T y_f,
-// with Y = L^{-1} N~, y_f = L^{-1} f~ and A_p = L L^T (Cholesky of the pinned
-// matrix).  Only the forward elimination is needed; no factor is stored.
+//     A_K = -N~^T A_p^{-1} N~,   E_K = N~^T A_p^{-1} f~,
+// which is what eliminating A_p from the matrix bordered by the loads leaves in the
+// border; no factor is stored.
 //
-// How.  A_p is block tridiagonal in the levels of the submesh (local_common.cuh).
-// The kernel slides a window over two consecutive levels held in shared memory:
-// rows [0, b) hold level lev (already reduced by the previous levels), rows
-// [b, b + b') the fresh level lev+1, the columns are the symmetric part (lower
-// triangle used) followed by the R = N_I + 1 right-hand sides.  It adds the
-// element matrices and loads of fine row lev (the only triangles touching both
-// levels), eliminates the b pivots of level lev by right-looking Cholesky on the
-// augmented rows (which produces L, W = L^{-1} C^T, the Schur complement of
-// level lev+1 and the forward-solved right-hand sides in one pass), accumulates
-// Y_lev^T Y_lev into the Gram matrix and moves the reduced level lev+1 to the
-// top of the window.
+// How.  Frontal elimination node by node in registers (front.cuh), one warp per coarse
+// triangle up to M = R + slots = 64 rows, 4 to 16 warps above.  Bound by the FP64 pipe: per
+// element of P1 r = 5, R = 19, 26.0 k FP64 warp instructions (16 clocks of the SM each), of
+// which 16.3 k are the algorithm's; 2048 elements in 3.44 ms with the pipe 79 % busy (8.69 ms
+// with a window over two levels in shared memory, 128 threads per element), 4480 elements of
+// P2 r = 4 in 7.9 ms (74.3 ms), 320 elements of P1 r = 7, R = 13 in 63 ms.
 //
-// Levels whose window does not fit in shared memory (P1 r = 7: 256 rows; P2 r = 5)
-// keep it in global memory instead, one workspace slot per block of a persistent
-// grid (one block per SM, so the slots stay in L2), and factor it panel by panel
-// through shared memory (wide_cholesky_level).
+// A level whose front is too large for that (P2 r = 7: 259 slots) slides a window over two
+// consecutive levels held in global memory, one workspace slot per block of a persistent
+// grid, and factors it panel by panel through shared memory (wide_cholesky_level).
 #include <cuda_runtime.h>
 
+#include "front.cuh"
 #include "local_common.cuh"
 #include "mixed_wide.h"
+#include "source_loads.cuh"
 
 namespace mhm {
 
 namespace {
 
-constexpr int kThreads = 128;
 constexpr int kThreadsWide = 512;   // wide window: one block per SM
 constexpr int kNBWide = 16;         // wide window: pivots per panel
 
@@ -58,6 +53,10 @@ struct Fp64Args {
     int32_t *status, *iters;
     const int32_t* kcount;   // launch indices >= *kcount do nothing (NULL: no bound)
     int fallback;            // 1: re-solving elements of a failed mixed refinement (iters = -1)
+    // frontal elimination: the level's step tables
+    const int4* ev;
+    const uint2* cp;
+    int steps;
 };
 
 struct KCtx {
@@ -234,19 +233,17 @@ inline size_t wide_smem_bytes(int rows, int R) {
            sizeof(double);
 }
 
-template <int RPL, bool WIDE>
-__global__ void __launch_bounds__(WIDE ? kThreadsWide : kThreads, WIDE ? 1 : 4) k_local_fp64(const Fp64Args g) {
+__global__ void __launch_bounds__(kThreadsWide, 1) k_local_fp64_wide(const Fp64Args g) {
     extern __shared__ double smem[];
     __shared__ KCtx c;
     __shared__ double red[32];
     const int R = g.R;
-    // window rows x ld: shared memory, or this block's workspace slot
-    double* W = WIDE ? g.win + (size_t)blockIdx.x * g.win_doubles : smem;
-    double* gram = WIDE ? smem : smem + (size_t)g.rows * g.ld;   // R x R, upper triangle used
-    double* Ps = smem + wide_gram_doubles(R);                      // (wide) panel
+    double* W = g.win + (size_t)blockIdx.x * g.win_doubles;   // window rows x ld: this block's workspace slot
+    double* gram = smem;                                       // R x R, upper triangle used
+    double* Ps = smem + wide_gram_doubles(R);                  // panel
     double* Rs = Ps + (size_t)g.rows * wide_panel_stride<kNBWide>();
     double* invd = Rs + (size_t)kNBWide * R;
-    // launch indices within the level: one per block, or (wide) strided over the grid
+    // launch indices within the level, strided over the grid
     for (int64_t ki = g.K0 + blockIdx.x; ki < g.K1; ki += gridDim.x) {
     if (g.kcount && ki >= *g.kcount) break;                        // (whole block)
     const int64_t K = g.dm.klist ? (int64_t)g.dm.klist[ki] : ki;  // coarse element
@@ -326,22 +323,8 @@ __global__ void __launch_bounds__(WIDE ? kThreadsWide : kThreads, WIDE ? 1 : 4) 
         }
         // Blocked right-looking Cholesky of the level's b pivots on the augmented window
         // rows; the right-hand-side columns (all window rows) are forward-substituted.
-        if constexpr (WIDE) {
-            // Gram += Y^T Y accumulated panel by panel
-            wide_cholesky_level<kNBWide>(W, g.ld, b, nr, W + g.rhs0, g.ld, nr, R, &c.bad, Ps, Rs, invd, gram);
-        } else {
-            blocked_cholesky_level<double, 8, RPL, 2>(W, g.ld, b, nr, W + g.rhs0, g.ld, nr, R, &c.bad);
-            // Gram += Y^T Y over the b rows of this level (upper triangle c1 <= c2)
-            for (int t = threadIdx.x; t < R * (R + 1) / 2; t += blockDim.x) {
-                int c1 = 0, c2 = t;   // t-th pair of the upper triangle, row by row
-                while (c2 >= R - c1) { c2 -= R - c1; ++c1; }
-                c2 += c1;
-                double s = 0.0;
-                for (int k = 0; k < b; ++k) s += W[k * g.ld + g.rhs0 + c1] * W[k * g.ld + g.rhs0 + c2];
-                gram[c1 * R + c2] += s;
-            }
-            __syncthreads();
-        }
+        // Gram += Y^T Y accumulated panel by panel
+        wide_cholesky_level<kNBWide>(W, g.ld, b, nr, W + g.rhs0, g.ld, nr, R, &c.bad, Ps, Rs, invd, gram);
         if (bn > 0) {
             // move the reduced level lev+1 (rows/cols [b, nr)) to the top; clear the next rows
             for (int t = threadIdx.x; t < bn * (bn + R); t += blockDim.x) {
@@ -383,6 +366,230 @@ __global__ void __launch_bounds__(WIDE ? kThreadsWide : kThreads, WIDE ? 1 : 4) 
     }
 }
 
+// Shared-memory layout (doubles) of one element of the frontal kernel.
+struct FrontSmem {
+    int Ke, mass, cproj, tab, src, total;
+};
+__host__ __device__ inline FrontSmem front_smem(int vec, int R, int kind, int P, int N) {
+    const int PN = P * N;
+    FrontSmem l;
+    int o = (int)front_shared_doubles(vec);
+    l.Ke = o, o += 72;       // element matrices, up then down
+    l.mass = o, o += 8;      // mass of a node on k fine triangles
+    l.cproj = o, o += R;     // projection coefficient of each right-hand side
+    l.tab = o, o += source_table_doubles(kind, PN);
+    l.src = o, o += kind == MHM_SRC_CONST ? 0 : (PN + 1) * (PN + 2) / 2;   // source load per node
+    l.total = o;
+    return l;
+}
+
+struct FrontCtx {
+    double X[3][2];
+    double area, flen[3], FK;
+    int sgn[3], rev[3], la1[3], bad, pin;
+};
+
+// choose_pin by one warp (kappa > 0 orders like its bits): x | y << 16.
+__device__ inline int choose_pin_warp(int P, int N, const double* kap) {
+    const int lane = threadIdx.x & 31, PN = P * N;
+    const int ymax = N == 1 ? (P == 1 ? 0 : 1) : (P == 1 ? 1 : 3), jmax = N == 1 ? 1 : 2;
+    long long best = -1;
+    for (int j = 0; j < jmax; ++j)
+        for (int t = lane; t < 2 * (N - j) - 1; t += 32) {
+            const long long k = __double_as_longlong(kap[j * (2 * N - j) + t]);
+            best = k > best ? k : best;
+        }
+    for (int o = 16; o > 0; o >>= 1) {
+        const long long k = __shfl_xor_sync(0xffffffffu, best, o);
+        best = k > best ? k : best;
+    }
+    int bd = 1 << 30;
+    for (int j = 0; j < jmax; ++j)
+        for (int t = lane; t < 2 * (N - j) - 1; t += 32) {
+            if (__double_as_longlong(kap[j * (2 * N - j) + t]) != best) continue;
+            int nx[6], ny[6];
+            element_nodes(P, t < N - j, t < N - j ? t : t - (N - j), j, nx, ny);
+            for (int a = 0; a < (P == 1 ? 3 : 6); ++a)
+                if (ny[a] <= ymax) bd = min(bd, ny[a] * (PN + 1) - ny[a] * (ny[a] - 1) / 2 + nx[a]);
+        }
+    bd = __reduce_min_sync(0xffffffffu, bd);
+    int y = 0;
+    while (bd >= PN + 1 - y) bd -= PN + 1 - y, ++y;
+    return (bd & 0xffff) | y << 16;
+}
+
+// Loads of a node in the bordered matrix: the face load -(s psi_j, phi_w)_{dK}, the
+// projection -(1^T g / |K|) m_w, the source load.  Lane q holds columns q and q + 32.
+struct FrontLoad {
+    const double *btab, *mass, *src;   // src NULL: constant source
+    int PN, NI;
+    double value;
+    double cp0, cp1, cf0, cf1;
+    int fc0, fc1;                      // face | reversed << 2 | table row << 3, -1: none
+    __device__ __forceinline__ double operator()(int x, int y, int info, int q) const {
+        const bool hi = q >= 32;
+        const double m = mass[info & 255];
+        double v = -(hi ? cp1 : cp0) * m;
+        if (info >> 8) {   // (the whole warp: a node on the boundary)
+            const int fc = hi ? fc1 : fc0;
+            if (fc >= 0 && ((info >> 8) >> (fc & 3)) & 1) {
+                const int kl = (fc & 3) == 2 ? x : (fc & 3) == 0 ? y : PN - y;
+                v = fma(hi ? cf1 : cf0, btab[(fc >> 3) * (PN + 1) + ((fc & 4) ? PN - kl : kl)], v);
+            }
+        }
+        if (q == NI) v = src ? v + src[y * (PN + 1) - y * (y - 1) / 2 + x] : fma(value, m, v);
+        return v;
+    }
+};
+
+// One block per coarse triangle at a time: NW compute warps (and one that prepares rows if NW > 1).
+template <class T, int NCP, int MINB>
+__global__ void __launch_bounds__(T::threads, MINB) k_local_fp64(const __grid_constant__ Fp64Args g) {
+    constexpr int NW = T::NW;
+    extern __shared__ double smem[];
+    __shared__ FrontCtx c;
+    const int P = g.P, N = g.N, PN = g.PN, R = g.R, NI = g.NI, tid = threadIdx.x, nthr = blockDim.x;
+    const FrontSmem L = front_smem(T::vec, R, g.src_kind, P, N);
+    const FrontShared sh = front_shared(smem, T::vec);
+    double* Ke = smem + L.Ke;
+    double* cproj = smem + L.cproj;
+    double* tab = smem + L.tab;
+    double* src = smem + L.src;
+
+    for (int64_t ki = g.K0 + blockIdx.x; ki < g.K1; ki += gridDim.x) {   // launch indices within the level
+    if (g.kcount && ki >= *g.kcount) break;                              // (whole block)
+    const int64_t K = g.dm.klist ? (int64_t)g.dm.klist[ki] : ki;         // coarse element
+    const double* kap = g.kappa + (g.dm.kap_off ? g.dm.kap_off[K] : K * (int64_t)N * N);
+
+    // ---- per-K setup
+    if (tid < 6) c.X[tid >> 1][tid & 1] = g.dm.geom[6 * K + tid];
+    if (tid < 3) {
+        c.sgn[tid] = g.dm.sign[3 * K + tid];
+        c.rev[tid] = g.dm.rev[3 * K + tid];
+        c.la1[tid] = face_la1(g.dm, K, tid);
+    }
+    if (tid < 32) {
+        const int pin = choose_pin_warp(P, N, kap);
+        if (tid == 0) c.pin = pin, c.bad = 0;
+    }
+    __syncthreads();
+    if (tid < 3) {
+        const double* P0 = c.X[(tid + 1) % 3];
+        const double* Q0 = c.X[(tid + 2) % 3];
+        c.flen[tid] = sqrt((Q0[0] - P0[0]) * (Q0[0] - P0[0]) + (Q0[1] - P0[1]) * (Q0[1] - P0[1]));
+    }
+    const double area = 0.5 * fabs((c.X[1][0] - c.X[0][0]) * (c.X[2][1] - c.X[0][1]) -
+                                   (c.X[2][0] - c.X[0][0]) * (c.X[1][1] - c.X[0][1]));
+    if (tid < 8) smem[L.mass + tid] = tid * (area / ((double)N * N) / 3.0);
+    element_stiffness_pair(P, N, c.X, Ke, tid, nthr);
+    source_tables(g.dm, g.src_kind, g.src_value, g.src_freq, P, N, c.X, tab, tid, nthr);
+    __syncthreads();
+    const double* vals = g.src_vals ? g.src_vals + 16 * (kap - g.kappa) : nullptr;
+    if (g.src_kind == MHM_SRC_CONST) {
+        if (tid == 0) c.FK = g.src_value * area;
+    } else {
+        const int n = (PN + 1) * (PN + 2) / 2;
+        int x = tid, y = 0;
+        for (int u = tid; u < n; u += nthr, x += nthr) {
+            while (x > PN - y) x -= PN + 1 - y, ++y;
+            src[u] = source_node(g.src_kind, P, N, x, y, tab, vals);
+        }
+        __syncthreads();
+        if (tid < 32) {
+            double s = 0.0;
+            for (int u = tid; u < n; u += 32) s += src[u];
+            for (int o = 16; o > 0; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
+            if (tid == 0) c.FK = s;
+        }
+    }
+    __syncthreads();
+    for (int col = tid; col < R; col += nthr) {
+        if (col == NI) cproj[col] = c.FK / area;
+        else {
+            const int a = col / g.dpf, jf = col - a * g.dpf;
+            const int row = face_row(jf, c.la1[a], g.dm.fm, g.dm.lmax1);
+            cproj[col] = row < 0 ? 0.0 : -c.sgn[a] * c.flen[a] * g.dm.btab_sum[row] / area;
+        }
+    }
+    __syncthreads();
+    FrontLoad load{g.dm.btab, smem + L.mass, g.src_kind == MHM_SRC_CONST ? nullptr : src, PN, NI, g.src_value,
+                   0.0, 0.0, 0.0, 0.0, -1, -1};
+    for (int h = 0; h < 2; ++h) {
+        const int col = (tid & 31) + 32 * h;
+        if (col >= R) break;
+        (h ? load.cp1 : load.cp0) = cproj[col];
+        if (col == NI) break;
+        const int a = col / g.dpf, row = face_row(col - a * g.dpf, c.la1[a], g.dm.fm, g.dm.lmax1);
+        (h ? load.cf1 : load.cf0) = -c.sgn[a] * c.flen[a];
+        if (row >= 0) (h ? load.fc1 : load.fc0) = a | (c.rev[a] ? 4 : 0) | row << 3;
+    }
+    FrontRows2D<NCP, FrontLoad> rows{g.cp, kap, Ke, g.steps, R, T::vec, c.pin, load};
+    if (NW == 1 || (tid >> 5) == NW) rows.start();
+
+    double A[T::NT];
+    front_eliminate<T>(rows, g.ev, g.steps, R, sh, A, &c.bad, nullptr, 0);
+
+    // ---- outputs
+    double* AK = g.AK + K * NI * NI;
+    front_result<T>(R, A, [&](int i, int j, double v) {
+        if (i < NI) {
+            AK[i * NI + j] = v;
+            AK[j * NI + i] = v;
+        } else if (j < NI) {
+            g.EK[K * NI + j] = -v;
+        }
+    });
+    for (int j = tid; j < NI; j += nthr) {
+        const int a = j / g.dpf, jf = j - a * g.dpf;
+        const int row = face_row(jf, c.la1[a], g.dm.fm, g.dm.lmax1);
+        g.BK[K * NI + j] = row < 0 ? 0.0 : c.sgn[a] * c.flen[a] * g.dm.btab_sum[row];
+    }
+    if (tid == 0) {
+        g.FK[K] = c.FK;
+        g.status[K] = c.bad ? MHM_ERR_INVALID_ARG : 0;
+        if (g.iters) g.iters[K] = g.fallback ? -1 : 1;
+        if (g.sword && (c.bad || g.fallback))
+            atomicOr(g.sword, (c.bad ? 1u << MHM_ERR_INVALID_ARG : 0u) | (g.fallback ? MHM_STATUS_REFINED_IN_FP64 : 0u));
+    }    __syncthreads();   // the context and the tables serve the next element
+    }
+}
+
+// The frontal kernel for a bordered matrix of M rows and step tables of ncp entries; NULL if
+// it is too large.  One warp holds up to 72 entries a lane; beyond, as many warps as keep a
+// lane's share near 40.
+struct FrontKernel {
+    void (*kern)(const Fp64Args) = nullptr;
+    int threads = 0, vec = 0;
+};
+template <class T, int NCP, int MINB>
+bool front_try(int M, FrontKernel* k) {
+    if (k->kern || M > T::rows) return false;
+    k->kern = k_local_fp64<T, NCP, MINB>;
+    k->threads = T::threads;
+    k->vec = T::vec;
+    return true;
+}
+template <int NCP>
+FrontKernel front_kernel_of(int M) {
+    FrontKernel k;
+    front_try<FrontTiles<1, 1, 4>, NCP, 16>(M, &k);
+    front_try<FrontTiles<1, 1, 7>, NCP, 16>(M, &k);
+    front_try<FrontTiles<1, 1, 10>, NCP, 14>(M, &k);
+    front_try<FrontTiles<1, 1, 13>, NCP, 12>(M, &k);
+    front_try<FrontTiles<1, 1, 14>, NCP, 8>(M, &k);
+    front_try<FrontTiles<1, 1, 16>, NCP, 8>(M, &k);
+    front_try<FrontTiles<4, 1, 5>, NCP, 4>(M, &k);
+    front_try<FrontTiles<4, 1, 7>, NCP, 2>(M, &k);
+    front_try<FrontTiles<4, 2, 9>, NCP, 1>(M, &k);
+    front_try<FrontTiles<4, 4, 12>, NCP, 1>(M, &k);
+    return k;
+}
+FrontKernel front_kernel(const mhm_mesh* mesh, const Level& lv) {
+    if (lv.fsteps == 0) return {};
+    const int M = (int)mesh->NI + 1 + lv.fslots;
+    return lv.fncp == 8 ? front_kernel_of<8>(M) : front_kernel_of<16>(M);
+}
+
 }  // namespace
 
 int fp64_window_rows(const mhm_mesh* mesh, const Level& lv) {
@@ -398,13 +605,12 @@ int fp64_window_rows(const mhm_mesh* mesh, const Level& lv) {
 
 namespace {
 
-// Window of a level: rows, leading dimension (even: 16-byte rows), shared memory, and
-// whether it lives in global memory (more rows than the register panel holds, or more
-// than the shared memory).
+// A level's frontal kernel, and for the levels without one the window in global memory:
+// rows, leading dimension (even: 16-byte rows), shared memory of the panel.
 struct Fp64Shape {
     int rows, ld, R;
     size_t smem, win_doubles;
-    bool wide;
+    FrontKernel front;   // no kernel: window in global memory
 };
 
 Fp64Shape fp64_shape(const mhm_mesh* mesh, const Level& lv) {
@@ -413,10 +619,9 @@ Fp64Shape fp64_shape(const mhm_mesh* mesh, const Level& lv) {
     sh.rows = fp64_window_rows(mesh, lv);
     sh.ld = sh.rows + sh.R;
     if (sh.ld % 2 == 1) sh.ld += 1;
-    sh.smem = ((size_t)sh.rows * sh.ld + (size_t)sh.R * sh.R) * sizeof(double);
-    sh.wide = sh.rows > 128 || sh.smem > 220 * 1024;
     sh.win_doubles = ((size_t)sh.rows * sh.ld + 31) & ~(size_t)31;   // 256-byte slots
-    if (sh.wide) sh.smem = wide_smem_bytes(sh.rows, sh.R);
+    sh.smem = wide_smem_bytes(sh.rows, sh.R);
+    sh.front = front_kernel(mesh, lv);
     return sh;
 }
 
@@ -431,19 +636,19 @@ int sm_count(const mhm_mesh* mesh) {
 size_t fp64_level_workspace(const mhm_mesh* mesh, const Level& lv) {
     if (mesh->device < 0) return 0;
     const Fp64Shape sh = fp64_shape(mesh, lv);
-    if (!sh.wide) return 0;
+    if (sh.front.kern) return 0;
     const int64_t slots = std::min<int64_t>(sm_count(mesh), std::max<int64_t>(lv.nK, 1));
     return (size_t)slots * sh.win_doubles * sizeof(double);
 }
 
 size_t fp64_slot_bytes(const mhm_mesh* mesh, const Level& lv) {
     const Fp64Shape sh = fp64_shape(mesh, lv);
-    return sh.wide ? sh.win_doubles * sizeof(double) : 0;
+    return sh.front.kern ? 0 : sh.win_doubles * sizeof(double);
 }
 
 bool fp64_level_launchable(const mhm_mesh* mesh, const Level& lv) {
     const Fp64Shape sh = fp64_shape(mesh, lv);
-    return sh.smem <= 220 * 1024 && sh.R <= 64;
+    return (sh.front.kern || sh.smem <= 220 * 1024) && sh.R <= 64;
 }
 
 static mhm_status launch_fp64(const mhm_mesh* mesh, const Level& lv, const double* kappa, const mhm_source& f,
@@ -480,16 +685,31 @@ static mhm_status launch_fp64(const mhm_mesh* mesh, const Level& lv, const doubl
     g.AK = AK; g.EK = EK; g.BK = BK; g.FK = FK;
     g.status = status;
     g.iters = iters;
-    if (sh.smem > 220 * 1024)
+    if (!sh.front.kern && sh.smem > 220 * 1024)
         return fail(MHM_ERR_UNSUPPORTED, "mhm_local_solve_batch: FP64 window panel exceeds shared memory (r too large)");
     if (g.R > 64)
         return fail(MHM_ERR_UNSUPPORTED, "mhm_local_solve_batch: FP64 path takes at most 64 right-hand sides");
     const int64_t nblk = K1 - K0;
     if (nblk <= 0) return MHM_OK;
-    void (*kern)(const Fp64Args);
+    void (*kern)(const Fp64Args) = sh.front.kern;
     int64_t grid = nblk;
-    int threads = kThreads;
-    if (sh.wide) {
+    int threads = sh.front.threads;
+    size_t smem = sh.smem;
+    if (kern) {
+        g.ev = lv.d_fev;
+        g.cp = lv.d_fcp;
+        g.steps = lv.fsteps;
+        smem = (size_t)front_smem(sh.front.vec, g.R, f.kind, g.P, g.N).total * sizeof(double);
+        // one wave of blocks, as many per SM as share the elements out evenly: left to the
+        // block scheduler, an SM that finishes early takes a whole second wave (2048 elements
+        // of P1 r = 5: 4.6 ms with 12 + 12 elements on some SMs where 14 are due)
+        int per_sm = 0;
+        MHM_CUDA_TRY(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
+        MHM_CUDA_TRY(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kern, threads, smem));
+        const int64_t sms = sm_count(mesh), each = (nblk + sms - 1) / sms;
+        const int64_t rounds = (each + std::max(per_sm, 1) - 1) / std::max(per_sm, 1);
+        grid = std::min(nblk, sms * ((each + rounds - 1) / rounds));
+    } else {
         // persistent grid: one block per SM and workspace slot
         const int64_t fit = ws ? (int64_t)(ws_bytes / (sh.win_doubles * sizeof(double))) : 0;
         grid = std::min<int64_t>(std::min<int64_t>(sm_count(mesh), fit), nblk);
@@ -499,15 +719,12 @@ static mhm_status launch_fp64(const mhm_mesh* mesh, const Level& lv, const doubl
         if (reinterpret_cast<uintptr_t>(ws) % 16 != 0)
             return fail(MHM_ERR_INVALID_ARG, "mhm_local_solve_batch: workspace must be 16-byte aligned");
         g.win = static_cast<double*>(ws);
-        kern = k_local_fp64<4, true>;
+        kern = k_local_fp64_wide;
         threads = kThreadsWide;
-    } else {
-        // register shape of the warp panel: window rows per lane
-        kern = sh.rows <= 64 ? k_local_fp64<2, false> : k_local_fp64<4, false>;
     }
-    MHM_CUDA_TRY(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sh.smem));
+    MHM_CUDA_TRY(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
     timing_mark(mesh, MHM_KERNEL_LOCAL_FP64, stream, true);
-    kern<<<(unsigned)grid, threads, sh.smem, stream>>>(g);
+    kern<<<(unsigned)grid, threads, smem, stream>>>(g);
     timing_mark(mesh, MHM_KERNEL_LOCAL_FP64, stream, false);
     MHM_CUDA_TRY(cudaGetLastError());
     return MHM_OK;

@@ -7,6 +7,7 @@
 #include <map>
 #include <utility>
 
+#include "front_plan.h"
 #include "mhm_internal.h"
 
 namespace {
@@ -94,6 +95,10 @@ void free_mesh_device(mhm_mesh* m) {
         if (lv.d_btab) cudaFree(lv.d_btab);
         lv.d_K = nullptr;
         lv.d_btab = nullptr;
+        if (lv.d_fev) cudaFree(lv.d_fev);
+        if (lv.d_fcp) cudaFree(lv.d_fcp);
+        lv.d_fev = nullptr;
+        lv.d_fcp = nullptr;
         if (lv.fstream) cudaStreamDestroy(lv.fstream);
         for (cudaEvent_t e : {lv.fstart, lv.fdone[0], lv.fdone[1], lv.mdone[0], lv.mdone[1]})
             if (e) cudaEventDestroy(e);
@@ -479,6 +484,14 @@ extern "C" mhm_status mhm_create_mesh(const mhm_mesh_desc* desc, int32_t device,
             if (!st) st = upload(lv.K, &lv.d_K);
             if (!st) st = upload(lv.btab, &lv.d_btab);
         }
+    }
+    for (mhm::Level& lv : m->levels) {
+        const mhm::FrontPlan plan = mhm::front_plan_2d(d.degree, lv.N);
+        lv.fsteps = plan.steps;
+        lv.fslots = plan.slots;
+        lv.fncp = plan.ncp;
+        if (!st) st = upload(plan.ev, (int32_t**)&lv.d_fev);
+        if (!st) st = upload(plan.cp, (uint32_t**)&lv.d_fcp);
     }
     if (st) {
         free_mesh_device(m);

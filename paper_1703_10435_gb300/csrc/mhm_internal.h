@@ -84,6 +84,10 @@ struct Level {
     std::vector<double> btab;      // face-load table of this level (dofs_per_face x (PN + 1))
     int32_t* d_K = nullptr;
     double* d_btab = nullptr;      // NULL: the mesh's table (uniform mesh)
+    // step tables of the frontal elimination (front_plan.h); fsteps 0: front too large
+    int fsteps = 0, fslots = 0, fncp = 0;
+    int4* d_fev = nullptr;
+    uint2* d_fcp = nullptr;
     // mixed path, several chunks: the factor launches run on their own stream, one chunk
     // ahead of the solve launches (created on first use)
     mutable Tuning tune;

@@ -1,0 +1,64 @@
+"""The FP64 frontal elimination at the sizes where its layout changes: the bordered matrix has
+M = R + slots rows (R = 3 m (l + 1) + 1 loads; P1: 2^r + 1 slots, P2: 2 2^r + 3), handled in
+4-row tiles by one warp up to M = 64 and by 4, 8 or 16 warps above, and by a window in global
+memory beyond (P2 r = 7).  Both elements of a one-square mesh, sin sin source (its loads by
+the addition theorem), against the oracle entry by entry."""
+import numpy as np
+import pytest
+
+torch = pytest.importorskip("torch")
+
+from oracle.local import solve_local
+from oracle.mesh import build_mesh
+from oracle.run import source_fn
+from paper_1703_10435_gb300 import mhm, workloads as W
+from tests._blocks import assert_blocks
+
+pytestmark = pytest.mark.gpu
+
+
+@pytest.fixture(scope="module", autouse=True)
+def built():
+    if not torch.cuda.is_available():
+        pytest.skip("no CUDA device")
+    from paper_1703_10435_gb300 import build
+    build.build()
+
+
+# (P, r, m, l): M and the warps that share it
+CASES = [(1, 0, 1, 0),    # 7, one warp, 4 rows of tiles
+         (1, 3, 2, 0),    # 16: the last size of 4 rows of tiles
+         (1, 3, 3, 0),    # 19
+         (1, 4, 2, 1),    # 30, not a multiple of 4
+         (1, 5, 2, 0),    # 40: the last of 10
+         (2, 4, 1, 1),    # 42
+         (1, 5, 3, 1),    # 52: the last of 13
+         (1, 5, 7, 0),    # 55
+         (1, 5, 10, 0),   # 64: the last for one warp
+         (1, 5, 11, 0),   # 67: four warps
+         (1, 5, 16, 0),   # 82
+         (2, 5, 1, 3),    # 80: the last of 5 rows of blocks, P2
+         (1, 6, 1, 3),    # 78
+         (1, 6, 8, 1),    # 114: eight warps
+         (1, 7, 1, 3),    # 142
+         (1, 7, 1, 4),    # 145: sixteen warps
+         (2, 6, 1, 4),    # 147
+         (2, 7, 1, 0)]    # no frontal kernel: the window in global memory
+
+
+@pytest.mark.parametrize("P,r,m,l", CASES)
+def test_blocks_vs_oracle_at_layout_edges(P, r, m, l):
+    from paper_1703_10435_gb300.pipeline import Pipeline
+    w = W.Workload("t", 1, 1, r, P, m, l, "log_uniform", "sinsin", 1.0, 1.0, seed=3)
+    kap = W.kappa_for(w) ** 0.25   # contrast 10
+    p = Pipeline.for_workload(w, 0, mhm.MHM_FP64)
+    p.local(torch.as_tensor(kap, device="cuda"), mhm.Source(mhm.MHM_SRC_SINSIN, 1.0, 1.0))
+    torch.cuda.synchronize()
+    assert int(p.status.abs().sum()) == 0 and p.iters.cpu().tolist() == [1, 1]
+    AK, EK, BK, FK = p.blocks()
+    mesh = build_mesh(1, 1, m, l)
+    n = (P * 2 ** r + 1) * (P * 2 ** r + 2) // 2
+    # 10 u cond; the P1 / P2 stiffness on n points has cond of about 12 n times the contrast
+    tol = max(1e-10, 10 * 1.1e-16 * 12 * n * 10)
+    for K in range(2):
+        assert_blocks(AK[K], EK[K], BK[K], FK[K], solve_local(mesh, K, r, P, kap[K], source_fn("sinsin", 1.0, 1.0)), tol, K)
