@@ -23,6 +23,7 @@
 #include <string>
 
 #include "local_common.cuh"
+#include "source_loads.cuh"
 
 namespace mhm {
 
@@ -115,33 +116,6 @@ __device__ __forceinline__ void fine_xy(const MCtx& c, int N, bool up, int i, in
         X[v][0] = c.X[0][0] + a[v][0] * e1x + a[v][1] * e2x;
         X[v][1] = c.X[0][1] + a[v][0] * e1y + a[v][1] * e2y;
     }
-}
-
-__device__ double cell_src(const MixedArgs& g, const double X[3][2], int P, int a, const double* fq) {
-    const double* gx = g.dm.gauss_x + 3 * kMaxGauss;
-    const double* gw = g.dm.gauss_w + 3 * kMaxGauss;
-    const double adet = fabs((X[1][0] - X[0][0]) * (X[2][1] - X[0][1]) - (X[2][0] - X[0][0]) * (X[1][1] - X[0][1]));
-    double s = 0.0;
-    for (int i = 0; i < 4; ++i)
-        for (int j = 0; j < 4; ++j) {
-            const double xi = gx[i], eta = gx[j] * (1.0 - gx[i]), w = gw[i] * gw[j] * (1.0 - gx[i]);
-            const double x = X[0][0] + xi * (X[1][0] - X[0][0]) + eta * (X[2][0] - X[0][0]);
-            const double y = X[0][1] + xi * (X[1][1] - X[0][1]) + eta * (X[2][1] - X[0][1]);
-            double phi = 1.0;
-            if (a >= 0) {
-                const double l0 = 1.0 - xi - eta, l1 = xi, l2 = eta;
-                if (P == 1) phi = a == 0 ? l0 : (a == 1 ? l1 : l2);
-                else {
-                    const double lam[3] = {l0, l1, l2};
-                    if (a < 3) phi = lam[a] * (2.0 * lam[a] - 1.0);
-                    else if (a == 3) phi = 4.0 * l1 * l2;
-                    else if (a == 4) phi = 4.0 * l2 * l0;
-                    else phi = 4.0 * l0 * l1;
-                }
-            }
-            s += w * adet * source_at(g.src_kind, g.src_value, g.src_freq, x, y, fq, 4 * i + j) * phi;
-        }
-    return s;
 }
 
 // Fine triangles incident to lattice point (X, Y) and the point's local index in
@@ -1367,6 +1341,7 @@ __device__ __forceinline__ void mixed_blocks(const MixedArgs& g) {
     float* opbuf = W;                                                   // nbuf x opmax staging (solves only)
     float* stage = W + (size_t)(SCHUR ? g.nbuf : 2) * g.opmax;          // staged solve operand(s) (solves only)
     float* cw = reinterpret_cast<float*>(smem_raw + g.off_cw);          // level-Schur path: 4 x nunk couplings
+    double* sload = reinterpret_cast<double*>(y);                       // source load per node (set-up only)
     __shared__ MCtx c;
     const LevelGeom lg{g.P, g.N, g.PN};
     const int R = g.R;
@@ -1454,15 +1429,18 @@ __device__ __forceinline__ void mixed_blocks(const MixedArgs& g) {
         if (g.src_kind == MHM_SRC_CONST) {
             if (threadIdx.x == 0) c.FK = g.src_value * c.area;
         } else {
+            // the source's load at every node (the pinned DOF 0 first) in y, which the solves
+            // overwrite after the right-hand sides have taken it; its tables in the window
+            double* tab = reinterpret_cast<double*>(W);
+            source_tables(g.dm, g.src_kind, g.src_value, g.src_freq, g.P, g.N, c.X, tab, threadIdx.x, blockDim.x);
+            __syncthreads();
+            const double* vals = g.src_vals ? g.src_vals + 16 * (kap - g.kappa) : nullptr;
             double s = 0.0;
-            for (int t = threadIdx.x; t < g.N * g.N; t += blockDim.x) {
-                int j = 0, rs = 0;
-                while (rs + 2 * (g.N - j) - 1 <= t) { rs += 2 * (g.N - j) - 1; ++j; }
-                const int o = t - rs;
-                const bool up = o < g.N - j;
-                double X[3][2];
-                fine_xy(c, g.N, up, up ? o : o - (g.N - j), j, X);
-                s += cell_src(g, X, g.P, -1, quad_of(g.src_vals, g.kappa, kap, g.N, up, up ? o : o - (g.N - j), j));
+            for (int u = threadIdx.x; u <= g.nunk; u += blockDim.x) {
+                int X = 0, Y = 0;
+                if (u > 0) lattice_of_unk(g.PN, u - 1, &X, &Y);
+                sload[u] = source_node(g.src_kind, g.P, g.N, X, Y, tab, vals);
+                s += sload[u];
             }
             for (int o = 16; o > 0; o >>= 1) s += __shfl_down_sync(0xffffffffu, s, o);
             if ((threadIdx.x & 31) == 0) c.red[threadIdx.x >> 5] = s;
@@ -1563,12 +1541,8 @@ __device__ __forceinline__ void mixed_blocks(const MixedArgs& g) {
                     const double mt = c.area_fine * element_mass_frac(1, ta[t]);
                     m += mt;
                     if (g.src_kind == MHM_SRC_CONST) fh += g.src_value * mt;
-                    else {
-                        double Xv[3][2];
-                        fine_xy(c, g.N, tup[t], ti[t], tj[t], Xv);
-                        fh += cell_src(g, Xv, 1, ta[t], quad_of(g.src_vals, g.kappa, kap, g.N, tup[t], ti[t], tj[t]));
-                    }
                 }
+                if (g.src_kind != MHM_SRC_CONST) fh = sload[u + 1];
                 const double su = sc[u];
                 smass[u] = su * m;
                 for (int col = 0; col < R; ++col) {
@@ -1764,12 +1738,8 @@ __device__ __forceinline__ void mixed_blocks(const MixedArgs& g) {
                     m += mt;
                     diag += kap[kap_index(g.N, tup[t], ti[t], tj[t])] * (tup[t] ? c.Sup : c.Sdn)[ta[t] * nb + ta[t]];
                     if (g.src_kind == MHM_SRC_CONST) fh += g.src_value * mt;
-                    else {
-                        double Xv[3][2];
-                        fine_xy(c, g.N, tup[t], ti[t], tj[t], Xv);
-                        fh += cell_src(g, Xv, g.P, ta[t], quad_of(g.src_vals, g.kappa, kap, g.N, tup[t], ti[t], tj[t]));
-                    }
                 }
+                if (g.src_kind != MHM_SRC_CONST) fh = sload[u + 1];
                 mass[u] = m;
                 scale[u] = 1.0 / sqrt(diag);
                 for (int col = 0; col < R; ++col) {
@@ -2563,6 +2533,8 @@ MixedLayout mixed_layout(const mhm_mesh* mesh, const Level& lv, bool split = tru
         if (win < (size_t)2 * L.opmax + (size_t)2 * L.stage_floats && L.mode != 3)
             win = (size_t)2 * L.opmax + (size_t)2 * L.stage_floats;
     }
+    // the source's tables (set-up only)
+    for (int kind : {MHM_SRC_SINSIN, MHM_SRC_QUAD}) win = std::max(win, (size_t)2 * source_table_doubles(kind, lv.PN));
     win = (win + 3) & ~(size_t)3;
     L.wfloats = (int)win;
     size_t yf = (size_t)L.nunk * L.Rp;

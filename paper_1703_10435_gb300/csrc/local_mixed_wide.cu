@@ -36,6 +36,7 @@
 #include <string>
 
 #include "local_common.cuh"
+#include "source_loads.cuh"
 #include "mixed_wide.h"
 
 namespace mhm {
@@ -168,42 +169,6 @@ __device__ __forceinline__ void fine_tri_vertices(const WCtx& c, int N, bool up,
         X[v][0] = c.X[0][0] + a[v][0] * e1x + a[v][1] * e2x;
         X[v][1] = c.X[0][1] + a[v][0] * e1y + a[v][1] * e2y;
     }
-}
-
-// int_T f lambda_a (a = -1: int_T f) over a fine triangle by the collapsed 4 x 4 Gauss rule.
-__device__ double tri_source(const WideArgs& g, const double X[3][2], int a, const double* fq) {
-    const double* gx = g.dm.gauss_x + 3 * kMaxGauss;
-    const double* gw = g.dm.gauss_w + 3 * kMaxGauss;
-    const double adet = fabs((X[1][0] - X[0][0]) * (X[2][1] - X[0][1]) - (X[2][0] - X[0][0]) * (X[1][1] - X[0][1]));
-    double s = 0.0;
-    for (int i = 0; i < 4; ++i)
-        for (int j = 0; j < 4; ++j) {
-            const double xi = gx[i], eta = gx[j] * (1.0 - gx[i]), w = gw[i] * gw[j] * (1.0 - gx[i]);
-            const double x = X[0][0] + xi * (X[1][0] - X[0][0]) + eta * (X[2][0] - X[0][0]);
-            const double y = X[0][1] + xi * (X[1][1] - X[0][1]) + eta * (X[2][1] - X[0][1]);
-            const double phi = a < 0 ? 1.0 : (a == 0 ? 1.0 - xi - eta : (a == 1 ? xi : eta));
-            s += w * adet * source_at(g.src_kind, g.src_value, g.src_freq, x, y, fq, 4 * i + j) * phi;
-        }
-    return s;
-}
-
-// (f, phi_w)_K of a source that is not constant: the cell integrals of the fine triangles
-// around vertex (x, y), each with the vertex's own barycentric weight.
-__device__ double vertex_source(const WideArgs& g, const WCtx& c, const double* kap, int x, int y) {
-    const int N = g.N;
-    double s = 0.0;
-    double X[3][2];
-    auto add = [&](bool up, int i, int j, int a) {
-        fine_tri_vertices(c, N, up, i, j, X);
-        s += tri_source(g, X, a, quad_of(g.src_vals, g.kappa, kap, N, up, i, j));
-    };
-    if (up_ok(N, x, y)) add(true, x, y, 0);
-    if (up_ok(N, x - 1, y)) add(true, x - 1, y, 1);
-    if (up_ok(N, x, y - 1)) add(true, x, y - 1, 2);
-    if (dn_ok(N, x - 1, y - 1)) add(false, x - 1, y - 1, 1);
-    if (dn_ok(N, x - 1, y)) add(false, x - 1, y, 0);
-    if (dn_ok(N, x, y - 1)) add(false, x, y - 1, 2);
-    return s;
 }
 
 // Sum over the block of up to kRp per-thread column values; out[c] for c < kRp (all
@@ -383,18 +348,18 @@ __global__ void __launch_bounds__(2 * BMAX, BMAX == 128 ? 2 : 4) k_local_mixed_w
             double acc[kRp];
 #pragma unroll
             for (int col = 0; col < kRp; ++col) acc[col] = 0.0;
-            for (int t = tid; t < N * N; t += NT) {
-                // fine triangle t in kappa order: row j starts at j (2N - j)
-                int j = (int)((double)N - sqrt((double)N * N - (double)t));
-                while (j > 0 && j * (2 * N - j) > t) --j;
-                while ((j + 1) * (2 * N - j - 1) <= t) ++j;
-                const int o = t - j * (2 * N - j);
-                const bool up = o < N - j;
-                const int ii = up ? o : o - (N - j);
-                double Xt[3][2];
-                fine_tri_vertices(c, N, up, ii, j, Xt);
-                acc[0] += tri_source(g, Xt, -1, quad_of(g.src_vals, g.kappa, kap, N, up, ii, j));
+            // the source's load per unknown in Q (free until the iteration), its tables in Tp
+            double* tab = reinterpret_cast<double*>(Tp);
+            source_tables(g.dm, g.src_kind, g.src_value, g.src_freq, 1, N, c.X, tab, tid, NT);
+            __syncthreads();
+            const double* vals = g.src_vals ? g.src_vals + 16 * (kap - g.kappa) : nullptr;
+            for (int u = tid; u < n; u += NT) {
+                int x, y;
+                node_of(c, lg, u, &x, &y);
+                Qv[u] = source_node(g.src_kind, 1, N, x, y, tab, vals);
+                acc[0] += Qv[u];
             }
+            if (tid == 0) acc[0] += source_node(g.src_kind, 1, N, c.pin_x, c.pin_y, tab, vals);
             block_sum_cols<NT>(acc, red, c.red);
             FK = c.red[0];
         }
@@ -435,7 +400,7 @@ __global__ void __launch_bounds__(2 * BMAX, BMAX == 128 ? 2 : 4) k_local_mixed_w
             q.w = (float)(su * w[kSelf] * su);
             cw[u] = q;
             const double m = vertex_mass(N, x, y, c.area_fine);
-            const double fsrc = g.src_kind == MHM_SRC_CONST ? g.src_value * m : vertex_source(g, c, kap, x, y);
+            const double fsrc = g.src_kind == MHM_SRC_CONST ? g.src_value * m : Qv[u];
             for (int col = 0; col < R; ++col) {
                 double val = -c.cproj[col] * m;
                 if (col == g.NI) {
