@@ -1,0 +1,100 @@
+// Set-up of one coarse triangle for the frontal kernels (local_fp64.cu, reconstruct.cu).
+#pragma once
+
+#include "front.cuh"
+#include "local_common.cuh"
+#include "source_loads.cuh"
+
+namespace mhm {
+
+struct FrontCtx {
+    double X[3][2];
+    double area, flen[3], FK;
+    int sgn[3], rev[3], la1[3], bad, pin;   // pin: lattice point x | y << 16
+};
+
+// choose_pin by one warp (kappa > 0 orders like its bits): x | y << 16.
+__device__ inline int choose_pin_warp(int P, int N, const double* kap) {
+    const int lane = threadIdx.x & 31, PN = P * N;
+    const int ymax = N == 1 ? (P == 1 ? 0 : 1) : (P == 1 ? 1 : 3), jmax = N == 1 ? 1 : 2;
+    long long best = -1;
+    for (int j = 0; j < jmax; ++j)
+        for (int t = lane; t < 2 * (N - j) - 1; t += 32) {
+            const long long k = __double_as_longlong(kap[j * (2 * N - j) + t]);
+            best = k > best ? k : best;
+        }
+    for (int o = 16; o > 0; o >>= 1) {
+        const long long k = __shfl_xor_sync(0xffffffffu, best, o);
+        best = k > best ? k : best;
+    }
+    int bd = 1 << 30;
+    for (int j = 0; j < jmax; ++j)
+        for (int t = lane; t < 2 * (N - j) - 1; t += 32) {
+            if (__double_as_longlong(kap[j * (2 * N - j) + t]) != best) continue;
+            int nx[6], ny[6];
+            element_nodes(P, t < N - j, t < N - j ? t : t - (N - j), j, nx, ny);
+            for (int a = 0; a < (P == 1 ? 3 : 6); ++a)
+                if (ny[a] <= ymax) bd = min(bd, ny[a] * (PN + 1) - ny[a] * (ny[a] - 1) / 2 + nx[a]);
+        }
+    bd = __reduce_min_sync(0xffffffffu, bd);
+    int y = 0;
+    while (bd >= PN + 1 - y) bd -= PN + 1 - y, ++y;
+    return (bd & 0xffff) | y << 16;
+}
+
+// Geometry, pin, element matrices (Ke, 72), mass of a node on k fine triangles (mass, 8) and
+// source tables of element K; all threads of the block, ends with a barrier.
+__device__ __forceinline__ void front_element(const DeviceMesh& dm, int64_t K, const double* kap, int P, int N,
+                                              int src_kind, double src_value, double src_freq, FrontCtx& c,
+                                              double* Ke, double* mass, double* tab) {
+    const int tid = threadIdx.x, nthr = blockDim.x;
+    if (tid < 6) c.X[tid >> 1][tid & 1] = dm.geom[6 * K + tid];
+    if (tid < 3) {
+        c.sgn[tid] = dm.sign[3 * K + tid];
+        c.rev[tid] = dm.rev[3 * K + tid];
+        c.la1[tid] = face_la1(dm, K, tid);
+    }
+    if (tid < 32) {
+        const int pin = choose_pin_warp(P, N, kap);
+        if (tid == 0) c.pin = pin, c.bad = 0;
+    }
+    __syncthreads();
+    if (tid < 3) {
+        const double* P0 = c.X[(tid + 1) % 3];
+        const double* Q0 = c.X[(tid + 2) % 3];
+        c.flen[tid] = sqrt((Q0[0] - P0[0]) * (Q0[0] - P0[0]) + (Q0[1] - P0[1]) * (Q0[1] - P0[1]));
+    }
+    const double area = 0.5 * fabs((c.X[1][0] - c.X[0][0]) * (c.X[2][1] - c.X[0][1]) -
+                                   (c.X[2][0] - c.X[0][0]) * (c.X[1][1] - c.X[0][1]));
+    if (tid == 0) c.area = area;
+    if (tid < 8) mass[tid] = tid * (area / ((double)N * N) / 3.0);
+    element_stiffness_pair(P, N, c.X, Ke, tid, nthr);
+    source_tables(dm, src_kind, src_value, src_freq, P, N, c.X, tab, tid, nthr);
+    __syncthreads();
+}
+
+// Source loads of all nodes to src (dof order) and their sum F_K to c.FK (a constant source:
+// c.FK alone); ends with a barrier.
+__device__ __forceinline__ void front_source(int kind, double value, int P, int N, const double* tab,
+                                             const double* vals, FrontCtx& c, double* src) {
+    const int tid = threadIdx.x, nthr = blockDim.x, PN = P * N, n = (PN + 1) * (PN + 2) / 2;
+    if (kind == MHM_SRC_CONST) {
+        if (tid == 0) c.FK = value * c.area;
+    } else {
+        int x = tid, y = 0;
+        for (int u = tid; u < n; u += nthr, x += nthr) {
+            while (x > PN - y) x -= PN + 1 - y, ++y;
+            src[u] = source_node(kind, P, N, x, y, tab, vals);
+        }
+        __syncthreads();
+        if (tid < 32) {
+            double s = 0.0;
+            for (int u = tid; u < n; u += 32) s += src[u];
+            for (int o = 16; o > 0; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
+            if (tid == 0) c.FK = s;
+        }
+    }
+    __syncthreads();
+}
+
+}  // namespace mhm

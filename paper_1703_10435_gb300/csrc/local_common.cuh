@@ -207,6 +207,25 @@ __device__ __forceinline__ double element_mass_frac(int P, int a) {
     return (P == 1 || a >= 3) ? (1.0 / 3.0) : 0.0;
 }
 
+// Mass m_w = int_K phi_w of lattice point (x, y) of the (P N)-lattice: a third of the fine
+// triangles around a P1 vertex; for P2 a third of the (one or two) triangles sharing an edge
+// midpoint, zero at a vertex.
+__device__ __forceinline__ double node_mass(int P, int N, int x, int y, double area_fine) {
+    auto up_ok = [&](int i, int j) { return i >= 0 && j >= 0 && i + j <= N - 1; };
+    auto dn_ok = [&](int i, int j) { return i >= 0 && j >= 0 && i + j <= N - 2; };
+    int n = 0;
+    if (P == 1) {
+        n = up_ok(x, y) + up_ok(x - 1, y) + up_ok(x, y - 1) + dn_ok(x - 1, y - 1) + dn_ok(x - 1, y) + dn_ok(x, y - 1);
+    } else if ((x & 1) && !(y & 1)) {          // horizontal edge midpoint
+        n = up_ok((x - 1) >> 1, y >> 1) + dn_ok((x - 1) >> 1, (y >> 1) - 1);
+    } else if (!(x & 1) && (y & 1)) {          // vertical edge midpoint
+        n = up_ok(x >> 1, (y - 1) >> 1) + dn_ok((x >> 1) - 1, (y - 1) >> 1);
+    } else if ((x & 1) && (y & 1)) {           // diagonal edge midpoint
+        n = up_ok((x - 1) >> 1, (y - 1) >> 1) + dn_ok((x - 1) >> 1, (y - 1) >> 1);
+    }
+    return n * (area_fine / 3.0);
+}
+
 __device__ __forceinline__ double source_value(int kind, double value, double freq, double x, double y) {
     if (kind == MHM_SRC_CONST) return value;
     const double c = 2.0 * (freq * M_PI) * (freq * M_PI) * value;

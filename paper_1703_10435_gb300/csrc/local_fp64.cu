@@ -23,10 +23,9 @@
 // grid, and factors it panel by panel through shared memory (wide_cholesky_level).
 #include <cuda_runtime.h>
 
-#include "front.cuh"
+#include "front2d.cuh"
 #include "local_common.cuh"
 #include "mixed_wide.h"
-#include "source_loads.cuh"
 
 namespace mhm {
 
@@ -129,25 +128,6 @@ __device__ __forceinline__ void fine_vertices(const KCtx& c, int N, bool up, int
         X[v][0] = c.X[0][0] + a[v][0] * e1x + a[v][1] * e2x;
         X[v][1] = c.X[0][1] + a[v][0] * e1y + a[v][1] * e2y;
     }
-}
-
-// Mass m_w = int_K phi_w of lattice point (x, y) of the (P N)-lattice: a third of the fine
-// triangles around a P1 vertex; for P2 a third of the (one or two) triangles sharing an edge
-// midpoint, zero at a vertex.
-__device__ __forceinline__ double node_mass(int P, int N, int x, int y, double area_fine) {
-    auto up_ok = [&](int i, int j) { return i >= 0 && j >= 0 && i + j <= N - 1; };
-    auto dn_ok = [&](int i, int j) { return i >= 0 && j >= 0 && i + j <= N - 2; };
-    int n = 0;
-    if (P == 1) {
-        n = up_ok(x, y) + up_ok(x - 1, y) + up_ok(x, y - 1) + dn_ok(x - 1, y - 1) + dn_ok(x - 1, y) + dn_ok(x, y - 1);
-    } else if ((x & 1) && !(y & 1)) {          // horizontal edge midpoint
-        n = up_ok((x - 1) >> 1, y >> 1) + dn_ok((x - 1) >> 1, (y >> 1) - 1);
-    } else if (!(x & 1) && (y & 1)) {          // vertical edge midpoint
-        n = up_ok(x >> 1, (y - 1) >> 1) + dn_ok((x >> 1) - 1, (y - 1) >> 1);
-    } else if ((x & 1) && (y & 1)) {           // diagonal edge midpoint
-        n = up_ok((x - 1) >> 1, (y - 1) >> 1) + dn_ok((x - 1) >> 1, (y - 1) >> 1);
-    }
-    return n * (area_fine / 3.0);
 }
 
 // Right-hand sides at the nodes of level lev (window rows row0 + p), once per node and
@@ -383,41 +363,6 @@ __host__ __device__ inline FrontSmem front_smem(int vec, int R, int kind, int P,
     return l;
 }
 
-struct FrontCtx {
-    double X[3][2];
-    double area, flen[3], FK;
-    int sgn[3], rev[3], la1[3], bad, pin;
-};
-
-// choose_pin by one warp (kappa > 0 orders like its bits): x | y << 16.
-__device__ inline int choose_pin_warp(int P, int N, const double* kap) {
-    const int lane = threadIdx.x & 31, PN = P * N;
-    const int ymax = N == 1 ? (P == 1 ? 0 : 1) : (P == 1 ? 1 : 3), jmax = N == 1 ? 1 : 2;
-    long long best = -1;
-    for (int j = 0; j < jmax; ++j)
-        for (int t = lane; t < 2 * (N - j) - 1; t += 32) {
-            const long long k = __double_as_longlong(kap[j * (2 * N - j) + t]);
-            best = k > best ? k : best;
-        }
-    for (int o = 16; o > 0; o >>= 1) {
-        const long long k = __shfl_xor_sync(0xffffffffu, best, o);
-        best = k > best ? k : best;
-    }
-    int bd = 1 << 30;
-    for (int j = 0; j < jmax; ++j)
-        for (int t = lane; t < 2 * (N - j) - 1; t += 32) {
-            if (__double_as_longlong(kap[j * (2 * N - j) + t]) != best) continue;
-            int nx[6], ny[6];
-            element_nodes(P, t < N - j, t < N - j ? t : t - (N - j), j, nx, ny);
-            for (int a = 0; a < (P == 1 ? 3 : 6); ++a)
-                if (ny[a] <= ymax) bd = min(bd, ny[a] * (PN + 1) - ny[a] * (ny[a] - 1) / 2 + nx[a]);
-        }
-    bd = __reduce_min_sync(0xffffffffu, bd);
-    int y = 0;
-    while (bd >= PN + 1 - y) bd -= PN + 1 - y, ++y;
-    return (bd & 0xffff) | y << 16;
-}
-
 // Loads of a node in the bordered matrix: the face load -(s psi_j, phi_w)_{dK}, the
 // projection -(1^T g / |K|) m_w, the source load.  Lane q holds columns q and q + 32.
 struct FrontLoad {
@@ -461,48 +406,9 @@ __global__ void __launch_bounds__(T::threads, MINB) k_local_fp64(const __grid_co
     const int64_t K = g.dm.klist ? (int64_t)g.dm.klist[ki] : ki;         // coarse element
     const double* kap = g.kappa + (g.dm.kap_off ? g.dm.kap_off[K] : K * (int64_t)N * N);
 
-    // ---- per-K setup
-    if (tid < 6) c.X[tid >> 1][tid & 1] = g.dm.geom[6 * K + tid];
-    if (tid < 3) {
-        c.sgn[tid] = g.dm.sign[3 * K + tid];
-        c.rev[tid] = g.dm.rev[3 * K + tid];
-        c.la1[tid] = face_la1(g.dm, K, tid);
-    }
-    if (tid < 32) {
-        const int pin = choose_pin_warp(P, N, kap);
-        if (tid == 0) c.pin = pin, c.bad = 0;
-    }
-    __syncthreads();
-    if (tid < 3) {
-        const double* P0 = c.X[(tid + 1) % 3];
-        const double* Q0 = c.X[(tid + 2) % 3];
-        c.flen[tid] = sqrt((Q0[0] - P0[0]) * (Q0[0] - P0[0]) + (Q0[1] - P0[1]) * (Q0[1] - P0[1]));
-    }
-    const double area = 0.5 * fabs((c.X[1][0] - c.X[0][0]) * (c.X[2][1] - c.X[0][1]) -
-                                   (c.X[2][0] - c.X[0][0]) * (c.X[1][1] - c.X[0][1]));
-    if (tid < 8) smem[L.mass + tid] = tid * (area / ((double)N * N) / 3.0);
-    element_stiffness_pair(P, N, c.X, Ke, tid, nthr);
-    source_tables(g.dm, g.src_kind, g.src_value, g.src_freq, P, N, c.X, tab, tid, nthr);
-    __syncthreads();
-    const double* vals = g.src_vals ? g.src_vals + 16 * (kap - g.kappa) : nullptr;
-    if (g.src_kind == MHM_SRC_CONST) {
-        if (tid == 0) c.FK = g.src_value * area;
-    } else {
-        const int n = (PN + 1) * (PN + 2) / 2;
-        int x = tid, y = 0;
-        for (int u = tid; u < n; u += nthr, x += nthr) {
-            while (x > PN - y) x -= PN + 1 - y, ++y;
-            src[u] = source_node(g.src_kind, P, N, x, y, tab, vals);
-        }
-        __syncthreads();
-        if (tid < 32) {
-            double s = 0.0;
-            for (int u = tid; u < n; u += 32) s += src[u];
-            for (int o = 16; o > 0; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
-            if (tid == 0) c.FK = s;
-        }
-    }
-    __syncthreads();
+    front_element(g.dm, K, kap, P, N, g.src_kind, g.src_value, g.src_freq, c, Ke, smem + L.mass, tab);
+    front_source(g.src_kind, g.src_value, P, N, tab, g.src_vals ? g.src_vals + 16 * (kap - g.kappa) : nullptr, c, src);
+    const double area = c.area;
     for (int col = tid; col < R; col += nthr) {
         if (col == NI) cproj[col] = c.FK / area;
         else {

@@ -96,7 +96,6 @@ void free_mesh_device(mhm_mesh* m) {
         lv.d_K = nullptr;
         lv.d_btab = nullptr;
         if (lv.d_fev) cudaFree(lv.d_fev);
-        if (lv.d_fcp) cudaFree(lv.d_fcp);
         lv.d_fev = nullptr;
         lv.d_fcp = nullptr;
         if (lv.fstream) cudaStreamDestroy(lv.fstream);
@@ -490,8 +489,10 @@ extern "C" mhm_status mhm_create_mesh(const mhm_mesh_desc* desc, int32_t device,
         lv.fsteps = plan.steps;
         lv.fslots = plan.slots;
         lv.fncp = plan.ncp;
-        if (!st) st = upload(plan.ev, (int32_t**)&lv.d_fev);
-        if (!st) st = upload(plan.cp, (uint32_t**)&lv.d_fcp);
+        std::vector<uint32_t> both(plan.ev.begin(), plan.ev.end());   // one allocation: steps, then couplings
+        both.insert(both.end(), plan.cp.begin(), plan.cp.end());
+        if (!st) st = upload(both, (uint32_t**)&lv.d_fev);
+        if (lv.d_fev) lv.d_fcp = reinterpret_cast<uint2*>(lv.d_fev + plan.steps);
     }
     if (st) {
         free_mesh_device(m);

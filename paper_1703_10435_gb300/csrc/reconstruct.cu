@@ -2,24 +2,27 @@
 // triangle K,  u_{H,h} = u0_K + sum_i k_i eta_i + eta_f.  By linearity this is
 // one zero-mean Neumann solve per K with the combined load
 //     g = sum_i k_i N~_i + f~      (k_i: global multipliers of K's local basis),
-// done here in FP64: the level-window Cholesky of the FP64 kernel with one
-// right-hand side, storing L_lev and L_{lev+1,lev} per level in scratch, then a
-// backward sweep by one warp.  Optional per-K squared L2 and broken-H1 errors
-// against an exact solution by the collapsed 4 x 4 Gauss rule per fine triangle.
-// Windows too large for shared memory (P1 r = 7, P2 r = 5) sit in the block's
-// scratch slot behind the stored factors and are factored panel by panel
-// (wide_cholesky_level).
+// done here in FP64: the frontal elimination of the FP64 local solves (front.cuh) with that
+// load as its one border row, which keeps every step's scaled pivot column w / d in scratch,
+// and a backward sweep over the steps by one warp, x_p = g_p / d - sum_j (w_j / d) x_j over
+// the front.  Optional per-K squared L2 and broken-H1 errors against an exact solution by the
+// collapsed 4 x 4 Gauss rule per fine triangle.
+// Levels whose front is too large (P2 r = 7) are refused.
+//
+// Bound by the FP64 pipe (81 % busy): 17.2 k FP64 warp instructions per element of P1 r = 5,
+// of which the update of the front takes 8 k, a step's fixed part (reciprocal, scaling,
+// couplings, the backward sum) the rest.  32768 elements: 33.3 ms (182.6 ms with a window
+// over two levels and a dense backward sweep).
 #include <cuda_runtime.h>
 
+#include <algorithm>
+
+#include "front2d.cuh"
 #include "local_common.cuh"
 
 namespace mhm {
 
 namespace {
-
-constexpr int kThreadsR = 128;
-constexpr int kThreadsRWide = 256;
-constexpr int kNBR = 16;   // wide window: pivots per panel
 
 struct RecArgs {
     DeviceMesh dm;
@@ -27,8 +30,7 @@ struct RecArgs {
     const double* lambda;
     const double* u0;
     const int32_t* k_lambda;    // n_K * N_I global multiplier ids
-    int P, N, PN, dpf, NI, nlev, nloc;
-    int rows, ld, rhs;          // window rows, leading dimension, right-hand-side column
+    int P, N, PN, dpf, NI, nloc;
     int src_kind;
     const double* src_vals;   // MHM_SRC_QUAD: 16 values per fine triangle, laid out like kappa
     double src_value, src_freq;
@@ -36,34 +38,24 @@ struct RecArgs {
     double ex[6];
     char* ws;
     size_t slot_bytes;
-    size_t win_offset;          // wide window: its byte offset in the slot (0: shared memory)
     int64_t nK;                 // launch indices of this level
     const int64_t* nod_off;     // first nodal value of each K in u_out (NULL: K * nloc)
     double* u_out;              // n_K * nloc (per-K levels: at nod_off)
     double* err_out;            // n_K * 2 (squared L2, squared H1 seminorm) or NULL
+    const int4* ev;             // frontal elimination: the level's step tables
+    const uint2* cp;
+    int steps, slots;
 };
 
-struct RCtx {
-    double X[3][2];
-    double Sup[36], Sdn[36];
-    double area, area_fine, FK, cl;
-    double flen[3];
-    int sgn[3], rev[3], la1[3];  // la1: degree + 1 of each face
-    int bad;
-    int pin_x, pin_y;            // the pinned lattice point (choose_pin)
-    double red[kThreadsRWide / 32];
-    double mz;
-};
-
-__device__ __forceinline__ void fine_xy(const RCtx& c, int N, bool up, int i, int j, double X[3][2]) {
-    const double e1x = (c.X[1][0] - c.X[0][0]) / N, e1y = (c.X[1][1] - c.X[0][1]) / N;
-    const double e2x = (c.X[2][0] - c.X[0][0]) / N, e2y = (c.X[2][1] - c.X[0][1]) / N;
+__device__ __forceinline__ void fine_xy(const double Xc[3][2], int N, bool up, int i, int j, double X[3][2]) {
+    const double e1x = (Xc[1][0] - Xc[0][0]) / N, e1y = (Xc[1][1] - Xc[0][1]) / N;
+    const double e2x = (Xc[2][0] - Xc[0][0]) / N, e2y = (Xc[2][1] - Xc[0][1]) / N;
     int a[3][2];
     if (up) { a[0][0] = i; a[0][1] = j; a[1][0] = i + 1; a[1][1] = j; a[2][0] = i; a[2][1] = j + 1; }
     else    { a[0][0] = i + 1; a[0][1] = j; a[1][0] = i + 1; a[1][1] = j + 1; a[2][0] = i; a[2][1] = j + 1; }
     for (int v = 0; v < 3; ++v) {
-        X[v][0] = c.X[0][0] + a[v][0] * e1x + a[v][1] * e2x;
-        X[v][1] = c.X[0][1] + a[v][0] * e1y + a[v][1] * e2y;
+        X[v][0] = Xc[0][0] + a[v][0] * e1x + a[v][1] * e2x;
+        X[v][1] = Xc[0][1] + a[v][0] * e1y + a[v][1] * e2y;
     }
 }
 
@@ -85,24 +77,6 @@ __device__ __forceinline__ void basis_eval(int P, double l0, double l1, double l
     dxi[5] = 4 * (l0 - l1); deta[5] = -4 * l1;
 }
 
-// Integral of f phi_a (a >= 0) or of f (a < 0) over a fine triangle, 4 x 4 collapsed Gauss.
-__device__ double cell_source(const RecArgs& g, const double X[3][2], int a, const double* fq) {
-    const double* gx = g.dm.gauss_x + 3 * kMaxGauss;
-    const double* gw = g.dm.gauss_w + 3 * kMaxGauss;
-    const double adet = fabs((X[1][0] - X[0][0]) * (X[2][1] - X[0][1]) - (X[2][0] - X[0][0]) * (X[1][1] - X[0][1]));
-    double s = 0.0;
-    for (int i = 0; i < 4; ++i)
-        for (int j = 0; j < 4; ++j) {
-            const double xi = gx[i], eta = gx[j] * (1.0 - gx[i]), w = gw[i] * gw[j] * (1.0 - gx[i]);
-            const double x = X[0][0] + xi * (X[1][0] - X[0][0]) + eta * (X[2][0] - X[0][0]);
-            const double y = X[0][1] + xi * (X[1][1] - X[0][1]) + eta * (X[2][1] - X[0][1]);
-            double phi[6], dx[6], dy[6];
-            basis_eval(g.P, 1.0 - xi - eta, xi, eta, phi, dx, dy);
-            s += w * adet * source_at(g.src_kind, g.src_value, g.src_freq, x, y, fq, 4 * i + j) * (a >= 0 ? phi[a] : 1.0);
-        }
-    return s;
-}
-
 __device__ void exact_eval(const RecArgs& g, double x, double y, double* u, double* ux, double* uy) {
     if (g.ex_kind == 1) {
         const double f = g.ex[0], amp = g.ex[1];
@@ -118,293 +92,221 @@ __device__ void exact_eval(const RecArgs& g, double x, double y, double* u, doub
     }
 }
 
-__device__ double block_sum(double v, RCtx& c) {
+__device__ double block_sum(double v, double* red) {
     for (int o = 16; o > 0; o >>= 1) v += __shfl_down_sync(0xffffffffu, v, o);
-    if ((threadIdx.x & 31) == 0) c.red[threadIdx.x >> 5] = v;
+    if ((threadIdx.x & 31) == 0) red[threadIdx.x >> 5] = v;
     __syncthreads();
     double s = 0.0;
-    for (int w = 0; w < (int)(blockDim.x >> 5); ++w) s += c.red[w];   // same order in every thread
+    for (int w = 0; w < (int)(blockDim.x >> 5); ++w) s += red[w];   // same order in every thread
     __syncthreads();
     return s;
 }
 
-template <bool WIDE>
-__global__ void __launch_bounds__(WIDE ? kThreadsRWide : kThreadsR) k_reconstruct(const RecArgs g) {
-    extern __shared__ double smem[];
-    __shared__ RCtx c;
-    const int rhs = g.rhs;
-    char* slot = g.ws + (size_t)blockIdx.x * g.slot_bytes;
-    double* Fst = reinterpret_cast<double*>(slot);   // per level: L (b x b), C (bn x b), y (b)
-    // window rows x ld (column rhs is the right-hand side): shared memory or the slot
-    double* W = WIDE ? reinterpret_cast<double*>(slot + g.win_offset) : smem;
-    double* zs = WIDE ? smem : smem + (size_t)g.rows * g.ld;   // nloc: the solution z (pinned DOF 0 = 0)
-    double* Ps = smem + (((size_t)g.nloc + 1) & ~(size_t)1);   // (wide) panel, 16-byte aligned
-    double* Rs = Ps + (size_t)g.rows * wide_panel_stride<kNBR>();
-    double* invd = Rs + kNBR;
-    const int nb = g.P == 1 ? 3 : 6, npair = nb * (nb + 1) / 2;
+// Squared L2 and H1 errors of u = zs + shift on element K (vertices Xc); all threads.
+__device__ void element_errors(const RecArgs& g, int64_t K, const double Xc[3][2], const double* zs, double shift,
+                               double* red) {
+    const double* gx = g.dm.gauss_x + 3 * kMaxGauss;
+    const double* gw = g.dm.gauss_w + 3 * kMaxGauss;
+    const int nb = g.P == 1 ? 3 : 6;
+    double e2 = 0.0, h2 = 0.0;
+    for (int t = threadIdx.x; t < g.N * g.N; t += blockDim.x) {
+        int j = 0, rs = 0;
+        while (rs + 2 * (g.N - j) - 1 <= t) { rs += 2 * (g.N - j) - 1; ++j; }
+        const int o = t - rs;
+        const bool up = o < g.N - j;
+        const int i = up ? o : o - (g.N - j);
+        int nx[6], ny[6];
+        element_nodes(g.P, up, i, j, nx, ny);
+        double X[3][2];
+        fine_xy(Xc, g.N, up, i, j, X);
+        const double j00 = X[1][0] - X[0][0], j10 = X[1][1] - X[0][1];
+        const double j01 = X[2][0] - X[0][0], j11 = X[2][1] - X[0][1];
+        const double det = j00 * j11 - j01 * j10;
+        double uv[6];
+        for (int a = 0; a < nb; ++a)
+            uv[a] = zs[ny[a] * (g.PN + 1) - ny[a] * (ny[a] - 1) / 2 + nx[a]] + shift;
+        for (int qi = 0; qi < 4; ++qi)
+            for (int qj = 0; qj < 4; ++qj) {
+                const double xi = gx[qi], eta = gx[qj] * (1.0 - gx[qi]);
+                const double w = gw[qi] * gw[qj] * (1.0 - gx[qi]) * fabs(det);
+                double phi[6], dxi[6], deta[6];
+                basis_eval(g.P, 1.0 - xi - eta, xi, eta, phi, dxi, deta);
+                double uh = 0.0, gxi = 0.0, geta = 0.0;
+                for (int a = 0; a < nb; ++a) {
+                    uh += phi[a] * uv[a];
+                    gxi += dxi[a] * uv[a];
+                    geta += deta[a] * uv[a];
+                }
+                // grad_x = J^{-T} grad_ref
+                const double ux = (j11 * gxi - j10 * geta) / det, uy = (-j01 * gxi + j00 * geta) / det;
+                const double x = X[0][0] + xi * j00 + eta * j01, y = X[0][1] + xi * j10 + eta * j11;
+                double ue, uex, uey;
+                exact_eval(g, x, y, &ue, &uex, &uey);
+                e2 += w * (uh - ue) * (uh - ue);
+                h2 += w * ((ux - uex) * (ux - uex) + (uy - uey) * (uy - uey));
+            }
+    }
+    const double E2 = block_sum(e2, red), H2 = block_sum(h2, red);
+    if (threadIdx.x == 0) {
+        g.err_out[2 * K] = E2;
+        g.err_out[2 * K + 1] = H2;
+    }
+}
 
+// Load of a node: the combined load of the nodes in dof order.
+struct RecLoad {
+    const double* gl;
+    int PN;
+    __device__ __forceinline__ double operator()(int x, int y, int, int) const {
+        return gl[y * (PN + 1) - y * (y - 1) / 2 + x];
+    }
+};
+
+struct RecSmem {
+    int Ke, mass, lamc, xs, red, tab, z, total;   // doubles
+};
+__host__ __device__ inline RecSmem rec_smem(int vec, int NI, int kind, int P, int N) {
+    const int PN = P * N;
+    RecSmem l;
+    int o = (int)front_shared_doubles(vec);
+    l.Ke = o, o += 72;
+    l.mass = o, o += 8;
+    l.lamc = o, o += NI;     // k_i (-s |F|) per local multiplier
+    l.xs = o, o += vec;      // solution at the front's slots
+    l.red = o, o += 32;
+    l.tab = o, o += source_table_doubles(kind, PN);
+    l.z = o, o += (PN + 1) * (PN + 2) / 2;   // load, then solution, per node
+    l.total = o;
+    return l;
+}
+
+// One block per coarse triangle at a time (front.cuh); SL: slots per lane of the backward sweep.
+template <class T, int NCP, int SL, int MINB>
+__global__ void __launch_bounds__(T::threads, MINB) k_reconstruct(const __grid_constant__ RecArgs g) {
+    extern __shared__ double smem[];
+    __shared__ FrontCtx c;
+    const int P = g.P, N = g.N, PN = g.PN, NI = g.NI, tid = threadIdx.x, nthr = blockDim.x, stride = g.slots + 1;
+    const RecSmem L = rec_smem(T::vec, NI, g.src_kind, P, N);
+    const FrontShared sh = front_shared(smem, T::vec);
+    double *Ke = smem + L.Ke, *lamc = smem + L.lamc, *xs = smem + L.xs, *z = smem + L.z;
+    double* keep = reinterpret_cast<double*>(g.ws + (size_t)blockIdx.x * g.slot_bytes);
     for (int64_t ki = blockIdx.x; ki < g.nK; ki += gridDim.x) {
-        const int64_t K = g.dm.klist ? (int64_t)g.dm.klist[ki] : ki;      // coarse element
-        const double* kap = g.kappa + (g.dm.kap_off ? g.dm.kap_off[K] : K * (int64_t)g.N * g.N);
-        if (threadIdx.x == 0) {
-            for (int v = 0; v < 3; ++v) {
-                c.X[v][0] = g.dm.geom[6 * K + 2 * v];
-                c.X[v][1] = g.dm.geom[6 * K + 2 * v + 1];
-            }
-            c.area = 0.5 * fabs((c.X[1][0] - c.X[0][0]) * (c.X[2][1] - c.X[0][1]) -
-                                (c.X[2][0] - c.X[0][0]) * (c.X[1][1] - c.X[0][1]));
-            c.area_fine = c.area / ((double)g.N * g.N);
-            for (int a = 0; a < 3; ++a) {
-                const double* P0 = c.X[(a + 1) % 3];
-                const double* Q0 = c.X[(a + 2) % 3];
-                c.flen[a] = sqrt((Q0[0] - P0[0]) * (Q0[0] - P0[0]) + (Q0[1] - P0[1]) * (Q0[1] - P0[1]));
-                c.sgn[a] = g.dm.sign[3 * K + a];
-                c.rev[a] = g.dm.rev[3 * K + a];
-                c.la1[a] = face_la1(g.dm, K, a);
-            }
-            double Xu[3][2], Xd[3][2];
-            fine_xy(c, g.N, true, 0, 0, Xu);
-            fine_xy(c, g.N, false, 0, 0, Xd);
-            element_stiffness(g.P, Xu, c.Sup);
-            element_stiffness(g.P, Xd, c.Sdn);
-            // sum_i k_i c_i, c_i = (1^T N_i) / |K| = -s |F| int psi / |K|
+        const int64_t K = g.dm.klist ? (int64_t)g.dm.klist[ki] : ki;
+        const double* kap = g.kappa + (g.dm.kap_off ? g.dm.kap_off[K] : K * (int64_t)N * N);
+        front_element(g.dm, K, kap, P, N, g.src_kind, g.src_value, g.src_freq, c, Ke, smem + L.mass, smem + L.tab);
+        front_source(g.src_kind, g.src_value, P, N, smem + L.tab,
+                     g.src_vals ? g.src_vals + 16 * (kap - g.kappa) : nullptr, c, z);
+        if (tid < 32) {   // k_i N_i's coefficients and sum_i k_i (1^T N_i) / |K|
             double cl = 0.0;
-            for (int i = 0; i < g.NI; ++i) {
-                const int a = i / g.dpf, jf = i - a * g.dpf;
-                const int row = face_row(jf, c.la1[a], g.dm.fm, g.dm.lmax1);
-                if (row < 0) continue;   // unused slot
-                cl += g.lambda[g.k_lambda[K * g.NI + i]] * (-c.sgn[a] * c.flen[a] * g.dm.btab_sum[row] / c.area);
+            for (int i = tid; i < NI; i += 32) {
+                const int a = i / g.dpf, row = face_row(i - a * g.dpf, c.la1[a], g.dm.fm, g.dm.lmax1);
+                lamc[i] = row < 0 ? 0.0 : g.lambda[g.k_lambda[K * NI + i]] * (-c.sgn[a] * c.flen[a]);
+                if (row >= 0) cl = fma(lamc[i], g.dm.btab_sum[row], cl);
             }
-            c.cl = cl;
-            c.bad = 0;
-            choose_pin(g.P, g.N, kap, &c.pin_x, &c.pin_y);
+            for (int o = 16; o > 0; o >>= 1) cl += __shfl_xor_sync(0xffffffffu, cl, o);
+            if (tid == 0) smem[L.red] = (cl + c.FK) / c.area;   // coefficient of the mass vector
         }
         __syncthreads();
-        const LevelGeom lg{g.P, g.N, g.PN, c.pin_x, c.pin_y};
-        double fk = 0.0;
-        if (g.src_kind == MHM_SRC_CONST) fk = g.src_value * c.area;
-        else {
-            double s = 0.0;
-            for (int t = threadIdx.x; t < g.N * g.N; t += blockDim.x) {
-                int j = 0, rs = 0;
-                while (rs + 2 * (g.N - j) - 1 <= t) { rs += 2 * (g.N - j) - 1; ++j; }
-                const int o = t - rs;
-                const bool up = o < g.N - j;
-                double X[3][2];
-                fine_xy(c, g.N, up, up ? o : o - (g.N - j), j, X);
-                s += cell_source(g, X, -1, quad_of(g.src_vals, g.kappa, kap, g.N, up, up ? o : o - (g.N - j), j));
-            }
-            fk = block_sum(s, c);
-        }
-        const double cm = fk / c.area + c.cl;     // coefficient of the mass vector in g
-        const int b0 = lg.size(0), b1 = g.nlev > 1 ? lg.size(1) : 0;
-        for (int t = threadIdx.x; t < (b0 + b1) * g.ld; t += blockDim.x) W[t] = 0.0;
-        __syncthreads();
-        size_t foff = 0;
-        for (int lev = 0; lev < g.nlev; ++lev) {
-            const int b = lg.size(lev);
-            const int bn = lev + 1 < g.nlev ? lg.size(lev + 1) : 0;
-            const int nr = b + bn;
-            // boundary loads sum_j k_j N_j of the fresh points (level 0 at the start too)
-            for (int pass = (lev == 0 ? 0 : 1); pass < 2; ++pass) {
-                const int l2 = lev + pass, row0 = pass ? b : 0;
-                if (l2 >= g.nlev) continue;
-                for (int p = threadIdx.x; p < lg.size(l2); p += blockDim.x) {
-                    int x, y;
-                    lg.point(l2, p, &x, &y);
-                    double v = 0.0;
-                    for (int a = 0; a < 3; ++a) {
-                        const int kl = face_position(g.PN, x, y, a);
-                        if (kl < 0) continue;
-                        const int kk = c.rev[a] ? g.PN - kl : kl;
-                        for (int jf = 0; jf < g.dpf; ++jf) {
-                            const int row = face_row(jf, c.la1[a], g.dm.fm, g.dm.lmax1);
-                            if (row < 0) continue;   // unused slot
-                            v += g.lambda[g.k_lambda[K * g.NI + a * g.dpf + jf]] *
-                                 (-c.sgn[a] * c.flen[a] * g.dm.btab[row * (g.PN + 1) + kk]);
-                        }
+        const double cm = smem[L.red], area_fine = c.area / ((double)N * N);
+        {
+            int x = tid, y = 0;
+            for (int u = tid; u < g.nloc; u += nthr, x += nthr) {
+                while (x > PN - y) x -= PN + 1 - y, ++y;
+                const double m = node_mass(P, N, x, y, area_fine);
+                double v = g.src_kind == MHM_SRC_CONST ? (g.src_value - cm) * m : fma(-cm, m, z[u]);
+                for (int a = 0; a < 3; ++a) {
+                    const int kl = face_position(PN, x, y, a);
+                    if (kl < 0) continue;
+                    const int kk = c.rev[a] ? PN - kl : kl;
+                    for (int jf = 0; jf < g.dpf; ++jf) {
+                        const int row = face_row(jf, c.la1[a], g.dm.fm, g.dm.lmax1);
+                        if (row >= 0) v = fma(lamc[a * g.dpf + jf], g.dm.btab[row * (PN + 1) + kk], v);
                     }
-                    W[(row0 + p) * g.ld + rhs] += v;
                 }
-                __syncthreads();
+                z[u] = v;
             }
-            if (bn > 0) {
-                // element matrices and loads of fine row lev, four colour classes
-                for (int cls = 0; cls < 4; ++cls) {
-                    const bool up = cls < 2;
-                    const int parity = cls & 1;
-                    const int ntri = up ? g.N - lev : g.N - 1 - lev;
-                    const int ncls = (ntri - parity + 1) / 2;
-                    const int per = npair + nb;
-                    for (int t = threadIdx.x; t < ncls * per; t += blockDim.x) {
-                        const int ti = t / per, item = t - ti * per;
-                        const int i = parity + 2 * ti;
-                        int nx[6], ny[6];
-                        element_nodes(g.P, up, i, lev, nx, ny);
-                        const double kt = kap[lev * (2 * g.N - lev) + (up ? i : (g.N - lev) + i)];
-                        const double* S = up ? c.Sup : c.Sdn;
-                        if (item < npair) {
-                            int a = 0, rem = item;
-                            while (rem >= nb - a) { rem -= nb - a; ++a; }
-                            const int bb = a + rem;
-                            const int pa = lg.pos(nx[a], ny[a]), pb = lg.pos(nx[bb], ny[bb]);
-                            if (pa < 0 || pb < 0) continue;
-                            const int ra = pa + (lg.level_of_row(ny[a]) == lev ? 0 : b);
-                            const int rb = pb + (lg.level_of_row(ny[bb]) == lev ? 0 : b);
-                            W[max(ra, rb) * g.ld + min(ra, rb)] += kt * S[a * nb + bb];
-                        } else {
-                            const int a = item - npair;
-                            const int pa = lg.pos(nx[a], ny[a]);
-                            if (pa < 0) continue;
-                            const int ra = pa + (lg.level_of_row(ny[a]) == lev ? 0 : b);
-                            const double mass = c.area_fine * element_mass_frac(g.P, a);
-                            double v = -cm * mass;
-                            if (g.src_kind == MHM_SRC_CONST) v += g.src_value * mass;
-                            else {
-                                double X[3][2];
-                                fine_xy(c, g.N, up, i, lev, X);
-                                v += cell_source(g, X, a, quad_of(g.src_vals, g.kappa, kap, g.N, up, i, lev));
-                            }
-                            W[ra * g.ld + rhs] += v;
-                        }
-                    }
-                    __syncthreads();
-                }
-            }
-            if constexpr (WIDE)
-                wide_cholesky_level<kNBR>(W, g.ld, b, nr, W + rhs, g.ld, nr, 1, &c.bad, Ps, Rs, invd, nullptr);
-            else
-                blocked_cholesky_level<double, 8, 4, 1>(W, g.ld, b, nr, W + rhs, g.ld, nr, 1, &c.bad);
-            // keep L_lev, L_{lev+1,lev} and y_lev for the backward sweep
-            for (int t = threadIdx.x; t < b * b + bn * b + b; t += blockDim.x) {
-                double v;
-                if (t < b * b) { const int i = t / b, k = t - i * b; v = k <= i ? W[i * g.ld + k] : 0.0; }
-                else if (t < b * b + bn * b) { const int q = t - b * b, i = q / b, k = q - i * b; v = W[(b + i) * g.ld + k]; }
-                else v = W[(t - b * b - bn * b) * g.ld + rhs];
-                Fst[foff + t] = v;
-            }
-            foff += (size_t)b * b + (size_t)bn * b + b;
-            __syncthreads();
-            if (bn > 0) {
-                for (int t = threadIdx.x; t < bn * bn; t += blockDim.x) {
-                    const int i = t / bn, jj = t - i * bn;
-                    if (jj <= i) W[i * g.ld + jj] = W[(b + i) * g.ld + b + jj];
-                }
-                for (int t = threadIdx.x; t < bn; t += blockDim.x) W[t * g.ld + rhs] = W[(b + t) * g.ld + rhs];
-                __syncthreads();
-                const int bnn = lev + 2 < g.nlev ? lg.size(lev + 2) : 0;
-                for (int t = threadIdx.x; t < bnn * g.ld; t += blockDim.x) W[bn * g.ld + t] = 0.0;
-                __syncthreads();
-            }
-        }
-        // backward sweep x_lev = L_lev^{-T} (y_lev - L_{lev+1,lev}^T x_{lev+1}) by warp 0
-        if (threadIdx.x < 32) {
-            const int lane = threadIdx.x;
-            size_t off = foff;
-            int bnext = 0, u0n = 0;
-            int ustart = g.nloc - 1;   // unknowns 0..nloc-2 at zs[1 ..]
-            for (int lev = g.nlev - 1; lev >= 0; --lev) {
-                const int b = lg.size(lev);
-                const int bn = lev + 1 < g.nlev ? lg.size(lev + 1) : 0;
-                off -= (size_t)b * b + (size_t)bn * b + b;
-                const double* Lm = Fst + off;
-                const double* Cm = Lm + (size_t)b * b;
-                const double* yv = Cm + (size_t)bn * b;
-                ustart -= b;
-                for (int k = lane; k < b; k += 32) {
-                    double t = yv[k];
-                    for (int i = 0; i < bnext; ++i) t -= Cm[i * b + k] * zs[1 + u0n + i];
-                    zs[1 + ustart + k] = t;
-                }
-                __syncwarp();
-                for (int k = b - 1; k >= 0; --k) {
-                    const double xk = zs[1 + ustart + k] / Lm[k * b + k];
-                    __syncwarp();
-                    for (int i = lane; i < k; i += 32) zs[1 + ustart + i] -= Lm[k * b + i] * xk;
-                    if (lane == 0) zs[1 + ustart + k] = xk;
-                    __syncwarp();
-                }
-                bnext = b;
-                u0n = ustart;
-            }
-            // zs[1 + u] holds unknown u; the unknowns are the local DOFs in order without the
-            // pinned one: shift the DOFs before it down by one and set the pinned DOF to 0
-            const int pd = lg.pin_y * (g.PN + 1) - lg.pin_y * (lg.pin_y - 1) / 2 + lg.pin_x;
-            for (int base = 0; base < pd; base += 32) {
-                const double v = base + lane < pd ? zs[base + lane + 1] : 0.0;
-                __syncwarp();
-                if (base + lane < pd) zs[base + lane] = v;
-                __syncwarp();
-            }
-            if (lane == 0) zs[pd] = 0.0;
         }
         __syncthreads();
-        // zero mean: eta = z - (m^T z) / |K|, m_w = sum of int phi_w over the fine triangles
-        double mzp = 0.0;
-        for (int t = threadIdx.x; t < g.N * g.N; t += blockDim.x) {
-            int j = 0, rs = 0;
-            while (rs + 2 * (g.N - j) - 1 <= t) { rs += 2 * (g.N - j) - 1; ++j; }
-            const int o = t - rs;
-            const bool up = o < g.N - j;
-            int nx[6], ny[6];
-            element_nodes(g.P, up, up ? o : o - (g.N - j), j, nx, ny);
-            for (int a = 0; a < nb; ++a) {
-                const int dof = ny[a] * (g.PN + 1) - ny[a] * (ny[a] - 1) / 2 + nx[a];
-                mzp += c.area_fine * element_mass_frac(g.P, a) * zs[dof];
+        FrontRows2D<NCP, RecLoad> rows{g.cp, kap, Ke, g.steps, 1, T::vec, c.pin, RecLoad{z, PN}};
+        if (T::NW == 1 || (tid >> 5) == T::NW) rows.start();
+        {
+            double A[T::NT];
+            front_eliminate<T>(rows, g.ev, g.steps, 1, sh, A, &c.bad, keep, stride);
+        }
+        __syncthreads();
+        // backward sweep; two steps' columns are in flight
+        if (tid < 32) {
+            for (int q = tid; q < T::vec; q += 32) xs[q] = 0.0;
+            struct Col { double s[SL], y; int4 v; };
+            auto fetch = [&](int e) {
+                Col k;
+                k.v = make_int4(kNoSlot | kNoSlot << 8, 0, 0, 0);
+                if (e >= 0) k.v = g.ev[e];
+                const bool on = (k.v.x & 255) != kNoSlot;
+                const int m = on ? (k.v.x >> 16) & 255 : 0;
+                const double* r = keep + (size_t)max(e, 0) * stride;
+                k.y = on ? r[0] : 0.0;
+#pragma unroll
+                for (int q = 0; q < SL; ++q) k.s[q] = tid + 32 * q < m ? r[1 + tid + 32 * q] : 0.0;
+                return k;
+            };
+            Col k0 = fetch(g.steps - 1), k1 = fetch(g.steps - 2);
+            __syncwarp();
+            for (int e = g.steps - 1; (k0.v.x & 255) != kNoSlot; --e) {
+                const Col k2 = fetch(e - 2);
+                double t = k0.s[0] * xs[tid];
+#pragma unroll
+                for (int q = 1; q < SL; ++q) t = fma(k0.s[q], xs[tid + 32 * q], t);
+                for (int o = 16; o > 0; o >>= 1) t += __shfl_xor_sync(0xffffffffu, t, o);
+                t = k0.y - t;
+                __syncwarp();
+                if (tid == 0) {
+                    const int x = k0.v.w & 0xffff, y = k0.v.w >> 16;
+                    xs[k0.v.x & 255] = t;
+                    z[y * (PN + 1) - y * (y - 1) / 2 + x] = t;
+                }
+                __syncwarp();
+                k0 = k1;
+                k1 = k2;
             }
         }
-        const double shift = g.u0[K] - block_sum(mzp, c) / c.area;
+        __syncthreads();
+        // zero mean, then u0
+        double mz = 0.0;
+        {
+            int x = tid, y = 0;
+            for (int u = tid; u < g.nloc; u += nthr, x += nthr) {
+                while (x > PN - y) x -= PN + 1 - y, ++y;
+                mz = fma(node_mass(P, N, x, y, area_fine), z[u], mz);
+            }
+        }
+        const double shift = g.u0[K] - block_sum(mz, smem + L.red) / c.area;
         double* uK = g.u_out + (g.nod_off ? g.nod_off[K] : K * (int64_t)g.nloc);
-        for (int w = threadIdx.x; w < g.nloc; w += blockDim.x) uK[w] = zs[w] + shift;
-        if (g.err_out) {
-            const double* gx = g.dm.gauss_x + 3 * kMaxGauss;
-            const double* gw = g.dm.gauss_w + 3 * kMaxGauss;
-            double e2 = 0.0, h2 = 0.0;
-            for (int t = threadIdx.x; t < g.N * g.N; t += blockDim.x) {
-                int j = 0, rs = 0;
-                while (rs + 2 * (g.N - j) - 1 <= t) { rs += 2 * (g.N - j) - 1; ++j; }
-                const int o = t - rs;
-                const bool up = o < g.N - j;
-                const int i = up ? o : o - (g.N - j);
-                int nx[6], ny[6];
-                element_nodes(g.P, up, i, j, nx, ny);
-                double X[3][2];
-                fine_xy(c, g.N, up, i, j, X);
-                const double j00 = X[1][0] - X[0][0], j10 = X[1][1] - X[0][1];
-                const double j01 = X[2][0] - X[0][0], j11 = X[2][1] - X[0][1];
-                const double det = j00 * j11 - j01 * j10;
-                double uv[6];
-                for (int a = 0; a < nb; ++a)
-                    uv[a] = zs[ny[a] * (g.PN + 1) - ny[a] * (ny[a] - 1) / 2 + nx[a]] + shift;
-                for (int qi = 0; qi < 4; ++qi)
-                    for (int qj = 0; qj < 4; ++qj) {
-                        const double xi = gx[qi], eta = gx[qj] * (1.0 - gx[qi]);
-                        const double w = gw[qi] * gw[qj] * (1.0 - gx[qi]) * fabs(det);
-                        double phi[6], dxi[6], deta[6];
-                        basis_eval(g.P, 1.0 - xi - eta, xi, eta, phi, dxi, deta);
-                        double uh = 0.0, gxi = 0.0, geta = 0.0;
-                        for (int a = 0; a < nb; ++a) {
-                            uh += phi[a] * uv[a];
-                            gxi += dxi[a] * uv[a];
-                            geta += deta[a] * uv[a];
-                        }
-                        // grad_x = J^{-T} grad_ref
-                        const double ux = (j11 * gxi - j10 * geta) / det, uy = (-j01 * gxi + j00 * geta) / det;
-                        const double x = X[0][0] + xi * j00 + eta * j01, y = X[0][1] + xi * j10 + eta * j11;
-                        double ue, uex, uey;
-                        exact_eval(g, x, y, &ue, &uex, &uey);
-                        e2 += w * (uh - ue) * (uh - ue);
-                        h2 += w * ((ux - uex) * (ux - uex) + (uy - uey) * (uy - uey));
-                    }
-            }
-            const double E2 = block_sum(e2, c), H2 = block_sum(h2, c);
-            if (threadIdx.x == 0) {
-                g.err_out[2 * K] = E2;
-                g.err_out[2 * K + 1] = H2;
-            }
-        }
+        for (int w = tid; w < g.nloc; w += nthr) uK[w] = z[w] + shift;
+        if (g.err_out) element_errors(g, K, c.X, z, shift, smem + L.red);
         __syncthreads();
     }
+}
+
+// The frontal kernel of a level (one border row); NULL if the front is too large.
+struct RecKernel {
+    void (*kern)(const RecArgs) = nullptr;
+    int threads = 0, vec = 0;
+};
+template <class T, int SL, int MINB>
+void rec_try(const Level& lv, RecKernel* k) {
+    if (k->kern || lv.fsteps == 0 || lv.fslots + 1 > T::rows || lv.fslots > 32 * SL) return;
+    k->kern = lv.fncp == 8 ? k_reconstruct<T, 8, SL, MINB> : k_reconstruct<T, 16, SL, MINB>;
+    k->threads = T::threads;
+    k->vec = T::vec;
+}
+RecKernel rec_kernel(const Level& lv) {
+    RecKernel k;
+    rec_try<FrontTiles<1, 1, 5>, 1, 16>(lv, &k);
+    rec_try<FrontTiles<1, 1, 9>, 2, 16>(lv, &k);
+    rec_try<FrontTiles<4, 1, 5>, 3, 3>(lv, &k);
+    rec_try<FrontTiles<4, 2, 9>, 5, 1>(lv, &k);
+    return k;
 }
 
 }  // namespace
@@ -441,51 +343,34 @@ extern "C" mhm_status mhm_reconstruct(const mhm_mesh* mesh, const double* kappa,
         g.PN = lv.PN;
         g.dpf = mesh->dpf;
         g.NI = (int)mesh->NI;
-        g.nlev = lv.N + 1;
         g.nloc = (int)lv.nloc;
-        auto size = [&](int lev) {
-            if (g.P == 1) return g.N + 1 - lev - (lev == 0);
-            if (lev == g.N) return 1;
-            return (2 * g.N - 2 * lev + 1) + (2 * g.N - 2 * lev) - (lev == 0);
-        };
-        g.rows = size(0) + (g.N >= 1 ? size(1) : 0);
-        g.rhs = g.rows;                      // right-hand side right after the symmetric part
-        g.ld = (g.rows + 2) & ~1;            // even: 16-byte rows for the vector panel loads
         g.src_kind = f->kind;
         g.src_vals = f->kind == MHM_SRC_QUAD ? f->values_dev : nullptr;
         g.src_value = f->value;
         g.src_freq = f->freq;
         g.ex_kind = exact ? (exact->kind == MHM_EXACT_SINSIN ? 1 : 2) : 0;
         for (int i = 0; i < 6; ++i) g.ex[i] = exact ? exact->c[i] : 0.0;
-        size_t per = 0;
-        for (int lev = 0; lev < g.nlev; ++lev) {
-            const int b = size(lev), bn = lev + 1 < g.nlev ? size(lev + 1) : 0;
-            per += (size_t)b * b + (size_t)bn * b + b;
-        }
-        g.slot_bytes = ((per * sizeof(double)) + 255) & ~(size_t)255;
         g.nK = lv.nK;
         g.nod_off = mesh->d_nod_off;
         g.u_out = u_nodal;
         g.err_out = err_sq;
-        size_t smem = ((size_t)g.rows * g.ld + (size_t)g.nloc) * sizeof(double);
-        const bool wide = g.rows > 128 || smem > 220 * 1024;
-        g.win_offset = 0;
-        if (wide) {
-            // the window behind the stored factors in the slot; shared memory keeps z and the panel
-            g.win_offset = g.slot_bytes;
-            g.slot_bytes += (((size_t)g.rows * g.ld * sizeof(double)) + 255) & ~(size_t)255;
-            smem = ((((size_t)g.nloc + 1) & ~(size_t)1) + (size_t)g.rows * wide_panel_stride<kNBR>() + 2 * kNBR) *
-                   sizeof(double);
-        }
-        if (smem > 220 * 1024) return fail(MHM_ERR_UNSUPPORTED, "mhm_reconstruct: window exceeds shared memory");
-        void (*kern)(const RecArgs) = wide ? k_reconstruct<true> : k_reconstruct<false>;
-        const int threads = wide ? kThreadsRWide : kThreadsR;
+        const RecKernel front = rec_kernel(lv);
+        g.ev = lv.d_fev;
+        g.cp = lv.d_fcp;
+        g.steps = lv.fsteps;
+        g.slots = lv.fslots;
+        if (!front.kern) return fail(MHM_ERR_UNSUPPORTED, "mhm_reconstruct: front too large (r too large)");
+        void (*kern)(const RecArgs) = front.kern;
+        const int threads = front.threads;
+        g.slot_bytes = ((size_t)g.steps * (g.slots + 1) * sizeof(double) + 255) & ~(size_t)255;
+        const size_t smem = (size_t)rec_smem(front.vec, g.NI, f->kind, g.P, g.N).total * sizeof(double);
         MHM_CUDA_TRY(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
         int sms = 0, occ = 0;
         cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, mesh->device);
         cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, kern, threads, smem);
-        int64_t grid = (int64_t)sms * (occ > 0 ? occ : 1);
-        if (grid > lv.nK) grid = lv.nK;
+        // one wave, the elements shared out evenly
+        const int64_t each = (lv.nK + sms - 1) / sms, rounds = (each + std::max(occ, 1) - 1) / std::max(occ, 1);
+        const int64_t grid = std::min(lv.nK, sms * ((each + rounds - 1) / rounds));
         char* ws = nullptr;
         cudaError_t e = cudaMallocAsync((void**)&ws, (size_t)grid * g.slot_bytes, s);
         if (e != cudaSuccess) return cuda_fail(e, "mhm_reconstruct: cudaMallocAsync");

@@ -62,3 +62,26 @@ def test_blocks_vs_oracle_at_layout_edges(P, r, m, l):
     tol = max(1e-10, 10 * 1.1e-16 * 12 * n * 10)
     for K in range(2):
         assert_blocks(AK[K], EK[K], BK[K], FK[K], solve_local(mesh, K, r, P, kap[K], source_fn("sinsin", 1.0, 1.0)), tol, K)
+
+
+@pytest.mark.parametrize("P,r,m,l", [(1, 0, 1, 0), (1, 3, 1, 1), (1, 4, 2, 0), (2, 4, 3, 1), (1, 5, 2, 2), (1, 6, 1, 3),
+                                     (2, 5, 1, 2), (1, 7, 1, 3), (2, 6, 1, 1)])
+def test_reconstruction_vs_oracle_at_layout_edges(P, r, m, l):
+    """u of both elements from given multipliers (fronts of 3 to 131 slots) against the oracle's
+    local solutions combined with the same multipliers."""
+    from paper_1703_10435_gb300.pipeline import Pipeline
+    w = W.Workload("t", 1, 1, r, P, m, l, "log_uniform", "sinsin", 1.0, 1.0, seed=3)
+    kap = W.kappa_for(w) ** 0.25
+    src = mhm.Source(mhm.MHM_SRC_SINSIN, 1.0, 1.0)
+    p = Pipeline.for_workload(w, 0, mhm.MHM_FP64)
+    rng = np.random.default_rng(7)
+    lam, u0 = rng.standard_normal(p.mesh.n_lambda), rng.standard_normal(2)
+    p.lam, p.u0 = torch.as_tensor(lam, device="cuda"), torch.as_tensor(u0, device="cuda")
+    u, _ = p.reconstruct(torch.as_tensor(kap, device="cuda"), src)
+    u = u.cpu().numpy()
+    mesh = build_mesh(1, 1, m, l)
+    for K in range(2):
+        o = solve_local(mesh, K, r, P, kap[K], source_fn("sinsin", 1.0, 1.0))
+        want = u0[K] + o.eta[:, :-1] @ lam[mesh.local_lambda(K)] + o.eta[:, -1]
+        tol = max(1e-10, 10 * 1.1e-16 * 12 * o.sub.n * 10)   # 10 u cond, as above
+        assert np.abs(u[K] - want).max() < tol * np.abs(want).max(), K
