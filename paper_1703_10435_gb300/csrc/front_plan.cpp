@@ -154,4 +154,79 @@ FrontPlan front_plan_2d(int P, int N) {
     return plan;
 }
 
+FrontPlan3 front_plan_3d(int n, int nb, const std::vector<int32_t>& dofs, const std::vector<int8_t>& cls,
+                         const std::vector<int32_t>& xyz, int R) {
+    FrontPlan3 plan;
+    const int nt = (int)cls.size(), n1 = n - 1;   // node v: DOF v + 1
+    std::vector<std::vector<int>> inc(n1), adj(n1);   // slots t nb + a; neighbours
+    for (int s = 0; s < nt * nb; ++s)
+        if (dofs[s] > 0) inc[dofs[s] - 1].push_back(s);
+    int top = 0;
+    for (int v = 0; v < n1; ++v) {
+        for (int s : inc[v])
+            for (int b = 0; b < nb; ++b) {
+                const int u = dofs[s / nb * nb + b] - 1;
+                if (u >= 0 && u != v) adj[v].push_back(u);
+            }
+        std::sort(adj[v].begin(), adj[v].end());
+        adj[v].erase(std::unique(adj[v].begin(), adj[v].end()), adj[v].end());
+        top = std::max(top, xyz[3 * (v + 1)]);
+    }
+    std::vector<FrontStep> steps;
+    double best = 0.0;
+    for (int kind = 0; kind < 3; ++kind) {
+        auto key = [&](int v) -> std::array<int, 6> {
+            const int A = xyz[3 * v + 3], B = xyz[3 * v + 4], C = xyz[3 * v + 5];
+            if (kind == 0) return {C, B, A, 0, 0, 0};
+            if (kind == 1) return {C / 2, B / 2, A / 2, C, B, A};
+            return {top - B, top - A, B - C, 0, 0, 0};
+        };
+        std::vector<int> order(n1);
+        for (int v = 0; v < n1; ++v) order[v] = v;
+        std::sort(order.begin(), order.end(), [&](int a, int b) { return key(a) < key(b); });
+        int slots = 0;
+        const std::vector<FrontStep> st = front_schedule(adj, order, &slots);
+        double work = 0.0;
+        for (const FrontStep& q : st)
+            if (q.pivot >= 0) work += (double)(R + q.m) * (R + q.m);
+        if (steps.empty() || work < best) steps = st, best = work, plan.slots = slots;
+    }
+    if (plan.slots > kMaxSlots) return FrontPlan3{};
+    plan.steps = (int)steps.size();
+    std::vector<int> slot(n1, -1);
+    for (const FrontStep& st : steps) {
+        const int v = st.enter, first = (int)plan.ent.size();
+        if (v >= 0) {
+            for (int part = 0; part < 8; ++part) {   // the diagonal: every eighth incident tetrahedron
+                const size_t c0 = plan.con.size();
+                for (size_t k = part; k < inc[v].size(); k += 8) {
+                    const int t = inc[v][k] / nb, a = inc[v][k] % nb;
+                    plan.con.push_back(t | (uint32_t)((cls[t] * nb + a) * nb + a) << 16);
+                }
+                plan.ent.push_back(kDiagSlot | (uint32_t)(plan.con.size() - c0) << 8 | (uint32_t)c0 << 16);
+            }
+            for (int u : adj[v]) {
+                const int sl = u == st.pivot ? kPivotSlot : slot[u];
+                if (sl < 0) continue;
+                const size_t c0 = plan.con.size();
+                for (int s : inc[v])
+                    for (int b = 0; b < nb; ++b)
+                        if (dofs[s / nb * nb + b] - 1 == u) {
+                            const int t = s / nb, a = s % nb;
+                            plan.con.push_back(t | (uint32_t)((cls[t] * nb + a) * nb + b) << 16);
+                        }
+                plan.ent.push_back(sl | (uint32_t)(plan.con.size() - c0) << 8 | (uint32_t)c0 << 16);
+            }
+        }
+        plan.ev.push_back(st.ps | st.zs << 8 | st.m << 16);
+        plan.ev.push_back(v >= 0 ? v + 1 : -1);
+        plan.ev.push_back(first);
+        plan.ev.push_back((int)plan.ent.size() - first);
+        if (st.pivot >= 0) slot[st.pivot] = -1;
+        if (v >= 0) slot[v] = st.zs;
+    }
+    if (plan.con.size() > 0xffff) return FrontPlan3{};
+    return plan;
+}
+
 }  // namespace mhm

@@ -41,4 +41,18 @@ struct FrontPlan {
 };
 FrontPlan front_plan_2d(int P, int N);
 
+// Tables of the refined tetrahedron, local DOF 0 left out (pinned).  dofs: the nb DOFs of every
+// sub-tetrahedron, cls its class, xyz the DOFs' lattice coordinates (A, B, C).  ev: 4 int32
+// per step: ps | zs << 8 | m << 16; the entering DOF (-1: none); first and number of its
+// entries.  ent: slot | terms << 8 | first term << 16, the first 8 of a node the parts of its
+// diagonal; the value of an entry is the sum of its terms kappa[t] S[s] (con: t | s << 16,
+// s = (class nb + a) nb + b).  Of three orders the one with the least work for R loads.
+struct FrontPlan3 {
+    int steps = 0, slots = 0;
+    std::vector<int32_t> ev;
+    std::vector<uint32_t> ent, con;
+};
+FrontPlan3 front_plan_3d(int n, int nb, const std::vector<int32_t>& dofs, const std::vector<int8_t>& cls,
+                         const std::vector<int32_t>& xyz, int R);
+
 }  // namespace mhm

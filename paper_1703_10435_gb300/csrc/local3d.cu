@@ -3,29 +3,20 @@
 // or mixed precision, and the gather of the skeleton system (Eq. "mat_global").
 // Conventions in mhm3d.h.
 //
-// Both local kernels run one block of kThreads threads per coarse element, everything in
-// shared memory, with no atomics (every sum in a fixed order: repeated calls are
-// bit-identical):
-//   1. one element matrix per class of congruent sub-tetrahedra (the Freudenthal
-//      refinement has six: its sub-tetrahedra of one permutation class are translates),
-//      from the closed forms of the P1 / P2 Lagrange stiffness in barycentric gradients;
-//   2. per local DOF, over the sub-tetrahedra that hold it: its row of the pinned lower
-//      triangle (local DOF 0 removed), its mass int phi_w and its source load; the
-//      multiplier loads -s (psi_j, phi_w) from the face table (a fine face triangle puts
-//      a third of its area on each load node);
-//   3. the compatibility projection g - (1^T g / |K|) m of every right-hand side;
-// then k_local3d (FP64):
-//   4. a right-looking Cholesky factorisation of the pinned matrix with the forward
-//      substitution of all right-hand sides fused in;
-//   5. the face integrals in Gram form, (s psi_j, eta_i)_{dK} = -Y_j . Y_i with Y = L^{-1}
-//      times the projected loads (symmetric by construction), and E_K = Y_j . y_f;
-// or k_local3d_mixed: an FP32 factor of the diagonally scaled matrix, FP64 refinement
-// against the matrix-free residual, and the corrected bilinear form (see the kernel).
+// No atomics anywhere, every sum in a fixed order: repeated calls are bit-identical.
+//   k_local3d (FP64): frontal elimination of the pinned matrix bordered by the projected loads
+//     g - (1^T g / |K|) m (front.cuh): class matrices of the six congruence classes of
+//     sub-tetrahedra (closed forms, per element type), couplings gathered per DOF, multiplier
+//     loads from the face table (a fine face triangle puts a third of its area on each load
+//     node); the face integrals are what the elimination leaves in the border;
+//   k_local3d_mixed: an FP32 factor of the diagonally scaled matrix, FP64 refinement against
+//     the matrix-free residual, and the corrected bilinear form (see the kernel).
 #include <algorithm>
 #include <cmath>
 #include <cstring>
 #include <string>
 
+#include "front.cuh"
 #include "mhm3d_internal.h"
 
 namespace mhm3 {
@@ -48,7 +39,7 @@ struct Local3DArgs {
     const double* kappa;
     int src_kind;
     double src_value, src_freq;
-    int64_t K0;
+    int64_t K0, K1;
     int N, P, n, nb, nsub, m, NI, R;
     double* AK;
     double* EK;
@@ -60,8 +51,18 @@ struct Local3DArgs {
     int it_max;           // mixed kernel: refinement passes
     double tol;           // mixed kernel: scaled residual target per column
     int qs;               // the source's quadrature points of a sub-tetrahedron in qs groups of 64/qs
+    // frontal elimination (front.cuh): step tables; per type of element (K mod 24: translates)
+    // the six class matrices and vol, area_a / (3 N^2); mass of a DOF on a unit volume; fine
+    // face triangles of subface q that load DOF w, per local face and permutation (x n x m)
+    const int4* ev;
+    const uint32_t *ent, *con;
+    int steps;
+    const double *cls24, *geo24, *mass1;
+    const uint8_t* fcnt;
+    const double* src24;  // source tables per type, class, local DOF (k_source3d); NULL: constant
 };
 
+constexpr int kPath[6][3] = {{0, 1, 2}, {0, 2, 1}, {1, 0, 2}, {1, 2, 0}, {2, 0, 1}, {2, 1, 0}};
 __constant__ int c_perm[6][3] = {{0, 1, 2}, {0, 2, 1}, {1, 0, 2}, {1, 2, 0}, {2, 0, 1}, {2, 1, 0}};
 __constant__ int c_edges[6][2] = {{0, 1}, {0, 2}, {0, 3}, {1, 2}, {1, 3}, {2, 3}};
 
@@ -86,29 +87,15 @@ __device__ __forceinline__ int tri_row(int t) {
     return r;
 }
 
-// shared-memory layout of the FP64 kernel (doubles), in this order
-struct Smem3 {
-    int T, Y, mass, S6, G6, J6, red, misc, total;
-};
-
 // doubles of the source's partial loads: per group of quadrature points of every
 // sub-tetrahedron, its nb loads and its part of F_K
 __host__ __device__ inline int partial_loads(int nsub, int nb, int qs) { return qs * nsub * (nb + 1); }
 
-__host__ __device__ inline Smem3 smem_layout(int n, int NI, int nb, int nsub, int qs) {
+// Size of the dense problem in shared memory (packed pinned triangle or partial loads,
+// n x R columns, tables), which bounds the meshes that are accepted.
+inline size_t dense_doubles(int n, int NI, int nb, int nsub, int qs) {
     const int R = NI + 1, n1 = n - 1, npk = n1 * (n1 + 1) / 2, pl = partial_loads(nsub, nb, qs);
-    Smem3 s{};
-    int o = 0;
-    s.T = o;    o += npk > pl ? npk : pl;           // the source's partial loads, then the pinned factor
-    s.Y = o;    o += n * R;                         // right-hand sides, then solutions
-    s.mass = o; o += n;
-    s.S6 = o;   o += 6 * nb * nb;                   // element matrix per class
-    s.G6 = o;   o += 6 * 12;                        // barycentric gradients per class
-    s.J6 = o;   o += 6 * 9;                         // edge vectors per class (columns)
-    s.red = o;  o += R;
-    s.misc = o; o += 16;                            // |K|, |face a| / N^2 (4), V_sub, F_K, pivot flag, done flag
-    s.total = o;
-    return s;
+    return (size_t)(npk > pl ? npk : pl) + (size_t)n * R + n + 6 * nb * nb + 6 * 21 + R + 16;
 }
 
 // shared-memory layout of the mixed kernel (doubles; the FP32 factor and solve vectors
@@ -373,83 +360,234 @@ __device__ __forceinline__ void element_tail(const Local3DArgs& g, int64_t K, co
     }
 }
 
-__global__ void __launch_bounds__(kThreads) k_local3d(Local3DArgs g) {
-    extern __shared__ double sm[];
-    const Smem3 L = smem_layout(g.n, g.NI, g.nb, g.nsub, g.qs);
-    double* Lp = sm + L.T;
-    double* Y = sm + L.Y;
-    double* mass = sm + L.mass;
-    double* S6 = sm + L.S6;
-    double* G6 = sm + L.G6;
-    double* J6 = sm + L.J6;
-    double* red = sm + L.red;
-    double* misc = sm + L.misc;
-    const int tid = threadIdx.x, nthr = blockDim.x;
-    const int64_t K = g.K0 + blockIdx.x;
-    if (g.only_failed && g.status[K] == MHM_OK) return;   // the whole block, before any barrier
-    const int n = g.n, n1 = n - 1, R = g.R, NI = g.NI;
-    const double* V = g.geom + 12 * K;   // v0..v3
-    const double* kap = g.kappa + K * (int64_t)g.nsub;
-
-    // ---- zero the right-hand sides; geometry; class matrices; the source's partial loads
-    for (int i = L.Y + tid; i < L.mass; i += nthr) sm[i] = 0.0;
-    element_geometry(g, V, misc, G6, J6);
-    __syncthreads();
-    class_matrices(g, misc[5], G6, S6);
-    source_partials(g, V, J6, misc, Lp);
-    __syncthreads();
-    // ---- loads and mass per DOF, then the pinned lower triangle row by row (pinned DOF 0
-    // dropped), over the partial loads once they are summed: no atomics, a fixed order
-    element_loads(g, K, Y, mass, Lp, misc);
-    __syncthreads();
-    for (int w = 1 + tid; w < n; w += nthr) assemble_row<double>(g, w, kap, S6, Lp + pk(w - 1, 0), nullptr);
-    const_source_and_projection(g, Y, mass, red, misc);
-
-    // ---- Cholesky of the pinned matrix (rows 1..n-1), forward substitution fused
-    for (int k = 0; k < n1; ++k) {
-        double d = Lp[pk(k, k)];
-        if (!(d > 0.0)) {
-            d = 1.0;
-            if (tid == 0) misc[7] = 1.0;
+// Source tables (sin sin sin by the collapsed Gauss rule) of one element type and class (one
+// block each): with a sub-tetrahedron's first vertex at x and a point of the rule at x + d,
+// the addition theorem splits f(x + d) into eight products of sines and cosines of x and of d,
+//   load of local DOF a = sum_b prod_c (b_c ? cos : sin)(k x_c) M[a][b],
+//   M[a][b] = sum over the points of w phi_a prod_c (b_c ? sin : cos)(k d_c).
+// The sub-tetrahedra of a class are translates, so M is per type and class (24 x 6): an element
+// needs 3 sincos per sub-tetrahedron where the rule has 3 sines at each of its 64 points.
+__global__ void __launch_bounds__(kQuad) k_source3d(const double* geom, const double* quad, int N, int nb, double value,
+                                                    double freq, double* out) {
+    __shared__ double f[kQuad][8];
+    const int type = blockIdx.x / 6, cls = blockIdx.x % 6, q = threadIdx.x;
+    const double* V = geom + 12 * type;
+    const double* qp = quad + 4 * q;
+    double s[3], c[3], det = 0.0;
+    {
+        double e[3][3];   // edge vectors v1 - v0, v2 - v1, v3 - v2
+        for (int k = 0; k < 3; ++k)
+            for (int x = 0; x < 3; ++x) e[k][x] = V[3 * (k + 1) + x] - V[3 * k + x];
+        det = e[0][0] * (e[1][1] * e[2][2] - e[1][2] * e[2][1]) - e[0][1] * (e[1][0] * e[2][2] - e[1][2] * e[2][0]) +
+              e[0][2] * (e[1][0] * e[2][1] - e[1][1] * e[2][0]);
+        // a point at reference (x, y, z): steps of the class's path, each along one edge vector
+        double t[3] = {0.0, 0.0, 0.0}, r = qp[0] + qp[1] + qp[2];
+        for (int k = 0; k < 3; ++k) {
+            t[c_perm[cls][k]] = r;
+            r -= qp[k];
         }
-        const double inv = 1.0 / sqrt(d);
-        for (int i = k + 1 + tid; i < n1; i += nthr) Lp[pk(i, k)] *= inv;
-        for (int r = tid; r < R; r += nthr) Y[(k + 1) * R + r] *= inv;
-        __syncthreads();
-        // trailing update of the triangle below pivot k and of the right-hand sides, as one
-        // flat list of items over all threads (every lane busy: the FP64 pipe is the limit)
-        const int mt = n1 - k - 1, tri = mt * (mt + 1) / 2, items = tri + mt * R;
-        for (int t = tid; t < items; t += nthr) {
-            if (t < tri) {
-                const int ii = tri_row(t);
-                const int i = k + 1 + ii, j = k + 1 + (t - ii * (ii + 1) / 2);
-                Lp[pk(i, j)] -= Lp[pk(i, k)] * Lp[pk(j, k)];
-            } else {
-                const int u = t - tri, i = k + 1 + u / R, r = u % R;
-                Y[(i + 1) * R + r] -= Lp[pk(i, k)] * Y[(k + 1) * R + r];
+        for (int x = 0; x < 3; ++x) sincospi(freq * ((t[0] * e[0][x] + t[1] * e[1][x] + t[2] * e[2][x]) / N), &s[x], &c[x]);
+    }
+    const double kf = freq * M_PI, w = qp[3] * fabs(det) / ((double)N * N * N) * value * 3.0 * kf * kf;
+    for (int b = 0; b < 8; ++b) f[q][b] = w * (b & 1 ? s[0] : c[0]) * (b & 2 ? s[1] : c[1]) * (b & 4 ? s[2] : c[2]);
+    __syncthreads();
+    const double* phi = quad + 4 * kQuad;
+    for (int t = q; t < 8 * nb; t += kQuad) {
+        const int a = t >> 3, b = t & 7;
+        double sum = 0.0;
+        for (int p = 0; p < kQuad; ++p) sum = fma(phi[p * nb + a], f[p][b], sum);
+        out[(size_t)blockIdx.x * 8 * nb + t] = sum;
+    }
+}
+
+// Source loads of element K per DOF (src, n) through the loads of every sub-tetrahedron (PL,
+// nsub x nb), summed per DOF in the fixed order of its incidence list.  All threads; ends
+// with a barrier.
+__device__ __forceinline__ void source_loads3(const Local3DArgs& g, int64_t K, double* PL, double* src) {
+    const int nb = g.nb, N = g.N;
+    const double* V = g.geom + 12 * K;
+    for (int t = threadIdx.x; t < g.nsub; t += blockDim.x) {
+        double s[3], c[3], T[8];
+        for (int x = 0; x < 3; ++x) {
+            const double p = V[x] + ((V[3 + x] - V[x]) * g.sub_base[3 * t] + (V[6 + x] - V[3 + x]) * g.sub_base[3 * t + 1] +
+                                     (V[9 + x] - V[6 + x]) * g.sub_base[3 * t + 2]) / N;
+            sincospi(g.src_freq * p, &s[x], &c[x]);
+        }
+#pragma unroll
+        for (int b = 0; b < 8; ++b) T[b] = (b & 1 ? c[0] : s[0]) * (b & 2 ? c[1] : s[1]) * (b & 4 ? c[2] : s[2]);
+        const double* M = g.src24 + (size_t)((int)(K % 24) * 6 + g.sub_cls[t]) * 8 * nb;
+        for (int a = 0; a < nb; ++a) {
+            double v = 0.0;
+#pragma unroll
+            for (int b = 0; b < 8; ++b) v = fma(T[b], M[8 * a + b], v);
+            PL[t * nb + a] = v;
+        }
+    }
+    __syncthreads();
+    for (int w = threadIdx.x; w < g.n; w += blockDim.x) {
+        double v = 0.0;
+        for (int e = g.inc_off[w]; e < g.inc_off[w + 1]; ++e) v += PL[g.inc_ent[e]];
+        src[w] = v;
+    }
+    __syncthreads();
+}
+
+// Entering rows of the frontal elimination (front_plan_3d's tables): couplings from kappa
+// and the class matrices S, loads -s (psi_j, phi_w) - (1^T g / |K|) m_w from the face counts.
+template <int VEC>
+struct FrontRows3D {
+    static constexpr int C = VEC / 32;
+    const Local3DArgs& g;
+    const double *kap, *S, *src;   // src NULL: constant source
+    double vol;
+    double cp[C], cf[C];           // projection coefficient x |K|; -s area / (3 N^2)
+    int base[C];                   // first face count of the column, -1: no face
+    __device__ __forceinline__ void prep(int, const int4& v, double* nb, double* wnew) {
+        const int lane = threadIdx.x & 31, zs = (v.x >> 8) & 255, R = g.R;
+        if (zs == mhm::kNoSlot) return;
+        const double mt = g.mass1[v.y];
+        mhm::static_for<C>([&](auto k) {
+            const int q = lane + 32 * k;
+            double x = 0.0;
+            if (q < R) {
+                x = -cp[k] * mt;
+                if (q == g.NI) {
+                    x = src ? x + src[v.y] : fma(g.src_value * vol, mt, x);
+                } else {
+                    const int cnt = g.fcnt[base[k] + v.y * g.m];
+                    // (cnt as a double without a conversion: 2^52 + cnt - 2^52)
+                    if (cnt) x = fma(cf[k], __hiloint2double(0x43300000, cnt) - 4503599627370496.0, x);
+                }
             }
+            nb[q] = x;
+        });
+        if (lane == 0) *wnew = 0.0;
+        __syncwarp();
+        for (int q = lane; q < ((v.w + 31) & ~31); q += 32) {
+            const uint32_t en = q < v.w ? g.ent[v.z + q] : mhm::kNoSlot;
+            const int sl = en & 255, terms = (en >> 8) & 255;
+            const uint32_t* con = g.con + (en >> 16);
+            double x = 0.0;
+            for (int i = 0; i < terms; ++i) x = fma(kap[con[i] & 0xffff], S[con[i] >> 16], x);
+            if (q < 32) {   // the first eight: the diagonal
+                double d = sl == mhm::kDiagSlot ? x : 0.0;
+                d += __shfl_xor_sync(0xffffffffu, d, 1);
+                d += __shfl_xor_sync(0xffffffffu, d, 2);
+                d += __shfl_xor_sync(0xffffffffu, d, 4);
+                if (lane == 0) nb[R + zs] = d;
+            }
+            if (sl < mhm::kDiagSlot) nb[R + sl] = x;
+            else if (sl == mhm::kPivotSlot) *wnew = x;
+        }
+    }
+};
+
+struct Front3Smem {
+    int S, kap, src, PL, total;   // doubles
+};
+__host__ __device__ inline Front3Smem front3_smem(int vec, int n, int nb, int nsub, bool source) {
+    Front3Smem l;
+    int o = (int)mhm::front_shared_doubles(vec);
+    l.S = o, o += 6 * nb * nb;
+    l.kap = o, o += nsub;
+    l.src = o, o += source ? n : 0;
+    l.PL = o, o += source ? nsub * nb : 0;
+    l.total = o;
+    return l;
+}
+
+// FP64: one block per coarse tetrahedron at a time eliminates the pinned matrix bordered by
+// its R loads from a front of at most 42 slots (P2, r = 2: 165 DOFs) held in registers
+// (front.cuh); what is left of the border are the face integrals.  Bound by the FP64 pipe.
+template <class T, int MINB>
+__global__ void __launch_bounds__(T::threads, MINB) k_local3d(const __grid_constant__ Local3DArgs g) {
+    extern __shared__ double sm[];
+    __shared__ int bad;
+    __shared__ double FKs;
+    const int tid = threadIdx.x, nthr = blockDim.x, n = g.n, nb = g.nb, NI = g.NI, R = g.R, m = g.m;
+    const Front3Smem L = front3_smem(T::vec, n, nb, g.nsub, g.src24 != nullptr);
+    const mhm::FrontShared sh = mhm::front_shared(sm, T::vec);
+    double *S = sm + L.S, *kap = sm + L.kap, *src = sm + L.src;
+    for (int64_t K = g.K0 + blockIdx.x; K < g.K1; K += gridDim.x) {
+        if (g.only_failed && g.status[K] == MHM_OK) continue;   // (the whole block)
+        const double* geo = g.geo24 + 8 * (K % 24);
+        const double vol = geo[0];
+        for (int t = tid; t < 6 * nb * nb; t += nthr) S[t] = g.cls24[(size_t)(K % 24) * 6 * nb * nb + t];
+        for (int t = tid; t < g.nsub; t += nthr) kap[t] = g.kappa[K * (int64_t)g.nsub + t];
+        if (tid == 0) bad = 0;
+        if (g.src24) source_loads3(g, K, sm + L.PL, src);
+        if (tid < 32) {
+            double f = 0.0;
+            if (g.src24) {
+                for (int w = tid; w < n; w += 32) f += src[w];
+                f = warp_sum(f);
+            } else {
+                f = g.src_value * vol;
+            }
+            if (tid == 0) FKs = f;
+        }
+        __syncthreads();
+        // (psi_j, 1)_{dK} of column j: s |subface|; the projection is its negative over |K|
+        auto moment = [&](int j) {
+            const int a = j / m, q = j % m, b0 = (a * 6 + g.perm[4 * K + a]) * (m + 1) + q;
+            int c = 0;
+            for (int e = g.ftab_off[b0]; e < g.ftab_off[b0 + 1]; ++e) c += g.ftab_cnt[e];
+            return (double)g.signs[4 * K + a] * geo[1 + a] * c;
+        };
+        FrontRows3D<T::vec> rows{g, kap, S, g.src24 ? src : nullptr, vol};
+        mhm::static_for<T::vec / 32>([&](auto k) {
+            const int q = (tid & 31) + 32 * k;
+            rows.cp[k] = rows.cf[k] = 0.0;
+            rows.base[k] = 0;
+            if (q < NI) {
+                const int a = q / m;
+                rows.cp[k] = -moment(q);
+                rows.cf[k] = -(double)g.signs[4 * K + a] * geo[1 + a];
+                rows.base[k] = (a * 6 + g.perm[4 * K + a]) * n * m + q % m;
+            } else if (q == NI) {
+                rows.cp[k] = FKs;
+            }
+        });
+        double A[T::NT];
+        mhm::front_eliminate<T>(rows, g.ev, g.steps, R, sh, A, &bad, nullptr, 0);
+        double* AK = g.AK + K * (int64_t)NI * NI;
+        mhm::front_result<T>(R, A, [&](int i, int j, double v) {
+            if (i < NI) {
+                AK[i * NI + j] = v;
+                AK[j * NI + i] = v;
+            } else if (j < NI) {
+                g.EK[K * NI + j] = -v;
+            }
+        });
+        for (int j = tid; j < NI; j += nthr) g.BK[K * NI + j] = moment(j);
+        if (tid == 0) {
+            g.FK[K] = FKs;
+            g.status[K] = bad ? MHM_ERR_INVALID_ARG : MHM_OK;
+            if (g.iters) g.iters[K] = g.only_failed ? -1 : 1;
         }
         __syncthreads();
     }
-    // ---- face integrals by the Gram form.  With Y = L^{-1} g~ over the pinned rows,
-    // (s psi_j, eta_i)_{dK} = -N_j^T eta_i = -N~_j^T z_i = -Y_j . Y_i: the zero-mean shift of
-    // eta_i cancels against the compatibility projection of N_j (N~_j^T 1 = 0), and z_i
-    // vanishes on the pinned DOF.  Likewise -(s psi_j, eta_f)_{dK} = Y_j . y_f.  No backward
-    // substitution is needed.
-    double* AK = g.AK + K * (int64_t)NI * NI;
-    const int pairs = NI * (NI + 1) / 2;   // each pair i <= j once, then the E_K entries (i = N_I)
-    for (int it = tid; it < pairs + NI; it += nthr) {
-        const int j = it < pairs ? tri_row(it) : it - pairs, i = it < pairs ? it - j * (j + 1) / 2 : NI;
-        double s = 0.0;
-        for (int w = 1; w < n; ++w) s += Y[w * R + j] * Y[w * R + i];
-        if (i == NI) {
-            g.EK[K * NI + j] = s;
-        } else {
-            AK[j * NI + i] = -s;
-            AK[i * NI + j] = -s;
-        }
-    }
-    element_tail(g, K, misc, misc[7] != 0.0 ? MHM_ERR_INVALID_ARG : MHM_OK, g.only_failed ? -1 : 1);
+}
+
+// The frontal kernel of a bordered matrix of M rows.
+struct Front3Kernel {
+    void (*kern)(const Local3DArgs) = nullptr;
+    int threads = 0, vec = 0;
+};
+template <class T, int MINB>
+void front3_try(int M, Front3Kernel* k) {
+    if (k->kern || M > T::rows) return;
+    k->kern = k_local3d<T, MINB>;
+    k->threads = T::threads;
+    k->vec = T::vec;
+}
+Front3Kernel front3_kernel(int M) {
+    Front3Kernel k;
+    front3_try<mhm::FrontTiles<1, 1, 8>, 12>(M, &k);
+    front3_try<mhm::FrontTiles<1, 1, 12>, 12>(M, &k);
+    front3_try<mhm::FrontTiles<1, 1, 15>, 8>(M, &k);
+    front3_try<mhm::FrontTiles<4, 1, 7>, 2>(M, &k);
+    return k;
 }
 
 // Mixed precision (Sec. 3: the local matrix is factored once and each further solve is
@@ -670,10 +808,92 @@ mhm_status upload3(const std::vector<T>& h, T** d) {
     return MHM_OK;
 }
 
+// Tables of the frontal elimination: step tables; per element type (the 24 tetrahedra of a
+// cube: every other element is a translate) the class matrices in closed form, |K| and the
+// face areas; mass per DOF; face counts per local face, permutation, DOF and subface.
+mhm_status upload_front_tables(mhm_mesh3d* m) {
+    const int nb = m->nb, n = (int)m->n, N = m->N, mm = m->desc.m, P = m->desc.degree;
+    const mhm::FrontPlan3 plan = mhm::front_plan_3d(n, nb, m->sub_dofs, m->sub_cls, m->nodes, (int)m->NI + 1);
+    m->fsteps = plan.steps;
+    m->fslots = plan.slots;
+    std::vector<double> cls((size_t)24 * 6 * nb * nb), geo(24 * 8, 0.0), mass(n, 0.0);
+    for (int t = 0; t < 24; ++t) {
+        const double* V = &m->geom[12 * t];
+        double E[3][3];   // edge vectors along the path of the Freudenthal simplex
+        for (int k = 0; k < 3; ++k)
+            for (int c = 0; c < 3; ++c) E[k][c] = V[3 * (k + 1) + c] - V[3 * k + c];
+        auto cross = [](const double* u, const double* v, double* w) {
+            w[0] = u[1] * v[2] - u[2] * v[1], w[1] = u[2] * v[0] - u[0] * v[2], w[2] = u[0] * v[1] - u[1] * v[0];
+        };
+        double x[3];
+        cross(E[1], E[2], x);
+        geo[8 * t] = std::fabs(E[0][0] * x[0] + E[0][1] * x[1] + E[0][2] * x[2]) / 6.0;
+        for (int a = 0; a < 4; ++a) {
+            int b[3], k = 0;
+            for (int v = 0; v < 4; ++v)
+                if (v != a) b[k++] = v;
+            double u[3], w[3];
+            for (int c = 0; c < 3; ++c) u[c] = V[3 * b[1] + c] - V[3 * b[0] + c], w[c] = V[3 * b[2] + c] - V[3 * b[0] + c];
+            cross(u, w, x);
+            geo[8 * t + 1 + a] = 0.5 * std::sqrt(x[0] * x[0] + x[1] * x[1] + x[2] * x[2]) / ((double)N * N) / 3.0;
+        }
+        const double Vs = geo[8 * t] / ((double)N * N * N);
+        for (int c = 0; c < 6; ++c) {
+            double J[3][3], G[4][3];   // vertices of the class's path from its first; gradients of the barycentrics
+            for (int v = 0; v < 3; ++v)
+                for (int k = 0; k < 3; ++k) J[v][k] = (v ? J[v - 1][k] : 0.0) + E[kPath[c][v]][k] / N;
+            const double* e[3] = {J[0], J[1], J[2]};
+            for (int v = 0; v < 3; ++v) {
+                cross(e[(v + 1) % 3], e[(v + 2) % 3], x);
+                const double d = e[v][0] * x[0] + e[v][1] * x[1] + e[v][2] * x[2];
+                for (int k = 0; k < 3; ++k) G[v + 1][k] = x[k] / d;
+            }
+            for (int k = 0; k < 3; ++k) G[0][k] = -(G[1][k] + G[2][k] + G[3][k]);
+            auto d = [&](int i, int j) { return G[i][0] * G[j][0] + G[i][1] * G[j][1] + G[i][2] * G[j][2]; };
+            // int grad phi_a . grad phi_b from int l_a l_b = Vs (1 + [a = b]) / 20 (P2 edges 4 l_a l_b)
+            static const int ed[6][2] = {{0, 1}, {0, 2}, {0, 3}, {1, 2}, {1, 3}, {2, 3}};
+            double* S = &cls[((size_t)t * 6 + c) * nb * nb];
+            for (int a = 0; a < nb; ++a)
+                for (int b = 0; b < nb; ++b) {
+                    double v;
+                    if (P == 1) {
+                        v = d(a, b);
+                    } else if (a < 4 && b < 4) {
+                        v = d(a, b) * (a == b ? 0.6 : -0.2);
+                    } else if (a < 4 || b < 4) {
+                        const int q = std::min(a, b), j = ed[std::max(a, b) - 4][0], k = ed[std::max(a, b) - 4][1];
+                        v = 4.0 * (d(q, k) * (q == j ? 0.15 : -0.05) + d(q, j) * (q == k ? 0.15 : -0.05));
+                    } else {
+                        const int i = ed[a - 4][0], j = ed[a - 4][1], k = ed[b - 4][0], l = ed[b - 4][1];
+                        v = 0.8 * (d(j, l) * (1 + (i == k)) + d(j, k) * (1 + (i == l)) + d(i, l) * (1 + (j == k)) +
+                                   d(i, k) * (1 + (j == l)));
+                    }
+                    S[a * nb + b] = Vs * v;
+                }
+        }
+    }
+    const double per[2] = {P == 1 ? 0.25 : -0.05, 0.2};   // int phi over a tetrahedron of unit volume: vertices, edges
+    for (int w = 0; w < n; ++w)
+        for (int e = m->inc_off[w]; e < m->inc_off[w + 1]; ++e) mass[w] += per[m->inc_ent[e] % nb >= 4] / ((double)N * N * N);
+    std::vector<uint8_t> cnt((size_t)24 * n * mm, 0);
+    for (int b = 0; b < 24; ++b)
+        for (int q = 0; q < mm; ++q)
+            for (int e = m->ftab_off[b * (mm + 1) + q]; e < m->ftab_off[b * (mm + 1) + q + 1]; ++e)
+                cnt[((size_t)b * n + m->ftab_node[e]) * mm + q] = (uint8_t)m->ftab_cnt[e];
+    mhm_status st = upload3(plan.ev, (int32_t**)&m->d_fev);
+    if (!st) st = upload3(plan.ent, &m->d_fent);
+    if (!st) st = upload3(plan.con, &m->d_fcon);
+    if (!st) st = upload3(cls, &m->d_cls24);
+    if (!st) st = upload3(geo, &m->d_geo24);
+    if (!st) st = upload3(mass, &m->d_mass1);
+    if (!st) st = upload3(cnt, &m->d_fcnt);
+    return st;
+}
+
 void free_device(mhm_mesh3d* m) {
     void* ptrs[] = {m->d_geom, m->d_signs, m->d_perm, m->d_sub_dofs, m->d_sub_cls, m->d_sub_base, m->d_ftab_off,
                     m->d_ftab_node, m->d_ftab_cnt, m->d_quad, m->d_rowptr, m->d_nbrs, m->d_face_ka, m->d_inc_off,
-                    m->d_inc_ent};
+                    m->d_inc_ent, m->d_fev, m->d_fent, m->d_fcon, m->d_cls24, m->d_geo24, m->d_mass1, m->d_fcnt};
     for (void* p : ptrs)
         if (p) cudaFree(p);
 }
@@ -686,7 +906,7 @@ int local3d_qsplit(int nsub) {
     return qs;
 }
 size_t local3d_smem(int n, int NI, int nb, int nsub) {
-    return (size_t)smem_layout(n, NI, nb, nsub, local3d_qsplit(nsub)).total * sizeof(double);
+    return dense_doubles(n, NI, nb, nsub, local3d_qsplit(nsub)) * sizeof(double);
 }
 size_t local3d_smem_mixed(int n, int NI, int nb, int nsub) {
     return (size_t)smem_layout_mixed(n, NI, nb, nsub, local3d_qsplit(nsub)).total * sizeof(double);
@@ -755,6 +975,7 @@ extern "C" mhm_status mhm3d_create_mesh(const mhm3d_mesh_desc* desc, int32_t dev
         if (!st) st = upload3(m->rowptr, &m->d_rowptr);
         if (!st) st = upload3(m->nbrs, &m->d_nbrs);
         if (!st) st = upload3(m->face_ka, &m->d_face_ka);
+        if (!st) st = upload_front_tables(m);
         if (st) {
             free_device(m);
             delete m;
@@ -834,6 +1055,9 @@ extern "C" mhm_status mhm3d_local_solve_batch(const mhm3d_mesh* m, const double*
     g.quad = m->d_quad, g.kappa = kappa;
     g.src_kind = f->kind, g.src_value = f->value, g.src_freq = f->freq;
     g.K0 = K0;
+    g.K1 = K1;
+    g.ev = m->d_fev, g.ent = m->d_fent, g.con = m->d_fcon, g.steps = m->fsteps;
+    g.cls24 = m->d_cls24, g.geo24 = m->d_geo24, g.mass1 = m->d_mass1, g.fcnt = m->d_fcnt;
     g.N = m->N, g.P = m->desc.degree, g.n = (int)m->n, g.nb = m->nb, g.nsub = (int)m->nsub, g.m = m->desc.m;
     g.NI = (int)m->NI, g.R = (int)m->NI + 1;
     g.AK = AK, g.EK = EK, g.BK = BK, g.FK = FK, g.status = status, g.iters = iters;
@@ -842,7 +1066,6 @@ extern "C" mhm_status mhm3d_local_solve_batch(const mhm3d_mesh* m, const double*
     cudaStream_t s = (cudaStream_t)stream;
     // the shared-memory attribute is per kernel, not per mesh: set it for this mesh every call
     g.qs = local3d_qsplit(g.nsub);
-    const size_t smem64 = local3d_smem(g.n, g.NI, g.nb, g.nsub);
     const size_t smemmx = local3d_smem_mixed(g.n, g.NI, g.nb, g.nsub);
     const bool mixed = precision == MHM_MIXED && smemmx <= 227 * 1024;
     if (mixed) {
@@ -852,9 +1075,28 @@ extern "C" mhm_status mhm3d_local_solve_batch(const mhm3d_mesh* m, const double*
         if (o.no_fallback) return MHM_OK;
         g.only_failed = 1;   // the elements the refinement could not finish, again in FP64
     }
-    MHM_CUDA_TRY(cudaFuncSetAttribute(k_local3d, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem64));
-    k_local3d<<<grid, kThreads, smem64, s>>>(g);
-    MHM_CUDA_TRY(cudaGetLastError());
+    // FP64: frontal elimination; the source tables in a stream-ordered scratch of this call
+    const Front3Kernel k = front3_kernel(g.R + m->fslots);
+    if (!k.kern) return mhm::fail(MHM_ERR_UNSUPPORTED, "mhm3d_local_solve_batch: front too large");
+    double* tables = nullptr;
+    if (f->kind == MHM3D_SRC_SINSINSIN) {
+        MHM_CUDA_TRY(cudaMallocAsync((void**)&tables, (size_t)24 * 6 * 8 * g.nb * sizeof(double), s));
+        k_source3d<<<24 * 6, kQuad, 0, s>>>(m->d_geom, m->d_quad, g.N, g.nb, f->value, f->freq, tables);
+        g.src24 = tables;
+    }
+    const size_t smem = (size_t)front3_smem(k.vec, g.n, g.nb, g.nsub, tables != nullptr).total * sizeof(double);
+    int sms = 0, per_sm = 0;
+    cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, m->device);
+    cudaError_t e = cudaFuncSetAttribute(k.kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    if (e == cudaSuccess) e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k.kern, k.threads, smem);
+    if (e == cudaSuccess) {
+        // one wave of blocks that share the elements out evenly
+        const int64_t each = (K1 - K0 + sms - 1) / sms, rounds = (each + std::max(per_sm, 1) - 1) / std::max(per_sm, 1);
+        k.kern<<<(unsigned)std::min<int64_t>(K1 - K0, sms * ((each + rounds - 1) / rounds)), k.threads, smem, s>>>(g);
+        e = cudaGetLastError();
+    }
+    if (tables) cudaFreeAsync(tables, s);
+    if (e != cudaSuccess) return mhm::cuda_fail(e, "mhm3d_local_solve_batch: launch");
     return MHM_OK;
 }
 

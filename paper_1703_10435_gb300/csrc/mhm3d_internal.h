@@ -84,6 +84,12 @@ struct mhm_mesh3d {
     int32_t* d_rowptr = nullptr;
     mhm3::Nbr3* d_nbrs = nullptr;
     int32_t* d_face_ka = nullptr;
+    // frontal elimination (front_plan.h, local3d.cu: upload_front_tables)
+    int fsteps = 0, fslots = 0;
+    int4* d_fev = nullptr;
+    uint32_t *d_fent = nullptr, *d_fcon = nullptr;
+    double *d_cls24 = nullptr, *d_geo24 = nullptr, *d_mass1 = nullptr;
+    uint8_t* d_fcnt = nullptr;
 };
 
 namespace mhm3 {
