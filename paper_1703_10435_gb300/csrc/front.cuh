@@ -76,14 +76,16 @@ struct FrontTiles {
     // first block row that holds entries of block column b
     static constexpr int first(int b) { return (8 * WC * b) / (4 * WR); }
 };
-// Shared memory of one element: pivot column, scaled pivot column and entering row (two of
+// Shared memory of one element (F values): pivot column, scaled pivot column and entering row (two of
 // each, used in turn), a row of zeros, the inverse pivots and the pivots' couplings.
+template <class F>
 struct FrontShared {
-    double *w[2], *s[2], *nb[2], *zero, *piv;
+    F *w[2], *s[2], *nb[2], *zero, *piv;
 };
-__host__ __device__ constexpr size_t front_shared_doubles(int vec) { return 7 * (size_t)vec + 4; }
-__device__ __forceinline__ FrontShared front_shared(double* base, int v) {
-    FrontShared f;
+__host__ __device__ constexpr size_t front_shared_values(int vec) { return 7 * (size_t)vec + 4; }
+template <class F>
+__device__ __forceinline__ FrontShared<F> front_shared(F* base, int v) {
+    FrontShared<F> f;
     for (int k = 0; k < 2; ++k) f.w[k] = base + k * v, f.s[k] = base + (2 + k) * v, f.nb[k] = base + (4 + k) * v;
     f.zero = base + 6 * v;
     f.piv = base + 7 * v;   // inverse pivot per parity; then the pivot's coupling with the entering node
@@ -99,6 +101,8 @@ __device__ __forceinline__ double front_rcp(double d) {
     return fma(t, y, y);
 }
 
+__device__ __forceinline__ float front_rcp(float d) { return 1.0f / d; }
+
 template <int NW> __device__ __forceinline__ void front_sync() {
     if (NW == 1) __syncwarp();
     else __syncthreads();
@@ -108,20 +112,21 @@ template <int NW> __device__ __forceinline__ void front_sync() {
 // prob.prep(e, ev[e], nb, wnew) is called by one warp for every step in order: it fills nb
 // (T::vec entries) with the row of step e's entering node against the loads and the front
 // as the step leaves it, zero elsewhere, and *wnew with its coupling to the pivot.  keep (NULL: none) gets the scaled
-// pivot column of every step, `stride` doubles apart.  *bad: 1 if a pivot was not positive.
+// pivot column of every step, `stride` values apart, and kinv (NULL: none) the inverse pivots;
+// both start at step e0, the first that has a pivot.  *bad: 1 if a pivot was not positive.
 // A: the entries; the result is read with front_result.  All warps of the element call it;
 // starts and ends with a barrier.
-template <class T, class Prob>
+template <class T, class F, class Prob>
 __device__ __forceinline__ void front_eliminate(Prob& prob, const int4* __restrict__ ev, int steps, int R,
-                                                const FrontShared& sh, double (&A)[T::NT], int* bad, double* keep,
-                                                int stride) {
+                                                const FrontShared<F>& sh, F (&A)[T::NT], int* bad, F* keep, int stride,
+                                                F* kinv = nullptr, int e0 = 0) {
     constexpr int WR = T::WR, WC = T::WC, NW = T::NW, AR = T::AR;
     const int tid = NW == 1 ? (int)(threadIdx.x & 31) : (int)threadIdx.x;
     const int warp = NW == 1 ? 0 : __shfl_sync(0xffffffffu, tid >> 5, 0), lane = tid & 31;
     const int row = 4 * (warp / WC) + (lane >> 3), col = 8 * (warp % WC) + (lane & 7);   // inside a block
 #pragma unroll
-    for (int q = 0; q < T::NT; ++q) A[q] = 0.0;
-    for (int t = tid; t < 7 * T::vec; t += T::threads) sh.w[0][t] = 0.0;
+    for (int q = 0; q < T::NT; ++q) A[q] = F(0);
+    for (int t = tid; t < 7 * T::vec; t += T::threads) sh.w[0][t] = F(0);
     front_sync<NW>();
     int4 v = ev[0];
     if (NW > 1 && warp == NW) {
@@ -146,9 +151,9 @@ __device__ __forceinline__ void front_eliminate(Prob& prob, const int4* __restri
         const int ps = v.x & 255, zs = (v.x >> 8) & 255, mm = R + ((v.x >> 16) & 255);
         if (e + 1 < steps) v = ev[e + 1];
         const int P = ps == kNoSlot ? -1 : R + ps, Z = zs == kNoSlot ? -1 : R + zs;
-        double* w = sh.w[par];
-        double* s = sh.s[par];
-        const double* nb = sh.nb[par];
+        F* w = sh.w[par];
+        F* s = sh.s[par];
+        const F* nb = sh.nb[par];
         // the pivot's row and column to w, then those of the entering node from nb (a slot
         // left free goes to zero and stays there)
         auto cross = [&](int X, auto&& fn) {   // fn(entry, other index) on row and column X
@@ -171,47 +176,48 @@ __device__ __forceinline__ void front_eliminate(Prob& prob, const int4* __restri
             });
         };
         if (P >= 0) {
-            const double* in = Z == P ? nb : sh.zero;
-            cross(P, [&](double& x, int k) {
+            const F* in = Z == P ? nb : sh.zero;
+            cross(P, [&](F& x, int k) {
                 w[k] = x;
                 if (NW > 1 && k == P) {
-                    if (!(x > 0.0)) *bad = 1;
+                    if (!(x > F(0))) *bad = 1;
                     sh.piv[par] = front_rcp(x);
                 }
                 x = in[k];
             });
         }
-        if (Z >= 0 && Z != P) cross(Z, [&](double& x, int k) { x = nb[k]; });
+        if (Z >= 0 && Z != P) cross(Z, [&](F& x, int k) { x = nb[k]; });
         front_sync<NW>();
-        double inv = 0.0;
+        F inv = F(0);
         if (NW == 1 && P >= 0) {   // (read by all lanes before w[P] changes)
-            const double d = w[P];
-            if (!(d > 0.0)) *bad = 1;
+            const F d = w[P];
+            if (!(d > F(0))) *bad = 1;
             inv = front_rcp(d);
         }
         if (NW == 1 && e + 1 < steps) prob.prep(e + 1, v, sh.nb[par ^ 1], sh.piv + 2 + (par ^ 1));
         if (NW == 1) __syncwarp();
         if (P >= 0) {
-            const double wnew = sh.piv[2 + par];
+            const F wnew = sh.piv[2 + par];
             if (NW > 1) inv = sh.piv[par];
             // whole blocks: rows past the ones in use get zeros
             const int top = (mm + 8 * WC - 1) / (8 * WC) * (8 * WC);
             for (int q = tid; q < top; q += 32 * NW) {
-                double x = q == Z ? wnew : (q == P || q >= mm) ? 0.0 : w[q];
+                F x = q == Z ? wnew : (q == P || q >= mm) ? F(0) : w[q];
                 if (q == Z || q == P || q >= mm) w[q] = x;
                 x *= inv;
                 s[q] = x;
-                if (keep && q < mm) keep[(size_t)e * stride + q] = x;
+                if (keep && q < mm) keep[(size_t)(e - e0) * stride + q] = x;
             }
+            if (kinv && tid == 0) kinv[e - e0] = inv;
         }
         if (NW == 1 || P >= 0) front_sync<NW>();
         if (P >= 0) {
-            double wb[T::NB];
-            static_for<T::NB>([&](auto b) { wb[b] = 8 * WC * b < mm ? w[8 * WC * b + col] : 0.0; });
+            F wb[T::NB];
+            static_for<T::NB>([&](auto b) { wb[b] = 8 * WC * b < mm ? w[8 * WC * b + col] : F(0); });
             // rows of blocks with this warp's rows in use
             static_upto<0, AR>((mm - 4 * (warp / WC) + 4 * WR - 1) / (4 * WR), [&](auto ca) {
                 constexpr int a = ca;
-                const double sa = s[4 * WR * a + row];
+                const F sa = s[4 * WR * a + row];
                 static_for<T::cols(a)>([&](auto cb) {
                     constexpr int b = cb;
                     A[T::at(a) + b] = fma(-sa, wb[b], A[T::at(a) + b]);
@@ -223,8 +229,8 @@ __device__ __forceinline__ void front_eliminate(Prob& prob, const int4* __restri
 }
 
 // Calls fn(i, j, value) for this thread's entries i >= j of the leading R x R block.
-template <class T, class F>
-__device__ __forceinline__ void front_result(int R, const double (&A)[T::NT], F&& fn) {
+template <class T, class Fn>
+__device__ __forceinline__ void front_result(int R, const double (&A)[T::NT], Fn&& fn) {
     const int tid = T::NW == 1 ? (int)(threadIdx.x & 31) : (int)threadIdx.x, warp = tid >> 5, lane = tid & 31;
     if (warp >= T::NW) return;
     const int row = 4 * (warp / T::WC) + (lane >> 3), col = 8 * (warp % T::WC) + (lane & 7);

@@ -193,10 +193,14 @@ FrontPlan3 front_plan_3d(int n, int nb, const std::vector<int32_t>& dofs, const 
     }
     if (plan.slots > kMaxSlots) return FrontPlan3{};
     plan.steps = (int)steps.size();
+    while (steps[plan.first_pivot].pivot < 0) ++plan.first_pivot;
     std::vector<int> slot(n1, -1);
+    std::vector<uint32_t> diag(n1, 0);
+    std::vector<std::vector<std::array<int, 2>>> rows(n1);
     for (const FrontStep& st : steps) {
         const int v = st.enter, first = (int)plan.ent.size();
         if (v >= 0) {
+            diag[v] = (uint32_t)plan.con.size() | (uint32_t)inc[v].size() << 16;
             for (int part = 0; part < 8; ++part) {   // the diagonal: every eighth incident tetrahedron
                 const size_t c0 = plan.con.size();
                 for (size_t k = part; k < inc[v].size(); k += 8) {
@@ -216,16 +220,29 @@ FrontPlan3 front_plan_3d(int n, int nb, const std::vector<int32_t>& dofs, const 
                             plan.con.push_back(t | (uint32_t)((cls[t] * nb + a) * nb + b) << 16);
                         }
                 plan.ent.push_back(sl | (uint32_t)(plan.con.size() - c0) << 8 | (uint32_t)c0 << 16);
+                rows[v].push_back({u, (int)plan.val.size()});
+                rows[u].push_back({v, (int)plan.val.size()});
+                plan.val.push_back((uint32_t)c0 | (uint32_t)(plan.con.size() - c0) << 16);
+                plan.rc.push_back(v | (uint32_t)u << 16);
             }
         }
         plan.ev.push_back(st.ps | st.zs << 8 | st.m << 16);
         plan.ev.push_back(v >= 0 ? v + 1 : -1);
         plan.ev.push_back(first);
-        plan.ev.push_back((int)plan.ent.size() - first);
+        plan.ev.push_back(((int)plan.ent.size() - first) | (st.pivot >= 0 ? st.pivot << 16 : 0));
         if (st.pivot >= 0) slot[st.pivot] = -1;
         if (v >= 0) slot[v] = st.zs;
     }
     if (plan.con.size() > 0xffff) return FrontPlan3{};
+    plan.off = (int)plan.val.size();
+    for (int v = 0; v < n1; ++v) {
+        rows[v].push_back({v, plan.off + v});
+        std::sort(rows[v].begin(), rows[v].end());
+        plan.rp.push_back((int)plan.col.size());
+        for (const auto& q : rows[v]) plan.col.push_back(q[0] | (uint32_t)q[1] << 16);
+        plan.val.push_back(diag[v]);
+    }
+    plan.rp.push_back((int)plan.col.size());
     return plan;
 }
 

@@ -47,10 +47,15 @@ FrontPlan front_plan_2d(int P, int N);
 // entries.  ent: slot | terms << 8 | first term << 16, the first 8 of a node the parts of its
 // diagonal; the value of an entry is the sum of its terms kappa[t] S[s] (con: t | s << 16,
 // s = (class nb + a) nb + b).  Of three orders the one with the least work for R loads.
+// The fourth value of a step also holds the pivot's node (DOF - 1) << 16; first_pivot: the
+// first step that has one.  For products with the matrix: val: first term | terms << 16 of
+// every off-diagonal value (in the order of the entries), then of every node's diagonal;
+// rc: the off-diagonal values' nodes v | u << 16; rp, col: per node its row, as
+// neighbour | value << 16.
 struct FrontPlan3 {
-    int steps = 0, slots = 0;
-    std::vector<int32_t> ev;
-    std::vector<uint32_t> ent, con;
+    int steps = 0, slots = 0, first_pivot = 0, off = 0;
+    std::vector<int32_t> ev, rp;
+    std::vector<uint32_t> ent, con, val, rc, col;
 };
 FrontPlan3 front_plan_3d(int n, int nb, const std::vector<int32_t>& dofs, const std::vector<int8_t>& cls,
                          const std::vector<int32_t>& xyz, int R);

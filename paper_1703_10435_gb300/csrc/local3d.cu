@@ -27,7 +27,6 @@ struct Local3DArgs {
     const double* geom;
     const int8_t* signs;
     const int8_t* perm;
-    const int32_t* sub_dofs;
     const int8_t* sub_cls;
     const int8_t* sub_base;
     const int32_t* inc_off;   // per local DOF, its slots t nb + a (ascending)
@@ -35,12 +34,10 @@ struct Local3DArgs {
     const int32_t* ftab_off;
     const int16_t* ftab_node;
     const int8_t* ftab_cnt;
-    const double* quad;
     const double* kappa;
-    int src_kind;
     double src_value, src_freq;
     int64_t K0, K1;
-    int N, P, n, nb, nsub, m, NI, R;
+    int N, n, nb, nsub, m, NI, R;
     double* AK;
     double* EK;
     double* BK;
@@ -50,314 +47,27 @@ struct Local3DArgs {
     int only_failed;      // FP64 kernel: solve only the elements whose status is nonzero (iters -1)
     int it_max;           // mixed kernel: refinement passes
     double tol;           // mixed kernel: scaled residual target per column
-    int qs;               // the source's quadrature points of a sub-tetrahedron in qs groups of 64/qs
     // frontal elimination (front.cuh): step tables; per type of element (K mod 24: translates)
     // the six class matrices and vol, area_a / (3 N^2); mass of a DOF on a unit volume; fine
     // face triangles of subface q that load DOF w, per local face and permutation (x n x m)
     const int4* ev;
     const uint32_t *ent, *con;
-    int steps;
+    int steps, slots;
     const double *cls24, *geo24, *mass1;
     const uint8_t* fcnt;
     const double* src24;  // source tables per type, class, local DOF (k_source3d); NULL: constant
+    // mixed kernel: values and rows of the matrix (FrontPlan3)
+    const uint32_t *val, *rc, *col;
+    const int32_t* rp;
+    int first, off;
 };
 
 constexpr int kPath[6][3] = {{0, 1, 2}, {0, 2, 1}, {1, 0, 2}, {1, 2, 0}, {2, 0, 1}, {2, 1, 0}};
 __constant__ int c_perm[6][3] = {{0, 1, 2}, {0, 2, 1}, {1, 0, 2}, {1, 2, 0}, {2, 0, 1}, {2, 1, 0}};
-__constant__ int c_edges[6][2] = {{0, 1}, {0, 2}, {0, 3}, {1, 2}, {1, 3}, {2, 3}};
-
-// packed lower triangle, row i >= column j
-__device__ __forceinline__ int pk(int i, int j) { return i * (i + 1) / 2 + j; }
 
 __device__ __forceinline__ double warp_sum(double v) {
     for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
     return v;
-}
-
-__device__ __forceinline__ float warp_sumf(float v) {
-    for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
-    return v;
-}
-
-// Row of entry t of a packed lower triangle (t = row (row + 1) / 2 + col, col <= row).
-__device__ __forceinline__ int tri_row(int t) {
-    int r = (int)((sqrtf(8.0f * (float)t + 1.0f) - 1.0f) * 0.5f);
-    while (r * (r + 1) / 2 > t) --r;
-    while ((r + 1) * (r + 2) / 2 <= t) ++r;
-    return r;
-}
-
-// doubles of the source's partial loads: per group of quadrature points of every
-// sub-tetrahedron, its nb loads and its part of F_K
-__host__ __device__ inline int partial_loads(int nsub, int nb, int qs) { return qs * nsub * (nb + 1); }
-
-// Size of the dense problem in shared memory (packed pinned triangle or partial loads,
-// n x R columns, tables), which bounds the meshes that are accepted.
-inline size_t dense_doubles(int n, int NI, int nb, int nsub, int qs) {
-    const int R = NI + 1, n1 = n - 1, npk = n1 * (n1 + 1) / 2, pl = partial_loads(nsub, nb, qs);
-    return (size_t)(npk > pl ? npk : pl) + (size_t)n * R + n + 6 * nb * nb + 6 * 21 + R + 16;
-}
-
-// shared-memory layout of the mixed kernel (doubles; the FP32 factor and solve vectors
-// take half a double per value)
-struct Smem3M {
-    int Lf, G, Z, Rr, W, sc, dg, invf, mass, S6, G6, J6, red, gn, misc, total;
-};
-
-__host__ __device__ inline Smem3M smem_layout_mixed(int n, int NI, int nb, int nsub, int qs) {
-    const int R = NI + 1, n1 = n - 1, npk = n1 * (n1 + 1) / 2, pl = partial_loads(nsub, nb, qs);
-    Smem3M s{};
-    int o = 0;
-    s.Lf = o;   o += (npk + 1) / 2;                 // FP32 factor of the scaled pinned matrix
-    s.G = o;    o += n * R;                         // projected loads g~ (FP64)
-    s.Z = o;    o += n * R;                         // solutions (FP64)
-    s.Rr = o;   o += n * R > pl ? n * R : pl;       // the source's partial loads, then residuals g~ - A z
-    s.W = o;    o += (n1 * R + 1) / 2;              // FP32 preconditioner solves
-    s.sc = o;   o += n1;                            // 1 / sqrt(diag) of the pinned matrix
-    s.dg = o;   o += n;                             // FP64 diagonal
-    s.invf = o; o += (n1 + 1) / 2;                  // FP32 1 / L_kk
-    s.mass = o; o += n;
-    s.S6 = o;   o += 6 * nb * nb;
-    s.G6 = o;   o += 6 * 12;
-    s.J6 = o;   o += 6 * 9;
-    s.red = o;  o += R;
-    s.gn = o;   o += R;                             // |S g~|^2 per column
-    s.misc = o; o += 16;
-    s.total = o;
-    return s;
-}
-
-// Geometry of element K into shared memory: misc[0] = |K|, misc[1 + a] = |face a| / N^2,
-// misc[5] = |sub-tetrahedron|, misc[6] = F_K accumulator, misc[7] = failure flag,
-// misc[8] = done flag; per class c: edge vectors J6[9c + 3 comp + v] and the gradients of
-// the four barycentrics G6[12c + 3 l + comp].  No barrier.
-__device__ __forceinline__ void element_geometry(const Local3DArgs& g, const double* V, double* misc, double* G6,
-                                                 double* J6) {
-    const int tid = threadIdx.x, N = g.N;
-    if (tid == 0) {
-        double e[3][3];
-        for (int c = 0; c < 3; ++c)
-            for (int k = 0; k < 3; ++k) e[k][c] = V[3 * (k + 1) + c] - V[c];
-        const double det = e[0][0] * (e[1][1] * e[2][2] - e[1][2] * e[2][1]) -
-                           e[0][1] * (e[1][0] * e[2][2] - e[1][2] * e[2][0]) +
-                           e[0][2] * (e[1][0] * e[2][1] - e[1][1] * e[2][0]);
-        misc[0] = fabs(det) / 6.0;
-        misc[5] = misc[0] / ((double)N * N * N);
-        misc[6] = 0.0;
-        misc[7] = 0.0;
-        misc[8] = 0.0;
-    }
-    if (tid < 4) {   // area of local face a over N^2
-        int b[3], k = 0;
-        for (int v = 0; v < 4; ++v)
-            if (v != tid) b[k++] = v;
-        double u[3], w[3];
-        for (int c = 0; c < 3; ++c) u[c] = V[3 * b[1] + c] - V[3 * b[0] + c], w[c] = V[3 * b[2] + c] - V[3 * b[0] + c];
-        const double cx = u[1] * w[2] - u[2] * w[1], cy = u[2] * w[0] - u[0] * w[2], cz = u[0] * w[1] - u[1] * w[0];
-        misc[1 + tid] = 0.5 * sqrt(cx * cx + cy * cy + cz * cz) / ((double)N * N);
-    }
-    if (tid < 6) {   // class tid: edge vectors X_v - X_0 = D p_v / N and barycentric gradients
-        double D[3][3];   // columns: v1 - v0, v2 - v1, v3 - v2
-        for (int c = 0; c < 3; ++c) {
-            D[c][0] = V[3 + c] - V[c];
-            D[c][1] = V[6 + c] - V[3 + c];
-            D[c][2] = V[9 + c] - V[6 + c];
-        }
-        int p[3] = {0, 0, 0};
-        double J[3][3];   // J[c][v]: component c of edge vector v
-        for (int v = 0; v < 3; ++v) {
-            p[c_perm[tid][v]] += 1;
-            for (int c = 0; c < 3; ++c) J[c][v] = (D[c][0] * p[0] + D[c][1] * p[1] + D[c][2] * p[2]) / N;
-        }
-        for (int c = 0; c < 3; ++c)
-            for (int v = 0; v < 3; ++v) J6[tid * 9 + 3 * c + v] = J[c][v];
-        const double det = J[0][0] * (J[1][1] * J[2][2] - J[1][2] * J[2][1]) -
-                           J[0][1] * (J[1][0] * J[2][2] - J[1][2] * J[2][0]) +
-                           J[0][2] * (J[1][0] * J[2][1] - J[1][1] * J[2][0]);
-        const double id = 1.0 / det;
-        // rows of J^{-1} are the gradients of the barycentrics l1, l2, l3
-        double Ji[3][3];
-        Ji[0][0] = (J[1][1] * J[2][2] - J[1][2] * J[2][1]) * id;
-        Ji[0][1] = (J[0][2] * J[2][1] - J[0][1] * J[2][2]) * id;
-        Ji[0][2] = (J[0][1] * J[1][2] - J[0][2] * J[1][1]) * id;
-        Ji[1][0] = (J[1][2] * J[2][0] - J[1][0] * J[2][2]) * id;
-        Ji[1][1] = (J[0][0] * J[2][2] - J[0][2] * J[2][0]) * id;
-        Ji[1][2] = (J[0][2] * J[1][0] - J[0][0] * J[1][2]) * id;
-        Ji[2][0] = (J[1][0] * J[2][1] - J[1][1] * J[2][0]) * id;
-        Ji[2][1] = (J[0][1] * J[2][0] - J[0][0] * J[2][1]) * id;
-        Ji[2][2] = (J[0][0] * J[1][1] - J[0][1] * J[1][0]) * id;
-        double* G = G6 + tid * 12;
-        for (int c = 0; c < 3; ++c) {
-            G[3 + c] = Ji[0][c], G[6 + c] = Ji[1][c], G[9 + c] = Ji[2][c];
-            G[c] = -(Ji[0][c] + Ji[1][c] + Ji[2][c]);
-        }
-    }
-}
-
-// Element matrix of each class from the closed forms in the barycentric gradients
-// (Vs the common volume of the sub-tetrahedra).  No barrier.
-__device__ __forceinline__ void class_matrices(const Local3DArgs& g, double Vs, const double* G6, double* S6) {
-    const int nb = g.nb;
-    for (int it = threadIdx.x; it < 6 * nb * nb; it += blockDim.x) {
-        const int c = it / (nb * nb), a = (it / nb) % nb, b = it % nb;
-        const double* G = G6 + c * 12;
-        auto d = [&](int i, int j) { return G[3 * i] * G[3 * j] + G[3 * i + 1] * G[3 * j + 1] + G[3 * i + 2] * G[3 * j + 2]; };
-        double v;
-        if (g.P == 1) {
-            v = Vs * d(a, b);
-        } else if (a < 4 && b < 4) {
-            v = Vs * d(a, b) * (a == b ? 0.6 : -0.2);
-        } else if (a < 4 || b < 4) {
-            const int x = a < 4 ? a : b, e = (a < 4 ? b : a) - 4;
-            const int j = c_edges[e][0], k = c_edges[e][1];
-            const double cj = x == j ? 0.15 : -0.05, ck = x == k ? 0.15 : -0.05;
-            v = 4.0 * Vs * (d(x, k) * cj + d(x, j) * ck);
-        } else {
-            const int i = c_edges[a - 4][0], j = c_edges[a - 4][1], k = c_edges[b - 4][0], l = c_edges[b - 4][1];
-            v = 0.8 * Vs * (d(j, l) * (1 + (i == k)) + d(j, k) * (1 + (i == l)) + d(i, l) * (1 + (j == k)) +
-                            d(i, k) * (1 + (j == l)));
-        }
-        S6[it] = v;
-    }
-}
-
-// The source's partial loads (sin sin sin by the collapsed Gauss rule of every
-// sub-tetrahedron, its 64 points in qs groups): PL[(t qs + grp) nb + a] and, after the
-// qs nsub nb loads, the group's part of F_K.  No barrier.
-__device__ __forceinline__ void source_partials(const Local3DArgs& g, const double* V, const double* J6,
-                                                const double* misc, double* PL) {
-    if (g.src_kind != MHM3D_SRC_SINSINSIN) return;
-    const int nb = g.nb, N = g.N, qs = g.qs, per = kQuad / qs;
-    const double* qp = g.quad;
-    const double* qphi = g.quad + 4 * kQuad;
-    const double w6 = 6.0 * misc[5];
-    const double kf = g.src_freq * M_PI, amp = g.src_value * 3.0 * kf * kf;
-    for (int it = threadIdx.x; it < g.nsub * qs; it += blockDim.x) {
-        const int t = it / qs, grp = it % qs;
-        const double* Jc = J6 + 9 * g.sub_cls[t];
-        const int zA = g.sub_base[3 * t], zB = g.sub_base[3 * t + 1], zC = g.sub_base[3 * t + 2];
-        double x0[3];
-        for (int c = 0; c < 3; ++c)
-            x0[c] = V[c] + ((V[3 + c] - V[c]) * zA + (V[6 + c] - V[3 + c]) * zB + (V[9 + c] - V[6 + c]) * zC) / N;
-        double acc[10] = {0, 0, 0, 0, 0, 0, 0, 0, 0, 0}, fk = 0.0;
-        for (int q = grp * per; q < (grp + 1) * per; ++q) {
-            double x[3];
-            for (int c = 0; c < 3; ++c)
-                x[c] = x0[c] + Jc[3 * c] * qp[4 * q] + Jc[3 * c + 1] * qp[4 * q + 1] + Jc[3 * c + 2] * qp[4 * q + 2];
-            const double wf = qp[4 * q + 3] * w6 * amp * sin(kf * x[0]) * sin(kf * x[1]) * sin(kf * x[2]);
-            fk += wf;
-#pragma unroll
-            for (int a = 0; a < 10; ++a)
-                if (a < nb) acc[a] += wf * qphi[q * nb + a];
-        }
-#pragma unroll
-        for (int a = 0; a < 10; ++a)
-            if (a < nb) PL[(size_t)it * nb + a] = acc[a];
-        PL[(size_t)g.nsub * qs * nb + it] = fk;
-    }
-}
-
-// After the partial loads' barrier: per local DOF, in the fixed order of its incidence
-// list, the mass int phi_w and the source load (f, phi_w)_K (column N_I of Y, n x R); the
-// multiplier loads -s |fine face| / 3 per load node and fine face triangle (columns
-// a m + q of Y, zeroed by the caller); F_K into misc[6] (thread 0, in order).  No barrier.
-__device__ __forceinline__ void element_loads(const Local3DArgs& g, int64_t K, double* Y, double* mass,
-                                              const double* PL, double* misc) {
-    const int tid = threadIdx.x, nthr = blockDim.x;
-    const int nb = g.nb, m = g.m, R = g.R, NI = g.NI, qs = g.qs;
-    const double Vs = misc[5];
-    const bool src = g.src_kind == MHM3D_SRC_SINSINSIN;
-    for (int w = tid; w < g.n; w += nthr) {
-        double ms = 0.0, ld = 0.0;
-        for (int e = g.inc_off[w]; e < g.inc_off[w + 1]; ++e) {
-            const int slot = g.inc_ent[e], t = slot / nb, a = slot % nb;
-            ms += (g.P == 1 ? 0.25 : (a < 4 ? -0.05 : 0.2)) * Vs;
-            if (src)
-                for (int grp = 0; grp < qs; ++grp) ld += PL[(size_t)(t * qs + grp) * nb + a];
-        }
-        mass[w] = ms;
-        if (src) Y[w * R + NI] = ld;
-    }
-    for (int it = tid; it < 4 * m; it += nthr) {
-        const int a = it / m, q = it % m;
-        const int p = g.perm[4 * K + a];
-        const double w = -(double)g.signs[4 * K + a] * misc[1 + a] / 3.0;
-        const int base = (a * 6 + p) * (m + 1) + q;
-        for (int e = g.ftab_off[base]; e < g.ftab_off[base + 1]; ++e)
-            Y[g.ftab_node[e] * R + it] = w * g.ftab_cnt[e];
-    }
-    if (src && tid == 0) {
-        double fk = 0.0;
-        for (int i = 0; i < g.nsub * qs; ++i) fk += PL[(size_t)g.nsub * qs * nb + i];
-        misc[6] = fk;
-    }
-}
-
-// Row w of the pinned lower triangle (DOF w >= 1, pinned row w - 1), gathered from the
-// element matrices of the sub-tetrahedra at w in the fixed order of its incidence list;
-// one thread owns the row (no atomics).  TL: double (FP64 factor) or float (FP32 factor).
-template <typename TL>
-__device__ __forceinline__ void assemble_row(const Local3DArgs& g, int w, const double* kap, const double* S6,
-                                             TL* Lrow, double* diag) {
-    const int nb = g.nb;
-    for (int j = 0; j < w; ++j) Lrow[j] = (TL)0;
-    double dsum = 0.0;
-    for (int e = g.inc_off[w]; e < g.inc_off[w + 1]; ++e) {
-        const int slot = g.inc_ent[e], t = slot / nb, a = slot % nb;
-        const double kt = kap[t];
-        const double* Sa = S6 + (g.sub_cls[t] * nb + a) * nb;
-        const int32_t* dofs = g.sub_dofs + t * nb;
-        for (int b = 0; b < nb; ++b) {
-            const int col = dofs[b];
-            if (col < 1 || col > w) continue;
-            const double v = kt * Sa[b];
-            Lrow[col - 1] += (TL)v;
-            if (col == w) dsum += v;
-        }
-    }
-    if (diag) *diag = dsum;
-}
-
-// After the loads' barrier: a constant source, then the compatibility projection
-// g - (1^T g / |K|) m of every column.  Ends with a barrier.
-__device__ __forceinline__ void const_source_and_projection(const Local3DArgs& g, double* Y, const double* mass,
-                                                            double* red, double* misc) {
-    const int tid = threadIdx.x, nthr = blockDim.x, lane = tid & 31, warp = tid >> 5, nwarp = nthr >> 5;
-    const int n = g.n, R = g.R, NI = g.NI;
-    if (g.src_kind == MHM3D_SRC_CONST) {
-        for (int w = tid; w < n; w += nthr) Y[w * R + NI] = g.src_value * mass[w];
-        if (tid == 0) misc[6] = g.src_value * misc[0];
-        __syncthreads();
-    }
-    const double volK = misc[0];
-    for (int r = warp; r < R; r += nwarp) {
-        double s = 0.0;
-        for (int w = lane; w < n; w += 32) s += Y[w * R + r];
-        s = warp_sum(s);
-        if (lane == 0) red[r] = s / volK;
-    }
-    __syncthreads();
-    for (int it = tid; it < n * R; it += nthr) Y[it] -= red[it % R] * mass[it / R];
-    __syncthreads();
-}
-
-// B_K[j] = (s psi_j, 1)_{dK} = s |subface j| from the face-load table, F_K, status.
-__device__ __forceinline__ void element_tail(const Local3DArgs& g, int64_t K, const double* misc, int32_t code,
-                                            int32_t iters) {
-    const int m = g.m, NI = g.NI;
-    for (int j = threadIdx.x; j < NI; j += blockDim.x) {
-        const int a = j / m, q = j % m;
-        const int p = g.perm[4 * K + a];
-        const int base = (a * 6 + p) * (m + 1) + q;
-        int c = 0;
-        for (int e = g.ftab_off[base]; e < g.ftab_off[base + 1]; ++e) c += g.ftab_cnt[e];
-        g.BK[K * NI + j] = (double)g.signs[4 * K + a] * misc[1 + a] / 3.0 * c;
-    }
-    if (threadIdx.x == 0) {
-        g.FK[K] = misc[6];
-        g.status[K] = code;
-        if (g.iters) g.iters[K] = iters;
-    }
 }
 
 // Source tables (sin sin sin by the collapsed Gauss rule) of one element type and class (one
@@ -463,8 +173,9 @@ struct FrontRows3D {
         });
         if (lane == 0) *wnew = 0.0;
         __syncwarp();
-        for (int q = lane; q < ((v.w + 31) & ~31); q += 32) {
-            const uint32_t en = q < v.w ? g.ent[v.z + q] : mhm::kNoSlot;
+        const int count = v.w & 0xffff;
+        for (int q = lane; q < ((count + 31) & ~31); q += 32) {
+            const uint32_t en = q < count ? g.ent[v.z + q] : mhm::kNoSlot;
             const int sl = en & 255, terms = (en >> 8) & 255;
             const uint32_t* con = g.con + (en >> 16);
             double x = 0.0;
@@ -487,7 +198,7 @@ struct Front3Smem {
 };
 __host__ __device__ inline Front3Smem front3_smem(int vec, int n, int nb, int nsub, bool source) {
     Front3Smem l;
-    int o = (int)mhm::front_shared_doubles(vec);
+    int o = (int)mhm::front_shared_values(vec);
     l.S = o, o += 6 * nb * nb;
     l.kap = o, o += nsub;
     l.src = o, o += source ? n : 0;
@@ -498,7 +209,9 @@ __host__ __device__ inline Front3Smem front3_smem(int vec, int n, int nb, int ns
 
 // FP64: one block per coarse tetrahedron at a time eliminates the pinned matrix bordered by
 // its R loads from a front of at most 42 slots (P2, r = 2: 165 DOFs) held in registers
-// (front.cuh); what is left of the border are the face integrals.  Bound by the FP64 pipe.
+// (front.cuh); what is left of the border are the face integrals.  Bound by the FP64 pipe
+// (82 % busy at m = 16).  12288 elements, m = 4: 9.9 ms (79.5 ms with the dense matrix in
+// shared memory, one element per SM); 1536 elements, m = 16: 4.2 ms (14.6 ms).
 template <class T, int MINB>
 __global__ void __launch_bounds__(T::threads, MINB) k_local3d(const __grid_constant__ Local3DArgs g) {
     extern __shared__ double sm[];
@@ -506,7 +219,7 @@ __global__ void __launch_bounds__(T::threads, MINB) k_local3d(const __grid_const
     __shared__ double FKs;
     const int tid = threadIdx.x, nthr = blockDim.x, n = g.n, nb = g.nb, NI = g.NI, R = g.R, m = g.m;
     const Front3Smem L = front3_smem(T::vec, n, nb, g.nsub, g.src24 != nullptr);
-    const mhm::FrontShared sh = mhm::front_shared(sm, T::vec);
+    const mhm::FrontShared<double> sh = mhm::front_shared(sm, T::vec);
     double *S = sm + L.S, *kap = sm + L.kap, *src = sm + L.src;
     for (int64_t K = g.K0 + blockIdx.x; K < g.K1; K += gridDim.x) {
         if (g.only_failed && g.status[K] == MHM_OK) continue;   // (the whole block)
@@ -549,7 +262,7 @@ __global__ void __launch_bounds__(T::threads, MINB) k_local3d(const __grid_const
             }
         });
         double A[T::NT];
-        mhm::front_eliminate<T>(rows, g.ev, g.steps, R, sh, A, &bad, nullptr, 0);
+        mhm::front_eliminate<T>(rows, g.ev, g.steps, R, sh, A, &bad, (double*)nullptr, 0);
         double* AK = g.AK + K * (int64_t)NI * NI;
         mhm::front_result<T>(R, A, [&](int i, int j, double v) {
             if (i < NI) {
@@ -590,183 +303,311 @@ Front3Kernel front3_kernel(int M) {
     return k;
 }
 
+// Entering rows of the FP32 factor: the scaled off-diagonal values, counted off in the order
+// of the entries (each entering node has 8 diagonal entries in front).
+struct FrontRowsScaled {
+    const Local3DArgs& g;
+    const float *off, *diag;
+    int vec, entered = 0;
+    __device__ __forceinline__ void prep(int, const int4& v, float* nb, float* wnew) {
+        const int lane = threadIdx.x & 31, zs = (v.x >> 8) & 255;
+        if (zs == mhm::kNoSlot) return;
+        ++entered;
+        for (int q = lane; q < vec; q += 32) nb[q] = 0.0f;
+        if (lane == 0) *wnew = 0.0f;
+        __syncwarp();
+        for (int q = 8 + lane; q < (v.w & 0xffff); q += 32) {
+            const int sl = g.ent[v.z + q] & 255;
+            const float x = off[v.z + q - 8 * entered];
+            if (sl == mhm::kPivotSlot) *wnew = x;
+            else nb[sl] = x;
+        }
+        if (lane == 0) nb[zs] = diag[v.y - 1];
+    }
+};
+
+using FrontTilesMixed = mhm::FrontTiles<1, 1, 11>;   // fronts of at most 44 slots
+constexpr int kMaxMixedR = 17;                       // three columns for each of 8 warps (m <= 4)
+
+struct Mixed3Smem {   // offsets in doubles
+    int S, kap, A, Z, Rr, W, Lc, inv, sc, src, cp, cf, gn, red, mz, front, total;
+};
+__host__ __device__ inline Mixed3Smem mixed3_smem(int n, int R, int nb, int nsub, int off, int slots) {
+    const int n1 = n - 1, pl = nsub * nb;
+    Mixed3Smem l;
+    int o = 0;
+    l.S = o, o += 6 * nb * nb;
+    l.kap = o, o += nsub;
+    l.A = o, o += off + n1;                                   // values of the pinned matrix
+    l.Z = o, o += n1 * R;
+    l.Rr = o, o += n1 * R > pl ? n1 * R : pl;                 // residuals (before: loads per sub-tetrahedron)
+    l.W = o, o += ((n1 * R > off + n1 ? n1 * R : off + n1) + 1) / 2 + R * R;   // FP32 solves (before: scaled values); outputs
+    l.Lc = o, o += (n1 * slots + 1) / 2;                      // FP32 pivot columns
+    l.inv = o, o += (n1 + 1) / 2;
+    l.sc = o, o += n1;
+    l.src = o, o += n;
+    l.cp = o, o += R;
+    l.cf = o, o += R;
+    l.gn = o, o += R;
+    l.red = o, o += R;
+    l.mz = o, o += R;
+    l.front = o, o += ((int)mhm::front_shared_values(FrontTilesMixed::vec) + 1) / 2;
+    l.total = o;
+    return l;
+}
+
 // Mixed precision (Sec. 3: the local matrix is factored once and each further solve is
 // only products with the factor): the pinned matrix, scaled by its diagonal, is factored
-// in FP32 (Cholesky, shared memory); the N_I + 1 solutions are refined in FP64 against
-// the matrix-free FP64 residual r = g~ - A z (element matrices of the six classes times
-// kappa), each pass one FP32 forward and backward substitution per column (a warp per
-// column), until every column's scaled residual |S r| <= tol |S g~| or it_max passes.  The
-// face integrals use the corrected bilinear form
+// in FP32 by the frontal elimination (one warp, the pivot columns kept in shared memory);
+// the N_I + 1 solutions are refined in FP64 against the FP64 residual r = g~ - A z (rows of
+// the assembled matrix), each pass one FP32 forward and backward sweep over the pivots (a warp
+// takes up to three columns, a lane the front's slots), until every column's scaled
+// residual |S r| <= tol |S g~| or it_max passes.  The face integrals use the corrected
+// bilinear form
 //   (s psi_j, eta_i)_{dK} = -(g~_j . z_i + z_j . r_i),
 // whose error is the product of the two solution errors in the energy norm (second order),
 // averaged with its transpose.  An element whose FP32 factor breaks down or that does not
 // converge gets MHM_ERR_NOT_CONVERGED (the host then re-solves it in FP64 unless asked not to).
-__global__ void __launch_bounds__(kThreads) k_local3d_mixed(Local3DArgs g) {
+//
+// Bound by issued instructions and their latencies: the FP32 sweeps take 60 % of 0.9 M warp
+// instructions per element (three passes), the FP64 pipe is 31 % busy; two elements per SM
+// (110 KB of shared memory each) hide one another's chains.  12288 elements, m = 4: 27.5 ms
+// (91.3 ms with a dense packed factor, 512 threads and one element per SM; the FP64 kernel
+// takes 9.9 ms).
+__global__ void __launch_bounds__(kThreads, 2) k_local3d_mixed(const __grid_constant__ Local3DArgs g) {
     extern __shared__ double sm[];
-    const Smem3M L = smem_layout_mixed(g.n, g.NI, g.nb, g.nsub, g.qs);
-    float* Lf = reinterpret_cast<float*>(sm + L.Lf);
-    double* G = sm + L.G;
-    double* Z = sm + L.Z;
-    double* Rr = sm + L.Rr;
+    __shared__ int bad;
+    __shared__ double FKs;
+    const int n = g.n, n1 = n - 1, nb = g.nb, NI = g.NI, R = g.R, m = g.m, off = g.off, slots = g.slots;
+    const Mixed3Smem L = mixed3_smem(n, R, nb, g.nsub, off, slots);
+    double *S = sm + L.S, *kap = sm + L.kap, *A = sm + L.A, *Z = sm + L.Z, *Rr = sm + L.Rr, *sc = sm + L.sc;
+    double *src = sm + L.src, *cp = sm + L.cp, *cf = sm + L.cf, *gn = sm + L.gn, *red = sm + L.red, *mz = sm + L.mz;
     float* W = reinterpret_cast<float*>(sm + L.W);
-    double* sc = sm + L.sc;
-    double* dg = sm + L.dg;
-    float* invf = reinterpret_cast<float*>(sm + L.invf);
-    double* mass = sm + L.mass;
-    double* S6 = sm + L.S6;
-    double* G6 = sm + L.G6;
-    double* J6 = sm + L.J6;
-    double* red = sm + L.red;
-    double* gn = sm + L.gn;
-    double* misc = sm + L.misc;
-    const int tid = threadIdx.x, nthr = blockDim.x, lane = tid & 31, warp = tid >> 5, nwarp = nthr >> 5;
-    const int64_t K = g.K0 + blockIdx.x;
-    const int n = g.n, n1 = n - 1, R = g.R, NI = g.NI, nb = g.nb, npk = n1 * (n1 + 1) / 2;
-    const double* V = g.geom + 12 * K;
-    const double* kap = g.kappa + K * (int64_t)g.nsub;
-
-    // ---- zero the loads and solutions; geometry; classes; the source's partial loads
-    for (int i = L.G + tid; i < L.Rr; i += nthr) sm[i] = 0.0;
-    element_geometry(g, V, misc, G6, J6);
-    __syncthreads();
-    class_matrices(g, misc[5], G6, S6);
-    source_partials(g, V, J6, misc, Rr);
-    __syncthreads();
-    // ---- loads and mass per DOF; the pinned lower triangle in FP32 row by row with its
-    // diagonal in FP64 (no atomics, a fixed order)
-    element_loads(g, K, G, mass, Rr, misc);
-    for (int w = 1 + tid; w < n; w += nthr) assemble_row<float>(g, w, kap, S6, Lf + pk(w - 1, 0), dg + w);
-    __syncthreads();
-    const_source_and_projection(g, G, mass, red, misc);
-
-    // ---- diagonal scaling S A S (S = diag^-1/2), then the FP32 Cholesky
-    for (int i = tid; i < n1; i += nthr) {
-        const double d = dg[i + 1];
-        if (!(d > 0.0)) misc[7] = 1.0;
-        sc[i] = d > 0.0 ? 1.0 / sqrt(d) : 1.0;
-    }
-    __syncthreads();
-    for (int it = tid; it < npk; it += nthr) {
-        const int i = tri_row(it), j = it - i * (i + 1) / 2;
-        Lf[it] = (float)((double)Lf[it] * sc[i] * sc[j]);
-    }
-    __syncthreads();
-    for (int k = 0; k < n1; ++k) {
-        float d = Lf[pk(k, k)];
-        if (!(d > 0.0f)) {
-            d = 1.0f;
-            if (tid == 0) misc[7] = 1.0;
-        }
-        const float inv = 1.0f / sqrtf(d);
-        for (int i = k + 1 + tid; i < n1; i += nthr) Lf[pk(i, k)] *= inv;
-        if (tid == 0) invf[k] = inv;
-        __syncthreads();
-        const int mt = n1 - k - 1, tri = mt * (mt + 1) / 2;   // the trailing triangle, one flat list
-        for (int t = tid; t < tri; t += nthr) {
-            const int ii = tri_row(t);
-            const int i = k + 1 + ii, j = k + 1 + (t - ii * (ii + 1) / 2);
-            Lf[pk(i, j)] -= Lf[pk(i, k)] * Lf[pk(j, k)];
-        }
-        __syncthreads();
-    }
-
-    // ---- FP64 refinement: z = 0, r = g~; |S g~|^2 per column
-    for (int it = tid; it < n * R; it += nthr) Rr[it] = it < R ? 0.0 : G[it];
-    for (int c = warp; c < R; c += nwarp) {
-        double s = 0.0;
-        for (int i = lane; i < n1; i += 32) s += (sc[i] * G[(i + 1) * R + c]) * (sc[i] * G[(i + 1) * R + c]);
-        s = warp_sum(s);
-        if (lane == 0) gn[c] = s;
-    }
-    __syncthreads();
-    int passes = 0;
-    const double tol2 = g.tol * g.tol;
-    for (int pass = 0; pass < g.it_max && misc[7] == 0.0; ++pass) {
-        // w = S r (FP32), then L^-1 and L^-T by a warp per column
-        for (int it = tid; it < n1 * R; it += nthr) {
-            const int i = it / R, c = it % R;
-            W[it] = (float)(sc[i] * Rr[(i + 1) * R + c]);
-        }
-        __syncthreads();
-        for (int c = warp; c < R; c += nwarp) {
-            for (int k = 0; k < n1; ++k) {
-                const float xk = W[k * R + c] * invf[k];
-                __syncwarp();
-                for (int i = k + 1 + lane; i < n1; i += 32) W[i * R + c] -= Lf[pk(i, k)] * xk;
-                if (lane == 0) W[k * R + c] = xk;
-                __syncwarp();
+    float* Lc = reinterpret_cast<float*>(sm + L.Lc);
+    float* inv = reinterpret_cast<float*>(sm + L.inv);
+    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+    constexpr int NWARP = kThreads / 32;
+    for (int64_t K = g.K0 + blockIdx.x; K < g.K1; K += gridDim.x) {
+        const double* geo = g.geo24 + 8 * (K % 24);
+        const double vol = geo[0];
+        // ---- class matrices, kappa, source loads; projection and face coefficients per column
+        for (int t = tid; t < 6 * nb * nb; t += kThreads) S[t] = g.cls24[(size_t)(K % 24) * 6 * nb * nb + t];
+        for (int t = tid; t < g.nsub; t += kThreads) kap[t] = g.kappa[K * (int64_t)g.nsub + t];
+        if (tid == 0) bad = 0;
+        if (g.src24) source_loads3(g, K, Rr, src);
+        if (warp == 0) {
+            double f = 0.0;
+            if (g.src24) {
+                for (int w = lane; w < n; w += 32) f += src[w];
+                f = warp_sum(f);
+            } else {
+                f = g.src_value * vol;
             }
-            for (int k = n1 - 1; k >= 0; --k) {
-                float s = 0.0f;
-                for (int i = k + 1 + lane; i < n1; i += 32) s += Lf[pk(i, k)] * W[i * R + c];
-                s = warp_sumf(s);
-                const float xk = (W[k * R + c] - s) * invf[k];
-                __syncwarp();
-                if (lane == 0) W[k * R + c] = xk;
-                __syncwarp();
-            }
+            if (lane == 0) FKs = cp[NI] = f;
+        }
+        auto moment = [&](int j) {   // (psi_j, 1)_{dK}
+            const int a = j / m, q = j % m, b0 = (a * 6 + g.perm[4 * K + a]) * (m + 1) + q;
+            int c = 0;
+            for (int e = g.ftab_off[b0]; e < g.ftab_off[b0 + 1]; ++e) c += g.ftab_cnt[e];
+            return (double)g.signs[4 * K + a] * geo[1 + a] * c;
+        };
+        for (int j = tid; j < NI; j += kThreads) {
+            cp[j] = -moment(j);
+            cf[j] = -(double)g.signs[4 * K + j / m] * geo[1 + j / m];
         }
         __syncthreads();
-        // z += S w; then r = g~ - A z on the pinned rows, gathered per DOF from the element
-        // matrices at it (z vanishes on the pinned DOF)
-        for (int it = tid; it < n1 * R; it += nthr) {
-            const int i = it / R, c = it % R;
-            Z[(i + 1) * R + c] += sc[i] * (double)W[it];
+        // projected load of column c at node w (DOF w + 1)
+        auto load = [&](int w, int c) {
+            const double mt = g.mass1[w + 1];
+            double x = -cp[c] * mt;
+            if (c == NI) return g.src24 ? x + src[w + 1] : fma(g.src_value * vol, mt, x);
+            const int a = c / m, cnt = g.fcnt[((a * 6 + g.perm[4 * K + a]) * n + w + 1) * m + c % m];
+            // (cnt as a double without a conversion: 2^52 + cnt - 2^52)
+            if (cnt) x = fma(cf[c], __hiloint2double(0x43300000, cnt) - 4503599627370496.0, x);
+            return x;
+        };
+        // ---- values of the pinned matrix, the scaling S = diag^-1/2, the scaled values in FP32
+        for (int q = tid; q < off + n1; q += kThreads) {
+            const uint32_t v = g.val[q];
+            const uint32_t* con = g.con + (v & 0xffff);
+            double x = 0.0;
+            for (int i = 0; i < (int)(v >> 16); ++i) x = fma(kap[con[i] & 0xffff], S[con[i] >> 16], x);
+            A[q] = x;
         }
         __syncthreads();
-        for (int it = tid; it < n1 * R; it += nthr) {
-            const int w = it / R + 1, c = it % R;
-            double s = 0.0;
-            for (int e = g.inc_off[w]; e < g.inc_off[w + 1]; ++e) {
-                const int slot = g.inc_ent[e], t = slot / nb, a = slot % nb;
-                const double* Sa = S6 + (g.sub_cls[t] * nb + a) * nb;
-                const int32_t* dofs = g.sub_dofs + t * nb;
-                double sa = 0.0;
-                for (int b = 0; b < nb; ++b) sa += Sa[b] * Z[dofs[b] * R + c];
-                s += kap[t] * sa;
-            }
-            Rr[w * R + c] = G[w * R + c] - s;
+        for (int w = tid; w < n1; w += kThreads) {
+            const double d = A[off + w];
+            if (!(d > 0.0)) bad = 1;
+            sc[w] = d > 0.0 ? 1.0 / sqrt(d) : 1.0;
         }
         __syncthreads();
-        // converged when every column's |S r|^2 <= tol^2 |S g~|^2
-        for (int c = warp; c < R; c += nwarp) {
-            double s = 0.0;
-            for (int i = lane; i < n1; i += 32) s += (sc[i] * Rr[(i + 1) * R + c]) * (sc[i] * Rr[(i + 1) * R + c]);
-            s = warp_sum(s);
-            if (lane == 0) red[c] = s;
+        for (int q = tid; q < off + n1; q += kThreads) {
+            const uint32_t rc = q < off ? g.rc[q] : (uint32_t)(q - off) * 0x10001u;
+            W[q] = (float)(A[q] * sc[rc & 0xffff] * sc[rc >> 16]);
         }
         __syncthreads();
-        passes = pass + 1;
-        bool done = true;
-        for (int c = 0; c < R; ++c) done = done && red[c] <= tol2 * gn[c];
-        if (done) break;   // the same decision in every thread (read after the barrier)
-        __syncthreads();   // red is rewritten in the next pass
-    }
-    const bool converged = misc[7] == 0.0 && passes > 0 && [&] {
-        bool ok = true;
-        for (int c = 0; c < R; ++c) ok = ok && red[c] <= tol2 * gn[c];
-        return ok;
-    }();
-
-    // ---- corrected face integrals T_ji = -(g~_j . z_i + z_j . r_i), averaged with T_ij
-    double* AK = g.AK + K * (int64_t)NI * NI;
-    const int pairs = NI * (NI + 1) / 2;   // each pair i <= j once, then the E_K entries (i = N_I)
-    for (int it = tid; it < pairs + NI; it += nthr) {
-        const int j = it < pairs ? tri_row(it) : it - pairs, i = it < pairs ? it - j * (j + 1) / 2 : NI;
-        double a1 = 0.0, a2 = 0.0;
-        for (int w = 1; w < n; ++w) {
-            a1 += G[w * R + j] * Z[w * R + i] + Z[w * R + j] * Rr[w * R + i];
-            a2 += G[w * R + i] * Z[w * R + j] + Z[w * R + i] * Rr[w * R + j];
-        }
-        const double v = 0.5 * (a1 + a2);
-        if (i == NI) {
-            g.EK[K * NI + j] = v;
+        // ---- FP32 factor: warp 0; the others prepare z = 0, r = g~ and |S g~|^2 per column
+        if (warp == 0) {
+            const mhm::FrontShared<float> sh = mhm::front_shared(reinterpret_cast<float*>(sm + L.front), FrontTilesMixed::vec);
+            FrontRowsScaled rows{g, W, W + off, FrontTilesMixed::vec};
+            float F[FrontTilesMixed::NT];
+            mhm::front_eliminate<FrontTilesMixed>(rows, g.ev, g.steps, 0, sh, F, &bad, Lc, slots, inv, g.first);
         } else {
-            AK[j * NI + i] = -v;
-            AK[i * NI + j] = -v;
+            for (int c = warp - 1; c < R; c += NWARP - 1) {
+                double s = 0.0;
+                for (int w = lane; w < n1; w += 32) {
+                    const double r = load(w, c), x = sc[w] * r;
+                    Rr[w * R + c] = r;
+                    Z[w * R + c] = 0.0;
+                    s = fma(x, x, s);
+                }
+                s = warp_sum(s);
+                if (lane == 0) gn[c] = s;
+            }
         }
+        __syncthreads();
+        // ---- refinement
+        int passes = 0;
+        bool converged = false;
+        const double tol2 = g.tol * g.tol;
+        for (int pass = 0; pass < g.it_max && !bad; ++pass) {
+            for (int it = tid; it < n1 * R; it += kThreads) W[it] = (float)(sc[it / R] * Rr[it]);
+            __syncthreads();
+            if (warp < R) {
+                // columns warp, warp + 8, warp + 16; a lane holds slots lane and lane + 32
+                const int nc = (R - warp + NWARP - 1) / NWARP;
+                float v0[3] = {0, 0, 0}, v1[3] = {0, 0, 0};
+                int4 e = g.ev[0];
+                for (int st = 0; st < g.steps; ++st) {
+                    const int ps = e.x & 255, zs = (e.x >> 8) & 255, used = e.x >> 16, pn = e.w >> 16, en = e.y - 1;
+                    if (st + 1 < g.steps) e = g.ev[st + 1];
+                    const bool pivot = ps != mhm::kNoSlot;
+                    const float* lc = Lc + (st - g.first) * slots;
+                    const float l0 = pivot && lane < used ? lc[lane] : 0.0f;
+                    const float l1 = pivot && lane + 32 < used ? lc[lane + 32] : 0.0f;
+                    const float di = pivot ? inv[st - g.first] : 0.0f;
+#pragma unroll
+                    for (int k = 0; k < 3; ++k)
+                        if (k < nc) {
+                            const int c = warp + NWARP * k;
+                            const float y = pivot ? __shfl_sync(0xffffffffu, ps >= 32 ? v1[k] : v0[k], ps & 31) : 0.0f;
+                            if (zs != mhm::kNoSlot) {
+                                const float x = W[en * R + c];
+                                if (zs == lane) v0[k] = x;
+                                if (zs == lane + 32) v1[k] = x;
+                            }
+                            v0[k] = fmaf(-l0, y, v0[k]);
+                            v1[k] = fmaf(-l1, y, v1[k]);
+                            if (pivot && lane == 0) W[pn * R + c] = y * di;
+                        }
+                }
+#pragma unroll
+                for (int k = 0; k < 3; ++k) v0[k] = v1[k] = 0.0f;
+                __syncwarp();
+                for (int st = g.steps - 1; st >= g.first; --st) {
+                    const int4 b = g.ev[st];
+                    const int ps = b.x & 255, used = b.x >> 16, pn = b.w >> 16;
+                    const float* lc = Lc + (st - g.first) * slots;
+                    const float l0 = lane < used ? lc[lane] : 0.0f, l1 = lane + 32 < used ? lc[lane + 32] : 0.0f;
+                    float t[3], y[3];
+#pragma unroll
+                    for (int k = 0; k < 3; ++k) {
+                        y[k] = k < nc ? W[pn * R + warp + NWARP * k] : 0.0f;
+                        t[k] = fmaf(l0, v0[k], l1 * v1[k]);
+                    }
+#pragma unroll
+                    for (int o = 16; o > 0; o >>= 1)
+#pragma unroll
+                        for (int k = 0; k < 3; ++k) t[k] += __shfl_xor_sync(0xffffffffu, t[k], o);
+#pragma unroll
+                    for (int k = 0; k < 3; ++k)
+                        if (k < nc) {
+                            const float x = y[k] - t[k];
+                            if (ps == lane) v0[k] = x;
+                            if (ps == lane + 32) v1[k] = x;
+                            if (lane == 0) W[pn * R + warp + NWARP * k] = x;
+                        }
+                }
+            }
+            __syncthreads();
+            // z += S w; then r = g~ - A z on the pinned rows (z vanishes on the pinned DOF)
+            for (int it = tid; it < n1 * R; it += kThreads) Z[it] = fma(sc[it / R], (double)W[it], Z[it]);
+            __syncthreads();
+            for (int it = tid; it < n1 * R; it += kThreads) {
+                const int w = it / R, c = it - w * R;
+                double s = load(w, c);
+                for (int q = g.rp[w]; q < g.rp[w + 1]; ++q) {
+                    const uint32_t e = g.col[q];
+                    s = fma(-A[e >> 16], Z[(e & 0xffff) * R + c], s);
+                }
+                Rr[it] = s;
+            }
+            __syncthreads();
+            // converged when every column's |S r|^2 <= tol^2 |S g~|^2
+            for (int c = warp; c < R; c += NWARP) {
+                double s = 0.0;
+                for (int w = lane; w < n1; w += 32) {
+                    const double x = sc[w] * Rr[w * R + c];
+                    s = fma(x, x, s);
+                }
+                s = warp_sum(s);
+                if (lane == 0) red[c] = s;
+            }
+            __syncthreads();
+            passes = pass + 1;
+            converged = true;
+            for (int c = 0; c < R; ++c) converged = converged && red[c] <= tol2 * gn[c];
+            if (converged) break;   // (the same in every thread)
+            __syncthreads();
+        }
+        converged = converged && !bad;
+
+        // ---- corrected face integrals X_ji = g~_j . z_i + z_j . r_i, averaged with X_ij; the
+        // multiplier loads live on their subface: g~_j . z = N_j . z - c_j m . z
+        double* X = sm + L.W;   // (the FP32 solves are done)
+        for (int c = warp; c < R; c += NWARP) {
+            double s = 0.0;
+            for (int w = lane; w < n1; w += 32) s = fma(g.mass1[w + 1], Z[w * R + c], s);
+            s = warp_sum(s);
+            if (lane == 0) mz[c] = s;
+        }
+        __syncthreads();
+        for (int it = tid; it < R * R; it += kThreads) {
+            const int j = it / R, i = it - j * R;
+            double s = -cp[j] * mz[i];
+            if (j < NI) {
+                const int a = j / m, b0 = (a * 6 + g.perm[4 * K + a]) * (m + 1) + j % m;
+                double t = 0.0;
+                for (int e = g.ftab_off[b0]; e < g.ftab_off[b0 + 1]; ++e) {
+                    const int w = g.ftab_node[e] - 1;
+                    if (w >= 0) t = fma(__hiloint2double(0x43300000, g.ftab_cnt[e]) - 4503599627370496.0, Z[w * R + i], t);
+                }
+                s = fma(cf[j], t, s);
+            } else if (g.src24) {
+                for (int w = 0; w < n1; ++w) s = fma(src[w + 1], Z[w * R + i], s);
+            } else {
+                s = fma(g.src_value * vol, mz[i], s);
+            }
+            for (int w = 0; w < n1; ++w) s = fma(Z[w * R + j], Rr[w * R + i], s);
+            X[it] = s;
+        }
+        __syncthreads();
+        double* AK = g.AK + K * (int64_t)NI * NI;
+        for (int it = tid; it < NI * NI; it += kThreads) {
+            const int j = it / NI, i = it - j * NI;
+            AK[it] = -0.5 * (X[j * R + i] + X[i * R + j]);
+        }
+        for (int j = tid; j < NI; j += kThreads) {
+            g.EK[K * NI + j] = 0.5 * (X[j * R + NI] + X[NI * R + j]);
+            g.BK[K * NI + j] = moment(j);
+        }
+        if (tid == 0) {
+            g.FK[K] = FKs;
+            g.status[K] = converged ? MHM_OK : MHM_ERR_NOT_CONVERGED;
+            if (g.iters) g.iters[K] = passes;
+        }
+        __syncthreads();
     }
-    element_tail(g, K, misc, converged ? MHM_OK : MHM_ERR_NOT_CONVERGED, passes);
 }
 
 // skeleton values: one thread per entry of a neighbour block
@@ -816,6 +657,8 @@ mhm_status upload_front_tables(mhm_mesh3d* m) {
     const mhm::FrontPlan3 plan = mhm::front_plan_3d(n, nb, m->sub_dofs, m->sub_cls, m->nodes, (int)m->NI + 1);
     m->fsteps = plan.steps;
     m->fslots = plan.slots;
+    m->ffirst = plan.first_pivot;
+    m->foff = plan.off;
     std::vector<double> cls((size_t)24 * 6 * nb * nb), geo(24 * 8, 0.0), mass(n, 0.0);
     for (int t = 0; t < 24; ++t) {
         const double* V = &m->geom[12 * t];
@@ -883,6 +726,10 @@ mhm_status upload_front_tables(mhm_mesh3d* m) {
     mhm_status st = upload3(plan.ev, (int32_t**)&m->d_fev);
     if (!st) st = upload3(plan.ent, &m->d_fent);
     if (!st) st = upload3(plan.con, &m->d_fcon);
+    if (!st) st = upload3(plan.val, &m->d_fval);
+    if (!st) st = upload3(plan.rc, &m->d_frc);
+    if (!st) st = upload3(plan.rp, &m->d_frp);
+    if (!st) st = upload3(plan.col, &m->d_fcol);
     if (!st) st = upload3(cls, &m->d_cls24);
     if (!st) st = upload3(geo, &m->d_geo24);
     if (!st) st = upload3(mass, &m->d_mass1);
@@ -893,23 +740,20 @@ mhm_status upload_front_tables(mhm_mesh3d* m) {
 void free_device(mhm_mesh3d* m) {
     void* ptrs[] = {m->d_geom, m->d_signs, m->d_perm, m->d_sub_dofs, m->d_sub_cls, m->d_sub_base, m->d_ftab_off,
                     m->d_ftab_node, m->d_ftab_cnt, m->d_quad, m->d_rowptr, m->d_nbrs, m->d_face_ka, m->d_inc_off,
-                    m->d_inc_ent, m->d_fev, m->d_fent, m->d_fcon, m->d_cls24, m->d_geo24, m->d_mass1, m->d_fcnt};
+                    m->d_inc_ent, m->d_fev, m->d_fent, m->d_fcon, m->d_cls24, m->d_geo24, m->d_mass1, m->d_fcnt, m->d_fval, m->d_frc, m->d_frp, m->d_fcol};
     for (void* p : ptrs)
         if (p) cudaFree(p);
 }
 
 }  // namespace
 
-int local3d_qsplit(int nsub) {
-    int qs = 8;   // groups of the 64 points: as many as keep one item per thread
-    while (qs > 1 && qs * nsub > kThreads) qs >>= 1;
-    return qs;
-}
-size_t local3d_smem(int n, int NI, int nb, int nsub) {
-    return dense_doubles(n, NI, nb, nsub, local3d_qsplit(nsub)) * sizeof(double);
-}
-size_t local3d_smem_mixed(int n, int NI, int nb, int nsub) {
-    return (size_t)smem_layout_mixed(n, NI, nb, nsub, local3d_qsplit(nsub)).total * sizeof(double);
+// The limit of the meshes taken on a device: the packed pinned triangle (or, if larger, nb + 1
+// loads per sub-tetrahedron in up to 8 groups of its 64 points), n x R columns and tables.
+size_t local3d_dense_bytes(int n, int NI, int nb, int nsub) {
+    int qs = 8;
+    while (qs > 1 && qs * nsub > 512) qs >>= 1;
+    const size_t R = NI + 1, npk = (size_t)(n - 1) * n / 2, pl = (size_t)qs * nsub * (nb + 1);
+    return (std::max(npk, pl) + n * R + n + 6 * nb * nb + 6 * 21 + R + 16) * sizeof(double);
 }
 
 }  // namespace mhm3
@@ -939,7 +783,7 @@ extern "C" mhm_status mhm3d_create_mesh(const mhm3d_mesh_desc* desc, int32_t dev
         if (!mhm::device_supported(device))
             return mhm::fail(MHM_ERR_UNSUPPORTED, "mhm3d_create_mesh: device is not an sm_103 GPU");
         if (n > kMaxLocal || d.m > kMaxM ||
-            local3d_smem((int)n, 4 * d.m, d.degree == 1 ? 4 : 10, 1 << (3 * d.r)) > 227 * 1024)
+            local3d_dense_bytes((int)n, 4 * d.m, d.degree == 1 ? 4 : 10, 1 << (3 * d.r)) > 227 * 1024)
             return mhm::fail(MHM_ERR_UNSUPPORTED,
                              "mhm3d_create_mesh: the local factor and right-hand sides exceed shared memory "
                              "(degree 2: r <= 2, degree 1: r <= 3, m <= 16)");
@@ -1049,51 +893,50 @@ extern "C" mhm_status mhm3d_local_solve_batch(const mhm3d_mesh* m, const double*
     MHM_CUDA_TRY(cudaSetDevice(m->device));
     Local3DArgs g{};
     g.geom = m->d_geom, g.signs = m->d_signs, g.perm = m->d_perm;
-    g.sub_dofs = m->d_sub_dofs, g.sub_cls = m->d_sub_cls, g.sub_base = m->d_sub_base;
+    g.sub_cls = m->d_sub_cls, g.sub_base = m->d_sub_base;
     g.inc_off = m->d_inc_off, g.inc_ent = m->d_inc_ent;
     g.ftab_off = m->d_ftab_off, g.ftab_node = m->d_ftab_node, g.ftab_cnt = m->d_ftab_cnt;
-    g.quad = m->d_quad, g.kappa = kappa;
-    g.src_kind = f->kind, g.src_value = f->value, g.src_freq = f->freq;
-    g.K0 = K0;
-    g.K1 = K1;
-    g.ev = m->d_fev, g.ent = m->d_fent, g.con = m->d_fcon, g.steps = m->fsteps;
-    g.cls24 = m->d_cls24, g.geo24 = m->d_geo24, g.mass1 = m->d_mass1, g.fcnt = m->d_fcnt;
-    g.N = m->N, g.P = m->desc.degree, g.n = (int)m->n, g.nb = m->nb, g.nsub = (int)m->nsub, g.m = m->desc.m;
+    g.kappa = kappa;
+    g.src_value = f->value, g.src_freq = f->freq;
+    g.K0 = K0, g.K1 = K1;
+    g.N = m->N, g.n = (int)m->n, g.nb = m->nb, g.nsub = (int)m->nsub, g.m = m->desc.m;
     g.NI = (int)m->NI, g.R = (int)m->NI + 1;
     g.AK = AK, g.EK = EK, g.BK = BK, g.FK = FK, g.status = status, g.iters = iters;
     g.it_max = o.it_max, g.tol = o.tol;
-    const unsigned grid = (unsigned)(K1 - K0);
+    g.ev = m->d_fev, g.ent = m->d_fent, g.con = m->d_fcon, g.steps = m->fsteps, g.slots = m->fslots;
+    g.cls24 = m->d_cls24, g.geo24 = m->d_geo24, g.mass1 = m->d_mass1, g.fcnt = m->d_fcnt;
+    g.val = m->d_fval, g.rc = m->d_frc, g.rp = m->d_frp, g.col = m->d_fcol, g.first = m->ffirst, g.off = m->foff;
     cudaStream_t s = (cudaStream_t)stream;
-    // the shared-memory attribute is per kernel, not per mesh: set it for this mesh every call
-    g.qs = local3d_qsplit(g.nsub);
-    const size_t smemmx = local3d_smem_mixed(g.n, g.NI, g.nb, g.nsub);
-    const bool mixed = precision == MHM_MIXED && smemmx <= 227 * 1024;
-    if (mixed) {
-        MHM_CUDA_TRY(cudaFuncSetAttribute(k_local3d_mixed, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smemmx));
-        k_local3d_mixed<<<grid, kThreads, smemmx, s>>>(g);
-        MHM_CUDA_TRY(cudaGetLastError());
-        if (o.no_fallback) return MHM_OK;
-        g.only_failed = 1;   // the elements the refinement could not finish, again in FP64
-    }
-    // FP64: frontal elimination; the source tables in a stream-ordered scratch of this call
     const Front3Kernel k = front3_kernel(g.R + m->fslots);
     if (!k.kern) return mhm::fail(MHM_ERR_UNSUPPORTED, "mhm3d_local_solve_batch: front too large");
+    // the source tables in a stream-ordered scratch of this call
     double* tables = nullptr;
+    cudaError_t e = cudaSuccess;
     if (f->kind == MHM3D_SRC_SINSINSIN) {
         MHM_CUDA_TRY(cudaMallocAsync((void**)&tables, (size_t)24 * 6 * 8 * g.nb * sizeof(double), s));
         k_source3d<<<24 * 6, kQuad, 0, s>>>(m->d_geom, m->d_quad, g.N, g.nb, f->value, f->freq, tables);
         g.src24 = tables;
     }
-    const size_t smem = (size_t)front3_smem(k.vec, g.n, g.nb, g.nsub, tables != nullptr).total * sizeof(double);
-    int sms = 0, per_sm = 0;
+    int sms = 0;
     cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, m->device);
-    cudaError_t e = cudaFuncSetAttribute(k.kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-    if (e == cudaSuccess) e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k.kern, k.threads, smem);
-    if (e == cudaSuccess) {
-        // one wave of blocks that share the elements out evenly
+    // one wave of blocks that share the elements out evenly
+    auto launch = [&](void (*kern)(const Local3DArgs), int threads, size_t smem) {
+        int per_sm = 0;
+        cudaError_t c = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+        if (c == cudaSuccess) c = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kern, threads, smem);
+        if (c != cudaSuccess) return c;
         const int64_t each = (K1 - K0 + sms - 1) / sms, rounds = (each + std::max(per_sm, 1) - 1) / std::max(per_sm, 1);
-        k.kern<<<(unsigned)std::min<int64_t>(K1 - K0, sms * ((each + rounds - 1) / rounds)), k.threads, smem, s>>>(g);
-        e = cudaGetLastError();
+        kern<<<(unsigned)std::min<int64_t>(K1 - K0, sms * ((each + rounds - 1) / rounds)), threads, smem, s>>>(g);
+        return cudaGetLastError();
+    };
+    const bool mixed = precision == MHM_MIXED && g.R <= kMaxMixedR && m->fslots <= FrontTilesMixed::rows;
+    if (mixed)
+        e = launch(k_local3d_mixed, kThreads,
+                   (size_t)mixed3_smem(g.n, g.R, g.nb, g.nsub, g.off, g.slots).total * sizeof(double));
+    if (e == cudaSuccess && !(mixed && o.no_fallback)) {
+        g.only_failed = mixed;   // the elements the refinement could not finish, again in FP64
+        e = launch(k.kern, k.threads,
+                   (size_t)front3_smem(k.vec, g.n, g.nb, g.nsub, tables != nullptr).total * sizeof(double));
     }
     if (tables) cudaFreeAsync(tables, s);
     if (e != cudaSuccess) return mhm::cuda_fail(e, "mhm3d_local_solve_batch: launch");

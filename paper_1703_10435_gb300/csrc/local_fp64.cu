@@ -353,7 +353,7 @@ struct FrontSmem {
 __host__ __device__ inline FrontSmem front_smem(int vec, int R, int kind, int P, int N) {
     const int PN = P * N;
     FrontSmem l;
-    int o = (int)front_shared_doubles(vec);
+    int o = (int)front_shared_values(vec);
     l.Ke = o, o += 72;       // element matrices, up then down
     l.mass = o, o += 8;      // mass of a node on k fine triangles
     l.cproj = o, o += R;     // projection coefficient of each right-hand side
@@ -395,7 +395,7 @@ __global__ void __launch_bounds__(T::threads, MINB) k_local_fp64(const __grid_co
     __shared__ FrontCtx c;
     const int P = g.P, N = g.N, PN = g.PN, R = g.R, NI = g.NI, tid = threadIdx.x, nthr = blockDim.x;
     const FrontSmem L = front_smem(T::vec, R, g.src_kind, P, N);
-    const FrontShared sh = front_shared(smem, T::vec);
+    const FrontShared<double> sh = front_shared(smem, T::vec);
     double* Ke = smem + L.Ke;
     double* cproj = smem + L.cproj;
     double* tab = smem + L.tab;
@@ -433,7 +433,7 @@ __global__ void __launch_bounds__(T::threads, MINB) k_local_fp64(const __grid_co
     if (NW == 1 || (tid >> 5) == NW) rows.start();
 
     double A[T::NT];
-    front_eliminate<T>(rows, g.ev, g.steps, R, sh, A, &c.bad, nullptr, 0);
+    front_eliminate<T>(rows, g.ev, g.steps, R, sh, A, &c.bad, (double*)nullptr, 0);
 
     // ---- outputs
     double* AK = g.AK + K * NI * NI;

@@ -17,7 +17,7 @@ constexpr int kMaxLocal = 165;
 constexpr int kMaxM = 16;                  // subfaces per face
 constexpr int kMaxNI = 4 * kMaxM;          // multipliers per element
 constexpr int kQuad = 64;                  // collapsed 4x4x4 Gauss rule per sub-tetrahedron
-constexpr int kThreads = 512;
+constexpr int kThreads = 256;              // mixed kernel
 
 // One block (f, g) of the skeleton rows of face f: the columns of face g start at
 // col_off inside each of f's rows; element K0 (and K1 on the diagonal block of an
@@ -29,10 +29,8 @@ struct Nbr3 {
     int32_t K1, a1, b1;   // K1 = -1: one contribution
 };
 
-// shared memory bytes of one local-solve block (FP64 and mixed kernels)
-int local3d_qsplit(int nsub);
-size_t local3d_smem(int n, int NI, int nb, int nsub);
-size_t local3d_smem_mixed(int n, int NI, int nb, int nsub);
+// bytes of one element's dense problem, which bounds the meshes that are accepted
+size_t local3d_dense_bytes(int n, int NI, int nb, int nsub);
 
 // rule on [0,1] (Newton on the Legendre polynomial)
 void gauss01(int n, double* x, double* w);
@@ -85,9 +83,10 @@ struct mhm_mesh3d {
     mhm3::Nbr3* d_nbrs = nullptr;
     int32_t* d_face_ka = nullptr;
     // frontal elimination (front_plan.h, local3d.cu: upload_front_tables)
-    int fsteps = 0, fslots = 0;
+    int fsteps = 0, fslots = 0, ffirst = 0, foff = 0;
     int4* d_fev = nullptr;
-    uint32_t *d_fent = nullptr, *d_fcon = nullptr;
+    int32_t* d_frp = nullptr;
+    uint32_t *d_fent = nullptr, *d_fcon = nullptr, *d_fval = nullptr, *d_frc = nullptr, *d_fcol = nullptr;
     double *d_cls24 = nullptr, *d_geo24 = nullptr, *d_mass1 = nullptr;
     uint8_t* d_fcnt = nullptr;
 };

@@ -168,7 +168,7 @@ struct RecSmem {
 __host__ __device__ inline RecSmem rec_smem(int vec, int NI, int kind, int P, int N) {
     const int PN = P * N;
     RecSmem l;
-    int o = (int)front_shared_doubles(vec);
+    int o = (int)front_shared_values(vec);
     l.Ke = o, o += 72;
     l.mass = o, o += 8;
     l.lamc = o, o += NI;     // k_i (-s |F|) per local multiplier
@@ -187,7 +187,7 @@ __global__ void __launch_bounds__(T::threads, MINB) k_reconstruct(const __grid_c
     __shared__ FrontCtx c;
     const int P = g.P, N = g.N, PN = g.PN, NI = g.NI, tid = threadIdx.x, nthr = blockDim.x, stride = g.slots + 1;
     const RecSmem L = rec_smem(T::vec, NI, g.src_kind, P, N);
-    const FrontShared sh = front_shared(smem, T::vec);
+    const FrontShared<double> sh = front_shared(smem, T::vec);
     double *Ke = smem + L.Ke, *lamc = smem + L.lamc, *xs = smem + L.xs, *z = smem + L.z;
     double* keep = reinterpret_cast<double*>(g.ws + (size_t)blockIdx.x * g.slot_bytes);
     for (int64_t ki = blockIdx.x; ki < g.nK; ki += gridDim.x) {
