@@ -359,9 +359,9 @@ mhm_status mhm_assemble_skeleton(const mhm_mesh* mesh, const double* AK_dev, con
  * saddle-point system [A B^T; B 0] [lambda; u0] = [E; F] in FP64 on the device,
  * with A_vals_dev / E_dev from mhm_assemble_skeleton, B from BK_dev
  * (B[K, K's local multiplier j] = BK_dev[K*N_I + j]) and F = FK_dev (n_K).
- * Writes lambda_dev (n_lambda) and u0_dev (n_K).  The matrix is assembled in CSR
- * and factored by cuSOLVER's sparse QR (a library direct solver; this stage is
- * outside the local-problem hot path).  Allocates temporary device memory.
+ * Writes lambda_dev (n_lambda) and u0_dev (n_K).  A multifrontal LDL^T in a nested
+ * dissection order of T_H, with one step of refinement; the plan and its device memory are
+ * made on the first call and kept by the mesh.  Synchronous (it reports a zero pivot).
  * Errors: INVALID_ARG (NULL, singular matrix), UNSUPPORTED, CUDA. */
 mhm_status mhm_solve_global(const mhm_mesh* mesh, const double* A_vals_dev, const double* E_dev,
                             const double* BK_dev, const double* FK_dev, double* lambda_dev, double* u0_dev,

@@ -21,13 +21,13 @@
 // Storage.  Every node has an F x F front (column-major, lower triangle) in one buffer:
 // after its factorisation its first k columns hold L (unit lower triangle, diagonal entries
 // replaced by D) and its trailing (F - k) x (F - k) block the update matrix its parent adds
-// in.  Small fronts are factored one per thread block with the panel in shared memory;
-// large separators holding multipliers only by the dense library routines (cuSOLVER potrf
-// of the negated pivot block, cuBLAS trsm and syrk), converted to the same LDL^T form.  One step of iterative
-// refinement against the assembled system follows the solve.
-#include <cublas_v2.h>
+// in.  All fronts of a depth are factored together, 32 pivots at a time: k_nd_panel factors the
+// diagonal block and solves the rows below it, k_nd_update subtracts L D L^T from the trailing
+// tiles.  (Library factorisations, one front after the other, took 93 of 132 ms at 128 x 128
+// squares with 6 multipliers per face; 5.0 G multiply-adds are 8.0 ms of the FP64 pipe.)
+// Forward and backward substitution take 32 pivots at a time too, one block per front.  One
+// step of iterative refinement against the assembled system follows the solve.
 #include <cuda_runtime.h>
-#include <cusolverDn.h>
 
 #include <algorithm>
 #include <functional>
@@ -46,41 +46,39 @@ struct NDNode {
     int64_t map_off[2] = {0, 0};         // children's update positions in this front
     std::vector<int32_t> idx;            // the front's unknowns: own (elimination order), then update
     int32_t deferred = -1;               // a u0 passed up to the parent (see dissect)
-    int64_t k_lam = 0;                   // own multipliers (the first k_lam own unknowns)
-    bool big = false;                    // factored by the library routines
 };
 
 struct NDPlan {
     std::vector<NDNode> nodes;              // post-order (children before parents)
     std::vector<std::vector<int>> by_depth;
-    int64_t n = 0, front_doubles = 0, vec_doubles = 0, map_ints = 0, idx_ints = 0;
-    int64_t max_big_k = 0;
+    struct Depth {              // the nodes of one depth in the list of all, and their largest sizes
+        int64_t first = 0, count = 0, k = 0, F = 0, child = 0;
+    };
+    std::vector<Depth> depth;
+    int64_t n = 0, front_doubles = 0, vec_doubles = 0;
     // device
     double* fronts = nullptr;
     double* vecs = nullptr;
     double* x = nullptr;       // solution
-    double* b = nullptr;       // right-hand side / residual
+    double* dx = nullptr;      // correction of the refinement step
+    double* b = nullptr;       // right-hand side
+    double* r = nullptr;       // residual
+    double* diag = nullptr;    // factored 32 x 32 diagonal blocks of the depth at hand, by node
+    int* list = nullptr;       // nodes by depth
     double* vals = nullptr;    // values of the assembled saddle-point CSR (refinement)
     int64_t* dst = nullptr;    // per saddle-point entry: its place in a front (lower triangle), or -1
     int32_t* maps = nullptr;   // children's update -> parent front positions
     int32_t* idx = nullptr;    // all fronts' unknowns
-    int64_t* idx_off = nullptr;
     int64_t* node_info = nullptr;   // per node: k, F, front_off, vec_off, map_off[0..1], child[0..1], idx offset
-    int* dinfo = nullptr;           // potrf status per large node
-    double* work = nullptr;         // potrf workspace
-    int lwork = 0;
-    cusolverDnHandle_t dn = nullptr;
-    cublasHandle_t bl = nullptr;
+    int* dinfo = nullptr;           // per node: a pivot was zero or not finite
 };
 
 void free_nd_plan(NDPlan* p) {
     if (!p) return;
-    for (void* q : {(void*)p->fronts, (void*)p->vecs, (void*)p->x, (void*)p->b, (void*)p->vals, (void*)p->dst,
-                    (void*)p->maps, (void*)p->idx, (void*)p->idx_off, (void*)p->node_info, (void*)p->dinfo,
-                    (void*)p->work})
+    for (void* q : {(void*)p->fronts, (void*)p->vecs, (void*)p->x, (void*)p->dx, (void*)p->b, (void*)p->r,
+                    (void*)p->diag, (void*)p->list, (void*)p->vals, (void*)p->dst, (void*)p->maps, (void*)p->idx,
+                    (void*)p->node_info, (void*)p->dinfo})
         if (q) cudaFree(q);
-    if (p->dn) cusolverDnDestroy(p->dn);
-    if (p->bl) cublasDestroy(p->bl);
     delete p;
 }
 
@@ -88,7 +86,8 @@ namespace {
 
 constexpr int kNodeInfo = 10;   // int64 fields per node on the device
 constexpr int kNdThreads = 256;
-constexpr size_t kSmallPanelBytes = 160 * 1024;   // panel (F x k doubles) of the one-block kernel
+constexpr int kNdPanel = 32;    // pivots per step
+constexpr int kNdRows = 128;    // rows per block of k_nd_panel
 
 // ---------------------------------------------------------------- symbolic ---
 
@@ -226,11 +225,24 @@ mhm_status build_nd_plan(const mhm_mesh* m, NDPlan** out) {
         P->front_doubles += nd.F * nd.F;
         nd.vec_off = P->vec_doubles;
         P->vec_doubles += nd.F;
-        nd.k_lam = 0;   // own multipliers come first, then the own u0
-        while (nd.k_lam < nd.k && nd.idx[nd.k_lam] < m->nlam) ++nd.k_lam;
-        nd.big = (size_t)nd.F * nd.k * sizeof(double) > kSmallPanelBytes && nd.k_lam > 0;
-        if (nd.big) P->max_big_k = std::max(P->max_big_k, nd.k_lam);
         P->by_depth[nd.depth].push_back((int)id);
+    }
+    std::vector<int32_t> list;
+    size_t widest = 1;
+    for (const std::vector<int>& ids : P->by_depth) {
+        NDPlan::Depth d;
+        d.first = (int64_t)list.size();
+        d.count = (int64_t)ids.size();
+        widest = std::max(widest, ids.size());
+        for (int id : ids) {
+            const NDNode& nd = P->nodes[id];
+            list.push_back(id);
+            d.k = std::max(d.k, nd.k);
+            d.F = std::max(d.F, nd.F);
+            for (int c : nd.child)
+                if (c >= 0) d.child = std::max(d.child, P->nodes[c].F - P->nodes[c].k);
+        }
+        P->depth.push_back(d);
     }
     // children's update positions in the parent's front
     std::vector<int32_t> maps;
@@ -251,7 +263,6 @@ mhm_status build_nd_plan(const mhm_mesh* m, NDPlan** out) {
             }
         }
     }
-    P->map_ints = (int64_t)maps.size();
     // each saddle-point entry (r, c) goes to the front of whichever of r, c is eliminated
     // first (post-order of the nodes, then the order inside the node), lower triangle only
     std::vector<int64_t> dst(m->aug_nnz, -1);
@@ -276,11 +287,10 @@ mhm_status build_nd_plan(const mhm_mesh* m, NDPlan** out) {
             if (pr >= pc) dst[t] = nd.front_off + pr + pc * nd.F;
         }
     }
-    std::vector<int64_t> info(P->nodes.size() * kNodeInfo), idx_off(P->nodes.size() + 1, 0);
+    std::vector<int64_t> info(P->nodes.size() * kNodeInfo);
     std::vector<int32_t> idx_all;
     for (size_t id = 0; id < P->nodes.size(); ++id) {
         const NDNode& nd = P->nodes[id];
-        idx_off[id] = (int64_t)idx_all.size();
         idx_all.insert(idx_all.end(), nd.idx.begin(), nd.idx.end());
         int64_t* q = &info[id * kNodeInfo];
         q[0] = nd.k;
@@ -294,8 +304,6 @@ mhm_status build_nd_plan(const mhm_mesh* m, NDPlan** out) {
         q[8] = (int64_t)idx_all.size() - nd.F;
         q[9] = nd.child[0] >= 0 ? P->nodes[nd.child[0]].F - P->nodes[nd.child[0]].k : 0;
     }
-    idx_off.back() = (int64_t)idx_all.size();
-    P->idx_ints = (int64_t)idx_all.size();
     // device
     auto up = [](const auto& v, auto** d) -> cudaError_t {
         using T = typename std::decay<decltype(v[0])>::type;
@@ -306,34 +314,20 @@ mhm_status build_nd_plan(const mhm_mesh* m, NDPlan** out) {
     cudaError_t e = cudaMalloc((void**)&P->fronts, P->front_doubles * sizeof(double));
     if (e == cudaSuccess) e = cudaMalloc((void**)&P->vecs, P->vec_doubles * sizeof(double));
     if (e == cudaSuccess) e = cudaMalloc((void**)&P->x, P->n * sizeof(double));
+    if (e == cudaSuccess) e = cudaMalloc((void**)&P->dx, P->n * sizeof(double));
     if (e == cudaSuccess) e = cudaMalloc((void**)&P->b, P->n * sizeof(double));
+    if (e == cudaSuccess) e = cudaMalloc((void**)&P->r, P->n * sizeof(double));
+    if (e == cudaSuccess) e = cudaMalloc((void**)&P->diag, widest * kNdPanel * kNdPanel * sizeof(double));
     if (e == cudaSuccess) e = cudaMalloc((void**)&P->vals, std::max<int64_t>(1, m->aug_nnz) * sizeof(double));
     if (e == cudaSuccess) e = up(dst, &P->dst);
     if (e == cudaSuccess) e = up(maps, &P->maps);
     if (e == cudaSuccess) e = up(idx_all, &P->idx);
-    if (e == cudaSuccess) e = up(idx_off, &P->idx_off);
+    if (e == cudaSuccess) e = up(list, &P->list);
     if (e == cudaSuccess) e = up(info, &P->node_info);
     if (e == cudaSuccess) e = cudaMalloc((void**)&P->dinfo, std::max<size_t>(1, P->nodes.size()) * sizeof(int));
     if (e != cudaSuccess) {
         free_nd_plan(P);
         return cuda_fail(e, "mhm_solve_global: device memory of the factorisation");
-    }
-    if (cusolverDnCreate(&P->dn) != CUSOLVER_STATUS_SUCCESS || cublasCreate(&P->bl) != CUBLAS_STATUS_SUCCESS) {
-        free_nd_plan(P);
-        return fail(MHM_ERR_CUDA, "mhm_solve_global: cuSOLVER / cuBLAS handles");
-    }
-    if (P->max_big_k > 0) {
-        int lw = 0;
-        if (cusolverDnDpotrf_bufferSize(P->dn, CUBLAS_FILL_MODE_LOWER, (int)P->max_big_k, P->fronts,
-                                        (int)P->max_big_k, &lw) != CUSOLVER_STATUS_SUCCESS) {
-            free_nd_plan(P);
-            return fail(MHM_ERR_CUDA, "mhm_solve_global: potrf workspace query");
-        }
-        P->lwork = lw;
-        if (cudaMalloc((void**)&P->work, std::max(1, lw) * sizeof(double)) != cudaSuccess) {
-            free_nd_plan(P);
-            return fail(MHM_ERR_OOM, "mhm_solve_global: potrf workspace");
-        }
     }
     *out = P;
     return MHM_OK;
@@ -356,136 +350,149 @@ __global__ void k_nd_assemble(int64_t nnz, const int64_t* dst, const double* val
 }
 
 // The update block of child slot s of every node in `list` added into the node's front
-// (lower triangles on both sides).
+// (lower triangles on both sides); grid (nodes, groups of the child's columns).
 __global__ void k_nd_extend_add(const int* list, int slot, const int64_t* info, const int32_t* maps, double* fronts) {
-    const int id = list[blockIdx.x];
-    const int64_t* q = info + (int64_t)id * kNodeInfo;
+    const int64_t* q = info + (int64_t)list[blockIdx.x] * kNodeInfo;
     const int64_t c = q[6 + slot];
     if (c < 0) return;
     const int64_t* qc = info + c * kNodeInfo;
-    const int64_t kc = qc[0], Fc = qc[1], nu = Fc - kc, Fp = q[1];
+    const int64_t kc = qc[0], Fc = qc[1], Fp = q[1];
+    const int nu = (int)(Fc - kc);
     const int32_t* map = maps + q[4 + slot];
     const double* C = fronts + qc[2];
     double* Pf = fronts + q[2];
-    for (int64_t t = threadIdx.x; t < nu * nu; t += blockDim.x) {
-        const int64_t j = t / nu, i = t - j * nu;
-        if (i < j) continue;
-        const int64_t pi = map[i], pj = map[j];
-        const int64_t hi = pi > pj ? pi : pj, lo = pi > pj ? pj : pi;
-        Pf[hi + lo * Fp] += C[(kc + i) + (kc + j) * Fc];
+    // a warp per column
+    for (int j = blockIdx.y * (blockDim.x >> 5) + (threadIdx.x >> 5); j < nu; j += gridDim.y * (blockDim.x >> 5)) {
+        const int64_t pj = map[j];
+        for (int i = j + (threadIdx.x & 31); i < nu; i += 32) {
+            const int64_t pi = map[i], hi = pi > pj ? pi : pj, lo = pi > pj ? pj : pi;
+            Pf[hi + lo * Fp] += C[(kc + i) + (kc + j) * Fc];
+        }
     }
 }
 
-// LDL^T without pivoting of the first k columns of a front (one block per front): the
-// F x k panel is factored in shared memory (column-major, right-looking, one pivot at a
-// time), written back (L below the diagonal, D on it), and the trailing block takes
-// U -= L21 D L21^T (lower triangle).
-__global__ void __launch_bounds__(kNdThreads) k_nd_factor_small(const int* list, const int64_t* info, double* fronts,
-                                                                int* bad) {
-    extern __shared__ double pan[];
+// One step of the LDL^T without pivoting of every front of a depth: the diagonal block of the
+// (up to) 32 pivots from p0 on and the rows below it, l = w / d with w_q = a_q - sum_{r<q}
+// w_r L_qr.  Grid (nodes, groups of 128 rows): every block factors the diagonal block for
+// itself in shared memory (about 5 us), a thread solves one row in registers.  The factored
+// diagonal block goes to `diag` (the other blocks of the front still read the old one);
+// k_nd_update puts it in place.
+__global__ void __launch_bounds__(kNdRows) k_nd_panel(const int* list, const int64_t* info, double* fronts, int p0,
+                                                      double* diag, int* bad) {
+    __shared__ double L[kNdPanel][kNdPanel + 1];
+    __shared__ double dinv[kNdPanel];
     const int id = list[blockIdx.x];
     const int64_t* q = info + (int64_t)id * kNodeInfo;
     const int k = (int)q[0], F = (int)q[1];
+    const int nb = min(kNdPanel, k - p0);
+    const int row0 = p0 + nb + blockIdx.y * kNdRows;
+    if (nb <= 0 || (blockIdx.y > 0 && row0 >= F)) return;
     double* Fr = fronts + q[2];
-    for (int t = threadIdx.x; t < F * k; t += blockDim.x) {
-        const int j = t / F, i = t - j * F;
-        pan[t] = i >= j ? Fr[i + (int64_t)j * F] : 0.0;
-    }
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    for (int j = warp; j < kNdPanel; j += kNdRows / 32)
+        L[lane][j] = lane >= j && lane < nb ? Fr[(p0 + lane) + (int64_t)(p0 + j) * F] : (lane == j ? 1.0 : 0.0);
     __syncthreads();
-    for (int p = 0; p < k; ++p) {
-        const double d = pan[p + p * F];
-        if (!(fabs(d) > 0.0) && threadIdx.x == 0) bad[id] = 1;   // zero or not finite
-        const double inv = 1.0 / d;
-        // rows below p of the remaining panel columns: P[i][j] -= P[i][p] P[j][p] / d
-        const int nr = F - p - 1, nc = k - p - 1;
-        for (int t = threadIdx.x; t < nr * nc; t += blockDim.x) {
-            const int jj = t / nr, ii = t - jj * nr;
-            const int i = p + 1 + ii, j = p + 1 + jj;
-            if (i >= j) pan[i + j * F] -= pan[i + p * F] * pan[j + p * F] * inv;
+    for (int p = 0; p < nb; ++p) {   // column p keeps w = l d until the end
+        const double d = L[p][p];
+        if (threadIdx.x == 0) {
+            if (!(fabs(d) > 0.0) && blockIdx.y == 0) bad[id] = 1;   // zero or not finite
+            dinv[p] = 1.0 / d;
         }
         __syncthreads();
-        for (int i = p + 1 + threadIdx.x; i < F; i += blockDim.x) pan[i + p * F] *= inv;
+        const double s = L[lane][p] * dinv[p];
+        for (int j = p + 1 + warp; j < nb; j += kNdRows / 32)
+            if (lane >= j) L[lane][j] -= s * L[j][p];
         __syncthreads();
     }
-    for (int t = threadIdx.x; t < F * k; t += blockDim.x) {
-        const int j = t / F, i = t - j * F;
-        if (i >= j) Fr[i + (int64_t)j * F] = pan[t];
-    }
-    // trailing update with the scaled columns: U[i][j] -= sum_p L[i][p] d_p L[j][p]
-    const int nu = F - k;
-    for (int64_t t = threadIdx.x; t < (int64_t)nu * nu; t += blockDim.x) {
-        const int jj = (int)(t / nu), ii = (int)(t - (int64_t)jj * nu);
-        if (ii < jj) continue;
-        const int i = k + ii, j = k + jj;
-        double s = 0.0;
-        for (int p = 0; p < k; ++p) s = fma(pan[i + p * F] * pan[p + p * F], pan[j + p * F], s);
-        Fr[i + (int64_t)j * F] -= s;
-    }
+    if (threadIdx.x >= nb && threadIdx.x < kNdPanel) dinv[threadIdx.x] = 1.0;
+    __syncthreads();
+    for (int j = warp; j < kNdPanel; j += kNdRows / 32)
+        if (lane > j) L[lane][j] *= dinv[j];
+    __syncthreads();
+    if (blockIdx.y == 0)
+        for (int j = warp; j < kNdPanel; j += kNdRows / 32)
+            diag[((int64_t)blockIdx.x * kNdPanel + j) * kNdPanel + lane] = L[lane][j];
+    const int i = row0 + threadIdx.x;
+    if (i >= F) return;
+    double w[kNdPanel];
+#pragma unroll
+    for (int c = 0; c < kNdPanel; ++c) w[c] = c < nb ? Fr[i + (int64_t)(p0 + c) * F] : 0.0;
+#pragma unroll
+    for (int c = 1; c < kNdPanel; ++c)
+#pragma unroll
+        for (int r = 0; r < c; ++r) w[c] = fma(-w[r], L[c][r], w[c]);
+#pragma unroll
+    for (int c = 0; c < kNdPanel; ++c)
+        if (c < nb) Fr[i + (int64_t)(p0 + c) * F] = w[c] * dinv[c];
 }
 
-// Negates the lower triangle of the k x k pivot block of a large front (potrf then
-// factors -F11 = C C^T).
-__global__ void k_nd_negate_pivots(double* Fr, int64_t F, int64_t k) {
-    for (int64_t t = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; t < k * k; t += (int64_t)gridDim.x * blockDim.x) {
-        const int64_t j = t / k, i = t - j * k;
-        if (i >= j) Fr[i + j * F] = -Fr[i + j * F];
+// The step's update of the trailing lower triangle, U -= L21 D L21^T, in TS x TS tiles (grid
+// (nodes, tiles)), a thread 4 x 4 entries; tile 0 also puts the factored diagonal block in place.
+template <int TS>
+__global__ void __launch_bounds__(TS * TS / 16) k_nd_update(const int* list, const int64_t* info, double* fronts, int p0,
+                                                            const double* diag) {
+    __shared__ double Ls[kNdPanel][TS], Ws[kNdPanel][TS];
+    constexpr int TH = TS / 4, NT = TH * TH;
+    const int64_t* q = info + (int64_t)list[blockIdx.x] * kNodeInfo;
+    const int k = (int)q[0], F = (int)q[1];
+    const int nb = min(kNdPanel, k - p0);
+    if (nb <= 0) return;
+    double* Fr = fronts + q[2];
+    const double* dg = diag + (int64_t)blockIdx.x * kNdPanel * kNdPanel;
+    if (blockIdx.y == 0)
+        for (int t = threadIdx.x; t < nb * kNdPanel; t += NT) {
+            const int j = t / kNdPanel, i = t % kNdPanel;
+            if (i >= j && i < nb) Fr[(p0 + i) + (int64_t)(p0 + j) * F] = dg[j * kNdPanel + i];
+        }
+    const int pe = p0 + nb, nt = (F - pe + TS - 1) / TS;
+    int ti = (int)((sqrtf(8.0f * blockIdx.y + 1.0f) - 1.0f) * 0.5f);   // tile row of the lower triangle
+    while (ti * (ti + 1) / 2 > (int)blockIdx.y) --ti;
+    while ((ti + 1) * (ti + 2) / 2 <= (int)blockIdx.y) ++ti;
+    const int tj = (int)blockIdx.y - ti * (ti + 1) / 2;
+    if (ti >= nt) return;
+    const int r0 = pe + ti * TS, c0 = pe + tj * TS;
+    for (int t = threadIdx.x; t < kNdPanel * TS; t += NT) {
+        const int c = t / TS, i = t % TS;
+        const double d = c < nb ? dg[c * kNdPanel + c] : 0.0;
+        Ls[c][i] = c < nb && r0 + i < F ? Fr[(r0 + i) + (int64_t)(p0 + c) * F] : 0.0;
+        Ws[c][i] = c < nb && c0 + i < F ? d * Fr[(c0 + i) + (int64_t)(p0 + c) * F] : 0.0;
     }
+    __syncthreads();
+    const int tx = threadIdx.x % TH, ty = threadIdx.x / TH;   // rows tx + TH a, columns ty + TH b
+    double acc[4][4] = {};
+    for (int c = 0; c < nb; ++c) {
+        double l[4], w[4];
+#pragma unroll
+        for (int a = 0; a < 4; ++a) l[a] = Ls[c][tx + TH * a], w[a] = Ws[c][ty + TH * a];
+#pragma unroll
+        for (int a = 0; a < 4; ++a)
+#pragma unroll
+            for (int b = 0; b < 4; ++b) acc[a][b] = fma(l[a], w[b], acc[a][b]);
+    }
+#pragma unroll
+    for (int b = 0; b < 4; ++b)
+#pragma unroll
+        for (int a = 0; a < 4; ++a) {
+            const int i = r0 + tx + TH * a, j = c0 + ty + TH * b;
+            if (i < F && j <= i) Fr[i + (int64_t)j * F] -= acc[a][b];
+        }
 }
 
-// From -F11 = C C^T and W = F21 C^-T to the LDL^T form: L11 = C diag(c)^-1, d = -c^2,
-// L21 = -W diag(c)^-1 (c the diagonal of C).
-__global__ void k_nd_to_ldlt(double* Fr, int64_t F, int64_t k) {
-    for (int64_t t = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; t < F * k; t += (int64_t)gridDim.x * blockDim.x) {
-        const int64_t j = t / F, i = t - j * F;
-        if (i < j) continue;
-        const double cj = Fr[j + j * F];
-        if (i == j) continue;
-        Fr[i + j * F] = i < k ? Fr[i + j * F] / cj : -Fr[i + j * F] / cj;
-    }
-}
-__global__ void k_nd_to_ldlt_diag(double* Fr, int64_t F, int64_t k) {
-    for (int64_t j = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; j < k; j += (int64_t)gridDim.x * blockDim.x) {
-        const double c = Fr[j + j * F];
-        Fr[j + j * F] = -c * c;
-    }
-}
-
-// One pivot p of a front (leading dimension F) eliminated right-looking over the trailing
-// block: Fr[i][j] -= Fr[i][p] Fr[j][p] / d for F > i >= j > p; then the column is scaled.
-__global__ void k_nd_pivot_update(double* Fr, int64_t F, int64_t p) {
-    const double inv = 1.0 / Fr[p + p * F];
-    const int64_t n = F - p - 1;
-    for (int64_t t = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; t < n * n; t += (int64_t)gridDim.x * blockDim.x) {
-        const int64_t jj = t / n, ii = t - jj * n;
-        if (ii < jj) continue;
-        const int64_t i = p + 1 + ii, j = p + 1 + jj;
-        Fr[i + j * F] -= Fr[i + p * F] * Fr[j + p * F] * inv;
-    }
-}
-__global__ void k_nd_pivot_scale(double* Fr, int64_t F, int64_t p, int* bad) {
-    const double d = Fr[p + p * F];
-    if (!(fabs(d) > 0.0)) {
-        if (blockIdx.x == 0 && threadIdx.x == 0) *bad = 1;
-        return;
-    }
-    for (int64_t i = p + 1 + (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < F; i += (int64_t)gridDim.x * blockDim.x)
-        Fr[i + p * F] /= d;
-}
-
-// Forward elimination and diagonal scaling of one level (one block per node): the front
-// vector takes the own right-hand sides and the children's update vectors; own pivots in
-// order, v[i] -= L[i][p] y_p for the rows below; then z = y / d on the own part.  The
-// update part stays for the parent.
+// Forward elimination and diagonal scaling of one depth (one block per node): the front
+// vector (shared memory, F values) takes the own right-hand sides and the children's update
+// vectors; 32 own pivots at a time, solved by one warp against the diagonal block, then
+// subtracted from the rows below; then z = y / d on the own part.  The update part stays for
+// the parent.
 __global__ void __launch_bounds__(kNdThreads) k_nd_forward(const int* list, const int64_t* info, const int32_t* maps,
                                                            const int32_t* idx, const double* fronts, double* vecs,
                                                            const double* b) {
-    const int id = list[blockIdx.x];
-    const int64_t* q = info + (int64_t)id * kNodeInfo;
-    const int64_t k = q[0], F = q[1];
+    extern __shared__ double v[];
+    __shared__ double L[kNdPanel][kNdPanel + 1];
+    const int64_t* q = info + (int64_t)list[blockIdx.x] * kNodeInfo;
+    const int k = (int)q[0], F = (int)q[1], lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     const double* Fr = fronts + q[2];
-    double* v = vecs + q[3];
     const int32_t* ix = idx + q[8];
-    for (int64_t i = threadIdx.x; i < F; i += blockDim.x) v[i] = i < k ? b[ix[i]] : 0.0;
+    for (int i = threadIdx.x; i < F; i += kNdThreads) v[i] = i < k ? b[ix[i]] : 0.0;
     __syncthreads();
     for (int s = 0; s < 2; ++s) {   // children in a fixed order
         const int64_t c = q[6 + s];
@@ -494,45 +501,74 @@ __global__ void __launch_bounds__(kNdThreads) k_nd_forward(const int* list, cons
         const int64_t kc = qc[0], nu = qc[1] - kc;
         const double* vc = vecs + qc[3];
         const int32_t* map = maps + q[4 + s];
-        for (int64_t i = threadIdx.x; i < nu; i += blockDim.x) v[map[i]] += vc[kc + i];
+        for (int64_t i = threadIdx.x; i < nu; i += kNdThreads) v[map[i]] += vc[kc + i];
         __syncthreads();
     }
-    for (int64_t p = 0; p < k; ++p) {
-        const double yp = v[p];
-        for (int64_t i = p + 1 + threadIdx.x; i < F; i += blockDim.x) v[i] = fma(-Fr[i + p * F], yp, v[i]);
+    for (int p0 = 0; p0 < k; p0 += kNdPanel) {
+        const int nb = min(kNdPanel, k - p0);
+        for (int j = warp; j < nb; j += kNdThreads / 32)
+            if (lane < nb) L[lane][j] = Fr[(p0 + lane) + (int64_t)(p0 + j) * F];
         __syncthreads();
-    }
-    for (int64_t p = threadIdx.x; p < k; p += blockDim.x) v[p] /= Fr[p + p * F];
-}
-
-// Back substitution of one level (one block per node, parents before children): x at the
-// update unknowns comes from the solution vector (ancestors); x_p = z_p - sum_{i > p}
-// L[i][p] x_i for the own pivots from last to first; the own x go to the solution vector.
-__global__ void __launch_bounds__(kNdThreads) k_nd_backward(const int* list, const int64_t* info, const int32_t* idx,
-                                                            const double* fronts, double* vecs, double* x) {
-    __shared__ double red[kNdThreads / 32];
-    const int id = list[blockIdx.x];
-    const int64_t* q = info + (int64_t)id * kNodeInfo;
-    const int64_t k = q[0], F = q[1];
-    const double* Fr = fronts + q[2];
-    double* v = vecs + q[3];
-    const int32_t* ix = idx + q[8];
-    for (int64_t i = k + threadIdx.x; i < F; i += blockDim.x) v[i] = x[ix[i]];
-    __syncthreads();
-    for (int64_t p = k - 1; p >= 0; --p) {
-        double s = 0.0;
-        for (int64_t i = p + 1 + threadIdx.x; i < F; i += blockDim.x) s = fma(Fr[i + p * F], v[i], s);
-        for (int o = 16; o > 0; o >>= 1) s += __shfl_down_sync(0xffffffffu, s, o);
-        if ((threadIdx.x & 31) == 0) red[threadIdx.x >> 5] = s;
+        if (warp == 0) {
+            double y = lane < nb ? v[p0 + lane] : 0.0;
+            for (int r = 0; r < nb; ++r) {
+                const double yr = __shfl_sync(0xffffffffu, y, r);
+                if (lane > r && lane < nb) y = fma(-L[lane][r], yr, y);
+            }
+            if (lane < nb) v[p0 + lane] = y;
+        }
         __syncthreads();
-        if (threadIdx.x == 0) {
-            double t = 0.0;
-            for (int w = 0; w < kNdThreads / 32; ++w) t += red[w];   // fixed order
-            v[p] -= t;
+        for (int i = p0 + nb + threadIdx.x; i < F; i += kNdThreads) {
+            const double* col = Fr + i + (int64_t)p0 * F;
+            double s = v[i];
+#pragma unroll 8
+            for (int c = 0; c < nb; ++c) s = fma(-col[(int64_t)c * F], v[p0 + c], s);
+            v[i] = s;
         }
         __syncthreads();
     }
-    for (int64_t p = threadIdx.x; p < k; p += blockDim.x) x[ix[p]] = v[p];
+    double* out = vecs + q[3];
+    for (int i = threadIdx.x; i < F; i += kNdThreads) out[i] = i < k ? v[i] / Fr[i + (int64_t)i * F] : v[i];
+}
+
+// Back substitution of one depth (one block per node, parents before children): x at the
+// update unknowns comes from the solution vector (ancestors); x_p = z_p - sum_{i > p}
+// L[i][p] x_i for the own pivots from last to first, 32 at a time (a warp per column for the
+// rows below the diagonal block, then one warp inside it); the own x go to the solution vector.
+__global__ void __launch_bounds__(kNdThreads) k_nd_backward(const int* list, const int64_t* info, const int32_t* idx,
+                                                            const double* fronts, const double* vecs, double* x) {
+    extern __shared__ double v[];
+    __shared__ double L[kNdPanel][kNdPanel + 1];
+    __shared__ double sum[kNdPanel];
+    const int64_t* q = info + (int64_t)list[blockIdx.x] * kNodeInfo;
+    const int k = (int)q[0], F = (int)q[1], lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    const double* Fr = fronts + q[2];
+    const double* z = vecs + q[3];
+    const int32_t* ix = idx + q[8];
+    for (int i = threadIdx.x; i < F; i += kNdThreads) v[i] = i < k ? z[i] : x[ix[i]];
+    __syncthreads();
+    for (int p0 = (k - 1) / kNdPanel * kNdPanel; p0 >= 0; p0 -= kNdPanel) {
+        const int nb = min(kNdPanel, k - p0);
+        for (int j = warp; j < nb; j += kNdThreads / 32) {
+            const double* col = Fr + (int64_t)(p0 + j) * F;
+            if (lane < nb) L[lane][j] = col[p0 + lane];
+            double s = 0.0;
+            for (int i = p0 + nb + lane; i < F; i += 32) s = fma(col[i], v[i], s);
+            for (int o = 16; o > 0; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
+            if (lane == 0) sum[j] = s;
+        }
+        __syncthreads();
+        if (warp == 0) {
+            double t = lane < nb ? v[p0 + lane] - sum[lane] : 0.0;
+            for (int r = nb - 1; r > 0; --r) {
+                const double xr = __shfl_sync(0xffffffffu, t, r);
+                if (lane < r) t = fma(-L[r][lane], xr, t);
+            }
+            if (lane < nb) v[p0 + lane] = t;
+        }
+        __syncthreads();
+    }
+    for (int p = threadIdx.x; p < k; p += kNdThreads) x[ix[p]] = v[p];
 }
 
 // r = b - M x for the assembled saddle-point CSR (one warp per row, fixed summation order).
@@ -561,17 +597,37 @@ __global__ void k_add_split(int64_t L, int64_t nK, const double* x, const double
 
 unsigned blocks_for(int64_t n, int threads) { return (unsigned)std::max<int64_t>(1, (n + threads - 1) / threads); }
 
-// Solves M x = rhs (in P->b) into x with the factors in the fronts, level by level.
-mhm_status nd_solve(NDPlan* P, const int* d_lists, const std::vector<int64_t>& list_off, double* x, cudaStream_t s) {
-    const int D = (int)P->by_depth.size();
-    for (int d = D - 1; d >= 0; --d) {
-        const int n = (int)P->by_depth[d].size();
-        k_nd_forward<<<n, kNdThreads, 0, s>>>(d_lists + list_off[d], P->node_info, P->maps, P->idx, P->fronts, P->vecs,
-                                              P->b);
+// Solves M x = rhs into x with the factors in the fronts, depth by depth.
+mhm_status nd_solve(const NDPlan* P, const double* rhs, double* x, cudaStream_t s) {
+    for (size_t d = P->depth.size(); d-- > 0;) {
+        const NDPlan::Depth& q = P->depth[d];
+        k_nd_forward<<<(unsigned)q.count, kNdThreads, q.F * sizeof(double), s>>>(P->list + q.first, P->node_info, P->maps,
+                                                                                P->idx, P->fronts, P->vecs, rhs);
     }
-    for (int d = 0; d < D; ++d) {
-        const int n = (int)P->by_depth[d].size();
-        k_nd_backward<<<n, kNdThreads, 0, s>>>(d_lists + list_off[d], P->node_info, P->idx, P->fronts, P->vecs, x);
+    for (const NDPlan::Depth& q : P->depth)
+        k_nd_backward<<<(unsigned)q.count, kNdThreads, q.F * sizeof(double), s>>>(P->list + q.first, P->node_info, P->idx,
+                                                                                  P->fronts, P->vecs, x);
+    MHM_CUDA_TRY(cudaGetLastError());
+    return MHM_OK;
+}
+
+// Factors the fronts of one depth: children's updates, then 32 pivots at a time.
+mhm_status nd_factor(const NDPlan* P, const NDPlan::Depth& q, cudaStream_t s) {
+    const int* list = P->list + q.first;
+    const unsigned n = (unsigned)q.count;
+    if (q.child > 0)
+        for (int slot = 0; slot < 2; ++slot)
+            k_nd_extend_add<<<dim3(n, (unsigned)std::min<int64_t>(64, (q.child + 7) / 8)), kNdThreads, 0, s>>>(
+                list, slot, P->node_info, P->maps, P->fronts);
+    for (int64_t p0 = 0; p0 < q.k; p0 += kNdPanel) {
+        const int64_t rest = std::max<int64_t>(q.F - p0 - 1, 1);
+        k_nd_panel<<<dim3(n, (unsigned)((rest + kNdRows - 1) / kNdRows)), kNdRows, 0, s>>>(list, P->node_info, P->fronts,
+                                                                                          (int)p0, P->diag, P->dinfo);
+        // small fronts: 32 x 32 tiles (a leaf's trailing block has 24 to 72 rows)
+        const int64_t ts = q.F >= 256 ? 64 : 32, t = (rest + ts - 1) / ts;
+        const dim3 grid(n, (unsigned)(t * (t + 1) / 2));
+        if (ts == 64) k_nd_update<64><<<grid, 256, 0, s>>>(list, P->node_info, P->fronts, (int)p0, P->diag);
+        else k_nd_update<32><<<grid, 64, 0, s>>>(list, P->node_info, P->fronts, (int)p0, P->diag);
     }
     MHM_CUDA_TRY(cudaGetLastError());
     return MHM_OK;
@@ -599,114 +655,33 @@ extern "C" mhm_status mhm_solve_global(const mhm_mesh* mesh, const double* A_val
         mesh->nd = P;
     }
     NDPlan* P = mesh->nd;
-    if (cusolverDnSetStream(P->dn, s) != CUSOLVER_STATUS_SUCCESS || cublasSetStream(P->bl, s) != CUBLAS_STATUS_SUCCESS)
-        return fail(MHM_ERR_CUDA, "mhm_solve_global: library stream");
-    const int D = (int)P->by_depth.size();
-    // node lists per depth (small and large fronts apart) in one device array
-    std::vector<int32_t> lists;
-    std::vector<int64_t> list_off(D), small_off(D), small_n(D);
-    for (int d = 0; d < D; ++d) {
-        list_off[d] = (int64_t)lists.size();
-        for (int id : P->by_depth[d]) lists.push_back(id);
-    }
-    for (int d = 0; d < D; ++d) {
-        small_off[d] = (int64_t)lists.size();
-        for (int id : P->by_depth[d])
-            if (!P->nodes[id].big) lists.push_back(id);
-        small_n[d] = (int64_t)lists.size() - small_off[d];
-    }
-    int* d_lists = nullptr;
-    MHM_CUDA_TRY(cudaMallocAsync((void**)&d_lists, lists.size() * sizeof(int), s));
-    MHM_CUDA_TRY(cudaMemcpyAsync(d_lists, lists.data(), lists.size() * sizeof(int), cudaMemcpyHostToDevice, s));
     const int thr = 256;
-    mhm_status st = MHM_OK;
     // assembled saddle-point values, fronts zeroed and filled with the original entries
     k_fill_saddle<<<blocks_for(mesh->aug_nnz, thr), thr, 0, s>>>(mesh->aug_nnz, mesh->d_aug_src, A_vals, BK, P->vals);
-    cudaMemsetAsync(P->fronts, 0, P->front_doubles * sizeof(double), s);
-    cudaMemsetAsync(P->dinfo, 0, P->nodes.size() * sizeof(int), s);
+    MHM_CUDA_TRY(cudaMemsetAsync(P->fronts, 0, P->front_doubles * sizeof(double), s));
+    MHM_CUDA_TRY(cudaMemsetAsync(P->dinfo, 0, P->nodes.size() * sizeof(int), s));
     k_nd_assemble<<<blocks_for(mesh->aug_nnz, thr), thr, 0, s>>>(mesh->aug_nnz, P->dst, P->vals, P->fronts);
-    cudaError_t e = cudaGetLastError();
-    if (e != cudaSuccess) st = cuda_fail(e, "mhm_solve_global: assembly");
-    size_t smem_max = 0;
-    for (const NDNode& nd : P->nodes)
-        if (!nd.big) smem_max = std::max(smem_max, (size_t)(nd.F * nd.k) * sizeof(double));
-    if (!st && smem_max > 48 * 1024)
-        e = cudaFuncSetAttribute(k_nd_factor_small, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem_max);
-    if (!st && e != cudaSuccess) st = cuda_fail(e, "mhm_solve_global: shared memory of the front kernel");
-    // numeric factorisation, deepest level first
-    for (int d = D - 1; d >= 0 && !st; --d) {
-        const int n = (int)P->by_depth[d].size();
-        for (int slot = 0; slot < 2; ++slot)
-            k_nd_extend_add<<<n, thr, 0, s>>>(d_lists + list_off[d], slot, P->node_info, P->maps, P->fronts);
-        if (small_n[d] > 0) {
-            size_t sm = 0;
-            for (int id : P->by_depth[d])
-                if (!P->nodes[id].big) sm = std::max(sm, (size_t)(P->nodes[id].F * P->nodes[id].k) * sizeof(double));
-            k_nd_factor_small<<<(unsigned)small_n[d], kNdThreads, sm, s>>>(d_lists + small_off[d], P->node_info,
-                                                                          P->fronts, P->dinfo);
-        }
-        for (int id : P->by_depth[d]) {
-            const NDNode& nd = P->nodes[id];
-            if (!nd.big) continue;
-            double* Fr = P->fronts + nd.front_off;
-            // the own multipliers by the library routines, then the own u0 (the trailing
-            // pivots, at most two) one at a time
-            const int64_t F = nd.F, k = nd.k_lam, nu = F - k;
-            k_nd_negate_pivots<<<blocks_for(k * k, thr), thr, 0, s>>>(Fr, F, k);
-            if (cusolverDnDpotrf(P->dn, CUBLAS_FILL_MODE_LOWER, (int)k, Fr, (int)F, P->work, P->lwork, P->dinfo + id) !=
-                CUSOLVER_STATUS_SUCCESS) {
-                st = fail(MHM_ERR_CUDA, "mhm_solve_global: potrf");
-                break;
-            }
-            if (nu > 0) {
-                const double one = 1.0;
-                if (cublasDtrsm(P->bl, CUBLAS_SIDE_RIGHT, CUBLAS_FILL_MODE_LOWER, CUBLAS_OP_T, CUBLAS_DIAG_NON_UNIT,
-                                (int)nu, (int)k, &one, Fr, (int)F, Fr + k, (int)F) != CUBLAS_STATUS_SUCCESS ||
-                    cublasDsyrk(P->bl, CUBLAS_FILL_MODE_LOWER, CUBLAS_OP_N, (int)nu, (int)k, &one, Fr + k, (int)F, &one,
-                                Fr + k + k * F, (int)F) != CUBLAS_STATUS_SUCCESS) {
-                    st = fail(MHM_ERR_CUDA, "mhm_solve_global: trsm / syrk");
-                    break;
-                }
-            }
-            k_nd_to_ldlt<<<blocks_for(F * k, thr), thr, 0, s>>>(Fr, F, k);
-            k_nd_to_ldlt_diag<<<blocks_for(k, thr), thr, 0, s>>>(Fr, F, k);
-            for (int64_t piv = k; piv < nd.k; ++piv) {
-                const int64_t rest = F - piv - 1;
-                k_nd_pivot_update<<<(unsigned)std::min<int64_t>(4096, blocks_for(rest * rest, thr)), thr, 0, s>>>(Fr, F, piv);
-                k_nd_pivot_scale<<<(unsigned)std::min<int64_t>(64, blocks_for(rest, thr)), thr, 0, s>>>(Fr, F, piv,
-                                                                                                   P->dinfo + id);
-            }
-        }
-        e = cudaGetLastError();
-        if (!st && e != cudaSuccess) st = cuda_fail(e, "mhm_solve_global: factorisation");
-    }
-    // solve, then one step of refinement against the assembled system
+    MHM_CUDA_TRY(cudaGetLastError());
+    mhm_status st = MHM_OK;
+    size_t vec_bytes = 0;   // a front vector in shared memory
+    for (const NDPlan::Depth& d : P->depth) vec_bytes = std::max(vec_bytes, (size_t)d.F * sizeof(double));
+    if (vec_bytes > 200 * 1024) return fail(MHM_ERR_UNSUPPORTED, "mhm_solve_global: a front vector exceeds shared memory");
+    MHM_CUDA_TRY(cudaFuncSetAttribute(k_nd_forward, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)vec_bytes));
+    MHM_CUDA_TRY(cudaFuncSetAttribute(k_nd_backward, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)vec_bytes));
+    // numeric factorisation, deepest level first; solve, then one step of refinement against
+    // the assembled system
+    for (size_t d = P->depth.size(); d-- > 0 && !st;) st = nd_factor(P, P->depth[d], s);
     if (!st) {
         k_rhs_saddle<<<blocks_for(P->n, thr), thr, 0, s>>>(mesh->nlam, mesh->nK, E, FK, P->b);
-        st = nd_solve(P, d_lists, list_off, P->x, s);
-    }
-    double* dx = nullptr;
-    if (!st) {
-        e = cudaMallocAsync((void**)&dx, P->n * sizeof(double), s);
-        if (e != cudaSuccess) st = cuda_fail(e, "mhm_solve_global: cudaMallocAsync");
+        st = nd_solve(P, P->b, P->x, s);
     }
     if (!st) {
-        double* rhs = nullptr;
-        e = cudaMallocAsync((void**)&rhs, P->n * sizeof(double), s);
-        if (e == cudaSuccess) {
-            k_rhs_saddle<<<blocks_for(P->n, thr), thr, 0, s>>>(mesh->nlam, mesh->nK, E, FK, rhs);
-            k_nd_residual<<<blocks_for(P->n * 32, thr), thr, 0, s>>>(P->n, mesh->d_aug_rowptr, mesh->d_aug_cols, P->vals,
-                                                                     P->x, rhs, P->b);
-            st = nd_solve(P, d_lists, list_off, dx, s);
-            if (!st) k_add_split<<<blocks_for(P->n, thr), thr, 0, s>>>(mesh->nlam, mesh->nK, P->x, dx, lambda, u0);
-            cudaFreeAsync(rhs, s);
-        } else {
-            st = cuda_fail(e, "mhm_solve_global: cudaMallocAsync");
-        }
+        k_nd_residual<<<blocks_for(P->n * 32, thr), thr, 0, s>>>(P->n, mesh->d_aug_rowptr, mesh->d_aug_cols, P->vals, P->x,
+                                                                 P->b, P->r);
+        st = nd_solve(P, P->r, P->dx, s);
     }
-    if (dx) cudaFreeAsync(dx, s);
-    cudaFreeAsync(d_lists, s);
-    e = cudaGetLastError();
+    if (!st) k_add_split<<<blocks_for(P->n, thr), thr, 0, s>>>(mesh->nlam, mesh->nK, P->x, P->dx, lambda, u0);
+    cudaError_t e = cudaGetLastError();
     if (!st && e != cudaSuccess) st = cuda_fail(e, "mhm_solve_global: solve");
     if (!st) {
         // a zero or non-finite pivot means a singular system: report it (synchronises)
