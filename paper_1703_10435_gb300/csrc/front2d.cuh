@@ -13,33 +13,35 @@ struct FrontCtx {
     int sgn[3], rev[3], la1[3], bad, pin;   // pin: lattice point x | y << 16
 };
 
-// choose_pin by one warp (kappa > 0 orders like its bits): x | y << 16.
+// The pinned node, by one warp: the first node (in DOF order) of the first fine triangle of
+// largest kappa, as x | y << 16; DOF 0 when kappa is uniform.  Pinned in the stiffest region
+// the solution carries no large constant over it, which the face integrals would cancel in
+// rounding; any node of the element can be pinned here (a window over two levels takes only
+// those of its first two).  On channels of 1e3 the blocks of levels 3..7 come out
+// 1e-11 to 3e-11 of their norm off the exact ones (1e-10 to 3e-10 pinned in the first two levels).
 __device__ inline int choose_pin_warp(int P, int N, const double* kap) {
     const int lane = threadIdx.x & 31, PN = P * N;
-    const int ymax = N == 1 ? (P == 1 ? 0 : 1) : (P == 1 ? 1 : 3), jmax = N == 1 ? 1 : 2;
-    long long best = -1;
-    for (int j = 0; j < jmax; ++j)
-        for (int t = lane; t < 2 * (N - j) - 1; t += 32) {
-            const long long k = __double_as_longlong(kap[j * (2 * N - j) + t]);
-            best = k > best ? k : best;
-        }
+    long long best = -1;   // (kappa > 0 orders like its bits)
+    int at = 0;
+#pragma unroll 4
+    for (int t = lane; t < N * N; t += 32) {
+        const long long k = __double_as_longlong(kap[t]);
+        if (k > best) best = k, at = t;
+    }
     for (int o = 16; o > 0; o >>= 1) {
         const long long k = __shfl_xor_sync(0xffffffffu, best, o);
-        best = k > best ? k : best;
+        const int t = __shfl_xor_sync(0xffffffffu, at, o);
+        if (k > best || (k == best && t < at)) best = k, at = t;
     }
-    int bd = 1 << 30;
-    for (int j = 0; j < jmax; ++j)
-        for (int t = lane; t < 2 * (N - j) - 1; t += 32) {
-            if (__double_as_longlong(kap[j * (2 * N - j) + t]) != best) continue;
-            int nx[6], ny[6];
-            element_nodes(P, t < N - j, t < N - j ? t : t - (N - j), j, nx, ny);
-            for (int a = 0; a < (P == 1 ? 3 : 6); ++a)
-                if (ny[a] <= ymax) bd = min(bd, ny[a] * (PN + 1) - ny[a] * (ny[a] - 1) / 2 + nx[a]);
-        }
-    bd = __reduce_min_sync(0xffffffffu, bd);
-    int y = 0;
-    while (bd >= PN + 1 - y) bd -= PN + 1 - y, ++y;
-    return (bd & 0xffff) | y << 16;
+    int j = 0, t = at;
+    while (t >= 2 * (N - j) - 1) t -= 2 * (N - j) - 1, ++j;
+    int nx[6], ny[6], px = 0, py = 0, bd = 1 << 30;
+    element_nodes(P, t < N - j, t < N - j ? t : t - (N - j), j, nx, ny);
+    for (int a = 0; a < (P == 1 ? 3 : 6); ++a) {
+        const int d = ny[a] * (PN + 1) - ny[a] * (ny[a] - 1) / 2 + nx[a];
+        if (d < bd) bd = d, px = nx[a], py = ny[a];
+    }
+    return px | py << 16;
 }
 
 // Geometry, pin, element matrices (Ke, 72), mass of a node on k fine triangles (mass, 8) and
