@@ -130,7 +130,9 @@ typedef struct {
  *     substitution of the N_I + 1 right-hand sides, the face integrals in Gram
  *     form (s psi_j, eta_i)_{dK} = -Y_j . Y_i with Y = L^{-1} times the
  *     projected loads.
- *   MHM_MIXED (N_I <= 16, i.e. m <= 4; larger m runs MHM_FP64): the pinned
+ *   MHM_MIXED (runs MHM_FP64, iters 1, where that is the faster way to the same quality:
+ *     m > 4, and meshes of 512 elements or more unless it_max is 1 or no_fallback is set):
+ *     the pinned
  *     matrix scaled by its diagonal is factored once in FP32 (Sec. 3: factor once,
  *     then only products with the factor), the solutions are refined in FP64
  *     against the matrix-free FP64 residual, and the face integrals use the

@@ -23,6 +23,7 @@
 // time up to the block's index; a further warp prepares the entering rows.
 #pragma once
 
+#include <cmath>
 #include <utility>
 
 #include "front_plan.h"
@@ -103,6 +104,13 @@ __device__ __forceinline__ double front_rcp(double d) {
 
 __device__ __forceinline__ float front_rcp(float d) { return 1.0f / d; }
 
+// d positive and finite (a double by its high word: no FP64 instruction)
+__device__ __forceinline__ bool front_positive(double d) {
+    const int h = __double2hiint(d);
+    return h > 0 && h < 0x7ff00000;
+}
+__device__ __forceinline__ bool front_positive(float d) { return d > 0.0f && d < INFINITY; }
+
 template <int NW> __device__ __forceinline__ void front_sync() {
     if (NW == 1) __syncwarp();
     else __syncthreads();
@@ -177,21 +185,25 @@ __device__ __forceinline__ void front_eliminate(Prob& prob, const int4* __restri
         };
         if (P >= 0) {
             const F* in = Z == P ? nb : sh.zero;
+            F d = F(0);
+            bool own = false;   // this lane holds the pivot
             cross(P, [&](F& x, int k) {
                 w[k] = x;
-                if (NW > 1 && k == P) {
-                    if (!(x > F(0))) *bad = 1;
-                    sh.piv[par] = front_rcp(x);
-                }
+                if (NW > 1 && k == P) d = x, own = true;
                 x = in[k];
             });
+            // (outside the row's loop: there the reciprocal would be issued for every entry)
+            if (NW > 1 && own) {
+                if (!front_positive(d)) *bad = 1;
+                sh.piv[par] = front_rcp(d);
+            }
         }
         if (Z >= 0 && Z != P) cross(Z, [&](F& x, int k) { x = nb[k]; });
         front_sync<NW>();
         F inv = F(0);
         if (NW == 1 && P >= 0) {   // (read by all lanes before w[P] changes)
             const F d = w[P];
-            if (!(d > F(0))) *bad = 1;
+            if (!front_positive(d)) *bad = 1;
             inv = front_rcp(d);
         }
         if (NW == 1 && e + 1 < steps) prob.prep(e + 1, v, sh.nb[par ^ 1], sh.piv + 2 + (par ^ 1));

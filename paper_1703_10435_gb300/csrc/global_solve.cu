@@ -87,7 +87,6 @@ namespace {
 constexpr int kNodeInfo = 10;   // int64 fields per node on the device
 constexpr int kNdThreads = 256;
 constexpr int kNdPanel = 32;    // pivots per step
-constexpr int kNdRows = 128;    // rows per block of k_nd_panel
 
 // ---------------------------------------------------------------- symbolic ---
 
@@ -373,54 +372,65 @@ __global__ void k_nd_extend_add(const int* list, int slot, const int64_t* info, 
 
 // One step of the LDL^T without pivoting of every front of a depth: the diagonal block of the
 // (up to) 32 pivots from p0 on and the rows below it, l = w / d with w_q = a_q - sum_{r<q}
-// w_r L_qr.  Grid (nodes, groups of 128 rows): every block factors the diagonal block for
-// itself in shared memory (about 5 us), a thread solves one row in registers.  The factored
-// diagonal block goes to `diag` (the other blocks of the front still read the old one);
-// k_nd_update puts it in place.
-__global__ void __launch_bounds__(kNdRows) k_nd_panel(const int* list, const int64_t* info, double* fronts, int p0,
-                                                      double* diag, int* bad) {
+// w_r L_qr.  Grid (nodes, groups of blockDim rows): one warp of every block factors the
+// diagonal block for itself (a lane a row, in registers; the pivot column through shared
+// memory), then a thread solves one row in registers.  A block of four warps takes 15 us of
+// the FP64 pipe for its rows, one of a single warp 4: depths with few fronts use single warps.
+// (The diagonal block by four warps with a barrier and a division per pivot: 40 us.)  The
+// factored diagonal block goes to `diag` (the other blocks of the front still read the old
+// one); k_nd_update puts it in place.
+__global__ void __launch_bounds__(128) k_nd_panel(const int* list, const int64_t* info, double* fronts, int p0,
+                                                  double* diag, int* bad) {
     __shared__ double L[kNdPanel][kNdPanel + 1];
-    __shared__ double dinv[kNdPanel];
+    __shared__ double dinv[kNdPanel], col[2][kNdPanel];
     const int id = list[blockIdx.x];
     const int64_t* q = info + (int64_t)id * kNodeInfo;
     const int k = (int)q[0], F = (int)q[1];
     const int nb = min(kNdPanel, k - p0);
-    const int row0 = p0 + nb + blockIdx.y * kNdRows;
+    const int row0 = p0 + nb + blockIdx.y * blockDim.x;
     if (nb <= 0 || (blockIdx.y > 0 && row0 >= F)) return;
     double* Fr = fronts + q[2];
-    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-    for (int j = warp; j < kNdPanel; j += kNdRows / 32)
-        L[lane][j] = lane >= j && lane < nb ? Fr[(p0 + lane) + (int64_t)(p0 + j) * F] : (lane == j ? 1.0 : 0.0);
-    __syncthreads();
-    for (int p = 0; p < nb; ++p) {   // column p keeps w = l d until the end
-        const double d = L[p][p];
-        if (threadIdx.x == 0) {
-            if (!(fabs(d) > 0.0) && blockIdx.y == 0) bad[id] = 1;   // zero or not finite
-            dinv[p] = 1.0 / d;
+    if (threadIdx.x < 32) {
+        const int lane = threadIdx.x;
+        double a[kNdPanel];   // row `lane`; rows and columns past nb: unit
+#pragma unroll
+        for (int j = 0; j < kNdPanel; ++j)
+            a[j] = lane >= j && lane < nb ? Fr[(p0 + lane) + (int64_t)(p0 + j) * F] : (lane == j ? 1.0 : 0.0);
+#pragma unroll
+        for (int p = 0; p < kNdPanel; ++p) {   // column p keeps w = l d until its turn is over
+            if (p < nb) {
+                double* w = col[p & 1];
+                w[lane] = a[p];
+                __syncwarp();
+                const double d = w[p], inv = 1.0 / d;
+                if (lane == 0) {
+                    dinv[p] = inv;
+                    if (!(fabs(d) > 0.0) && blockIdx.y == 0) bad[id] = 1;   // zero or not finite
+                }
+                const double l = a[p] * inv;
+#pragma unroll
+                for (int j = p + 1; j < kNdPanel; ++j) a[j] = fma(-l, w[j], a[j]);   // (j > lane: not used)
+                if (lane > p) a[p] = l;
+            } else if (lane == p) {
+                dinv[p] = 1.0;
+            }
         }
-        __syncthreads();
-        const double s = L[lane][p] * dinv[p];
-        for (int j = p + 1 + warp; j < nb; j += kNdRows / 32)
-            if (lane >= j) L[lane][j] -= s * L[j][p];
-        __syncthreads();
+#pragma unroll
+        for (int j = 0; j < kNdPanel; ++j) {
+            L[lane][j] = a[j];
+            if (blockIdx.y == 0) diag[((int64_t)blockIdx.x * kNdPanel + j) * kNdPanel + lane] = a[j];
+        }
     }
-    if (threadIdx.x >= nb && threadIdx.x < kNdPanel) dinv[threadIdx.x] = 1.0;
     __syncthreads();
-    for (int j = warp; j < kNdPanel; j += kNdRows / 32)
-        if (lane > j) L[lane][j] *= dinv[j];
-    __syncthreads();
-    if (blockIdx.y == 0)
-        for (int j = warp; j < kNdPanel; j += kNdRows / 32)
-            diag[((int64_t)blockIdx.x * kNdPanel + j) * kNdPanel + lane] = L[lane][j];
     const int i = row0 + threadIdx.x;
     if (i >= F) return;
     double w[kNdPanel];
 #pragma unroll
     for (int c = 0; c < kNdPanel; ++c) w[c] = c < nb ? Fr[i + (int64_t)(p0 + c) * F] : 0.0;
 #pragma unroll
-    for (int c = 1; c < kNdPanel; ++c)
+    for (int r = 0; r < kNdPanel; ++r)
 #pragma unroll
-        for (int r = 0; r < c; ++r) w[c] = fma(-w[r], L[c][r], w[c]);
+        for (int c = r + 1; c < kNdPanel; ++c) w[c] = fma(-w[r], L[c][r], w[c]);
 #pragma unroll
     for (int c = 0; c < kNdPanel; ++c)
         if (c < nb) Fr[i + (int64_t)(p0 + c) * F] = w[c] * dinv[c];
@@ -521,8 +531,12 @@ __global__ void __launch_bounds__(kNdThreads) k_nd_forward(const int* list, cons
         for (int i = p0 + nb + threadIdx.x; i < F; i += kNdThreads) {
             const double* col = Fr + i + (int64_t)p0 * F;
             double s = v[i];
-#pragma unroll 8
-            for (int c = 0; c < nb; ++c) s = fma(-col[(int64_t)c * F], v[p0 + c], s);
+            if (nb == kNdPanel) {   // (all loads in flight)
+#pragma unroll
+                for (int c = 0; c < kNdPanel; ++c) s = fma(-col[(int64_t)c * F], v[p0 + c], s);
+            } else {
+                for (int c = 0; c < nb; ++c) s = fma(-col[(int64_t)c * F], v[p0 + c], s);
+            }
             v[i] = s;
         }
         __syncthreads();
@@ -549,13 +563,28 @@ __global__ void __launch_bounds__(kNdThreads) k_nd_backward(const int* list, con
     __syncthreads();
     for (int p0 = (k - 1) / kNdPanel * kNdPanel; p0 >= 0; p0 -= kNdPanel) {
         const int nb = min(kNdPanel, k - p0);
-        for (int j = warp; j < nb; j += kNdThreads / 32) {
-            const double* col = Fr + (int64_t)(p0 + j) * F;
-            if (lane < nb) L[lane][j] = col[p0 + lane];
-            double s = 0.0;
-            for (int i = p0 + nb + lane; i < F; i += 32) s = fma(col[i], v[i], s);
-            for (int o = 16; o > 0; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
-            if (lane == 0) sum[j] = s;
+        {   // a warp takes columns warp, warp + 8, .. together
+            constexpr int W = kNdThreads / 32, C = kNdPanel / W;
+            const double* col[C];
+            double s[C];
+#pragma unroll
+            for (int c = 0; c < C; ++c) {
+                const int j = min(warp + W * c, nb - 1);   // (past nb: the last column again, not kept)
+                col[c] = Fr + (int64_t)(p0 + j) * F;
+                s[c] = 0.0;
+                if (lane < nb) L[lane][j] = col[c][p0 + lane];
+            }
+#pragma unroll 4
+            for (int i = p0 + nb + lane; i < F; i += 32) {
+                const double x = v[i];
+#pragma unroll
+                for (int c = 0; c < C; ++c) s[c] = fma(col[c][i], x, s[c]);
+            }
+#pragma unroll
+            for (int c = 0; c < C; ++c) {
+                for (int o = 16; o > 0; o >>= 1) s[c] += __shfl_xor_sync(0xffffffffu, s[c], o);
+                if (lane == 0 && warp + W * c < nb) sum[warp + W * c] = s[c];
+            }
         }
         __syncthreads();
         if (warp == 0) {
@@ -621,8 +650,9 @@ mhm_status nd_factor(const NDPlan* P, const NDPlan::Depth& q, cudaStream_t s) {
                 list, slot, P->node_info, P->maps, P->fronts);
     for (int64_t p0 = 0; p0 < q.k; p0 += kNdPanel) {
         const int64_t rest = std::max<int64_t>(q.F - p0 - 1, 1);
-        k_nd_panel<<<dim3(n, (unsigned)((rest + kNdRows - 1) / kNdRows)), kNdRows, 0, s>>>(list, P->node_info, P->fronts,
-                                                                                          (int)p0, P->diag, P->dinfo);
+        const int rows = n >= 128 ? 128 : 32;   // (rows per block: k_nd_panel)
+        k_nd_panel<<<dim3(n, (unsigned)((rest + rows - 1) / rows)), rows, 0, s>>>(list, P->node_info, P->fronts, (int)p0,
+                                                                                 P->diag, P->dinfo);
         // small fronts: 32 x 32 tiles (a leaf's trailing block has 24 to 72 rows)
         const int64_t ts = q.F >= 256 ? 64 : 32, t = (rest + ts - 1) / ts;
         const dim3 grid(n, (unsigned)(t * (t + 1) / 2));

@@ -294,8 +294,15 @@ void front3_try(int M, Front3Kernel* k) {
     k->threads = T::threads;
     k->vec = T::vec;
 }
-Front3Kernel front3_kernel(int M) {
+// few: no more elements than three per SM: 4 warps (and one for the rows) share an element, which
+// shortens a step where a single warp's latency is what counts (24 elements, m = 4: 0.86 -> 0.48
+// ms); the same results bit for bit.
+Front3Kernel front3_kernel(int M, bool few) {
     Front3Kernel k;
+    if (few) {
+        front3_try<mhm::FrontTiles<4, 1, 2>, 4>(M, &k);
+        front3_try<mhm::FrontTiles<4, 1, 4>, 4>(M, &k);
+    }
     front3_try<mhm::FrontTiles<1, 1, 8>, 12>(M, &k);
     front3_try<mhm::FrontTiles<1, 1, 12>, 12>(M, &k);
     front3_try<mhm::FrontTiles<1, 1, 15>, 8>(M, &k);
@@ -907,7 +914,9 @@ extern "C" mhm_status mhm3d_local_solve_batch(const mhm3d_mesh* m, const double*
     g.cls24 = m->d_cls24, g.geo24 = m->d_geo24, g.mass1 = m->d_mass1, g.fcnt = m->d_fcnt;
     g.val = m->d_fval, g.rc = m->d_frc, g.rp = m->d_frp, g.col = m->d_fcol, g.first = m->ffirst, g.off = m->foff;
     cudaStream_t s = (cudaStream_t)stream;
-    const Front3Kernel k = front3_kernel(g.R + m->fslots);
+    int sms = 0;
+    cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, m->device);
+    const Front3Kernel k = front3_kernel(g.R + m->fslots, K1 - K0 <= 3 * (int64_t)sms);
     if (!k.kern) return mhm::fail(MHM_ERR_UNSUPPORTED, "mhm3d_local_solve_batch: front too large");
     // the source tables in a stream-ordered scratch of this call
     double* tables = nullptr;
@@ -917,8 +926,6 @@ extern "C" mhm_status mhm3d_local_solve_batch(const mhm3d_mesh* m, const double*
         k_source3d<<<24 * 6, kQuad, 0, s>>>(m->d_geom, m->d_quad, g.N, g.nb, f->value, f->freq, tables);
         g.src24 = tables;
     }
-    int sms = 0;
-    cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, m->device);
     // one wave of blocks that share the elements out evenly
     auto launch = [&](void (*kern)(const Local3DArgs), int threads, size_t smem) {
         int per_sm = 0;
@@ -929,7 +936,13 @@ extern "C" mhm_status mhm3d_local_solve_batch(const mhm3d_mesh* m, const double*
         kern<<<(unsigned)std::min<int64_t>(K1 - K0, sms * ((each + rounds - 1) / rounds)), threads, smem, s>>>(g);
         return cudaGetLastError();
     };
-    const bool mixed = precision == MHM_MIXED && g.R <= kMaxMixedR && m->fslots <= FrontTilesMixed::rows;
+    // MIXED with room to refine and the FP64 re-solve allowed ends with FP64-quality blocks on
+    // either kernel, and the FP64 one is the faster from 512 elements on (12288 elements, m = 4:
+    // 9.9 against 27.4 ms, 1536: 1.6 against 4.1; m = 1: 6.9 against 19.2, 1.0 against 2.9; P1
+    // r = 3: 10.9 against 24.3, 1.7 against 3.7; at 192 elements the two are within 12 %).  The
+    // rule goes by the mesh and not by the call's range: a range gives the full call's bits.
+    const bool direct = o.it_max >= 2 && !o.no_fallback && m->nK >= 512;
+    const bool mixed = precision == MHM_MIXED && !direct && g.R <= kMaxMixedR && m->fslots <= FrontTilesMixed::rows;
     if (mixed)
         e = launch(k_local3d_mixed, kThreads,
                    (size_t)mixed3_smem(g.n, g.R, g.nb, g.nsub, g.off, g.slots).total * sizeof(double));

@@ -462,7 +462,11 @@ __global__ void __launch_bounds__(T::threads, MINB) k_local_fp64(const __grid_co
 
 // The frontal kernel for a bordered matrix of M rows and step tables of ncp entries; NULL if
 // it is too large.  One warp holds up to 72 entries a lane; beyond, as many warps as keep a
-// lane's share near 40.
+// lane's share near 40.  few: the mesh's only level has no more
+// elements than three per SM.  A step of one warp takes about
+// 5 k clocks by itself (P1 r = 5), with 4 warps and a fifth preparing the rows 3 k: 32 elements
+// 1.56 -> 0.87 ms, P1 r = 4 0.38 -> 0.23 ms; from 3 to 4 elements per SM on the two meet (512
+// elements P1 r = 5, R = 19: 1.58 and 1.60 ms).  The results are the same bit for bit.
 struct FrontKernel {
     void (*kern)(const Fp64Args) = nullptr;
     int threads = 0, vec = 0;
@@ -476,8 +480,12 @@ bool front_try(int M, FrontKernel* k) {
     return true;
 }
 template <int NCP>
-FrontKernel front_kernel_of(int M) {
+FrontKernel front_kernel_of(int M, bool few) {
     FrontKernel k;
+    if (few) {
+        front_try<FrontTiles<4, 1, 2>, NCP, 4>(M, &k);
+        front_try<FrontTiles<4, 1, 4>, NCP, 4>(M, &k);
+    }
     front_try<FrontTiles<1, 1, 4>, NCP, 16>(M, &k);
     front_try<FrontTiles<1, 1, 7>, NCP, 16>(M, &k);
     front_try<FrontTiles<1, 1, 10>, NCP, 14>(M, &k);
@@ -490,10 +498,10 @@ FrontKernel front_kernel_of(int M) {
     front_try<FrontTiles<4, 4, 12>, NCP, 1>(M, &k);
     return k;
 }
-FrontKernel front_kernel(const mhm_mesh* mesh, const Level& lv) {
+FrontKernel front_kernel(const mhm_mesh* mesh, const Level& lv, bool few) {
     if (lv.fsteps == 0) return {};
     const int M = (int)mesh->NI + 1 + lv.fslots;
-    return lv.fncp == 8 ? front_kernel_of<8>(M) : front_kernel_of<16>(M);
+    return lv.fncp == 8 ? front_kernel_of<8>(M, few) : front_kernel_of<16>(M, few);
 }
 
 }  // namespace
@@ -519,7 +527,7 @@ struct Fp64Shape {
     FrontKernel front;   // no kernel: window in global memory
 };
 
-Fp64Shape fp64_shape(const mhm_mesh* mesh, const Level& lv) {
+Fp64Shape fp64_shape(const mhm_mesh* mesh, const Level& lv, bool few = false) {
     Fp64Shape sh;
     sh.R = (int)mesh->NI + 1;
     sh.rows = fp64_window_rows(mesh, lv);
@@ -527,7 +535,7 @@ Fp64Shape fp64_shape(const mhm_mesh* mesh, const Level& lv) {
     if (sh.ld % 2 == 1) sh.ld += 1;
     sh.win_doubles = ((size_t)sh.rows * sh.ld + 31) & ~(size_t)31;   // 256-byte slots
     sh.smem = wide_smem_bytes(sh.rows, sh.R);
-    sh.front = front_kernel(mesh, lv);
+    sh.front = front_kernel(mesh, lv, few);
     return sh;
 }
 
@@ -574,7 +582,7 @@ static mhm_status launch_fp64(const mhm_mesh* mesh, const Level& lv, const doubl
     g.L = mesh->desc.l;
     g.dpf = mesh->dpf;
     g.NI = (int)mesh->NI;
-    const Fp64Shape sh = fp64_shape(mesh, lv);
+    const Fp64Shape sh = fp64_shape(mesh, lv, mesh->levels.size() == 1 && K1 - K0 <= 3 * sm_count(mesh));
     g.R = sh.R;
     g.rows = sh.rows;
     g.rhs0 = sh.rows;

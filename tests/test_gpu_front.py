@@ -85,3 +85,29 @@ def test_reconstruction_vs_oracle_at_layout_edges(P, r, m, l):
         want = u0[K] + o.eta[:, :-1] @ lam[mesh.local_lambda(K)] + o.eta[:, -1]
         tol = max(1e-10, 10 * 1.1e-16 * 12 * o.sub.n * 10)   # 10 u cond, as above
         assert np.abs(u[K] - want).max() < tol * np.abs(want).max(), K
+
+
+@pytest.mark.parametrize("P,r,m", [(2, 2, 4), (2, 1, 1), (1, 3, 4)])
+def test_3d_mixed_on_large_meshes_is_the_fp64_path(P, r, m):
+    """MIXED on a mesh of 512 elements or more with room to refine runs the FP64 elimination (the
+    same bits, iters 1); one pass or no re-solve runs the refinement, whose blocks agree with it
+    to the mixed tolerance."""
+    M = mhm.Mesh3D(3, r, P, m, device=0)   # 648 elements
+    kappa = 10.0 ** torch.as_tensor(np.random.default_rng(5).uniform(-1, 1, (M.n_K, 8 ** r)), device="cuda")
+    src = mhm.Source3D(mhm.MHM3D_SRC_SINSINSIN, 1.0, 2.0)
+
+    def run(precision, opts=None):
+        f64 = dict(dtype=torch.float64, device="cuda")
+        o = [torch.zeros(M.n_K, M.n_I, M.n_I, **f64), torch.zeros(M.n_K, M.n_I, **f64), torch.zeros(M.n_K, M.n_I, **f64),
+             torch.zeros(M.n_K, **f64), torch.full((M.n_K,), -7, dtype=torch.int32, device="cuda"),
+             torch.full((M.n_K,), -7, dtype=torch.int32, device="cuda")]
+        mhm.mhm3d_local_solve_batch(M, kappa, src, *o[:5], precision=precision, opts=opts, iters=o[5])
+        return o
+    ref, default, explicit = run(mhm.MHM_FP64), run(mhm.MHM_MIXED), run(mhm.MHM_MIXED, mhm.Opts3D(8, 1e-9, 0))
+    for got in (default, explicit):
+        assert all(torch.equal(a, b) for a, b in zip(ref, got)) and bool((got[5] == 1).all())
+    mixed = run(mhm.MHM_MIXED, mhm.Opts3D(8, 1e-9, 1))
+    assert int(mixed[4].abs().sum()) == 0 and int(mixed[5].min()) >= 2
+    d = ref[0].diagonal(dim1=1, dim2=2).abs().sqrt()
+    assert float(((mixed[0] - ref[0]).abs() / (d[:, :, None] * d[:, None]).clamp_min(1e-300)).max()) < 1e-9
+    assert float((mixed[1] - ref[1]).abs().max()) < 1e-9 * float(ref[1].abs().max())
