@@ -70,7 +70,7 @@ __device__ __forceinline__ void front_element(const DeviceMesh& dm, int64_t K, c
                                    (c.X[2][0] - c.X[0][0]) * (c.X[1][1] - c.X[0][1]));
     if (tid == 0) c.area = area;
     if (tid < 8) mass[tid] = tid * (area / ((double)N * N) / 3.0);
-    element_stiffness_pair(P, N, c.X, Ke, tid, nthr);
+    element_stiffness_pair(P, N, c.X, Ke, Ke + 36, tid, nthr);
     source_tables(dm, src_kind, src_value, src_freq, P, N, c.X, tab, tid, nthr);
     __syncthreads();
 }

@@ -105,19 +105,6 @@ struct MCtx {
     int timeout;
 };
 
-// Fine-triangle vertices in physical coordinates.
-__device__ __forceinline__ void fine_xy(const MCtx& c, int N, bool up, int i, int j, double X[3][2]) {
-    const double e1x = (c.X[1][0] - c.X[0][0]) / N, e1y = (c.X[1][1] - c.X[0][1]) / N;
-    const double e2x = (c.X[2][0] - c.X[0][0]) / N, e2y = (c.X[2][1] - c.X[0][1]) / N;
-    int a[3][2];
-    if (up) { a[0][0] = i; a[0][1] = j; a[1][0] = i + 1; a[1][1] = j; a[2][0] = i; a[2][1] = j + 1; }
-    else    { a[0][0] = i + 1; a[0][1] = j; a[1][0] = i + 1; a[1][1] = j + 1; a[2][0] = i; a[2][1] = j + 1; }
-    for (int v = 0; v < 3; ++v) {
-        X[v][0] = c.X[0][0] + a[v][0] * e1x + a[v][1] * e2x;
-        X[v][1] = c.X[0][1] + a[v][0] * e1y + a[v][1] * e2y;
-    }
-}
-
 // Fine triangles incident to lattice point (X, Y) and the point's local index in
 // each: up to 6 for a vertex, 2 for a P2 edge midpoint.  Returns the count.
 __device__ int incident(int P, int N, int X, int Y, int ti[6], int tj[6], bool tup[6], int ta[6]) {
@@ -1413,11 +1400,6 @@ __device__ __forceinline__ void mixed_blocks(const MixedArgs& g) {
                 c.rev[a] = g.dm.rev[3 * K + a];
                 c.la1[a] = face_la1(g.dm, K, a);
             }
-            double Xu[3][2], Xd[3][2];
-            fine_xy(c, g.N, true, 0, 0, Xu);
-            fine_xy(c, g.N, false, 0, 0, Xd);
-            element_stiffness(g.P, Xu, c.Sup);
-            element_stiffness(g.P, Xd, c.Sdn);
             c.bad = 0;
             c.col_fail = 0;
             c.timeout = 0;
@@ -1426,6 +1408,7 @@ __device__ __forceinline__ void mixed_blocks(const MixedArgs& g) {
         }
         for (int col = threadIdx.x; col < R; col += blockDim.x) c.col_done[col] = c.col_frozen[col] = 0;
         __syncthreads();
+        if constexpr (MODE != 2) element_stiffness_pair(g.P, g.N, c.X, c.Sup, c.Sdn, threadIdx.x, blockDim.x);
         if (g.src_kind == MHM_SRC_CONST) {
             if (threadIdx.x == 0) c.FK = g.src_value * c.area;
         } else {
@@ -2096,21 +2079,13 @@ __device__ __forceinline__ void schur_factor_block(const MixedArgs& g, int blk) 
     const int64_t kk = ki - g.Kbase;
     float* cw = g.cwall + kk * 4 * (int64_t)nu;
     float* T = g.Tall + kk * (int64_t)g.t_stride;
-    if (lane < 2) {
-        // the two fine-triangle shapes of the uniform refinement: up (lane 0), down (lane 1)
+    {
         double V[3][2];
         for (int v = 0; v < 3; ++v) {
             V[v][0] = g.dm.geom[6 * K + 2 * v];
             V[v][1] = g.dm.geom[6 * K + 2 * v + 1];
         }
-        const double e1x = (V[1][0] - V[0][0]) / g.N, e1y = (V[1][1] - V[0][1]) / g.N;
-        const double e2x = (V[2][0] - V[0][0]) / g.N, e2y = (V[2][1] - V[0][1]) / g.N;
-        const double Xu[3][2] = {{V[0][0], V[0][1]}, {V[0][0] + e1x, V[0][1] + e1y}, {V[0][0] + e2x, V[0][1] + e2y}};
-        const double Xd[3][2] = {{V[0][0] + e1x, V[0][1] + e1y},
-                                 {V[0][0] + e1x + e2x, V[0][1] + e1y + e2y},
-                                 {V[0][0] + e2x, V[0][1] + e2y}};
-        if (lane == 0) element_stiffness(1, Xu, fs.Su);
-        else element_stiffness(1, Xd, fs.Sd);
+        element_stiffness_pair(1, g.N, V, fs.Su, fs.Sd, lane, 32);
         if (lane == 0) fs.bad = 0;
     }
     __syncwarp();
@@ -2322,22 +2297,14 @@ __global__ void __launch_bounds__(kGenThreads) k_schur_factor_gen(const MixedArg
     for (int t = p; t < g.N * g.N; t += kGenThreads) kap[t] = d2f_bits(kapg[t]);
     const int64_t kk = ki - g.Kbase;
     float* F = g.Tall + kk * (int64_t)g.t_stride;
-    if (p == 0) {
-        // the two fine-triangle shapes (up and down) of the uniform refinement
+    {
         double V[3][2];
         for (int v = 0; v < 3; ++v) {
             V[v][0] = g.dm.geom[6 * K + 2 * v];
             V[v][1] = g.dm.geom[6 * K + 2 * v + 1];
         }
-        const double e1x = (V[1][0] - V[0][0]) / g.N, e1y = (V[1][1] - V[0][1]) / g.N;
-        const double e2x = (V[2][0] - V[0][0]) / g.N, e2y = (V[2][1] - V[0][1]) / g.N;
-        const double Xu[3][2] = {{V[0][0], V[0][1]}, {V[0][0] + e1x, V[0][1] + e1y}, {V[0][0] + e2x, V[0][1] + e2y}};
-        const double Xd[3][2] = {{V[0][0] + e1x, V[0][1] + e1y},
-                                 {V[0][0] + e1x + e2x, V[0][1] + e1y + e2y},
-                                 {V[0][0] + e2x, V[0][1] + e2y}};
-        element_stiffness(g.P, Xu, s.Su);
-        element_stiffness(g.P, Xd, s.Sd);
-        s.bad = 0;
+        element_stiffness_pair(g.P, g.N, V, s.Su, s.Sd, p, kGenThreads);
+        if (p == 0) s.bad = 0;
     }
     __syncthreads();
     if (p < 36) {

@@ -159,18 +159,6 @@ __device__ __forceinline__ double vertex_mass(int N, int x, int y, double area_f
     return n * (area_fine / 3.0);
 }
 
-__device__ __forceinline__ void fine_tri_vertices(const WCtx& c, int N, bool up, int i, int j, double X[3][2]) {
-    const double e1x = (c.X[1][0] - c.X[0][0]) / N, e1y = (c.X[1][1] - c.X[0][1]) / N;
-    const double e2x = (c.X[2][0] - c.X[0][0]) / N, e2y = (c.X[2][1] - c.X[0][1]) / N;
-    int a[3][2];
-    if (up) { a[0][0] = i; a[0][1] = j; a[1][0] = i + 1; a[1][1] = j; a[2][0] = i; a[2][1] = j + 1; }
-    else    { a[0][0] = i + 1; a[0][1] = j; a[1][0] = i + 1; a[1][1] = j + 1; a[2][0] = i; a[2][1] = j + 1; }
-    for (int v = 0; v < 3; ++v) {
-        X[v][0] = c.X[0][0] + a[v][0] * e1x + a[v][1] * e2x;
-        X[v][1] = c.X[0][1] + a[v][0] * e1y + a[v][1] * e2y;
-    }
-}
-
 // Sum over the block of up to kRp per-thread column values; out[c] for c < kRp (all
 // threads see it after the call).
 template <int NT>
@@ -304,11 +292,6 @@ __global__ void __launch_bounds__(2 * BMAX, BMAX == 128 ? 2 : 4) k_local_mixed_w
                 c.rev[a] = g.dm.rev[3 * K + a];
                 c.la1[a] = face_la1(g.dm, K, a);
             }
-            double Xu[3][2], Xd[3][2];
-            fine_tri_vertices(c, N, true, 0, 0, Xu);
-            fine_tri_vertices(c, N, false, 0, 0, Xd);
-            element_stiffness(1, Xu, c.Sup);
-            element_stiffness(1, Xd, c.Sdn);
             choose_pin(1, N, kap, &c.pin_x, &c.pin_y);
             c.bad = 0;
             const LevelGeom lg0{1, N, N, c.pin_x, c.pin_y};
@@ -323,6 +306,8 @@ __global__ void __launch_bounds__(2 * BMAX, BMAX == 128 ? 2 : 4) k_local_mixed_w
             c.u0[N + 1] = u;
             c.toff[N + 1] = t;
         }
+        __syncthreads();
+        element_stiffness_pair(1, N, c.X, c.Sup, c.Sdn, tid, NT);
         __syncthreads();
         if (c.pin_y != 0) {
             // pinned DOF on lattice row 1: level 0 keeps all N + 1 points of row 0, one more
@@ -432,7 +417,13 @@ __global__ void __launch_bounds__(2 * BMAX, BMAX == 128 ? 2 : 4) k_local_mixed_w
             const int b = lg.size(lev), ub = c.u0[lev];
             for (int p = tid; p < b; p += NT) cws[p] = cw[ub + p];
             __syncthreads();
-            // row i of S_lev = Ah_ll - C T_{lev-1} C^T in registers (positions 64 h .. of this half)
+            // row i of S_lev = Ah_ll - C T_{lev-1} C^T in registers: the two threads of a row take
+            // the columns four and four in turn (column 8 q + 4 h + e in a[4 q + e]), so both run
+            // out of columns as the levels get narrower; blocks of 32 columns past b and warps
+            // whose rows are past b are skipped (half of the padded 128 x 128 work over a level-7
+            // element)
+            const int nq = (b + 7) / 8;
+            const bool busy = (tid >> 5) * 16 < b;   // (the whole warp)
             float a[H];
             float dd = 0.0f;
             {
@@ -453,7 +444,7 @@ __global__ void __launch_bounds__(2 * BMAX, BMAX == 128 ? 2 : 4) k_local_mixed_w
                 }
 #pragma unroll
                 for (int jj = 0; jj < H; ++jj) {
-                    const int j = h * H + jj;
+                    const int j = 8 * (jj >> 2) + 4 * h + (jj & 3);
                     float v = 0.0f;
                     if (row_ok && j < b) {
                         const float4 cwj = cws[j];
@@ -474,7 +465,7 @@ __global__ void __launch_bounds__(2 * BMAX, BMAX == 128 ? 2 : 4) k_local_mixed_w
                     a[jj] = v;
                     if (j == i) dd = v;
                 }
-                if (row_ok && h == i / H) dg[i] = dd;
+                if (row_ok && h == ((i >> 2) & 1)) dg[i] = dd;
             }
             __syncthreads();
             // symmetric sweep: per pivot k the pivot row (entry k replaced by d - 1) is
@@ -483,38 +474,42 @@ __global__ void __launch_bounds__(2 * BMAX, BMAX == 128 ? 2 : 4) k_local_mixed_w
             for (int k = 0; k < b; ++k) {
                 float* rbk = rb + (k & 1) * BMAX;
                 if (i == k) {
-                    float4* dst = reinterpret_cast<float4*>(rbk + h * H);
+                    float4* dst = reinterpret_cast<float4*>(rbk) + h;
 #pragma unroll
-                    for (int q = 0; q < H / 4; ++q) dst[q] = make_float4(a[4 * q], a[4 * q + 1], a[4 * q + 2], a[4 * q + 3]);
-                    if (h == k / H) {
+                    for (int q = 0; q < H / 4; ++q)
+                        if (q < nq) dst[2 * q] = make_float4(a[4 * q], a[4 * q + 1], a[4 * q + 2], a[4 * q + 3]);
+                    if (h == ((k >> 2) & 1)) {
                         const float d = dg[k];
                         rbk[k] = d - 1.0f;
-                        dsh[k & 1] = d;
+                        if (!(d > 0.0f)) c.bad = 1;
+                        dsh[k & 1] = d > 0.0f ? 1.0f / d : 0.0f;
                     }
                 }
                 __syncthreads();
-                const float d = dsh[k & 1];
-                float dinv = 0.0f;
-                if (d > 0.0f) dinv = 1.0f / d;
-                else if (tid == 0) c.bad = 1;
-                const float m = rbk[i];
-                const float s = m * dinv;
-                const float4* src = reinterpret_cast<const float4*>(rbk + h * H);
+                if (busy) {
+                    const float m = rbk[i];
+                    const float s = m * dsh[k & 1];
+                    const float4* src = reinterpret_cast<const float4*>(rbk) + h;
 #pragma unroll
-                for (int q = 0; q < H / 4; ++q) {
-                    const float4 r4 = src[q];
-                    a[4 * q] = fmaf(-s, r4.x, a[4 * q]);
-                    a[4 * q + 1] = fmaf(-s, r4.y, a[4 * q + 1]);
-                    a[4 * q + 2] = fmaf(-s, r4.z, a[4 * q + 2]);
-                    a[4 * q + 3] = fmaf(-s, r4.w, a[4 * q + 3]);
+                    for (int q0 = 0; q0 < H / 4; q0 += 4)
+                        if (q0 < nq) {
+#pragma unroll
+                            for (int q = q0; q < q0 + 4; ++q) {
+                                const float4 r4 = src[2 * q];
+                                a[4 * q] = fmaf(-s, r4.x, a[4 * q]);
+                                a[4 * q + 1] = fmaf(-s, r4.y, a[4 * q + 1]);
+                                a[4 * q + 2] = fmaf(-s, r4.z, a[4 * q + 2]);
+                                a[4 * q + 3] = fmaf(-s, r4.w, a[4 * q + 3]);
+                            }
+                        }
+                    if (i < b && h == ((i >> 2) & 1)) dg[i] = fmaf(-s, m, dg[i]);
                 }
-                if (i < b && h == i / H) dg[i] = fmaf(-s, m, dg[i]);
             }
             __syncthreads();
             if (i < b) {
 #pragma unroll
                 for (int jj = 0; jj < H; ++jj) {
-                    const int j = h * H + jj;
+                    const int j = 8 * (jj >> 2) + 4 * h + (jj & 3);
                     if (j < b) Tp[i * LDT + j] = (j == i) ? 2.0f - a[jj] : -a[jj];
                 }
             }
