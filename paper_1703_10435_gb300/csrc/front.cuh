@@ -259,7 +259,8 @@ __device__ __forceinline__ void front_result(int R, const double (&A)[T::NT], Fn
 
 // Entering rows of the 2-D local problems (FrontPlan's tables): couplings from kappa and the
 // two element matrices, ahead of their use by one batch of 32 / ncp steps (loads of the batch
-// after it in flight).  load(x, y, mass count | faces << 8, column) gives the node's load.  The pinned
+// after it in flight).  load.node(info), then load(x, y, info,
+// column) gives the node's load (info: mass count | faces << 8).  The pinned
 // node is kept as a node coupled to nothing, with a unit pivot and no loads.
 template <int NCP, class Load>
 struct FrontRows2D {
@@ -301,6 +302,7 @@ struct FrontRows2D {
         const int ps = v.x & 255, zs = (v.x >> 8) & 255;
         if (zs != kNoSlot) {
             const bool pinned = v.y == pin;
+            load.node(v.z);
             for (int q = lane; q < vec; q += 32) nb[q] = q < R && !pinned ? load(v.y & 0xffff, v.y >> 16, v.z, q) : 0.0;
             if (lane == 0) *wnew = 0.0;
             __syncwarp();

@@ -35,6 +35,7 @@
 #include <string>
 #include <vector>
 
+#include "front.cuh"
 #include "mhm_internal.h"
 
 namespace mhm {
@@ -402,7 +403,7 @@ __global__ void __launch_bounds__(128) k_nd_panel(const int* list, const int64_t
                 double* w = col[p & 1];
                 w[lane] = a[p];
                 __syncwarp();
-                const double d = w[p], inv = 1.0 / d;
+                const double d = w[p], inv = front_rcp(d);
                 if (lane == 0) {
                     dinv[p] = inv;
                     if (!(fabs(d) > 0.0) && blockIdx.y == 0) bad[id] = 1;   // zero or not finite

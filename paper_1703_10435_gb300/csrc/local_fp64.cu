@@ -368,13 +368,20 @@ __host__ __device__ inline FrontSmem front_smem(int vec, int R, int kind, int P,
 struct FrontLoad {
     const double *btab, *mass, *src;   // src NULL: constant source
     int PN, NI;
-    double value;
-    double cp0, cp1, cf0, cf1;
+    double cp0, cp1, cf0, cf1;         // load per mass; -s |face|
     int fc0, fc1;                      // face | reversed << 2 | table row << 3, -1: none
+    int last = -1;                     // mass count of the products kept in v0, v1
+    double v0 = 0.0, v1 = 0.0;         // (nodes of equal mass follow one another: no FP64 work)
+    __device__ __forceinline__ void node(int info) {
+        if ((info & 255) == last) return;
+        last = info & 255;
+        const double m = mass[last];
+        v0 = cp0 * m;
+        v1 = cp1 * m;
+    }
     __device__ __forceinline__ double operator()(int x, int y, int info, int q) const {
         const bool hi = q >= 32;
-        const double m = mass[info & 255];
-        double v = -(hi ? cp1 : cp0) * m;
+        double v = hi ? v1 : v0;
         if (info >> 8) {   // (the whole warp: a node on the boundary)
             const int fc = hi ? fc1 : fc0;
             if (fc >= 0 && ((info >> 8) >> (fc & 3)) & 1) {
@@ -382,7 +389,7 @@ struct FrontLoad {
                 v = fma(hi ? cf1 : cf0, btab[(fc >> 3) * (PN + 1) + ((fc & 4) ? PN - kl : kl)], v);
             }
         }
-        if (q == NI) v = src ? v + src[y * (PN + 1) - y * (y - 1) / 2 + x] : fma(value, m, v);
+        if (src && q == NI) v += src[y * (PN + 1) - y * (y - 1) / 2 + x];
         return v;
     }
 };
@@ -418,12 +425,12 @@ __global__ void __launch_bounds__(T::threads, MINB) k_local_fp64(const __grid_co
         }
     }
     __syncthreads();
-    FrontLoad load{g.dm.btab, smem + L.mass, g.src_kind == MHM_SRC_CONST ? nullptr : src, PN, NI, g.src_value,
+    FrontLoad load{g.dm.btab, smem + L.mass, g.src_kind == MHM_SRC_CONST ? nullptr : src, PN, NI,
                    0.0, 0.0, 0.0, 0.0, -1, -1};
     for (int h = 0; h < 2; ++h) {
         const int col = (tid & 31) + 32 * h;
         if (col >= R) break;
-        (h ? load.cp1 : load.cp0) = cproj[col];
+        (h ? load.cp1 : load.cp0) = (col == NI && !load.src ? g.src_value : 0.0) - cproj[col];
         if (col == NI) break;
         const int a = col / g.dpf, row = face_row(col - a * g.dpf, c.la1[a], g.dm.fm, g.dm.lmax1);
         (h ? load.cf1 : load.cf0) = -c.sgn[a] * c.flen[a];

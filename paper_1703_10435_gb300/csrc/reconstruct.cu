@@ -157,6 +157,7 @@ __device__ void element_errors(const RecArgs& g, int64_t K, const double Xc[3][2
 struct RecLoad {
     const double* gl;
     int PN;
+    __device__ __forceinline__ void node(int) {}
     __device__ __forceinline__ double operator()(int x, int y, int, int) const {
         return gl[y * (PN + 1) - y * (y - 1) / 2 + x];
     }
@@ -300,8 +301,13 @@ void rec_try(const Level& lv, RecKernel* k) {
     k->threads = T::threads;
     k->vec = T::vec;
 }
-RecKernel rec_kernel(const Level& lv) {
+// (few: no more elements than three per SM, which four warps each finish sooner: front.cuh)
+RecKernel rec_kernel(const Level& lv, bool few) {
     RecKernel k;
+    if (few) {
+        rec_try<FrontTiles<4, 1, 2>, 1, 4>(lv, &k);
+        rec_try<FrontTiles<4, 1, 3>, 2, 4>(lv, &k);
+    }
     rec_try<FrontTiles<1, 1, 5>, 1, 16>(lv, &k);
     rec_try<FrontTiles<1, 1, 9>, 2, 16>(lv, &k);
     rec_try<FrontTiles<4, 1, 5>, 3, 3>(lv, &k);
@@ -354,7 +360,9 @@ extern "C" mhm_status mhm_reconstruct(const mhm_mesh* mesh, const double* kappa,
         g.nod_off = mesh->d_nod_off;
         g.u_out = u_nodal;
         g.err_out = err_sq;
-        const RecKernel front = rec_kernel(lv);
+        int sms = 0, occ = 0;
+        cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, mesh->device);
+        const RecKernel front = rec_kernel(lv, lv.nK <= 3 * (int64_t)sms);
         g.ev = lv.d_fev;
         g.cp = lv.d_fcp;
         g.steps = lv.fsteps;
@@ -365,8 +373,6 @@ extern "C" mhm_status mhm_reconstruct(const mhm_mesh* mesh, const double* kappa,
         g.slot_bytes = ((size_t)g.steps * (g.slots + 1) * sizeof(double) + 255) & ~(size_t)255;
         const size_t smem = (size_t)rec_smem(front.vec, g.NI, f->kind, g.P, g.N).total * sizeof(double);
         MHM_CUDA_TRY(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
-        int sms = 0, occ = 0;
-        cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, mesh->device);
         cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, kern, threads, smem);
         // one wave, the elements shared out evenly
         const int64_t each = (lv.nK + sms - 1) / sms, rounds = (each + std::max(occ, 1) - 1) / std::max(occ, 1);
