@@ -62,13 +62,23 @@ struct DeviceMesh {
 // autotuner's choices; defaults below): see mhm_tuning in mhm.h.
 struct Tuning {
     int chunk = 8192;        // elements per factor + solve launch pair (<= kChunkMax)
-    int blocks_per_sm = 3;   // resident solve blocks per SM (<= the kernel's occupancy)
+    int blocks_per_sm = 3;   // resident solve blocks per SM (default_blocks_per_sm sets it per level)
     int nbuf = 2;            // staged level operators in the shared-memory ring (2..4)
     int l2pf = 0;            // L2 prefetch distance in level steps (0: none)
     int pf_all = 0;          // 1: prefetch the element's whole operator set into L2 per solve
     int op_policy = 1;       // L2 policy of the operator copies: 0 default, 1 evict first, 2 evict last
     int tuned = 0;           // 1: set by the autotuner or a tuning cache
 };
+
+// Blocks of the mixed solve kernel per SM before any tuning: four (64 registers a thread) where
+// an element's level steps are short and their serial chains hold it back; three (80
+// registers) where the columns fill the threads.
+// Three against four blocks, ms on 152 SMs: r = 3, 7 columns, 4608 elements 0.773 / 0.653;
+// r = 4, 10 columns, 1702 elements 0.791 / 0.739; r = 4, 19 columns, 18432 elements 8.21 / 7.62;
+// r = 5, 7 columns, 3200 elements 3.03 / 2.77; r = 5, 19 columns, 18432 elements 44.4 / 48.1.
+inline int default_blocks_per_sm(int degree, int N, int n_I) {
+    return degree == 1 && (N <= 16 || n_I + 1 <= 8) ? 4 : 3;
+}
 
 // Multifrontal factorisation plan of the global saddle-point system (mhm_solve_global):
 // built on the first call, kept by the mesh.
