@@ -303,34 +303,8 @@ __device__ __forceinline__ void assembled_row(int P, int N, int PN, int nunk, co
     for (int k = 7; k < 19; ++k) { w[k] = T(0); v[k] = u; }
 }
 
-// Res(u, :) -= (A_p D)(u, :) for the columns still refining, in FP64, and the next
-// FP32 right-hand side y(u, :) = s_u Res(u, :), from the assembled row of u (the sum
-// over the fine triangles T containing u of kappa_T S_T[a_u][b]): 7 entries for P1,
-// up to 19 for P2.
-__device__ void apply_residual(const MixedArgs& g, const MCtx& c, const double* kap, int u, const double* D,
-                               double* Res, float* y, const double s_u) {
-    int X, Y;
-    lattice_of_unk(g.PN, u, &X, &Y);
-    const size_t ld = (size_t)g.nunk;
-    double w[19];
-    int v[19];
-    assembled_row(g.P, g.N, g.PN, g.nunk, c.Sup, c.Sdn, kap, X, Y, u, w, v);
-    uint32_t nz = 0;   // non-zero weights (zero: edges at right angles), tested on the integer pipe
-#pragma unroll
-    for (int k = 0; k < 19; ++k)
-        if ((__double_as_longlong(w[k]) << 1) != 0) nz |= 1u << k;
-    for (int col = 0; col < g.R; ++col) {
-        if (c.col_done[col]) continue;
-        const double* Dc = D + col * ld;
-        double a = 0.0;
-#pragma unroll
-        for (int k = 0; k < 19; ++k)
-            if (nz >> k & 1) a = fma(w[k], Dc[v[k]], a);
-        const double rn = Res[col * ld + u] - a;
-        Res[col * ld + u] = rn;
-        y[(size_t)u * g.Rp + col] = d2f_bits(rn * s_u);
-    }
-}
+// Row stride of the staged solution and residual columns of the outputs (64 nodes and one).
+constexpr int kOutLd = 65;
 
 // out[c] = sum_u Res(u, c) s(u) y(u, c) for the columns still refining (warp per
 // column, fixed summation order).
@@ -1142,6 +1116,96 @@ __device__ __noinline__ void fused_residual(int PN, int nu, int R, const double*
     }
 }
 
+// Z += D and Res -= A_p D, D = S y, for the columns still refining, in FP64, with the assembled
+// row of each node (the sum over the fine triangles T containing u of kappa_T S_T[a_u][b]: 7
+// entries for P1, 19 at a vertex and 9 at a midpoint for P2).
+// The FP64 pipe bounds it (one warp instruction per 64 clocks and scheduler): a warp takes nodes
+// of one class (vertices, then the three kinds of midpoints), whose rows have the same zeros
+// (no neighbour there, or an edge at a right angle), and leaves those entries out by a branch;
+// as predicated instructions they cost what the others do.  The columns of S are put into the
+// row once per node; y is read in shared memory, four columns at a time, with their Z and Res
+// loaded ahead.  P2 r = 4, 19 columns: 385000 -> KRES clocks per pass.
+__device__ __noinline__ void refine_residual(const MixedArgs& g, const MCtx& c, const double* kap, const float* y,
+                                             const double* scale, double* Z, double* Res) {
+    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    const int ncls = g.P == 2 ? 4 : 1, nver = (g.N + 1) * (g.N + 2) / 2 - 1, nmid = g.N * (g.N + 1) / 2;
+    const int wver = (nver + 31) >> 5, wmid = (nmid + 31) >> 5, ntask = wver + (ncls - 1) * wmid;
+    const uint32_t y_s = smem_u32(y);
+    const size_t ld = (size_t)g.nunk;
+    uint64_t done = 0;
+    for (int col = 0; col < g.R; ++col)
+        if (c.col_done[col]) done |= 1ull << col;
+    for (int task = warp; task < ntask; task += kWarpsM) {
+        const int cls = task < wver ? 0 : 1 + (task - wver) / wmid;
+        const int q = (cls == 0 ? task : (task - wver) - (cls - 1) * wmid) * 32 + lane;
+        const bool in = q < (cls == 0 ? nver : nmid);
+        int X = 0, Y = 0;
+        if (in) lattice_of_unk(cls == 0 ? g.N : g.N - 1, cls == 0 ? q : q - 1, &X, &Y);
+        if (g.P == 2) {
+            X = 2 * X + (cls == 1 || cls == 3);
+            Y = 2 * Y + (cls >= 2);
+        }
+        const int u = in ? unk(g.PN, X, Y) : 0;
+        double w[19];
+        int v[19];
+        uint32_t nz = 0;
+        const double su = scale[u];
+        if (in) {
+            assembled_row(g.P, g.N, g.PN, g.nunk, c.Sup, c.Sdn, kap, X, Y, u, w, v);
+#pragma unroll
+            for (int k = 0; k < 19; ++k)
+                if (!is_zero(w[k])) nz |= 1u << k;
+        } else {
+#pragma unroll
+            for (int k = 0; k < 19; ++k) { w[k] = 0.0; v[k] = 0; }
+        }
+        const uint32_t any = __reduce_or_sync(0xffffffffu, nz);
+#pragma unroll
+        for (int k = 0; k < 19; ++k) {
+            if (any >> k & 1) w[k] *= -scale[v[k]];
+            v[k] = (int)(y_s + 4u * (uint32_t)(v[k] * g.Rp));
+        }
+        for (int c0 = 0; c0 < g.R; c0 += 4) {
+            double r[4], z[4];
+            bool on[4];
+#pragma unroll
+            for (int j = 0; j < 4; ++j) {
+                const int col = c0 + j;
+                on[j] = in && col < g.R && !(done >> col & 1);
+                r[j] = on[j] ? Res[col * ld + u] : 0.0;
+                z[j] = on[j] ? Z[col * ld + u] : 0.0;
+            }
+            const uint32_t yc = 4u * (uint32_t)c0;
+#pragma unroll
+            for (int j = 0; j < 4; ++j)
+                if (c0 + j < g.R) {
+                    const double d0 = f2d_bits(lds1((uint32_t)v[0] + yc + 4u * j));
+                    z[j] = fma(su, d0, z[j]);
+                    r[j] = fma(w[0], d0, r[j]);
+                }
+#pragma unroll
+            for (int k = 1; k < 19; ++k)
+                if (any >> k & 1) {
+                    const uint32_t ya = (uint32_t)v[k] + yc;
+                    r[0] = fma(w[k], f2d_bits(lds1(ya)), r[0]);
+                    if (c0 + 1 < g.R) {
+                        r[1] = fma(w[k], f2d_bits(lds1(ya + 4u)), r[1]);
+                        if (c0 + 2 < g.R) {
+                            r[2] = fma(w[k], f2d_bits(lds1(ya + 8u)), r[2]);
+                            if (c0 + 3 < g.R) r[3] = fma(w[k], f2d_bits(lds1(ya + 12u)), r[3]);
+                        }
+                    }
+                }
+#pragma unroll
+            for (int j = 0; j < 4; ++j)
+                if (on[j]) {
+                    Res[(c0 + j) * ld + u] = r[j];
+                    Z[(c0 + j) * ld + u] = z[j];
+                }
+        }
+    }
+}
+
 // The level factorisation, the solves and the column dots run out of line: each
 // then keeps its working set (register panel, accumulator tiles) in registers
 // instead of sharing the kernel's register budget with the per-K state live
@@ -1622,23 +1686,38 @@ __device__ __forceinline__ void mixed_blocks(const MixedArgs& g) {
                 for (int i = 0; i < 32; ++i) acc[i] = 0.0f;
                 double mzp = 0.0;
                 int par = 0;
-                for (int u = warp; u < nu; u += kWarpsM) {
-                    const double zh = lc ? Zh[(size_t)u * R + lane] : 0.0;
-                    const double rh = lc ? Rh[(size_t)u * R + lane] : 0.0;
-                    mzp = fma(smass[u], zh, mzp);
-                    const float zf = d2f_bits(zh);
-                    float* rb = rowb + par * 32;
-                    par ^= 1;
-                    rb[lane] = d2f_bits(rh);
-                    __syncwarp();
+                // four nodes' rows are loaded ahead of their products: one node at a time the
+                // loop waits for memory (the outputs of an r = 5 element with 19 columns took
+                // 270000 clocks of its 1.1 million)
+                constexpr int kAhead = 4;
+                for (int ub = warp; ub < nu; ub += kAhead * kWarpsM) {
+                    double zh[kAhead], rh[kAhead], sm[kAhead];
 #pragma unroll
-                    for (int q = 0; q < 8; ++q) {
-                        if (4 * q < R) {
-                            const float4 r4 = *reinterpret_cast<const float4*>(rb + 4 * q);
-                            acc[4 * q] = fmaf(zf, r4.x, acc[4 * q]);
-                            if (4 * q + 1 < R) acc[4 * q + 1] = fmaf(zf, r4.y, acc[4 * q + 1]);
-                            if (4 * q + 2 < R) acc[4 * q + 2] = fmaf(zf, r4.z, acc[4 * q + 2]);
-                            if (4 * q + 3 < R) acc[4 * q + 3] = fmaf(zf, r4.w, acc[4 * q + 3]);
+                    for (int e = 0; e < kAhead; ++e) {
+                        const int u = ub + e * kWarpsM;
+                        const bool on = lc && u < nu;
+                        zh[e] = on ? Zh[(size_t)u * R + lane] : 0.0;
+                        rh[e] = on ? Rh[(size_t)u * R + lane] : 0.0;
+                        sm[e] = on ? smass[u] : 0.0;
+                    }
+#pragma unroll
+                    for (int e = 0; e < kAhead; ++e) {
+                        if (ub + e * kWarpsM >= nu) break;
+                        mzp = fma(sm[e], zh[e], mzp);
+                        const float zf = d2f_bits(zh[e]);
+                        float* rb = rowb + par * 32;
+                        par ^= 1;
+                        rb[lane] = d2f_bits(rh[e]);
+                        __syncwarp();
+#pragma unroll
+                        for (int q = 0; q < 8; ++q) {
+                            if (4 * q < R) {
+                                const float4 r4 = *reinterpret_cast<const float4*>(rb + 4 * q);
+                                acc[4 * q] = fmaf(zf, r4.x, acc[4 * q]);
+                                if (4 * q + 1 < R) acc[4 * q + 1] = fmaf(zf, r4.y, acc[4 * q + 1]);
+                                if (4 * q + 2 < R) acc[4 * q + 2] = fmaf(zf, r4.z, acc[4 * q + 2]);
+                                if (4 * q + 3 < R) acc[4 * q + 3] = fmaf(zf, r4.w, acc[4 * q + 3]);
+                            }
                         }
                     }
                 }
@@ -1660,29 +1739,47 @@ __device__ __forceinline__ void mixed_blocks(const MixedArgs& g) {
                     c.mz[threadIdx.x] = mz;
                 }
                 __syncthreads();
-                // boundary terms (S N_j)^T Zh: warp per face, lane = column, FP64
-                if (warp < 3 && lc) {
-                    const int a = warp;
-                    double sb[kMaxFaceDofs];
-                    for (int jf = 0; jf < g.dpf; ++jf) sb[jf] = 0.0;
-                    for (int kl = 0; kl <= g.PN; ++kl) {
-                        int X, Y;
-                        if (a == 2) { X = kl; Y = 0; }
-                        else if (a == 0) { X = g.PN - kl; Y = kl; }
-                        else { X = 0; Y = g.PN - kl; }
-                        const int u = unk(g.PN, X, Y);
-                        if (u < 0) continue;
-                        const int kk2 = c.rev[a] ? g.PN - kl : kl;
-                        const double zs = sc[u] * Zh[(size_t)u * R + lane] * (-c.sgn[a] * c.flen[a]);
-                        for (int jf = 0; jf < g.dpf; ++jf) {
-                            const int row = face_row(jf, c.la1[a], g.dm.fm, g.dm.lmax1);
-                            if (row >= 0) sb[jf] = fma(g.dm.btab[row * (g.PN + 1) + kk2], zs, sb[jf]);
+                // boundary terms (S N_j)^T Zh: a warp takes three multipliers of a face, lane =
+                // column, FP64; four points loaded ahead
+                const int ng = (g.dpf + 2) / 3;
+                for (int it = warp; it < 3 * ng && lc; it += kWarpsM) {
+                    const int a = it / ng, jf0 = 3 * (it - a * ng), nj = min(3, g.dpf - jf0);
+                    double sb[3] = {0.0, 0.0, 0.0};
+                    const double* tb[3];
+                    bool on[3];
+#pragma unroll
+                    for (int q = 0; q < 3; ++q) {
+                        const int row = q < nj ? face_row(jf0 + q, c.la1[a], g.dm.fm, g.dm.lmax1) : -1;
+                        on[q] = row >= 0;
+                        tb[q] = g.dm.btab + (size_t)max(row, 0) * (g.PN + 1);
+                    }
+                    const double fs = -c.sgn[a] * c.flen[a];
+                    for (int kb = 0; kb <= g.PN; kb += 4) {
+                        double z4[4], s4[4], t4[3][4];
+#pragma unroll
+                        for (int e = 0; e < 4; ++e) {
+                            const int kl = min(kb + e, g.PN);
+                            const int X = a == 2 ? kl : a == 0 ? g.PN - kl : 0, Y = a == 2 ? 0 : a == 0 ? kl : g.PN - kl;
+                            const int u = unk(g.PN, X, Y), kk2 = c.rev[a] ? g.PN - kl : kl;
+                            const bool in = u >= 0 && kb + e <= g.PN;
+                            z4[e] = in ? Zh[(size_t)u * R + lane] : 0.0;
+                            s4[e] = in ? sc[u] : 0.0;
+#pragma unroll
+                            for (int q = 0; q < 3; ++q) t4[q][e] = tb[q][kk2];
+                        }
+#pragma unroll
+                        for (int e = 0; e < 4; ++e) {
+                            const double zs = s4[e] * z4[e] * fs;
+#pragma unroll
+                            for (int q = 0; q < 3; ++q) sb[q] = fma(t4[q][e], zs, sb[q]);
                         }
                     }
-                    for (int jf = 0; jf < g.dpf; ++jf) {
-                        const int j = a * g.dpf + jf;
-                        xbuf[j * R + lane] += sb[jf] - c.cproj[j] * c.mz[lane];
-                    }
+#pragma unroll
+                    for (int q = 0; q < 3; ++q)
+                        if (q < nj) {
+                            const int j = a * g.dpf + jf0 + q;
+                            xbuf[j * R + lane] += (on[q] ? sb[q] : 0.0) - c.cproj[j] * c.mz[lane];
+                        }
                 }
                 __syncthreads();
             }
@@ -1860,13 +1957,11 @@ __device__ __forceinline__ void mixed_blocks(const MixedArgs& g) {
             // bilinear form N~^T Z + Z^T Res, whose error e^T A_p e is quadratic in the
             // error e of Z; eps_c = Res_c^T M Res_c estimates ||e_c||^2_{A_p}.
             double* Res = G;
-            double* D64 = reinterpret_cast<double*>(slot + g.off_D);
-            const int total = g.nunk * R;
             for (int t = threadIdx.x; t < g.nunk * g.Rp; t += blockDim.x) {
                 const int u = t / g.Rp, col = t - u * g.Rp;
                 y[t] = col < R ? d2f_bits(Res[(size_t)col * g.nunk + u] * scale[u]) : 0.0f;
             }
-            for (int t = threadIdx.x; t < total; t += blockDim.x) Z[t] = 0.0;
+            for (int t = threadIdx.x; t < g.nunk * R; t += blockDim.x) Z[t] = 0.0;
             __syncthreads();
             // gamma_c = G_c^T M G_c ~ ||z_c||^2_{A_p}
             if constexpr (MODE == 3) solve_gen(g, F, sinfo, y, opbuf, stage, c);
@@ -1892,17 +1987,7 @@ __device__ __forceinline__ void mixed_blocks(const MixedArgs& g) {
             __syncthreads();
             int pass = 0;
             while (!c.all_done) {
-                // D = s . y (FP64), Z += D
-                for (int t = threadIdx.x; t < total; t += blockDim.x) {
-                    const int col = t / g.nunk, u = t - col * g.nunk;
-                    if (c.col_done[col]) continue;
-                    const double d = f2d_bits(y[(size_t)u * g.Rp + col]) * scale[u];
-                    D64[t] = d;
-                    Z[t] += d;
-                }
-                __syncthreads();
-                // Res -= A_p D (FP64, from kappa and the element matrices); y = s . Res
-                for (int u = threadIdx.x; u < g.nunk; u += blockDim.x) apply_residual(g, c, kap, u, D64, Res, y, scale[u]);
+                refine_residual(g, c, kap, y, scale, Z, Res);
                 ++pass;
                 __syncthreads();
                 if (threadIdx.x == 0) {
@@ -1916,6 +2001,12 @@ __device__ __forceinline__ void mixed_blocks(const MixedArgs& g) {
                 }
                 __syncthreads();
                 if (c.all_done) break;
+                for (int u = threadIdx.x; u < g.nunk; u += blockDim.x) {   // the next solves' y = S Res
+                    const double su = scale[u];
+                    for (int col = 0; col < R; ++col)
+                        if (!c.col_done[col]) y[(size_t)u * g.Rp + col] = d2f_bits(Res[(size_t)col * g.nunk + u] * su);
+                }
+                __syncthreads();
                 if constexpr (MODE == 3) solve_gen(g, F, sinfo, y, opbuf, stage, c);
                 else solve_factor(g, F, sinfo, y, opbuf, stage, c);
                 __syncthreads();
@@ -1954,22 +2045,24 @@ __device__ __forceinline__ void mixed_blocks(const MixedArgs& g) {
             float corr[(kMaxNI + 1) * (kMaxNI + 1) / kThreadsM + 1];
             const int npair = R * R;
             for (int q = 0; q * kThreadsM < npair; ++q) corr[q] = 0.0f;
-            constexpr int kChunk = 64;
-            float* zs = y;                       // R x kChunk
-            float* rs = y + R * kChunk;          // R x kChunk
+            // (rows one float apart from a multiple of 32 banks: the columns i of a warp's pairs
+            // are 19 rows on one bank otherwise)
+            constexpr int kChunk = 64, kLd = kOutLd;
+            float* zs = y;                       // R x kLd
+            float* rs = y + R * kLd;             // R x kLd
             for (int base = 0; base < g.nunk; base += kChunk) {
                 const int cnt = min(kChunk, g.nunk - base);
                 __syncthreads();
                 for (int t = threadIdx.x; t < R * kChunk; t += blockDim.x) {
                     const int col = t / kChunk, uu = t - col * kChunk;
-                    zs[t] = uu < cnt ? d2f_bits(Z[(size_t)col * g.nunk + base + uu]) : 0.0f;
-                    rs[t] = uu < cnt ? d2f_bits(Res[(size_t)col * g.nunk + base + uu]) : 0.0f;
+                    zs[col * kLd + uu] = uu < cnt ? d2f_bits(Z[(size_t)col * g.nunk + base + uu]) : 0.0f;
+                    rs[col * kLd + uu] = uu < cnt ? d2f_bits(Res[(size_t)col * g.nunk + base + uu]) : 0.0f;
                 }
                 __syncthreads();
                 for (int q = 0; q * kThreadsM + (int)threadIdx.x < npair; ++q) {
                     const int t = q * kThreadsM + threadIdx.x, j = t / R, i = t - j * R;
                     float a = 0.0f;
-                    for (int uu = 0; uu < kChunk; ++uu) a = fmaf(zs[j * kChunk + uu], rs[i * kChunk + uu], a);
+                    for (int uu = 0; uu < kChunk; ++uu) a = fmaf(zs[j * kLd + uu], rs[i * kLd + uu], a);
                     corr[q] += a;
                 }
             }
@@ -1982,16 +2075,20 @@ __device__ __forceinline__ void mixed_blocks(const MixedArgs& g) {
                 const int a = j / g.dpf, jf = j - a * g.dpf;
                 const int row = face_row(jf, c.la1[a], g.dm.fm, g.dm.lmax1);
                 const double* zc = Z + (size_t)col * g.nunk;
+                const double fs = -c.sgn[a] * c.flen[a];
                 double s = 0.0;
-                for (int kl = 0; kl <= g.PN && row >= 0; ++kl) {
-                    int X, Y;
-                    if (a == 2) { X = kl; Y = 0; }
-                    else if (a == 0) { X = g.PN - kl; Y = kl; }
-                    else { X = 0; Y = g.PN - kl; }
-                    const int u = unk(g.PN, X, Y);
-                    if (u < 0) continue;
-                    const int kk = c.rev[a] ? g.PN - kl : kl;
-                    s += (-c.sgn[a] * c.flen[a] * g.dm.btab[row * (g.PN + 1) + kk]) * zc[u];
+                for (int kb = 0; kb <= g.PN && row >= 0; kb += 4) {   // four points loaded ahead
+                    double z4[4], t4[4];
+#pragma unroll
+                    for (int e = 0; e < 4; ++e) {
+                        const int kl = min(kb + e, g.PN);
+                        const int X = a == 2 ? kl : a == 0 ? g.PN - kl : 0, Y = a == 2 ? 0 : a == 0 ? kl : g.PN - kl;
+                        const int u = unk(g.PN, X, Y);
+                        z4[e] = u >= 0 && kb + e <= g.PN ? zc[u] : 0.0;
+                        t4[e] = g.dm.btab[row * (g.PN + 1) + (c.rev[a] ? g.PN - kl : kl)];
+                    }
+#pragma unroll
+                    for (int e = 0; e < 4; ++e) s += (fs * t4[e]) * z4[e];
                 }
                 xbuf[j * R + col] += s - c.cproj[j] * c.mz[col];
             }
@@ -2473,7 +2570,9 @@ MixedLayout mixed_layout(const mhm_mesh* mesh, const Level& lv, bool split = tru
     L.off_mass = L.off_Z + al((size_t)L.nunk * R * sizeof(double));
     L.off_scale = L.off_mass + al((size_t)L.nunk * sizeof(double));
     L.off_D = L.off_scale + al((size_t)L.nunk * sizeof(double));
-    L.slot_bytes = L.off_D + al((size_t)L.nunk * R * sizeof(double));
+    // MODE 1: the scaled matrix, 7 values per node (MODE 0 keeps the room: its slot decides what
+    // the allocation-free entry takes)
+    L.slot_bytes = L.off_D + (L.mode >= 2 ? 0 : al((size_t)L.nunk * std::max(R, 7) * sizeof(double)));
     size_t win = (size_t)L.wrows * L.wld;
     if (win < (size_t)R * R * 2) win = (size_t)R * R * 2;
     // staged solve operand: K-tiles x n-tiles x 64 floats, K = b + b' of the largest step
@@ -2505,7 +2604,7 @@ MixedLayout mixed_layout(const mhm_mesh* mesh, const Level& lv, bool split = tru
     win = (win + 3) & ~(size_t)3;
     L.wfloats = (int)win;
     size_t yf = (size_t)L.nunk * L.Rp;
-    if (yf < (size_t)2 * R * 64) yf = (size_t)2 * R * 64;   // also holds two R x 64 staging chunks
+    if (yf < (size_t)2 * R * kOutLd) yf = (size_t)2 * R * kOutLd;   // also holds two R x 64 staging chunks
     L.ldr = (2 * bmax + 3) & ~3;
     if (L.mode == 0 && yf < (size_t)bmax * L.ldr) yf = (size_t)bmax * L.ldr;   // and the level right-hand sides while factoring
     if (L.schur) yf = std::max(yf, (size_t)(10 * R * R + 16 * R + 8 + 4 + kWarpsM * 64));   // and the output partials
