@@ -1486,12 +1486,19 @@ __device__ __forceinline__ void mixed_blocks(const MixedArgs& g) {
             double* tab = reinterpret_cast<double*>(W);
             source_tables(g.dm, g.src_kind, g.src_value, g.src_freq, g.P, g.N, c.X, tab, threadIdx.x, blockDim.x);
             __syncthreads();
-            const double* vals = g.src_vals ? g.src_vals + 16 * (kap - g.kappa) : nullptr;
+            // values: the triangles' integrals (P1: 3 N^2, P2: 6 N^2) in the room of G and Z, free
+            // until the right-hand sides (2 n R doubles, n > N^2 / 2 or 2 N^2, R >= 4)
+            const bool quad = g.src_kind == MHM_SRC_QUAD;
+            if (quad) {
+                source_triangles(g.P, g.N, tab, g.src_vals + 16 * (kap - g.kappa), G, threadIdx.x, blockDim.x);
+                __syncthreads();
+            }
             double s = 0.0;
             for (int u = threadIdx.x; u <= g.nunk; u += blockDim.x) {
                 int X = 0, Y = 0;
                 if (u > 0) lattice_of_unk(g.PN, u - 1, &X, &Y);
-                sload[u] = source_node(g.src_kind, g.P, g.N, X, Y, tab, vals);
+                sload[u] = quad ? source_node_of_triangles(g.P, g.N, X, Y, G)
+                                : source_node(g.src_kind, g.P, g.N, X, Y, tab, nullptr);
                 s += sload[u];
             }
             for (int o = 16; o > 0; o >>= 1) s += __shfl_down_sync(0xffffffffu, s, o);
