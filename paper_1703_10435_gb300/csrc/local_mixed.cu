@@ -42,7 +42,7 @@ struct MixedArgs {
     int yfloats;                  // floats reserved for the right-hand-side block (>= nunk Rp)
     int bmax;                     // largest level size
     int opmax;                    // floats of the largest level operator (fragment order, multiple of 128)
-    int stage_floats;             // floats of one staged solve operand (fragment order)
+    int stage_floats, tab_floats; // floats of one staged solve operand (fragment order), of one staged coupling table
     int ldr;                      // leading dimension of the level right-hand sides (multiple of 4)
     int src_kind;
     const double* src_vals;       // MHM_SRC_QUAD: 16 values per fine triangle, laid out like kappa
@@ -1277,8 +1277,9 @@ __device__ inline int4 gen_step_info(const LevelGeom& lg, int nlev, const int* u
 // Forward + backward solve of the generic path for every column still refining, in place
 // in y (node-major: y[u * R + col]): per level step the operand is staged from y through
 // the coupling tables, then one b x b by b x R product with T_lev on the tensor cores
-// (three-term TF32 split, as in solve_factor); T_lev streams into two shared-memory
-// buffers by bulk copies, one step ahead.
+// (three-term TF32 split, as in solve_factor); T_lev and the step's coupling table stream
+// into two shared-memory buffers by bulk copies, one step ahead (the tables read in place:
+// 132000 clocks per solve of P2 r = 4 with 19 columns, copied 116000).
 __device__ __noinline__ void solve_gen(const MixedArgs& g, const float* F, const int4* sinfo, float* y,
                                        float* opbuf, float* stage, MCtx& c) {
     const int R = g.R, NT = (R + 7) >> 3;
@@ -1290,12 +1291,16 @@ __device__ __noinline__ void solve_gen(const MixedArgs& g, const float* F, const
     uint64_t frozen = 0;
     for (int col = 0; col < R; ++col)
         if (c.col_frozen[col]) frozen |= 1ull << col;
+    float* tabbuf = stage + g.stage_floats;   // 2 x tab_floats
+    const uint32_t tab_s = smem_u32(tabbuf);
     auto issue = [&](int st) {
         const int4 si = sinfo[st];
         const int b = si.x & 0xff;
         const uint32_t bytes = (uint32_t)frag_op_floats(b, b) * 4u;
+        const uint32_t tbytes = (si.x >> 8 & 1) ? 8u * kTabF * b : 8u * kTabQ * (uint32_t)(si.x >> 16);
         fence_proxy_async_shared();
-        mbar_arrive_expect_tx(&c.bar[st & 1], bytes);
+        mbar_arrive_expect_tx(&c.bar[st & 1], bytes + tbytes);
+        if (tbytes) bulk_copy_g2s(tabbuf + (size_t)(st & 1) * g.tab_floats, F + si.z, tbytes, &c.bar[st & 1]);
         bulk_copy_g2s(opbuf + (size_t)(st & 1) * g.opmax, F + si.w, bytes, &c.bar[st & 1]);
     };
     const bool issuer = threadIdx.x == kThreadsM - 32;
@@ -1306,9 +1311,12 @@ __device__ __noinline__ void solve_gen(const MixedArgs& g, const float* F, const
         const int4 si = sinfo[st];
         const int b = si.x & 0xff, dir = (si.x >> 8) & 1, l0 = si.x >> 16;
         const int ulev = si.y & 0xffff, uo = si.y >> 16;
-        const float2* tab = reinterpret_cast<const float2*>(F + si.z);
+        const uint32_t tab = tab_s + (uint32_t)((st & 1) * g.tab_floats) * 4u;
         // the other buffer was last read in step st - 1, which ended with a barrier
         if (issuer && st + 1 < nsteps) issue(st + 1);
+        const uint32_t par = (st & 1) ? ph1 : ph0;
+        if (!mbar_wait_bounded(&c.bar[st & 1], par)) c.timeout = 1;
+        if (st & 1) ph1 ^= 1u; else ph0 ^= 1u;
         // operand (b x R, fragment order): forward r_lev - C_lev v_{lev-1}, backward
         // C_{lev+1}^T x_{lev+1}
         {
@@ -1319,18 +1327,20 @@ __device__ __noinline__ void solve_gen(const MixedArgs& g, const float* F, const
                     v = lds1(y_s + 4u * (uint32_t)((ulev + i) * R + col));
                     if (i < l0) {
 #pragma unroll
-                        for (int m = 0; m < kTabQ; ++m) {
-                            const float2 e = tab[i * kTabQ + m];
-                            const int pos = __float_as_int(e.x);
+                        for (int m = 0; m < kTabQ; m += 2) {
+                            const float4 e = lds4(tab + 8u * (uint32_t)(i * kTabQ + m));
+                            const int pos = __float_as_int(e.x), pos2 = __float_as_int(e.z);
                             if (pos >= 0) v = fmaf(-e.y, lds1(y_s + 4u * (uint32_t)((uo + pos) * R + col)), v);
+                            if (pos2 >= 0) v = fmaf(-e.w, lds1(y_s + 4u * (uint32_t)((uo + pos2) * R + col)), v);
                         }
                     }
                 } else {
 #pragma unroll
-                    for (int m = 0; m < kTabF; ++m) {
-                        const float2 e = tab[i * kTabF + m];
-                        const int pos = __float_as_int(e.x);
+                    for (int m = 0; m < kTabF; m += 2) {
+                        const float4 e = lds4(tab + 8u * (uint32_t)(i * kTabF + m));
+                        const int pos = __float_as_int(e.x), pos2 = __float_as_int(e.z);
                         if (pos >= 0) v = fmaf(e.y, lds1(y_s + 4u * (uint32_t)((uo + pos) * R + col)), v);
+                        if (pos2 >= 0) v = fmaf(e.w, lds1(y_s + 4u * (uint32_t)((uo + pos2) * R + col)), v);
                     }
                 }
                 sts1(st_s + 4u * frag_b_pos(i, col, NT), v);
@@ -1339,9 +1349,6 @@ __device__ __noinline__ void solve_gen(const MixedArgs& g, const float* F, const
                 if (col >= R) { col -= R; ++i; }
             }
         }
-        const uint32_t par = (st & 1) ? ph1 : ph0;
-        if (!mbar_wait_bounded(&c.bar[st & 1], par)) c.timeout = 1;
-        if (st & 1) ph1 ^= 1u; else ph0 ^= 1u;
         __syncthreads();
         const int KT = (b + 7) >> 3, MT = (b + 15) >> 4;
         const uint32_t op0 = op_s + (uint32_t)((st & 1) * g.opmax) * 4u;
@@ -2522,7 +2529,7 @@ size_t gen_factor_smem_bytes(int nunk, int N) {
 }
 
 struct MixedLayout {
-    int nlev, nunk, wrows, wld, wfloats, yfloats, bmax, opmax, ldr, Rp, stage_floats;
+    int nlev, nunk, wrows, wld, wfloats, yfloats, bmax, opmax, ldr, Rp, stage_floats, tab_floats;
     size_t factor_floats, slot_bytes, off_G, off_Z, off_mass, off_scale, off_D, smem;
     size_t off_kap_smem, off_scale_smem, off_sinfo, off_cw;
     int kap_in_smem, rpl, cpl;
@@ -2566,6 +2573,7 @@ MixedLayout mixed_layout(const mhm_mesh* mesh, const Level& lv, bool split = tru
             if (L.mode == 3) {   // coupling tables: forward (first rows of levels >= 1), backward
                 const int l0 = P == 1 || lev == N ? b : 2 * N - 2 * lev + 1 - (lev == 0);
                 if (lev >= 1) f += (size_t)2 * kTabQ * l0;
+                L.tab_floats = std::max(L.tab_floats, 2 * std::max(kTabQ * l0, kTabF * b));
                 if (lev + 1 < L.nlev) f += (size_t)2 * kTabF * b;
             }
         } else {
@@ -2610,7 +2618,7 @@ MixedLayout mixed_layout(const mhm_mesh* mesh, const Level& lv, bool split = tru
         if (L.mode == 3) {
             // no factorisation window: two operator buffers and one staged operand of K = b
             L.stage_floats = ((bmax + 7) / 8) * ((R + 7) / 8) * 64;
-            win = std::max((size_t)R * R * 2, (size_t)2 * L.opmax + (size_t)L.stage_floats);
+            win = std::max((size_t)R * R * 2, (size_t)2 * L.opmax + (size_t)L.stage_floats + (size_t)2 * L.tab_floats);
         }
         if (win < (size_t)2 * L.opmax + (size_t)2 * L.stage_floats && L.mode != 3)
             win = (size_t)2 * L.opmax + (size_t)2 * L.stage_floats;
@@ -2713,6 +2721,7 @@ MixedArgs mixed_args(const mhm_mesh* mesh, const Level& lv, const MixedLayout& L
     g.bmax = L.bmax;
     g.opmax = L.opmax;
     g.stage_floats = L.stage_floats;
+    g.tab_floats = L.tab_floats;
     g.ldr = L.ldr;
     g.src_kind = f.kind;
     g.src_vals = f.kind == MHM_SRC_QUAD ? f.values_dev : nullptr;
