@@ -22,6 +22,7 @@ on 4 or 16 subfaces) is timed last, FP64, in `three_d`.  Prints one JSON line.
 from __future__ import annotations
 
 import argparse
+import functools
 import json
 import math
 import os
@@ -39,28 +40,43 @@ SECONDARY = "c2_hetero_fp64"
 MORE = "c5_p2_large,c4_channels"
 
 
-def algorithmic_fmas(P, N, R):
-    """Multiply-adds of the block-tridiagonal forward elimination of one K: per
-    level, Cholesky of the b x b block, W = L^-1 C^T, the Schur update W^T W,
-    the forward solve of R right-hand sides, their update W^T Y and the Gram
-    matrix Y^T Y (symmetric halves counted once)."""
-    def size(lev):
-        if P == 1:
-            return N + 1 - lev - (lev == 0)
-        if lev == N:
-            return 1
-        return (2 * N - 2 * lev + 1) + (2 * N - 2 * lev) - (lev == 0)
+def elimination_fmas(cliques, R):
+    """Multiply-adds of eliminating the nodes of a local matrix in ascending order from the
+    matrix bordered by R load columns, node 0 pinned (left out): with s later neighbours in the
+    filled graph, one step updates the lower triangle of s + R rows and scales its column.
+    cliques: the node numbers of every fine element."""
+    later = {}
+    for q in cliques:
+        for a in q:
+            if a:
+                later.setdefault(a, set()).update(b for b in q if b > a)
     tot = 0.0
-    for lev in range(N + 1):
-        b = size(lev)
-        bn = size(lev + 1) if lev < N else 0
-        tot += b * (b - 1) * (b + 1) / 6.0           # Cholesky
-        tot += bn * b * (b + 1) / 2.0                 # W = L^-1 C^T
-        tot += b * bn * (bn + 1) / 2.0                # S' -= W^T W
-        tot += R * b * (b + 1) / 2.0                  # Y = L^-1 G
-        tot += bn * R * b                             # G' -= W^T Y
-        tot += b * R * (R + 1) / 2.0                  # Gram += Y^T Y
+    for a in sorted(later):
+        nb = later[a]
+        if nb:
+            later[min(nb)] |= nb - {min(nb)}      # the fill reaches the rest through the first of them
+        k = len(nb) + R
+        tot += k * (k + 1) / 2.0 + k
     return tot
+
+
+@functools.lru_cache(maxsize=None)
+def algorithmic_fmas(P, N, R):
+    """elimination_fmas of one K: degree P on N^2 fine triangles, nodes by lattice rows."""
+    PN = P * N
+    num = lambda x, y: y * (PN + 1) - y * (y - 1) // 2 + x
+    tri = []
+    for j in range(N):
+        for i in range(N - j):
+            for up in (True, False):
+                if not up and i + j > N - 2:
+                    continue
+                v = [(i, j), (i + 1, j), (i, j + 1)] if up else [(i + 1, j), (i + 1, j + 1), (i, j + 1)]
+                pts = [(P * x, P * y) for x, y in v]
+                if P == 2:
+                    pts += [(a[0] + b[0], a[1] + b[1]) for a, b in ((v[1], v[2]), (v[2], v[0]), (v[0], v[1]))]
+                tri.append([num(x, y) for x, y in pts])
+    return elimination_fmas(tri, R)
 
 
 class ClockSampler:
@@ -195,8 +211,9 @@ def measured_peaks():
 # Kernel sources whose hash a recorded ncu traffic figure belongs to; the summary of
 # kernel k on workload w is profiles/<k>_<short name of w>.md.
 TRAFFIC_SOURCES = {
-    "k_local_mixed": ["local_mixed.cu", "local_common.cuh", "mhm_internal.h"],
-    "k_local_fp64": ["local_fp64.cu", "local_common.cuh", "mhm_internal.h"],
+    "k_local_mixed": ["local_mixed.cu", "source_loads.cuh", "local_common.cuh", "mhm_internal.h"],
+    "k_local_fp64": ["local_fp64.cu", "front.cuh", "front2d.cuh", "front_plan.cpp", "source_loads.cuh", "local_common.cuh",
+                     "mhm_internal.h"],
 }
 PROFILE_TAG = {"c2_hetero_fp64": "c2", "c3_grf_mixed": "c3", "c5_p2_large": "c5", "c4_channels": "c4"}
 
@@ -534,12 +551,10 @@ def solution_errors(args, w, p64, pmx, kap, src):
 THREE_D = [(8, 2, 2, 4), (4, 2, 2, 16)]   # (nc, r, k, m): 12288 and 1536 coarse tetrahedra
 
 
-def local3d_flops(n, NI):
-    """FP64 flops of one 3-D local solve: Cholesky of the pinned n - 1 unknowns
-    ((n-1)^3 / 3), the forward substitution of N_I + 1 right-hand sides ((n-1)^2 (N_I + 1))
-    and the Gram products of the face integrals (2 (n-1) (N_I (N_I + 1) / 2 + N_I))."""
-    n1 = n - 1
-    return n1 ** 3 / 3.0 + n1 * n1 * (NI + 1.0) + 2.0 * n1 * (NI * (NI + 1) / 2.0 + NI)
+def local3d_flops(sub, NI):
+    """FP64 flops of one 3-D local solve: two per multiply-add of elimination_fmas on the
+    submesh's tetrahedra with the N_I + 1 loads."""
+    return 2.0 * elimination_fmas([[int(d) for d in q] for q in sub.dofs], NI + 1)
 
 
 def local3d_mixed_fp64_flops(n, NI, n_sub, nb, passes):
@@ -608,7 +623,7 @@ def run_three_d(dev, flush, peak64, steps=5, warmup=3, n_check=2):
             return t_step, t_local, err, t_or, itv
 
         t64, l64, e64, t_or, _ = timed(mhm.MHM_FP64)
-        fl64 = local3d_flops(M.n_local, M.n_I) * M.n_K
+        fl64 = local3d_flops(T.Submesh3D(np.vstack([np.zeros(3), np.eye(3)]), r, P), M.n_I) * M.n_K
         entry = {"workload": "cube_%dx%dx%d_tets%d_sub%d_k%d_m%d" % (nc, nc, nc, M.n_K, M.n_sub, P, m),
                  "n_K": M.n_K, "local_dofs": M.n_local, "n_I": M.n_I, "lambda_unknowns": M.n_lambda,
                  "unit": "coarse elements/s",
@@ -626,12 +641,13 @@ def run_three_d(dev, flush, peak64, steps=5, warmup=3, n_check=2):
         if M.n_I <= 16:
             tmx, lmx, emx, _, itv = timed(mhm.MHM_MIXED)
             passes = float(itv[itv > 0].mean()) if np.any(itv > 0) else 0.0
-            flmx = local3d_mixed_fp64_flops(M.n_local, M.n_I, M.n_sub, nb, passes) * M.n_K
+            direct = bool(np.all(itv == 1))   # MIXED ran the FP64 elimination
+            flmx = fl64 if direct else local3d_mixed_fp64_flops(M.n_local, M.n_I, M.n_sub, nb, passes) * M.n_K
             entry["mixed"] = {"value": M.n_K / (tmx * 1e-3), "ms_per_step": tmx, "local_ms": lmx,
                               "skeleton_ms": tmx - lmx, "refinement_passes_mean": passes,
                               "fp64_resolved_elements": int(np.sum(itv < 0)),
-                              "roofline": {"kernel": "k_local3d_mixed", "bound": "alu",
-                                           "pipe": "fp64 (residuals and corrected face integrals)",
+                              "roofline": {"kernel": "k_local3d" if direct else "k_local3d_mixed", "bound": "alu",
+                                           "pipe": "fp64" if direct else "fp64 (residuals and corrected face integrals)",
                                            "flops_per_step": flmx, "achieved": flmx / (lmx * 1e-3) / 1e12,
                                            "peak": peak64, "unit": "TFLOP/s",
                                            "frac": flmx / (lmx * 1e-3) / 1e12 / peak64},

@@ -210,8 +210,7 @@ mhm_status mhm_mesh_query(const mhm_mesh* mesh, int32_t what, void* host_out, si
 /* Bytes of device scratch memory mhm_local_solve_batch needs for `precision`: a
  * region per refinement level of the mesh, one after the other.  MHM_FP64 levels
  * eliminated in registers need none (0 for a mesh of those only); the others
- * (P2 r = 7) keep a level window in one slot per SM of
- * rows x (rows + N_I + 1) doubles.  MHM_MIXED adds its per-level buffers. */
+ * (P2 r = 7) keep a level window in one slot per SM of rows x (rows + N_I + 1) doubles.  MHM_MIXED adds its per-level buffers. */
 mhm_status mhm_local_workspace_size(const mhm_mesh* mesh, int32_t precision, size_t* bytes);
 
 /* Bytes of the factor store that mhm_solve_opts.factor_store points to: 0 when no level
@@ -293,7 +292,7 @@ mhm_status mhm_local_solve_waves(const mhm_mesh* mesh, const double* kappa_host,
  * allocates nothing.  Coarse elements whose per-element scratch exceeds 32 MiB
  * are rejected with MHM_ERR_INVALID_ARG; a large batch runs with as many
  * concurrent blocks as fit in the array (the FP64 levels of the MIXED precision
- * with windows wider than shared memory too).  The first call on a device looks up
+ * with a window in global memory too).  The first call on a device looks up
  * the array's device address (cudaGetSymbolAddress) with that device current:
  * make that first call before any stream capture.  All calls share the array,
  * and each call overwrites what the previous one left there: calls that can
@@ -378,10 +377,9 @@ mhm_status mhm_solve_global(const mhm_mesh* mesh, const double* A_vals_dev, cons
  * `exact`), also writes err_sq_dev[2K] = ||u_{H,h} - u||^2_{L2(K)} and
  * err_sq_dev[2K+1] = |u_{H,h} - u|^2_{H1(K)}, by the collapsed 4 x 4 Gauss rule
  * on every fine triangle.  Allocates temporary device memory, stream-ordered: per
- * resident block the level factors of one element (2/3 (PN+1)^3 doubles for P1, about
- * 11 MB at r = 7, with its level window behind them when that exceeds shared memory),
- * i.e. a few GB for a level-7 launch.
- * Errors: INVALID_ARG, UNSUPPORTED (window panel beyond shared memory), OOM, CUDA. */
+ * resident block the scaled pivot columns of one element (n (slots + 1) doubles for n nodes
+ * and a front of PN + 1 slots (P2: PN + 3): 150 KB at P1 r = 5, 9 MB at P1 r = 7).
+ * Errors: INVALID_ARG, UNSUPPORTED (P2 r = 7: front too large), OOM, CUDA. */
 mhm_status mhm_reconstruct(const mhm_mesh* mesh, const double* kappa_dev, const mhm_source* f,
                            const double* lambda_dev, const double* u0_dev, const mhm_exact* exact,
                            double* u_nodal_dev, double* err_sq_dev, void* stream);

@@ -126,18 +126,16 @@ typedef struct {
  * loads N_i = -(s psi_i, phi_w)_{dK} and (f, phi_w)_K (a collapsed 4x4x4 Gauss
  * rule per sub-tetrahedron for the non-constant f), the compatibility
  * projection, and the face integrals of the zero-mean solutions.
- *   MHM_FP64: a Cholesky factorisation with local DOF 0 pinned and the forward
- *     substitution of the N_I + 1 right-hand sides, the face integrals in Gram
- *     form (s psi_j, eta_i)_{dK} = -Y_j . Y_i with Y = L^{-1} times the
- *     projected loads.
- *   MHM_MIXED (runs MHM_FP64, iters 1, where that is the faster way to the same quality:
- *     m > 4, and meshes of 512 elements or more unless it_max is 1 or no_fallback is set):
- *     the pinned
- *     matrix scaled by its diagonal is factored once in FP32 (Sec. 3: factor once,
- *     then only products with the factor), the solutions are refined in FP64
- *     against the matrix-free FP64 residual, and the face integrals use the
+ *   MHM_FP64: the matrix with one DOF pinned, bordered by the N_I + 1 projected
+ *     loads g~, is eliminated node by node; the border is then left with the face
+ *     integrals (s psi_j, eta_i)_{dK} = -g~_j . A^{-1} g~_i.
+ *   MHM_MIXED: the pinned matrix scaled by its diagonal is factored once in FP32
+ *     (Sec. 3: factor once, then only products with the factor), the solutions are
+ *     refined in FP64 against the FP64 residual, and the face integrals use the
  *     corrected bilinear form -(g~_j . z_i + z_j . r_i), second order in the
- *     solution error.
+ *     solution error.  Runs MHM_FP64 (iters 1) where that is the faster way to the
+ *     same quality: m > 4, and meshes of 512 elements or more unless it_max is 1 or
+ *     no_fallback is set.
  * Outputs (device, caller-owned, indexed by K):
  *   AK_dev[K][j][i] = (s psi_j, eta_i)_{dK}  (N_I x N_I, symmetric)
  *   EK_dev[K][j]    = -(s psi_j, eta_f)_{dK}
@@ -146,7 +144,7 @@ typedef struct {
  *   status_dev[K]   = 0, MHM_ERR_INVALID_ARG (FP64: non-positive pivot), or
  *                     MHM_ERR_NOT_CONVERGED (MIXED with no_fallback: FP32 breakdown or
  *                     it_max passes without convergence)
- *   iters_dev[K]    = refinement passes (1 for FP64; -1: solved again in FP64 after
+ *   iters_dev[K]    = refinement passes (1 for FP64 and for MIXED that runs it; -1: solved again in FP64 after
  *                     the mixed refinement failed); may be NULL.
  * kappa_dev: 8^r values per K (sub-tetrahedron order above), > 0.
  * Errors: INVALID_ARG (NULL pointers, range, source kind, precision, options),

@@ -9,9 +9,9 @@
 // M = R + slots rows: 33 slots for P1 at N = 32, 35 for P2 at N = 16 (an elimination level by
 // level works on windows of two levels, 64 and 127 rows).
 //
-// How.  This GPU has two FP64 multiply-adds per clock and SM: one warp instruction takes 16
-// clocks of the whole SM, however many of its lanes work, and about 60 other instructions
-// per scheduler fit beside it.  So the layout is made for full FP64 instructions: the lower
+// How.  This GPU has two FP64 multiply-adds per clock and SM, half a lane per scheduler: a
+// warp's FP64 instruction holds its scheduler's unit for 64 clocks, however many of its lanes
+// work, and about 60 other instructions fit beside it.  So the layout is made for full FP64 instructions: the lower
 // triangle lives in registers in tiles of 4 x 8 entries, one entry per lane, and a step is one
 // multiply-add per tile of the rows in use, a_ij -= (w_i / d) w_j with w the pivot's column in
 // shared memory.  The step's other FP64 work is the reciprocal (3), the scaling of w and the

@@ -379,8 +379,8 @@ __host__ __device__ inline Mixed3Smem mixed3_smem(int n, int R, int nb, int nsub
 // Bound by issued instructions and their latencies: the FP32 sweeps take 60 % of 0.9 M warp
 // instructions per element (three passes), the FP64 pipe is 31 % busy; two elements per SM
 // (110 KB of shared memory each) hide one another's chains.  12288 elements, m = 4: 27.5 ms
-// (91.3 ms with a dense packed factor, 512 threads and one element per SM; the FP64 kernel
-// takes 9.9 ms).
+// (91.3 ms with a dense packed factor, 512 threads and one element per SM).  The FP64 kernel
+// takes 9.7 ms, so meshes of 512 elements or more come here only with it_max 1 or no re-solve.
 __global__ void __launch_bounds__(kThreads, 2) k_local3d_mixed(const __grid_constant__ Local3DArgs g) {
     extern __shared__ double sm[];
     __shared__ int bad;

@@ -4,8 +4,7 @@
 // What is computed.  With A the stiffness matrix of a(.,.)_K on the submesh,
 // m_w = int_K phi_w, and the loads N_i = -(s psi_i, phi_w)_{dK}, F = (f, phi_w)_K,
 // the zero-mean solutions are eta = z - (m^T z / |K|) 1 where z solves the
-// system pinned at one DOF (choose_pin: inside the stiffest region touching the
-// first two levels) with the compatible loads g~ = g - (1^T g / |K|) m.
+// system pinned at one DOF (choose_pin_warp: a node of the stiffest fine triangle) with the compatible loads g~ = g - (1^T g / |K|) m.
 // The face integrals of Eq. "mat_global" then reduce to a Gram matrix:
 //     A_K = -N~^T A_p^{-1} N~,   E_K = N~^T A_p^{-1} f~,
 // which is what eliminating A_p from the matrix bordered by the loads leaves in the
@@ -13,13 +12,13 @@
 //
 // How.  Frontal elimination node by node in registers (front.cuh), one warp per coarse
 // triangle up to M = R + slots = 64 rows, 4 to 16 warps above.  Bound by the FP64 pipe: per
-// element of P1 r = 5, R = 19, 26.0 k FP64 warp instructions (16 clocks of the SM each), of
-// which 16.3 k are the algorithm's; 2048 elements in 3.44 ms with the pipe 79 % busy (8.69 ms
+// element of P1 r = 5, R = 19, 26.0 k FP64 warp instructions (64 clocks of a scheduler each), of
+// which 16.3 k are the algorithm's; 2048 elements in 3.30 ms with the pipe about 80 % busy (8.69 ms
 // with a window over two levels in shared memory, 128 threads per element), 4480 elements of
-// P2 r = 4 in 7.9 ms (74.3 ms), 320 elements of P1 r = 7, R = 13 in 63 ms.
+// P2 r = 4 in 7.7 ms (74.3 ms), 320 elements of P1 r = 7, R = 13 in 63 ms.
 //
 // A level whose front is too large for that (P2 r = 7: 259 slots) slides a window over two
-// consecutive levels held in global memory, one workspace slot per block of a persistent
+// consecutive levels held in global memory (pinned by choose_pin within the first two levels), one workspace slot per block of a persistent
 // grid, and factors it panel by panel through shared memory (wide_cholesky_level).
 #include <cuda_runtime.h>
 

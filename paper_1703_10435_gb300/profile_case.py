@@ -12,7 +12,7 @@ factor + solve launch pair of the bench's mixed path:
     python -m paper_1703_10435_gb300.profile_case --workload c3_grf_mixed --n-k 8192
 
 --level r puts every coarse triangle of the workload at refinement level r (its
-kappa field sampled at that level), e.g. the 256-row level windows of r = 7:
+kappa field sampled at that level), e.g. the widest fronts, of r = 7:
 
     python -m paper_1703_10435_gb300.profile_case --workload c4_channels --level 7 \
         --precision fp64 --n-k 152

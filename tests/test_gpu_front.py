@@ -100,7 +100,7 @@ def test_one_warp_per_element(P, r, m, l):
         assert np.array_equal(a, b)
 
 
-@pytest.mark.parametrize("P,r,m", [(1, 1, 1), (1, 2, 1), (2, 1, 2), (1, 3, 1), (2, 2, 4), (1, 3, 4)])
+@pytest.mark.parametrize("P,r,m", [(1, 1, 1), (1, 2, 1), (2, 1, 4), (1, 3, 1), (2, 2, 4), (1, 3, 4)])
 def test_3d_one_warp_and_few_elements_agree(P, r, m):
     """648 tetrahedra in one call (one warp per element) against ranges of 324 (four warps per
     element where the front has room): the same bits."""
