@@ -1616,7 +1616,7 @@ __device__ __forceinline__ void mixed_blocks(const MixedArgs& g) {
             __syncthreads();
             // entry by entry the projections' part (coalesced, one product), then the face
             // loads, which only boundary nodes have (node by node, with the face tests in every
-            // column: 42.1 against 39.9 ms for 18432 elements r = 5, 19 columns)
+            // column: 42.1 against 39.9 ms for 32768 elements r = 5, 19 columns)
             for (int t = threadIdx.x, u = t / R, col = t - u * R; t < nu * R;) {
                 double v = -c.cproj[col] * smass[u];
                 if (col == g.NI) v += Zh[t];

@@ -75,7 +75,7 @@ struct Tuning {
 // registers) where the columns fill the threads.
 // Three against four blocks, ms on 152 SMs: r = 3, 7 columns, 4608 elements 0.773 / 0.653;
 // r = 4, 10 columns, 1702 elements 0.791 / 0.739; r = 4, 19 columns, 18432 elements 8.21 / 7.62;
-// r = 5, 7 columns, 3200 elements 3.03 / 2.77; r = 5, 19 columns, 18432 elements 44.4 / 48.1.
+// r = 5, 7 columns, 3200 elements 3.03 / 2.77; r = 5, 19 columns, 32768 elements 44.4 / 48.1.
 inline int default_blocks_per_sm(int degree, int N, int n_I) {
     return degree == 1 && (N <= 16 || n_I + 1 <= 8) ? 4 : 3;
 }
