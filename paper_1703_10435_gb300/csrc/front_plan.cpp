@@ -157,26 +157,32 @@ FrontPlan front_plan_2d(int P, int N) {
 FrontPlan3 front_plan_3d(int n, int nb, const std::vector<int32_t>& dofs, const std::vector<int8_t>& cls,
                          const std::vector<int32_t>& xyz, int R) {
     FrontPlan3 plan;
-    const int nt = (int)cls.size(), n1 = n - 1;   // node v: DOF v + 1
+    const int nt = (int)cls.size(), n1 = n - 1;
+    std::vector<int> deg(n, 0);
+    for (int s = 0; s < nt * nb; ++s) ++deg[dofs[s]];
+    const int pin = (int)(std::max_element(deg.begin(), deg.end()) - deg.begin());
+    plan.pin = pin;
+    auto dof = [&](int v) { return v + (v >= pin); };
+    auto node = [&](int d) { return d == pin ? -1 : d - (d > pin); };
     std::vector<std::vector<int>> inc(n1), adj(n1);   // slots t nb + a; neighbours
     for (int s = 0; s < nt * nb; ++s)
-        if (dofs[s] > 0) inc[dofs[s] - 1].push_back(s);
+        if (dofs[s] != pin) inc[node(dofs[s])].push_back(s);
     int top = 0;
     for (int v = 0; v < n1; ++v) {
         for (int s : inc[v])
             for (int b = 0; b < nb; ++b) {
-                const int u = dofs[s / nb * nb + b] - 1;
+                const int u = node(dofs[s / nb * nb + b]);
                 if (u >= 0 && u != v) adj[v].push_back(u);
             }
         std::sort(adj[v].begin(), adj[v].end());
         adj[v].erase(std::unique(adj[v].begin(), adj[v].end()), adj[v].end());
-        top = std::max(top, xyz[3 * (v + 1)]);
+        top = std::max(top, xyz[3 * dof(v)]);
     }
     std::vector<FrontStep> steps;
     double best = 0.0;
     for (int kind = 0; kind < 3; ++kind) {
         auto key = [&](int v) -> std::array<int, 6> {
-            const int A = xyz[3 * v + 3], B = xyz[3 * v + 4], C = xyz[3 * v + 5];
+            const int A = xyz[3 * dof(v)], B = xyz[3 * dof(v) + 1], C = xyz[3 * dof(v) + 2];
             if (kind == 0) return {C, B, A, 0, 0, 0};
             if (kind == 1) return {C / 2, B / 2, A / 2, C, B, A};
             return {top - B, top - A, B - C, 0, 0, 0};
@@ -215,7 +221,7 @@ FrontPlan3 front_plan_3d(int n, int nb, const std::vector<int32_t>& dofs, const 
                 const size_t c0 = plan.con.size();
                 for (int s : inc[v])
                     for (int b = 0; b < nb; ++b)
-                        if (dofs[s / nb * nb + b] - 1 == u) {
+                        if (node(dofs[s / nb * nb + b]) == u) {
                             const int t = s / nb, a = s % nb;
                             plan.con.push_back(t | (uint32_t)((cls[t] * nb + a) * nb + b) << 16);
                         }
@@ -227,7 +233,7 @@ FrontPlan3 front_plan_3d(int n, int nb, const std::vector<int32_t>& dofs, const 
             }
         }
         plan.ev.push_back(st.ps | st.zs << 8 | st.m << 16);
-        plan.ev.push_back(v >= 0 ? v + 1 : -1);
+        plan.ev.push_back(v >= 0 ? dof(v) : -1);
         plan.ev.push_back(first);
         plan.ev.push_back(((int)plan.ent.size() - first) | (st.pivot >= 0 ? st.pivot << 16 : 0));
         if (st.pivot >= 0) slot[st.pivot] = -1;

@@ -41,19 +41,21 @@ struct FrontPlan {
 };
 FrontPlan front_plan_2d(int P, int N);
 
-// Tables of the refined tetrahedron, local DOF 0 left out (pinned).  dofs: the nb DOFs of every
+// Tables of the refined tetrahedron, the DOF of most sub-tetrahedra left out (pinned; in the
+// interior the pin holds the constants 3 to 10 times closer than a corner of one sub-tetrahedron
+// does); node v is DOF v, or v + 1 from the pinned one on.  dofs: the nb DOFs of every
 // sub-tetrahedron, cls its class, xyz the DOFs' lattice coordinates (A, B, C).  ev: 4 int32
 // per step: ps | zs << 8 | m << 16; the entering DOF (-1: none); first and number of its
 // entries.  ent: slot | terms << 8 | first term << 16, the first 8 of a node the parts of its
 // diagonal; the value of an entry is the sum of its terms kappa[t] S[s] (con: t | s << 16,
 // s = (class nb + a) nb + b).  Of three orders the one with the least work for R loads.
-// The fourth value of a step also holds the pivot's node (DOF - 1) << 16; first_pivot: the
+// The fourth value of a step also holds the pivot's node << 16; first_pivot: the
 // first step that has one.  For products with the matrix: val: first term | terms << 16 of
 // every off-diagonal value (in the order of the entries), then of every node's diagonal;
 // rc: the off-diagonal values' nodes v | u << 16; rp, col: per node its row, as
 // neighbour | value << 16.
 struct FrontPlan3 {
-    int steps = 0, slots = 0, first_pivot = 0, off = 0;
+    int steps = 0, slots = 0, first_pivot = 0, off = 0, pin = 0;
     std::vector<int32_t> ev, rp;
     std::vector<uint32_t> ent, con, val, rc, col;
 };

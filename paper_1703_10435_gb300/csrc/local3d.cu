@@ -59,7 +59,7 @@ struct Local3DArgs {
     // mixed kernel: values and rows of the matrix (FrontPlan3)
     const uint32_t *val, *rc, *col;
     const int32_t* rp;
-    int first, off;
+    int first, off, pin;
 };
 
 constexpr int kPath[6][3] = {{0, 1, 2}, {0, 2, 1}, {1, 0, 2}, {1, 2, 0}, {2, 0, 1}, {2, 1, 0}};
@@ -208,10 +208,10 @@ __host__ __device__ inline Front3Smem front3_smem(int vec, int n, int nb, int ns
 }
 
 // FP64: one block per coarse tetrahedron at a time eliminates the pinned matrix bordered by
-// its R loads from a front of at most 42 slots (P2, r = 2: 165 DOFs) held in registers
+// its R loads from a front of at most 41 slots (P2, r = 2: 165 DOFs) held in registers
 // (front.cuh); what is left of the border are the face integrals.  Bound by the FP64 pipe
-// (82 % busy at m = 16).  12288 elements, m = 4: 9.9 ms (79.5 ms with the dense matrix in
-// shared memory, one element per SM); 1536 elements, m = 16: 4.2 ms (14.6 ms).
+// (82 % busy at m = 16).  12288 elements, m = 4: 9.5 ms (79.5 ms with the dense matrix in
+// shared memory, one element per SM); 1536 elements, m = 16: 4.0 ms (14.6 ms).
 template <class T, int MINB>
 __global__ void __launch_bounds__(T::threads, MINB) k_local3d(const __grid_constant__ Local3DArgs g) {
     extern __shared__ double sm[];
@@ -329,7 +329,7 @@ struct FrontRowsScaled {
             if (sl == mhm::kPivotSlot) *wnew = x;
             else nb[sl] = x;
         }
-        if (lane == 0) nb[zs] = diag[v.y - 1];
+        if (lane == 0) nb[zs] = diag[v.y - (v.y > g.pin)];
     }
 };
 
@@ -380,7 +380,7 @@ __host__ __device__ inline Mixed3Smem mixed3_smem(int n, int R, int nb, int nsub
 // instructions per element (three passes), the FP64 pipe is 31 % busy; two elements per SM
 // (110 KB of shared memory each) hide one another's chains.  12288 elements, m = 4: 27.5 ms
 // (91.3 ms with a dense packed factor, 512 threads and one element per SM).  The FP64 kernel
-// takes 9.7 ms, so meshes of 512 elements or more come here only with it_max 1 or no re-solve.
+// takes 9.5 ms, so meshes of 512 elements or more come here only with it_max 1 or no re-solve.
 __global__ void __launch_bounds__(kThreads, 2) k_local3d_mixed(const __grid_constant__ Local3DArgs g) {
     extern __shared__ double sm[];
     __shared__ int bad;
@@ -423,12 +423,13 @@ __global__ void __launch_bounds__(kThreads, 2) k_local3d_mixed(const __grid_cons
             cf[j] = -(double)g.signs[4 * K + j / m] * geo[1 + j / m];
         }
         __syncthreads();
-        // projected load of column c at node w (DOF w + 1)
+        // projected load of column c at node w
         auto load = [&](int w, int c) {
-            const double mt = g.mass1[w + 1];
+            const int d = w + (w >= g.pin);
+            const double mt = g.mass1[d];
             double x = -cp[c] * mt;
-            if (c == NI) return g.src24 ? x + src[w + 1] : fma(g.src_value * vol, mt, x);
-            const int a = c / m, cnt = g.fcnt[((a * 6 + g.perm[4 * K + a]) * n + w + 1) * m + c % m];
+            if (c == NI) return g.src24 ? x + src[d] : fma(g.src_value * vol, mt, x);
+            const int a = c / m, cnt = g.fcnt[((a * 6 + g.perm[4 * K + a]) * n + d) * m + c % m];
             // (cnt as a double without a conversion: 2^52 + cnt - 2^52)
             if (cnt) x = fma(cf[c], __hiloint2double(0x43300000, cnt) - 4503599627370496.0, x);
             return x;
@@ -486,7 +487,7 @@ __global__ void __launch_bounds__(kThreads, 2) k_local3d_mixed(const __grid_cons
                 float v0[3] = {0, 0, 0}, v1[3] = {0, 0, 0};
                 int4 e = g.ev[0];
                 for (int st = 0; st < g.steps; ++st) {
-                    const int ps = e.x & 255, zs = (e.x >> 8) & 255, used = e.x >> 16, pn = e.w >> 16, en = e.y - 1;
+                    const int ps = e.x & 255, zs = (e.x >> 8) & 255, used = e.x >> 16, pn = e.w >> 16, en = e.y - (e.y > g.pin);
                     if (st + 1 < g.steps) e = g.ev[st + 1];
                     const bool pivot = ps != mhm::kNoSlot;
                     const float* lc = Lc + (st - g.first) * slots;
@@ -574,7 +575,7 @@ __global__ void __launch_bounds__(kThreads, 2) k_local3d_mixed(const __grid_cons
         double* X = sm + L.W;   // (the FP32 solves are done)
         for (int c = warp; c < R; c += NWARP) {
             double s = 0.0;
-            for (int w = lane; w < n1; w += 32) s = fma(g.mass1[w + 1], Z[w * R + c], s);
+            for (int w = lane; w < n1; w += 32) s = fma(g.mass1[w + (w >= g.pin)], Z[w * R + c], s);
             s = warp_sum(s);
             if (lane == 0) mz[c] = s;
         }
@@ -586,12 +587,12 @@ __global__ void __launch_bounds__(kThreads, 2) k_local3d_mixed(const __grid_cons
                 const int a = j / m, b0 = (a * 6 + g.perm[4 * K + a]) * (m + 1) + j % m;
                 double t = 0.0;
                 for (int e = g.ftab_off[b0]; e < g.ftab_off[b0 + 1]; ++e) {
-                    const int w = g.ftab_node[e] - 1;
-                    if (w >= 0) t = fma(__hiloint2double(0x43300000, g.ftab_cnt[e]) - 4503599627370496.0, Z[w * R + i], t);
+                    const int d = g.ftab_node[e], w = d - (d > g.pin);
+                    if (d != g.pin) t = fma(__hiloint2double(0x43300000, g.ftab_cnt[e]) - 4503599627370496.0, Z[w * R + i], t);
                 }
                 s = fma(cf[j], t, s);
             } else if (g.src24) {
-                for (int w = 0; w < n1; ++w) s = fma(src[w + 1], Z[w * R + i], s);
+                for (int w = 0; w < n1; ++w) s = fma(src[w + (w >= g.pin)], Z[w * R + i], s);
             } else {
                 s = fma(g.src_value * vol, mz[i], s);
             }
@@ -665,6 +666,7 @@ mhm_status upload_front_tables(mhm_mesh3d* m) {
     m->fsteps = plan.steps;
     m->fslots = plan.slots;
     m->ffirst = plan.first_pivot;
+    m->fpin = plan.pin;
     m->foff = plan.off;
     std::vector<double> cls((size_t)24 * 6 * nb * nb), geo(24 * 8, 0.0), mass(n, 0.0);
     for (int t = 0; t < 24; ++t) {
@@ -910,7 +912,7 @@ extern "C" mhm_status mhm3d_local_solve_batch(const mhm3d_mesh* m, const double*
     g.NI = (int)m->NI, g.R = (int)m->NI + 1;
     g.AK = AK, g.EK = EK, g.BK = BK, g.FK = FK, g.status = status, g.iters = iters;
     g.it_max = o.it_max, g.tol = o.tol;
-    g.ev = m->d_fev, g.ent = m->d_fent, g.con = m->d_fcon, g.steps = m->fsteps, g.slots = m->fslots;
+    g.ev = m->d_fev, g.ent = m->d_fent, g.con = m->d_fcon, g.steps = m->fsteps, g.slots = m->fslots, g.pin = m->fpin;
     g.cls24 = m->d_cls24, g.geo24 = m->d_geo24, g.mass1 = m->d_mass1, g.fcnt = m->d_fcnt;
     g.val = m->d_fval, g.rc = m->d_frc, g.rp = m->d_frp, g.col = m->d_fcol, g.first = m->ffirst, g.off = m->foff;
     cudaStream_t s = (cudaStream_t)stream;

@@ -83,7 +83,7 @@ struct mhm_mesh3d {
     mhm3::Nbr3* d_nbrs = nullptr;
     int32_t* d_face_ka = nullptr;
     // frontal elimination (front_plan.h, local3d.cu: upload_front_tables)
-    int fsteps = 0, fslots = 0, ffirst = 0, foff = 0;
+    int fsteps = 0, fslots = 0, ffirst = 0, foff = 0, fpin = 0;
     int4* d_fev = nullptr;
     int32_t* d_frp = nullptr;
     uint32_t *d_fent = nullptr, *d_fcon = nullptr, *d_fval = nullptr, *d_frc = nullptr, *d_fcol = nullptr;
