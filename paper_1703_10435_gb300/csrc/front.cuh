@@ -93,8 +93,9 @@ __device__ __forceinline__ FrontShared<F> front_shared(F* base, int v) {
     return f;
 }
 
-// 1 / d for a normal d by one third-order step y (1 + e + e^2), e = 1 - d y, from the
-// hardware's estimate (relative error below 2^-20): truncation below 2^-60.
+// 1 / d for 2^-1022 <= |d| < 2^1021 (the estimate flushes subnormals, d or 1 / d) by one
+// third-order step y (1 + e + e^2), e = 1 - d y, from the hardware's estimate (relative error below
+// 2^-20): truncation below 2^-60.
 __device__ __forceinline__ double front_rcp(double d) {
     double y;
     asm("rcp.approx.ftz.f64 %0, %1;" : "=d"(y) : "d"(d));
@@ -104,12 +105,23 @@ __device__ __forceinline__ double front_rcp(double d) {
 
 __device__ __forceinline__ float front_rcp(float d) { return 1.0f / d; }
 
-// d positive and finite (a double by its high word: no FP64 instruction)
+// d positive and where front_rcp holds (a double by its high word: no FP64 instruction)
 __device__ __forceinline__ bool front_positive(double d) {
-    const int h = __double2hiint(d);
-    return h > 0 && h < 0x7ff00000;
+    return (unsigned)__double2hiint(d) - 0x00100000u < 0x7fc00000u - 0x00100000u;
 }
 __device__ __forceinline__ bool front_positive(float d) { return d > 0.0f && d < INFINITY; }
+
+// Power of two by which an element's matrix is scaled, from the high words of its largest and
+// smallest positive kappa.  1 unless one of them is beyond 2^+-900; then the largest goes to 2^800 (by
+// 2^1000 at most), so that every pivot and its reciprocal stay normal numbers for a contrast of up to
+// about 2^1700 (front_rcp takes 2^-1022 to 2^1021, and a pivot is a few kappa).  The loads are not
+// scaled: what the border is left with has to be multiplied by the scale.  Exact, so results do
+// not depend on it.  Returned as the exponent, so that asking for 0 takes no FP64 instruction.
+__device__ __forceinline__ int front_scale(int kmax, int kmin) {
+    const int emax = (kmax >> 20) - 1023, emin = (kmin >> 20) - 1023;
+    return kmax < 0 || (emax <= 900 && emin >= -900) ? 0 : min(1000, 800 - emax);
+}
+__device__ __forceinline__ double exp2_of(int e) { return __hiloint2double((1023 + e) << 20, 0); }
 
 template <int NW> __device__ __forceinline__ void front_sync() {
     if (NW == 1) __syncwarp();

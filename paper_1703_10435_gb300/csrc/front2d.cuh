@@ -10,7 +10,7 @@ namespace mhm {
 struct FrontCtx {
     double X[3][2];
     double area, flen[3], FK;
-    int sgn[3], rev[3], la1[3], bad, pin;   // pin: lattice point x | y << 16
+    int sgn[3], rev[3], la1[3], bad, pin, scale;   // pin: lattice point x | y << 16; scale: front_scale
 };
 
 // The pinned node, by one warp: the first node (in DOF order) of the first fine triangle of
@@ -19,20 +19,23 @@ struct FrontCtx {
 // rounding; any node of the element can be pinned here (a window over two levels takes only
 // those of its first two).  On channels of 1e3 the blocks of levels 3..7 come out
 // 1e-11 to 3e-11 of their norm off the exact ones (1e-10 to 3e-10 pinned in the first two levels).
-__device__ inline int choose_pin_warp(int P, int N, const double* kap) {
+// *scale: the matrix's (front_scale).
+__device__ inline int choose_pin_warp(int P, int N, const double* kap, int* scale) {
     const int lane = threadIdx.x & 31, PN = P * N;
     long long best = -1;   // (kappa > 0 orders like its bits)
-    int at = 0;
+    int at = 0, least = 0x7fffffff;
 #pragma unroll 4
     for (int t = lane; t < N * N; t += 32) {
         const long long k = __double_as_longlong(kap[t]);
         if (k > best) best = k, at = t;
+        if (k > 0) least = min(least, (int)(k >> 32));
     }
     for (int o = 16; o > 0; o >>= 1) {
         const long long k = __shfl_xor_sync(0xffffffffu, best, o);
         const int t = __shfl_xor_sync(0xffffffffu, at, o);
         if (k > best || (k == best && t < at)) best = k, at = t;
     }
+    *scale = front_scale((int)(best >> 32), __reduce_min_sync(0xffffffffu, least));
     int j = 0, t = at;
     while (t >= 2 * (N - j) - 1) t -= 2 * (N - j) - 1, ++j;
     int nx[6], ny[6], px = 0, py = 0, bd = 1 << 30;
@@ -44,7 +47,7 @@ __device__ inline int choose_pin_warp(int P, int N, const double* kap) {
     return px | py << 16;
 }
 
-// Geometry, pin, element matrices (Ke, 72), mass of a node on k fine triangles (mass, 8) and
+// Geometry, pin, scaled element matrices (Ke, 72), mass of a node on k fine triangles (mass, 8) and
 // source tables of element K; all threads of the block, ends with a barrier.
 __device__ __forceinline__ void front_element(const DeviceMesh& dm, int64_t K, const double* kap, int P, int N,
                                               int src_kind, double src_value, double src_freq, FrontCtx& c,
@@ -57,8 +60,9 @@ __device__ __forceinline__ void front_element(const DeviceMesh& dm, int64_t K, c
         c.la1[tid] = face_la1(dm, K, tid);
     }
     if (tid < 32) {
-        const int pin = choose_pin_warp(P, N, kap);
-        if (tid == 0) c.pin = pin, c.bad = 0;
+        int scale;
+        const int pin = choose_pin_warp(P, N, kap, &scale);
+        if (tid == 0) c.pin = pin, c.scale = scale, c.bad = 0;
     }
     __syncthreads();
     if (tid < 3) {
@@ -73,6 +77,10 @@ __device__ __forceinline__ void front_element(const DeviceMesh& dm, int64_t K, c
     element_stiffness_pair(P, N, c.X, Ke, Ke + 36, tid, nthr);
     source_tables(dm, src_kind, src_value, src_freq, P, N, c.X, tab, tid, nthr);
     __syncthreads();
+    if (c.scale != 0) {
+        for (int t = tid; t < 72; t += nthr) Ke[t] *= exp2_of(c.scale);
+        __syncthreads();
+    }
 }
 
 // Source loads of all nodes to src (dof order) and their sum F_K to c.FK (a constant source:

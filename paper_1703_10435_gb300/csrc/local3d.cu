@@ -215,7 +215,7 @@ __host__ __device__ inline Front3Smem front3_smem(int vec, int n, int nb, int ns
 template <class T, int MINB>
 __global__ void __launch_bounds__(T::threads, MINB) k_local3d(const __grid_constant__ Local3DArgs g) {
     extern __shared__ double sm[];
-    __shared__ int bad;
+    __shared__ int bad, scales;
     __shared__ double FKs;
     const int tid = threadIdx.x, nthr = blockDim.x, n = g.n, nb = g.nb, NI = g.NI, R = g.R, m = g.m;
     const Front3Smem L = front3_smem(T::vec, n, nb, g.nsub, g.src24 != nullptr);
@@ -237,9 +237,21 @@ __global__ void __launch_bounds__(T::threads, MINB) k_local3d(const __grid_const
             } else {
                 f = g.src_value * vol;
             }
-            if (tid == 0) FKs = f;
+            int most = -1, least = 0x7fffffff;
+            for (int t = tid; t < g.nsub; t += 32) {
+                const long long k = __double_as_longlong(g.kappa[K * (int64_t)g.nsub + t]);
+                if (k > 0) most = max(most, (int)(k >> 32)), least = min(least, (int)(k >> 32));
+            }
+            most = __reduce_max_sync(0xffffffffu, most);
+            least = __reduce_min_sync(0xffffffffu, least);
+            if (tid == 0) FKs = f, scales = mhm::front_scale(most, least);
         }
         __syncthreads();
+        const int scale = scales;
+        if (scale != 0) {
+            for (int t = tid; t < 6 * nb * nb; t += nthr) S[t] *= mhm::exp2_of(scale);
+            __syncthreads();
+        }
         // (psi_j, 1)_{dK} of column j: s |subface|; the projection is its negative over |K|
         auto moment = [&](int j) {
             const int a = j / m, q = j % m, b0 = (a * 6 + g.perm[4 * K + a]) * (m + 1) + q;
@@ -265,6 +277,7 @@ __global__ void __launch_bounds__(T::threads, MINB) k_local3d(const __grid_const
         mhm::front_eliminate<T>(rows, g.ev, g.steps, R, sh, A, &bad, (double*)nullptr, 0);
         double* AK = g.AK + K * (int64_t)NI * NI;
         mhm::front_result<T>(R, A, [&](int i, int j, double v) {
+            if (scale != 0) v *= mhm::exp2_of(scale);
             if (i < NI) {
                 AK[i * NI + j] = v;
                 AK[j * NI + i] = v;

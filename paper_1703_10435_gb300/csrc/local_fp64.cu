@@ -443,7 +443,9 @@ __global__ void __launch_bounds__(T::threads, MINB) k_local_fp64(const __grid_co
 
     // ---- outputs
     double* AK = g.AK + K * NI * NI;
+    const int scale = c.scale;
     front_result<T>(R, A, [&](int i, int j, double v) {
+        if (scale != 0) v *= exp2_of(scale);
         if (i < NI) {
             AK[i * NI + j] = v;
             AK[j * NI + i] = v;

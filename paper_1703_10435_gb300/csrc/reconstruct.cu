@@ -281,7 +281,13 @@ __global__ void __launch_bounds__(T::threads, MINB) k_reconstruct(const __grid_c
                 mz = fma(node_mass(P, N, x, y, area_fine), z[u], mz);
             }
         }
-        const double shift = g.u0[K] - block_sum(mz, smem + L.red) / c.area;
+        const double mean = block_sum(mz, smem + L.red) / c.area;
+        double shift = g.u0[K] - mean;
+        if (c.scale != 0) {   // (the mean in the scaled range: mass times z can underflow in the other)
+            for (int u = tid; u < g.nloc; u += nthr) z[u] = (z[u] - mean) * exp2_of(c.scale);
+            __syncthreads();
+            shift = g.u0[K];
+        }
         double* uK = g.u_out + (g.nod_off ? g.nod_off[K] : K * (int64_t)g.nloc);
         for (int w = tid; w < g.nloc; w += nthr) uK[w] = z[w] + shift;
         if (g.err_out) element_errors(g, K, c.X, z, shift, smem + L.red);
