@@ -16,7 +16,8 @@
 // Pivoting.  A is negative definite, so eliminating a node's multipliers before its u0
 // gives negative pivots and then positive ones (the Schur complement B (-A)^-1 B^T is
 // positive definite on the u0 a block can fix: see "constant modes" at dissect).  So an
-// LDL^T without pivoting is stable in this order and the fronts keep a fixed structure.
+// LDL^T without pivoting is stable in this order and the fronts keep a fixed structure.  Large
+// fronts check the sign of their multipliers' pivots (kSignedPanel).
 //
 // Storage.  Every node has an F x F front (column-major, lower triangle) in one buffer:
 // after its factorisation its first k columns hold L (unit lower triangle, diagonal entries
@@ -71,8 +72,10 @@ struct NDPlan {
     int64_t* dst = nullptr;    // per saddle-point entry: its place in a front (lower triangle), or -1
     int32_t* maps = nullptr;   // children's update -> parent front positions
     int32_t* idx = nullptr;    // all fronts' unknowns
-    int64_t* node_info = nullptr;   // per node: k, F, front_off, vec_off, map_off[0..1], child[0..1], idx offset
-    int* dinfo = nullptr;           // per node: a pivot was zero or not finite
+    // per node: k, F, front_off, vec_off, map_off[0..1], child[0..1], idx offset, size of the first
+    // child's update, pivots that have to be negative
+    int64_t* node_info = nullptr;
+    int* dinfo = nullptr;           // per node: a pivot was refused (k_nd_panel)
 };
 
 void free_nd_plan(NDPlan* p) {
@@ -86,9 +89,13 @@ void free_nd_plan(NDPlan* p) {
 
 namespace {
 
-constexpr int kNodeInfo = 10;   // int64 fields per node on the device
+constexpr int kNodeInfo = 11;   // int64 fields per node on the device
 constexpr int kNdThreads = 256;
 constexpr int kNdPanel = 32;    // pivots per step
+// Fronts with a larger F x k panel (doubles) are refused if a multiplier's pivot is not negative:
+// A is then not negative definite, and an indefinite front of hundreds of unknowns is not
+// stable without pivoting.  In smaller ones only pivots that cannot be divided by are refused.
+constexpr int64_t kSignedPanel = 20 * 1024;
 
 // ---------------------------------------------------------------- symbolic ---
 
@@ -304,6 +311,8 @@ mhm_status build_nd_plan(const mhm_mesh* m, NDPlan** out) {
         q[7] = nd.child[1];
         q[8] = (int64_t)idx_all.size() - nd.F;
         q[9] = nd.child[0] >= 0 ? P->nodes[nd.child[0]].F - P->nodes[nd.child[0]].k : 0;
+        q[10] = 0;   // pivots that have to be negative: the own multipliers, which come first
+        while (nd.F * nd.k > kSignedPanel && q[10] < nd.k && nd.idx[q[10]] < m->nlam) ++q[10];
     }
     // device
     auto up = [](const auto& v, auto** d) -> cudaError_t {
@@ -407,7 +416,9 @@ __global__ void __launch_bounds__(128) k_nd_panel(const int* list, const int64_t
                 const double d = w[p], inv = front_rcp(d);
                 if (lane == 0) {
                     dinv[p] = inv;
-                    if (!(fabs(d) > 0.0) && blockIdx.y == 0) bad[id] = 1;   // zero or not finite
+                    // zero, not finite or where front_rcp does not hold; of the wrong sign
+                    const int h = __double2hiint(d);
+                    if (blockIdx.y == 0 && (!front_positive(fabs(d)) || (p0 + p < q[10] && h >= 0))) bad[id] = 1;
                 }
                 const double l = a[p] * inv;
 #pragma unroll
@@ -716,13 +727,13 @@ extern "C" mhm_status mhm_solve_global(const mhm_mesh* mesh, const double* A_val
     cudaError_t e = cudaGetLastError();
     if (!st && e != cudaSuccess) st = cuda_fail(e, "mhm_solve_global: solve");
     if (!st) {
-        // a zero or non-finite pivot means a singular system: report it (synchronises)
+        // a refused pivot means a singular or (in a large front) indefinite system: report it (synchronises)
         std::vector<int> bad(P->nodes.size());
         e = cudaMemcpyAsync(bad.data(), P->dinfo, bad.size() * sizeof(int), cudaMemcpyDeviceToHost, s);
         if (e == cudaSuccess) e = cudaStreamSynchronize(s);
         if (e != cudaSuccess) return cuda_fail(e, "mhm_solve_global: status");
         for (int v : bad)
-            if (v != 0) return fail(MHM_ERR_INVALID_ARG, "mhm_solve_global: singular saddle-point system (zero pivot)");
+            if (v != 0) return fail(MHM_ERR_INVALID_ARG, "mhm_solve_global: singular saddle-point system (zero, non-finite or wrong-sign pivot)");
     }
     return st;
 }
