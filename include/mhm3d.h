@@ -147,6 +147,7 @@ typedef struct {
  *   iters_dev[K]    = refinement passes (1 for FP64 and for MIXED that runs it; -1: solved again in FP64 after
  *                     the mixed refinement failed); may be NULL.
  * kappa_dev: 8^r values per K (sub-tetrahedron order above), > 0.
+ * Allocates no device memory.
  * Errors: INVALID_ARG (NULL pointers, range, source kind, precision, options),
  * UNSUPPORTED (host-only mesh), CUDA (launch). */
 mhm_status mhm3d_local_solve_batch(const mhm3d_mesh* mesh, const double* kappa_dev, const mhm3d_source* f,

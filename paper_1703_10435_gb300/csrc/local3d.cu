@@ -55,7 +55,7 @@ struct Local3DArgs {
     int steps, slots;
     const double *cls24, *geo24, *mass1;
     const uint8_t* fcnt;
-    const double* src24;  // source tables per type, class, local DOF (k_source3d); NULL: constant
+    int source;           // 1: sin sin sin, by Source3; 0: constant
     // mixed kernel: values and rows of the matrix (FrontPlan3)
     const uint32_t *val, *rc, *col;
     const int32_t* rp;
@@ -63,73 +63,52 @@ struct Local3DArgs {
 };
 
 constexpr int kPath[6][3] = {{0, 1, 2}, {0, 2, 1}, {1, 0, 2}, {1, 2, 0}, {2, 0, 1}, {2, 1, 0}};
-__constant__ int c_perm[6][3] = {{0, 1, 2}, {0, 2, 1}, {1, 0, 2}, {1, 2, 0}, {2, 0, 1}, {2, 1, 0}};
+
+// Source tables (sin sin sin by the collapsed Gauss rule).  With a sub-tetrahedron's first vertex at
+// x and a point of the rule at x + d, the addition theorem splits f(x + d) into eight products of
+// sines and cosines of x and of d,
+//   load of local DOF a = sum_b prod_c (b_c ? cos : sin)(k x_c) M[a][b],
+//   M[a][b] = sum over the points of w phi_a prod_c (b_c ? sin : cos)(k d_c),
+// so an element needs 3 sincos per sub-tetrahedron where the rule has 3 sines at each of its 64
+// points.  The sub-tetrahedra of a class are translates, and the 24 types of element (K mod 24) are
+// images of type 0 under permutations and reflections of the axes, so the M of the six classes
+// of type 0 serve all: 480 values (P2) that the host forms for every call (source_tables) and the
+// kernels take as a parameter: the call allocates nothing and has one launch.  (1536 elements of P2
+// r = 1, m = 4, whole call: 0.285 ms with tables of all types formed by a kernel in memory from the
+// stream-ordered pool, 0.465 formed by every block for itself, 0.197 as a parameter.)
+struct Source3 {
+    double M[6 * 10 * 8];    // per class, local DOF, b
+    uint8_t axis[24][4];     // per type: axis that type 0's x, y, z goes to, + 4 if reflected
+};
 
 __device__ __forceinline__ double warp_sum(double v) {
     for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
     return v;
 }
 
-// Source tables (sin sin sin by the collapsed Gauss rule) of one element type and class (one
-// block each): with a sub-tetrahedron's first vertex at x and a point of the rule at x + d,
-// the addition theorem splits f(x + d) into eight products of sines and cosines of x and of d,
-//   load of local DOF a = sum_b prod_c (b_c ? cos : sin)(k x_c) M[a][b],
-//   M[a][b] = sum over the points of w phi_a prod_c (b_c ? sin : cos)(k d_c).
-// The sub-tetrahedra of a class are translates, so M is per type and class (24 x 6): an element
-// needs 3 sincos per sub-tetrahedron where the rule has 3 sines at each of its 64 points.
-__global__ void __launch_bounds__(kQuad) k_source3d(const double* geom, const double* quad, int N, int nb, double value,
-                                                    double freq, double* out) {
-    __shared__ double f[kQuad][8];
-    const int type = blockIdx.x / 6, cls = blockIdx.x % 6, q = threadIdx.x;
-    const double* V = geom + 12 * type;
-    const double* qp = quad + 4 * q;
-    double s[3], c[3], det = 0.0;
-    {
-        double e[3][3];   // edge vectors v1 - v0, v2 - v1, v3 - v2
-        for (int k = 0; k < 3; ++k)
-            for (int x = 0; x < 3; ++x) e[k][x] = V[3 * (k + 1) + x] - V[3 * k + x];
-        det = e[0][0] * (e[1][1] * e[2][2] - e[1][2] * e[2][1]) - e[0][1] * (e[1][0] * e[2][2] - e[1][2] * e[2][0]) +
-              e[0][2] * (e[1][0] * e[2][1] - e[1][1] * e[2][0]);
-        // a point at reference (x, y, z): steps of the class's path, each along one edge vector
-        double t[3] = {0.0, 0.0, 0.0}, r = qp[0] + qp[1] + qp[2];
-        for (int k = 0; k < 3; ++k) {
-            t[c_perm[cls][k]] = r;
-            r -= qp[k];
-        }
-        for (int x = 0; x < 3; ++x) sincospi(freq * ((t[0] * e[0][x] + t[1] * e[1][x] + t[2] * e[2][x]) / N), &s[x], &c[x]);
-    }
-    const double kf = freq * M_PI, w = qp[3] * fabs(det) / ((double)N * N * N) * value * 3.0 * kf * kf;
-    for (int b = 0; b < 8; ++b) f[q][b] = w * (b & 1 ? s[0] : c[0]) * (b & 2 ? s[1] : c[1]) * (b & 4 ? s[2] : c[2]);
-    __syncthreads();
-    const double* phi = quad + 4 * kQuad;
-    for (int t = q; t < 8 * nb; t += kQuad) {
-        const int a = t >> 3, b = t & 7;
-        double sum = 0.0;
-        for (int p = 0; p < kQuad; ++p) sum = fma(phi[p * nb + a], f[p][b], sum);
-        out[(size_t)blockIdx.x * 8 * nb + t] = sum;
-    }
-}
-
 // Source loads of element K per DOF (src, n) through the loads of every sub-tetrahedron (PL,
 // nsub x nb), summed per DOF in the fixed order of its incidence list.  All threads; ends
 // with a barrier.
-__device__ __forceinline__ void source_loads3(const Local3DArgs& g, int64_t K, double* PL, double* src) {
+__device__ __forceinline__ void source_loads3(const Local3DArgs& g, const Source3& q, int64_t K, double* PL, double* src) {
     const int nb = g.nb, N = g.N;
     const double* V = g.geom + 12 * K;
+    const uint8_t* axis = q.axis[K % 24];
     for (int t = threadIdx.x; t < g.nsub; t += blockDim.x) {
-        double s[3], c[3], T[8];
-        for (int x = 0; x < 3; ++x) {
+        double s[3], c[3], T[8];   // along type 0's axes
+        for (int y = 0; y < 3; ++y) {
+            const int x = axis[y] & 3;
             const double p = V[x] + ((V[3 + x] - V[x]) * g.sub_base[3 * t] + (V[6 + x] - V[3 + x]) * g.sub_base[3 * t + 1] +
                                      (V[9 + x] - V[6 + x]) * g.sub_base[3 * t + 2]) / N;
-            sincospi(g.src_freq * p, &s[x], &c[x]);
+            sincospi(g.src_freq * p, &s[y], &c[y]);
+            if (axis[y] & 4) c[y] = -c[y];   // (the cosine goes with the sine of d)
         }
 #pragma unroll
         for (int b = 0; b < 8; ++b) T[b] = (b & 1 ? c[0] : s[0]) * (b & 2 ? c[1] : s[1]) * (b & 4 ? c[2] : s[2]);
-        const double* M = g.src24 + (size_t)((int)(K % 24) * 6 + g.sub_cls[t]) * 8 * nb;
+        const int m0 = g.sub_cls[t] * 8 * nb;
         for (int a = 0; a < nb; ++a) {
             double v = 0.0;
 #pragma unroll
-            for (int b = 0; b < 8; ++b) v = fma(T[b], M[8 * a + b], v);
+            for (int b = 0; b < 8; ++b) v = fma(T[b], q.M[m0 + 8 * a + b], v);
             PL[t * nb + a] = v;
         }
     }
@@ -213,12 +192,13 @@ __host__ __device__ inline Front3Smem front3_smem(int vec, int n, int nb, int ns
 // (82 % busy at m = 16).  12288 elements, m = 4: 9.5 ms (79.5 ms with the dense matrix in
 // shared memory, one element per SM); 1536 elements, m = 16: 4.0 ms (14.6 ms).
 template <class T, int MINB>
-__global__ void __launch_bounds__(T::threads, MINB) k_local3d(const __grid_constant__ Local3DArgs g) {
+__global__ void __launch_bounds__(T::threads, MINB) k_local3d(const __grid_constant__ Local3DArgs g,
+                                                             const __grid_constant__ Source3 source) {
     extern __shared__ double sm[];
     __shared__ int bad, scales;
     __shared__ double FKs;
     const int tid = threadIdx.x, nthr = blockDim.x, n = g.n, nb = g.nb, NI = g.NI, R = g.R, m = g.m;
-    const Front3Smem L = front3_smem(T::vec, n, nb, g.nsub, g.src24 != nullptr);
+    const Front3Smem L = front3_smem(T::vec, n, nb, g.nsub, g.source != 0);
     const mhm::FrontShared<double> sh = mhm::front_shared(sm, T::vec);
     double *S = sm + L.S, *kap = sm + L.kap, *src = sm + L.src;
     for (int64_t K = g.K0 + blockIdx.x; K < g.K1; K += gridDim.x) {
@@ -228,10 +208,10 @@ __global__ void __launch_bounds__(T::threads, MINB) k_local3d(const __grid_const
         for (int t = tid; t < 6 * nb * nb; t += nthr) S[t] = g.cls24[(size_t)(K % 24) * 6 * nb * nb + t];
         for (int t = tid; t < g.nsub; t += nthr) kap[t] = g.kappa[K * (int64_t)g.nsub + t];
         if (tid == 0) bad = 0;
-        if (g.src24) source_loads3(g, K, sm + L.PL, src);
+        if (g.source) source_loads3(g, source, K, sm + L.PL, src);
         if (tid < 32) {
             double f = 0.0;
-            if (g.src24) {
+            if (g.source) {
                 for (int w = tid; w < n; w += 32) f += src[w];
                 f = warp_sum(f);
             } else {
@@ -259,7 +239,7 @@ __global__ void __launch_bounds__(T::threads, MINB) k_local3d(const __grid_const
             for (int e = g.ftab_off[b0]; e < g.ftab_off[b0 + 1]; ++e) c += g.ftab_cnt[e];
             return (double)g.signs[4 * K + a] * geo[1 + a] * c;
         };
-        FrontRows3D<T::vec> rows{g, kap, S, g.src24 ? src : nullptr, vol};
+        FrontRows3D<T::vec> rows{g, kap, S, g.source ? src : nullptr, vol};
         mhm::static_for<T::vec / 32>([&](auto k) {
             const int q = (tid & 31) + 32 * k;
             rows.cp[k] = rows.cf[k] = 0.0;
@@ -297,7 +277,7 @@ __global__ void __launch_bounds__(T::threads, MINB) k_local3d(const __grid_const
 
 // The frontal kernel of a bordered matrix of M rows.
 struct Front3Kernel {
-    void (*kern)(const Local3DArgs) = nullptr;
+    void (*kern)(const Local3DArgs, const Source3) = nullptr;
     int threads = 0, vec = 0;
 };
 template <class T, int MINB>
@@ -394,7 +374,8 @@ __host__ __device__ inline Mixed3Smem mixed3_smem(int n, int R, int nb, int nsub
 // (110 KB of shared memory each) hide one another's chains.  12288 elements, m = 4: 27.5 ms
 // (91.3 ms with a dense packed factor, 512 threads and one element per SM).  The FP64 kernel
 // takes 9.5 ms, so meshes of 512 elements or more come here only with it_max 1 or no re-solve.
-__global__ void __launch_bounds__(kThreads, 2) k_local3d_mixed(const __grid_constant__ Local3DArgs g) {
+__global__ void __launch_bounds__(kThreads, 2) k_local3d_mixed(const __grid_constant__ Local3DArgs g,
+                                                               const __grid_constant__ Source3 source) {
     extern __shared__ double sm[];
     __shared__ int bad;
     __shared__ double FKs;
@@ -414,10 +395,10 @@ __global__ void __launch_bounds__(kThreads, 2) k_local3d_mixed(const __grid_cons
         for (int t = tid; t < 6 * nb * nb; t += kThreads) S[t] = g.cls24[(size_t)(K % 24) * 6 * nb * nb + t];
         for (int t = tid; t < g.nsub; t += kThreads) kap[t] = g.kappa[K * (int64_t)g.nsub + t];
         if (tid == 0) bad = 0;
-        if (g.src24) source_loads3(g, K, Rr, src);
+        if (g.source) source_loads3(g, source, K, Rr, src);
         if (warp == 0) {
             double f = 0.0;
-            if (g.src24) {
+            if (g.source) {
                 for (int w = lane; w < n; w += 32) f += src[w];
                 f = warp_sum(f);
             } else {
@@ -441,7 +422,7 @@ __global__ void __launch_bounds__(kThreads, 2) k_local3d_mixed(const __grid_cons
             const int d = w + (w >= g.pin);
             const double mt = g.mass1[d];
             double x = -cp[c] * mt;
-            if (c == NI) return g.src24 ? x + src[d] : fma(g.src_value * vol, mt, x);
+            if (c == NI) return g.source ? x + src[d] : fma(g.src_value * vol, mt, x);
             const int a = c / m, cnt = g.fcnt[((a * 6 + g.perm[4 * K + a]) * n + d) * m + c % m];
             // (cnt as a double without a conversion: 2^52 + cnt - 2^52)
             if (cnt) x = fma(cf[c], __hiloint2double(0x43300000, cnt) - 4503599627370496.0, x);
@@ -604,7 +585,7 @@ __global__ void __launch_bounds__(kThreads, 2) k_local3d_mixed(const __grid_cons
                     if (d != g.pin) t = fma(__hiloint2double(0x43300000, g.ftab_cnt[e]) - 4503599627370496.0, Z[w * R + i], t);
                 }
                 s = fma(cf[j], t, s);
-            } else if (g.src24) {
+            } else if (g.source) {
                 for (int w = 0; w < n1; ++w) s = fma(src[w + (w >= g.pin)], Z[w * R + i], s);
             } else {
                 s = fma(g.src_value * vol, mz[i], s);
@@ -670,6 +651,44 @@ mhm_status upload3(const std::vector<T>& h, T** d) {
     return MHM_OK;
 }
 
+// sin and cos of pi x; x mod 2 is exact, so the argument of sin is rounded once.
+void sincospi_host(double x, double* s, double* c) {
+    const double y = M_PI * (x - 2.0 * std::rint(0.5 * x));
+    *s = std::sin(y);
+    *c = std::cos(y);
+}
+
+// Source3 for f = value 3 k^2 sin sin sin, k = freq pi.  Type 0 of h = 1 / nc has the edge vectors
+// h (-1/2, 0, 0), h (0, -1/2, -1/2), h (0, 1, 0), and a point of class (p0, p1, p2) takes steps
+// r0 >= r1 >= r2 along edges p0, p1, p2, so d = h / N (-t0 / 2, t2 - t1 / 2, -t1 / 2) with t[p_k] = r_k:
+// three arguments t0, t1 and six pairs (t1, t2) per point for the six classes.
+void source_tables(const mhm_mesh3d* m, double value, double freq, Source3* out) {
+    const int nb = m->nb;
+    const double h = 1.0 / m->desc.nc / m->N, kf = freq * M_PI;
+    const double amp = h * h * h / 4.0 * value * 3.0 * kf * kf;   // 6 |sub-tetrahedron| = h^3 / 4
+    double f[6][8];
+    std::fill(out->M, out->M + 6 * 8 * nb, 0.0);
+    for (int q = 0; q < kQuad; ++q) {
+        const double* qp = &m->quad[4 * q];
+        const double* phi = &m->quad[4 * kQuad + (size_t)q * nb];
+        const double r[3] = {qp[0] + qp[1] + qp[2], qp[1] + qp[2], qp[2]};
+        double sx[3], cx[3];
+        for (int k = 0; k < 3; ++k) sincospi_host(freq * (-0.5 * h * r[k]), &sx[k], &cx[k]);
+        for (int cls = 0; cls < 6; ++cls) {
+            int at[3];   // step along each edge
+            for (int k = 0; k < 3; ++k) at[kPath[cls][k]] = k;
+            double sy, cy;
+            sincospi_host(freq * (h * (r[at[2]] - 0.5 * r[at[1]])), &sy, &cy);
+            for (int b = 0; b < 8; ++b)
+                f[cls][b] = qp[3] * amp * (b & 1 ? sx[at[0]] : cx[at[0]]) * (b & 2 ? sy : cy) * (b & 4 ? sx[at[1]] : cx[at[1]]);
+            double* M = out->M + cls * 8 * nb;
+            for (int a = 0; a < nb; ++a)
+                for (int b = 0; b < 8; ++b) M[8 * a + b] += phi[a] * f[cls][b];
+        }
+    }
+    std::copy(&m->axis[0][0], &m->axis[0][0] + 24 * 4, &out->axis[0][0]);
+}
+
 // Tables of the frontal elimination: step tables; per element type (the 24 tetrahedra of a
 // cube: every other element is a translate) the class matrices in closed form, |K| and the
 // face areas; mass per DOF; face counts per local face, permutation, DOF and subface.
@@ -701,6 +720,15 @@ mhm_status upload_front_tables(mhm_mesh3d* m) {
             for (int c = 0; c < 3; ++c) u[c] = V[3 * b[1] + c] - V[3 * b[0] + c], w[c] = V[3 * b[2] + c] - V[3 * b[0] + c];
             cross(u, w, x);
             geo[8 * t + 1 + a] = 0.5 * std::sqrt(x[0] * x[0] + x[1] * x[1] + x[2] * x[2]) / ((double)N * N) / 3.0;
+        }
+        // edges 0 and 2 are the images of type 0's along -x and y, edge 1 of -(y + z) / 2
+        const double sign[3] = {-1.0, 1.0, -1.0};
+        const int edge[3] = {0, 2, 1};
+        for (int y = 0; y < 3; ++y) {
+            int x = 0;
+            for (int c = 1; c < 3; ++c)
+                if (y < 2 ? std::fabs(E[edge[y]][c]) > std::fabs(E[edge[y]][x]) : c != m->axis[t][0] % 4 && c != m->axis[t][1] % 4) x = c;
+            m->axis[t][y] = (uint8_t)(x + (sign[y] * E[edge[y]][x] < 0.0 ? 4 : 0));
         }
         const double Vs = geo[8 * t] / ((double)N * N * N);
         for (int c = 0; c < 6; ++c) {
@@ -933,22 +961,18 @@ extern "C" mhm_status mhm3d_local_solve_batch(const mhm3d_mesh* m, const double*
     cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, m->device);
     const Front3Kernel k = front3_kernel(g.R + m->fslots, K1 - K0 <= 3 * (int64_t)sms);
     if (!k.kern) return mhm::fail(MHM_ERR_UNSUPPORTED, "mhm3d_local_solve_batch: front too large");
-    // the source tables in a stream-ordered scratch of this call
-    double* tables = nullptr;
+    Source3 source{};
+    g.source = f->kind == MHM3D_SRC_SINSINSIN;
+    if (g.source) source_tables(m, f->value, f->freq, &source);
     cudaError_t e = cudaSuccess;
-    if (f->kind == MHM3D_SRC_SINSINSIN) {
-        MHM_CUDA_TRY(cudaMallocAsync((void**)&tables, (size_t)24 * 6 * 8 * g.nb * sizeof(double), s));
-        k_source3d<<<24 * 6, kQuad, 0, s>>>(m->d_geom, m->d_quad, g.N, g.nb, f->value, f->freq, tables);
-        g.src24 = tables;
-    }
     // one wave of blocks that share the elements out evenly
-    auto launch = [&](void (*kern)(const Local3DArgs), int threads, size_t smem) {
+    auto launch = [&](void (*kern)(const Local3DArgs, const Source3), int threads, size_t smem) {
         int per_sm = 0;
         cudaError_t c = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
         if (c == cudaSuccess) c = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kern, threads, smem);
         if (c != cudaSuccess) return c;
         const int64_t each = (K1 - K0 + sms - 1) / sms, rounds = (each + std::max(per_sm, 1) - 1) / std::max(per_sm, 1);
-        kern<<<(unsigned)std::min<int64_t>(K1 - K0, sms * ((each + rounds - 1) / rounds)), threads, smem, s>>>(g);
+        kern<<<(unsigned)std::min<int64_t>(K1 - K0, sms * ((each + rounds - 1) / rounds)), threads, smem, s>>>(g, source);
         return cudaGetLastError();
     };
     // MIXED with room to refine and the FP64 re-solve allowed ends with FP64-quality blocks on
@@ -964,9 +988,8 @@ extern "C" mhm_status mhm3d_local_solve_batch(const mhm3d_mesh* m, const double*
     if (e == cudaSuccess && !(mixed && o.no_fallback)) {
         g.only_failed = mixed;   // the elements the refinement could not finish, again in FP64
         e = launch(k.kern, k.threads,
-                   (size_t)front3_smem(k.vec, g.n, g.nb, g.nsub, tables != nullptr).total * sizeof(double));
+                   (size_t)front3_smem(k.vec, g.n, g.nb, g.nsub, g.source != 0).total * sizeof(double));
     }
-    if (tables) cudaFreeAsync(tables, s);
     if (e != cudaSuccess) return mhm::cuda_fail(e, "mhm3d_local_solve_batch: launch");
     return MHM_OK;
 }

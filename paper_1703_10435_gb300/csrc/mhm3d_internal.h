@@ -63,6 +63,7 @@ struct mhm_mesh3d {
     std::vector<int16_t> ftab_node;   // local DOF
     std::vector<int8_t> ftab_cnt;     // fine face triangles of the subface that hold the DOF as a load node
     std::vector<double> quad;         // kQuad*4: x, y, z, w of the reference rule, then kQuad*nb basis values
+    uint8_t axis[24][4] = {};         // per element type, axis of type 0's x, y, z, + 4: reflected (local3d.cu)
     std::vector<int32_t> rowptr, cols;
     std::vector<mhm3::Nbr3> nbrs;
 
