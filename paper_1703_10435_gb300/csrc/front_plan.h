@@ -24,20 +24,20 @@ constexpr int kPivotSlot = 254;   // coupling entry: with the node eliminated in
 constexpr int kDiagSlot = 253;    // coupling entry: a part of the entering node's diagonal
 
 // Steps that eliminate the nodes in `order`, each node entering as late as one entry per
-// step allows; *slots gets the largest front.  adj[v]: the nodes v couples with.
-std::vector<FrontStep> front_schedule(const std::vector<std::vector<int>>& adj, const std::vector<int>& order,
+// step allows; *slots gets the largest front (none if it exceeds kMaxSlots).  cliques: nb nodes
+// each, which couple with one another (fine triangles or sub-tetrahedra; -1: no node).
+std::vector<FrontStep> front_schedule(const std::vector<int>& cliques, int nb, const std::vector<int>& order,
                                       int* slots);
 
 // Tables of the 2-D refined triangle (N segments per face, degree P) as the kernels read
-// them.  ev: 4 int32 per step: ps | zs << 8 | m << 16; lattice point x | y << 16 of the
+// them, in one array.  Steps first, 4 int32 each: ps | zs << 8 | m << 16; lattice point x | y << 16 of the
 // entering node; the number of its fine triangles that carry its mass, and bit 8 + a if it
-// lies on local face a; lattice point of the pivot.  cp: per step ncp entries of 2 uint32: slot | e0 << 8 | e1 << 16 and t0 | t1 << 16:
-// the value kappa[t0] Ke[e0] + kappa[t1] Ke[e1] (t1 = 0xffff: one term; Ke[36 down + 6 a + b]),
+// lies on local face a; lattice point of the pivot.  Then the couplings, per step ncp entries
+// of 2 uint32: slot | e0 << 8 | e1 << 16 and t0 | t1 << 16: the value kappa[t0] Ke[e0] + kappa[t1] Ke[e1] (t1 = 0xffff: one term; Ke[36 down + 6 a + b]),
 // unused entries with slot kNoSlot; the last three hold the diagonal's (up to six) terms.
 struct FrontPlan {
     int steps = 0, slots = 0, ncp = 0;   // steps = 0: no plan (front too large)
-    std::vector<int32_t> ev;
-    std::vector<uint32_t> cp;
+    std::vector<uint32_t> tab;
 };
 FrontPlan front_plan_2d(int P, int N);
 

@@ -689,10 +689,29 @@ void source_tables(const mhm_mesh3d* m, double value, double freq, Source3* out)
     std::copy(&m->axis[0][0], &m->axis[0][0] + 24 * 4, &out->axis[0][0]);
 }
 
+// The mesh's small tables, gathered into one allocation and one copy (a cudaMalloc and a copy each
+// take longer than the tables' contents).
+struct Pack3 {
+    std::vector<char> bytes;
+    std::vector<std::pair<void**, size_t>> at;
+    template <typename T, typename D>
+    void add(const std::vector<T>& h, D** d) {
+        at.emplace_back((void**)d, bytes.size());
+        const char* p = reinterpret_cast<const char*>(h.data());
+        bytes.insert(bytes.end(), p, p + h.size() * sizeof(T));
+        bytes.resize((bytes.size() + 255) & ~(size_t)255);
+    }
+    mhm_status upload(char** base) {
+        const mhm_status st = upload3(bytes, base);
+        for (const auto& q : at) *q.first = st ? nullptr : *base + q.second;
+        return st;
+    }
+};
+
 // Tables of the frontal elimination: step tables; per element type (the 24 tetrahedra of a
 // cube: every other element is a translate) the class matrices in closed form, |K| and the
 // face areas; mass per DOF; face counts per local face, permutation, DOF and subface.
-mhm_status upload_front_tables(mhm_mesh3d* m) {
+void add_front_tables(mhm_mesh3d* m, Pack3* pack) {
     const int nb = m->nb, n = (int)m->n, N = m->N, mm = m->desc.m, P = m->desc.degree;
     const mhm::FrontPlan3 plan = mhm::front_plan_3d(n, nb, m->sub_dofs, m->sub_cls, m->nodes, (int)m->NI + 1);
     m->fsteps = plan.steps;
@@ -773,24 +792,21 @@ mhm_status upload_front_tables(mhm_mesh3d* m) {
         for (int q = 0; q < mm; ++q)
             for (int e = m->ftab_off[b * (mm + 1) + q]; e < m->ftab_off[b * (mm + 1) + q + 1]; ++e)
                 cnt[((size_t)b * n + m->ftab_node[e]) * mm + q] = (uint8_t)m->ftab_cnt[e];
-    mhm_status st = upload3(plan.ev, (int32_t**)&m->d_fev);
-    if (!st) st = upload3(plan.ent, &m->d_fent);
-    if (!st) st = upload3(plan.con, &m->d_fcon);
-    if (!st) st = upload3(plan.val, &m->d_fval);
-    if (!st) st = upload3(plan.rc, &m->d_frc);
-    if (!st) st = upload3(plan.rp, &m->d_frp);
-    if (!st) st = upload3(plan.col, &m->d_fcol);
-    if (!st) st = upload3(cls, &m->d_cls24);
-    if (!st) st = upload3(geo, &m->d_geo24);
-    if (!st) st = upload3(mass, &m->d_mass1);
-    if (!st) st = upload3(cnt, &m->d_fcnt);
-    return st;
+    pack->add(plan.ev, &m->d_fev);
+    pack->add(plan.ent, &m->d_fent);
+    pack->add(plan.con, &m->d_fcon);
+    pack->add(plan.val, &m->d_fval);
+    pack->add(plan.rc, &m->d_frc);
+    pack->add(plan.rp, &m->d_frp);
+    pack->add(plan.col, &m->d_fcol);
+    pack->add(cls, &m->d_cls24);
+    pack->add(geo, &m->d_geo24);
+    pack->add(mass, &m->d_mass1);
+    pack->add(cnt, &m->d_fcnt);
 }
 
 void free_device(mhm_mesh3d* m) {
-    void* ptrs[] = {m->d_geom, m->d_signs, m->d_perm, m->d_sub_dofs, m->d_sub_cls, m->d_sub_base, m->d_ftab_off,
-                    m->d_ftab_node, m->d_ftab_cnt, m->d_quad, m->d_rowptr, m->d_nbrs, m->d_face_ka, m->d_inc_off,
-                    m->d_inc_ent, m->d_fev, m->d_fent, m->d_fcon, m->d_cls24, m->d_geo24, m->d_mass1, m->d_fcnt, m->d_fval, m->d_frc, m->d_frp, m->d_fcol};
+    void* ptrs[] = {m->d_geom, m->d_signs, m->d_perm, m->d_rowptr, m->d_nbrs, m->d_face_ka, m->d_tables};
     for (void* p : ptrs)
         if (p) cudaFree(p);
 }
@@ -857,19 +873,19 @@ extern "C" mhm_status mhm3d_create_mesh(const mhm3d_mesh_desc* desc, int32_t dev
         if (!st) st = upload3(m->geom, &m->d_geom);
         if (!st) st = upload3(m->signs, &m->d_signs);
         if (!st) st = upload3(m->perm, &m->d_perm);
-        if (!st) st = upload3(m->sub_dofs, &m->d_sub_dofs);
-        if (!st) st = upload3(m->sub_cls, &m->d_sub_cls);
-        if (!st) st = upload3(m->sub_base, &m->d_sub_base);
-        if (!st) st = upload3(m->inc_off, &m->d_inc_off);
-        if (!st) st = upload3(m->inc_ent, &m->d_inc_ent);
-        if (!st) st = upload3(m->ftab_off, &m->d_ftab_off);
-        if (!st) st = upload3(m->ftab_node, &m->d_ftab_node);
-        if (!st) st = upload3(m->ftab_cnt, &m->d_ftab_cnt);
-        if (!st) st = upload3(m->quad, &m->d_quad);
         if (!st) st = upload3(m->rowptr, &m->d_rowptr);
         if (!st) st = upload3(m->nbrs, &m->d_nbrs);
         if (!st) st = upload3(m->face_ka, &m->d_face_ka);
-        if (!st) st = upload_front_tables(m);
+        Pack3 pack;
+        pack.add(m->sub_cls, &m->d_sub_cls);
+        pack.add(m->sub_base, &m->d_sub_base);
+        pack.add(m->inc_off, &m->d_inc_off);
+        pack.add(m->inc_ent, &m->d_inc_ent);
+        pack.add(m->ftab_off, &m->d_ftab_off);
+        pack.add(m->ftab_node, &m->d_ftab_node);
+        pack.add(m->ftab_cnt, &m->d_ftab_cnt);
+        add_front_tables(m, &pack);
+        if (!st) st = pack.upload(&m->d_tables);
         if (st) {
             free_device(m);
             delete m;

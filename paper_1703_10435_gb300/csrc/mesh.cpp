@@ -4,6 +4,7 @@
 #include <algorithm>
 #include <climits>
 #include <cmath>
+#include <cstring>
 #include <map>
 #include <utility>
 
@@ -80,8 +81,7 @@ mhm_status upload(const std::vector<T>& h, T** d) {
 }  // namespace
 
 void free_mesh_device(mhm_mesh* m) {
-    void* ptrs[] = {m->d_geom, m->d_sign, m->d_rev, m->d_btab, m->d_btab_sum, m->d_gauss_x,
-                    m->d_gauss_w, m->d_face_v, m->d_face_K, m->d_tri_f, m->d_vxy, m->d_lam_off,
+    void* ptrs[] = {m->d_geom, m->d_sign, m->d_rev, m->d_btab, m->d_gauss_x, m->d_face_v, m->d_face_K, m->d_tri_f, m->d_vxy, m->d_lam_off,
                     m->d_csr_rowptr, m->d_nbr_ptr, m->d_nbrs, m->d_aug_rowptr, m->d_aug_cols, m->d_aug_src, m->d_k_lambda,
                     m->d_lam_face, m->d_lface};
     for (void* p : ptrs)
@@ -91,11 +91,10 @@ void free_mesh_device(mhm_mesh* m) {
     if (m->d_sword) cudaFree(m->d_sword);
     m->d_sword = nullptr;
     for (mhm::Level& lv : m->levels) {
-        if (lv.d_K) cudaFree(lv.d_K);
-        if (lv.d_btab) cudaFree(lv.d_btab);
+        if (lv.d_all) cudaFree(lv.d_all);
+        lv.d_all = nullptr;
         lv.d_K = nullptr;
         lv.d_btab = nullptr;
-        if (lv.d_fev) cudaFree(lv.d_fev);
         lv.d_fev = nullptr;
         lv.d_fcp = nullptr;
         if (lv.fstream) cudaStreamDestroy(lv.fstream);
@@ -458,9 +457,14 @@ extern "C" mhm_status mhm_create_mesh(const mhm_mesh_desc* desc, int32_t device,
     if (!st) st = upload(m->tri_s, &m->d_sign);
     if (!st) st = upload(m->tri_rev, &m->d_rev);
     if (!st) st = upload(m->btab, &m->d_btab);
-    if (!st) st = upload(m->btab_sum, &m->d_btab_sum);
-    if (!st) st = upload(m->gauss_x, &m->d_gauss_x);
-    if (!st) st = upload(m->gauss_w, &m->d_gauss_w);
+    {   // one allocation: Gauss nodes and weights, the multipliers' integrals
+        std::vector<double> g = m->gauss_x;
+        g.insert(g.end(), m->gauss_w.begin(), m->gauss_w.end());
+        g.insert(g.end(), m->btab_sum.begin(), m->btab_sum.end());
+        if (!st) st = upload(g, &m->d_gauss_x);
+        if (m->d_gauss_x) m->d_gauss_w = m->d_gauss_x + m->gauss_x.size();
+        if (m->d_gauss_x) m->d_btab_sum = m->d_gauss_w + m->gauss_w.size();
+    }
     if (!st) st = upload(m->face_v, &m->d_face_v);
     if (!st) st = upload(m->face_K, &m->d_face_K);
     if (!st) st = upload(m->tri_f, &m->d_tri_f);
@@ -479,10 +483,6 @@ extern "C" mhm_status mhm_create_mesh(const mhm_mesh_desc* desc, int32_t device,
     if (m->per_k_levels) {
         if (!st) st = upload(m->kap_off, &m->d_kap_off);
         if (!st) st = upload(m->nod_off, &m->d_nod_off);
-        for (mhm::Level& lv : m->levels) {
-            if (!st) st = upload(lv.K, &lv.d_K);
-            if (!st) st = upload(lv.btab, &lv.d_btab);
-        }
     }
     for (mhm::Level& lv : m->levels) {
         lv.tune.blocks_per_sm = mhm::default_blocks_per_sm(d.degree, lv.N, (int)m->NI);
@@ -490,10 +490,19 @@ extern "C" mhm_status mhm_create_mesh(const mhm_mesh_desc* desc, int32_t device,
         lv.fsteps = plan.steps;
         lv.fslots = plan.slots;
         lv.fncp = plan.ncp;
-        std::vector<uint32_t> both(plan.ev.begin(), plan.ev.end());   // one allocation: steps, then couplings
-        both.insert(both.end(), plan.cp.begin(), plan.cp.end());
-        if (!st) st = upload(both, (uint32_t**)&lv.d_fev);
-        if (lv.d_fev) lv.d_fcp = reinterpret_cast<uint2*>(lv.d_fev + plan.steps);
+        // one allocation: steps, couplings, face-load table, elements
+        std::vector<uint32_t> all = plan.tab;
+        const size_t btab = all.size(), words = 2 * lv.btab.size();
+        all.resize(btab + words + lv.K.size());
+        if (words) std::memcpy(&all[btab], lv.btab.data(), 4 * words);
+        if (!lv.K.empty()) std::memcpy(&all[btab + words], lv.K.data(), 4 * lv.K.size());
+        if (!st) st = upload(all, &lv.d_all);
+        if (lv.d_all && plan.steps) {
+            lv.d_fev = reinterpret_cast<int4*>(lv.d_all);
+            lv.d_fcp = reinterpret_cast<uint2*>(lv.d_fev + plan.steps);
+        }
+        if (lv.d_all && words) lv.d_btab = reinterpret_cast<double*>(lv.d_all + btab);
+        if (lv.d_all && !lv.K.empty()) lv.d_K = reinterpret_cast<int32_t*>(lv.d_all + btab + words);
     }
     if (st) {
         free_mesh_device(m);

@@ -71,7 +71,7 @@ struct mhm_mesh3d {
     double* d_geom = nullptr;
     int8_t* d_signs = nullptr;
     int8_t* d_perm = nullptr;
-    int32_t* d_sub_dofs = nullptr;
+    char* d_tables = nullptr;   // holds every table below but the skeleton's
     int8_t* d_sub_cls = nullptr;
     int8_t* d_sub_base = nullptr;
     int32_t* d_inc_off = nullptr;
@@ -79,11 +79,10 @@ struct mhm_mesh3d {
     int32_t* d_ftab_off = nullptr;
     int16_t* d_ftab_node = nullptr;
     int8_t* d_ftab_cnt = nullptr;
-    double* d_quad = nullptr;
     int32_t* d_rowptr = nullptr;
     mhm3::Nbr3* d_nbrs = nullptr;
     int32_t* d_face_ka = nullptr;
-    // frontal elimination (front_plan.h, local3d.cu: upload_front_tables)
+    // frontal elimination (front_plan.h, local3d.cu: add_front_tables)
     int fsteps = 0, fslots = 0, ffirst = 0, foff = 0, fpin = 0;
     int4* d_fev = nullptr;
     int32_t* d_frp = nullptr;

@@ -97,7 +97,8 @@ struct Level {
     // step tables of the frontal elimination (front_plan.h); fsteps 0: front too large
     int fsteps = 0, fslots = 0, fncp = 0;
     int4* d_fev = nullptr;
-    uint2* d_fcp = nullptr;   // (behind the steps, in d_fev's allocation)
+    uint2* d_fcp = nullptr;
+    uint32_t* d_all = nullptr;   // the allocation that holds the step tables, d_btab and d_K
     // mixed path, several chunks: the factor launches run on their own stream, one chunk
     // ahead of the solve launches (created on first use)
     mutable Tuning tune;
