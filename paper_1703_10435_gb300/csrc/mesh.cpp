@@ -485,7 +485,7 @@ extern "C" mhm_status mhm_create_mesh(const mhm_mesh_desc* desc, int32_t device,
         if (!st) st = upload(m->nod_off, &m->d_nod_off);
     }
     for (mhm::Level& lv : m->levels) {
-        lv.tune.blocks_per_sm = mhm::default_blocks_per_sm(d.degree, lv.N, (int)m->NI);
+        lv.tune = mhm::untuned(d.degree, lv.N, (int)m->NI);
         const mhm::FrontPlan plan = mhm::front_plan_2d(d.degree, lv.N);
         lv.fsteps = plan.steps;
         lv.fslots = plan.slots;

@@ -62,7 +62,7 @@ struct DeviceMesh {
 // autotuner's choices; defaults below): see mhm_tuning in mhm.h.
 struct Tuning {
     int chunk = 8192;        // elements per factor + solve launch pair (<= kChunkMax)
-    int blocks_per_sm = 3;   // resident solve blocks per SM (default_blocks_per_sm sets it per level)
+    int blocks_per_sm = 3;   // resident solve blocks per SM (untuned() sets it per level)
     int nbuf = 2;            // staged level operators in the shared-memory ring (2..4)
     int l2pf = 0;            // L2 prefetch distance in level steps (0: none)
     int pf_all = 0;          // 1: prefetch the element's whole operator set into L2 per solve
@@ -78,6 +78,11 @@ struct Tuning {
 // r = 5, 7 columns, 3200 elements 3.03 / 2.77; r = 5, 19 columns, 32768 elements 44.4 / 48.1.
 inline int default_blocks_per_sm(int degree, int N, int n_I) {
     return degree == 1 && (N <= 16 || n_I + 1 <= 8) ? 4 : 3;
+}
+inline Tuning untuned(int degree, int N, int n_I) {
+    Tuning t;
+    t.blocks_per_sm = default_blocks_per_sm(degree, N, n_I);
+    return t;
 }
 
 // Multifrontal factorisation plan of the global saddle-point system (mhm_solve_global):

@@ -5,8 +5,7 @@
 // level operators, the L2 prefetch of the operators ahead of use and the L2 policy of their
 // copies.  The shapes change speed only; every shape computes the same results.
 //
-// The search is a coordinate descent: each field in turn over its candidate values, the
-// other fields fixed at the best values so far, two sweeps; every candidate runs the
+// The search is a coordinate descent from the level's untuned shape (tune_search.h); every candidate runs the
 // level's first elements (up to kTuneSample) once to warm up and twice timed with CUDA
 // events on the caller's stream, the faster run counting.  Results go to a text cache, one
 // line per key (degree, level, right-hand sides, device name, SM count); the last line of a
@@ -21,6 +20,7 @@
 #include <vector>
 
 #include "mhm_internal.h"
+#include "tune_search.h"
 
 namespace mhm {
 
@@ -140,35 +140,15 @@ mhm_status search_level(const mhm_mesh* mesh, const Level& lv, const double* kap
     mhm_solve_opts to = o;
     to.factor_store = nullptr;   // timing runs factor every element
     to.factor_reuse = 0;
-    Tuning best = Tuning();
-    best.chunk = (int)std::min<int64_t>(8192, std::max<int64_t>(256, lv.nK));
-    lv.tune = best;
+    mhm_status st = MHM_OK;
     double best_t = 0.0;
-    mhm_status st = time_level(mesh, lv, kappa, f, to, AK, EK, BK, FK, status, iters, ws, ws_bytes, s, e0, e1, &best_t);
-    struct Field {
-        int Tuning::*m;
-        std::vector<int> values;
-    };
-    const std::vector<Field> fields = {{&Tuning::nbuf, {2, 3, 4}},          {&Tuning::pf_all, {0, 1}},
-                                       {&Tuning::l2pf, {0, 2, 4, 8}},       {&Tuning::op_policy, {0, 1, 2}},
-                                       {&Tuning::blocks_per_sm, {2, 3, 4}},    {&Tuning::chunk, {2048, 4096, 8192}}};
-    for (int sweep = 0; sweep < 2 && !st; ++sweep) {
-        for (const Field& fd : fields) {
-            for (int v : fd.values) {
-                if (st) break;
-                if (best.*(fd.m) == v) continue;
-                Tuning cand = best;
-                cand.*(fd.m) = v;
-                lv.tune = cand;
-                double t = 0.0;
-                st = time_level(mesh, lv, kappa, f, to, AK, EK, BK, FK, status, iters, ws, ws_bytes, s, e0, e1, &t);
-                if (!st && t < best_t) {
-                    best_t = t;
-                    best = cand;
-                }
-            }
-        }
-    }
+    Tuning best = untuned(mesh->desc.degree, lv.N, (int)mesh->NI);
+    best.chunk = (int)std::min<int64_t>(best.chunk, std::max<int64_t>(256, lv.nK));   // (the chunk it runs)
+    best = tune_descend(best, &best_t, [&](const Tuning& shape, double* ms) {
+        lv.tune = shape;
+        st = time_level(mesh, lv, kappa, f, to, AK, EK, BK, FK, status, iters, ws, ws_bytes, s, e0, e1, ms);
+        return st == MHM_OK;
+    });
     cudaEventDestroy(e0);
     cudaEventDestroy(e1);
     best.tuned = 1;
