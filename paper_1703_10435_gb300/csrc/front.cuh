@@ -93,9 +93,12 @@ __device__ __forceinline__ FrontShared<F> front_shared(F* base, int v) {
     return f;
 }
 
-// 1 / d for 2^-1022 <= |d| < 2^1021 (the estimate flushes subnormals, d or 1 / d) by one
-// third-order step y (1 + e + e^2), e = 1 - d y, from the hardware's estimate (relative error below
-// 2^-20): truncation below 2^-60.
+// 1 / d for 2^-1022 <= |d| < 2^1021 (the estimate flushes subnormals, d or 1 / d): one step of the
+// hyperpower iteration of order three (M. Altman, Pacific J. Math. 10, 1960), y (1 + e + e^2)
+// with e = 1 - d y, from the hardware's estimate y.  The estimate reads and gives 20 bits of
+// mantissa, so |e| <= 2^-19; 1 / d = y (1 + e + e^2 + e^3 + ..), so the step leaves out 2^-57, a
+// sixteenth of an ulp at most, and with its roundings ends within 0.57 ulp: the division's value or
+// the one next to it.  Three FP64 instructions after the estimate.
 __device__ __forceinline__ double front_rcp(double d) {
     double y;
     asm("rcp.approx.ftz.f64 %0, %1;" : "=d"(y) : "d"(d));
