@@ -813,15 +813,6 @@ void free_device(mhm_mesh3d* m) {
 
 }  // namespace
 
-// The limit of the meshes taken on a device: the packed pinned triangle (or, if larger, nb + 1
-// loads per sub-tetrahedron in up to 8 groups of its 64 points), n x R columns and tables.
-size_t local3d_dense_bytes(int n, int NI, int nb, int nsub) {
-    int qs = 8;
-    while (qs > 1 && qs * nsub > 512) qs >>= 1;
-    const size_t R = NI + 1, npk = (size_t)(n - 1) * n / 2, pl = (size_t)qs * nsub * (nb + 1);
-    return (std::max(npk, pl) + n * R + n + 6 * nb * nb + 6 * 21 + R + 16) * sizeof(double);
-}
-
 }  // namespace mhm3
 
 using namespace mhm3;
@@ -848,10 +839,9 @@ extern "C" mhm_status mhm3d_create_mesh(const mhm3d_mesh_desc* desc, int32_t dev
     if (device >= 0) {
         if (!mhm::device_supported(device))
             return mhm::fail(MHM_ERR_UNSUPPORTED, "mhm3d_create_mesh: device is not an sm_103 GPU");
-        if (n > kMaxLocal || d.m > kMaxM ||
-            local3d_dense_bytes((int)n, 4 * d.m, d.degree == 1 ? 4 : 10, 1 << (3 * d.r)) > 227 * 1024)
+        if (n > kMaxLocal || d.m > kMaxM)
             return mhm::fail(MHM_ERR_UNSUPPORTED,
-                             "mhm3d_create_mesh: the local factor and right-hand sides exceed shared memory "
+                             "mhm3d_create_mesh: more local DOFs or multipliers than the kernels take "
                              "(degree 2: r <= 2, degree 1: r <= 3, m <= 16)");
     }
     mhm_mesh3d* m = new mhm_mesh3d();

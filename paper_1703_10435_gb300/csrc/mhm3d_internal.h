@@ -11,8 +11,8 @@
 
 namespace mhm3 {
 
-// Largest local space whose pinned factor (packed lower triangle) and right-hand
-// sides are held in one block's shared memory: 165 DOFs (k = 2, r = 2; k = 1, r = 3).
+// Largest local space taken on a device: 165 DOFs (k = 2, r = 2; k = 1, r = 3), whose fronts have at
+// most 41 slots; with 65 loads (m = 16) 106 of the 112 rows of the largest kernel.
 constexpr int kMaxLocal = 165;
 constexpr int kMaxM = 16;                  // subfaces per face
 constexpr int kMaxNI = 4 * kMaxM;          // multipliers per element
@@ -28,9 +28,6 @@ struct Nbr3 {
     int32_t K0, a0, b0;
     int32_t K1, a1, b1;   // K1 = -1: one contribution
 };
-
-// bytes of one element's dense problem, which bounds the meshes that are accepted
-size_t local3d_dense_bytes(int n, int NI, int nb, int nsub);
 
 // rule on [0,1] (Newton on the Legendre polynomial)
 void gauss01(int n, double* x, double* w);
