@@ -361,7 +361,8 @@ mhm_status mhm_assemble_skeleton(const mhm_mesh* mesh, const double* AK_dev, con
  * Writes lambda_dev (n_lambda) and u0_dev (n_K).  A multifrontal LDL^T in a nested
  * dissection order of T_H, with one step of refinement; the plan and its device memory are
  * made on the first call and kept by the mesh.  Synchronous (it reports a zero pivot).
- * Errors: INVALID_ARG (NULL, singular matrix), UNSUPPORTED, CUDA. */
+ * Errors: INVALID_ARG (NULL; a singular matrix, or one whose A is not negative definite in a large
+ * front: a zero, non-finite or wrong-sign pivot), UNSUPPORTED, CUDA. */
 mhm_status mhm_solve_global(const mhm_mesh* mesh, const double* A_vals_dev, const double* E_dev,
                             const double* BK_dev, const double* FK_dev, double* lambda_dev, double* u0_dev,
                             void* stream);
@@ -377,8 +378,9 @@ mhm_status mhm_solve_global(const mhm_mesh* mesh, const double* A_vals_dev, cons
  * `exact`), also writes err_sq_dev[2K] = ||u_{H,h} - u||^2_{L2(K)} and
  * err_sq_dev[2K+1] = |u_{H,h} - u|^2_{H1(K)}, by the collapsed 4 x 4 Gauss rule
  * on every fine triangle.  Allocates temporary device memory, stream-ordered: per
- * resident block the scaled pivot columns of one element (n (slots + 1) doubles for n nodes
- * and a front of PN + 1 slots (P2: PN + 3): 150 KB at P1 r = 5, 9 MB at P1 r = 7).
+ * resident block the scaled pivot columns of one element (slots + 1 doubles for each of its
+ * steps, n nodes and the slots of the first front, with PN + 1 slots (P2: PN + 3): 162 KB at P1
+ * r = 5, 8.9 MB at P1 r = 7).
  * Errors: INVALID_ARG, UNSUPPORTED (P2 r = 7: front too large), OOM, CUDA. */
 mhm_status mhm_reconstruct(const mhm_mesh* mesh, const double* kappa_dev, const mhm_source* f,
                            const double* lambda_dev, const double* u0_dev, const mhm_exact* exact,

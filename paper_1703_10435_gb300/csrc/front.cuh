@@ -53,7 +53,7 @@ template <int LO, int HI, class F> __device__ __forceinline__ void static_select
 }
 // fn(0), fn(1), .. fn(n - 1) for a run-time n <= N, each index a constant.  The rest of the
 // range hangs in one branch: under a loop of conditions the compiler issues every
-// instruction with a predicate, and a switched-off FP64 instruction takes its 16 clocks too.
+// instruction with a predicate, and a switched-off FP64 instruction holds the scheduler for its 64 clocks too.
 template <int I, int N, class F> __device__ __forceinline__ void static_upto(int n, F&& fn) {
     if constexpr (I < N) {
         if (n > I) {

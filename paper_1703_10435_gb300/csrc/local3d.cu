@@ -189,8 +189,9 @@ __host__ __device__ inline Front3Smem front3_smem(int vec, int n, int nb, int ns
 // FP64: one block per coarse tetrahedron at a time eliminates the pinned matrix bordered by
 // its R loads from a front of at most 41 slots (P2, r = 2: 165 DOFs) held in registers
 // (front.cuh); what is left of the border are the face integrals.  Bound by the FP64 pipe
-// (82 % busy at m = 16).  12288 elements, m = 4: 9.5 ms (79.5 ms with the dense matrix in
-// shared memory, one element per SM); 1536 elements, m = 16: 4.0 ms (14.6 ms).
+// (84 % busy at m = 4, 12.4 k warp instructions per element; 81 % at m = 16).  12288 elements,
+// m = 4, sin sin sin: 9.4 ms (79.5 ms with the dense matrix in shared memory, one element per SM);
+// 1536 elements, m = 16: 4.0 ms (14.6 ms).
 template <class T, int MINB>
 __global__ void __launch_bounds__(T::threads, MINB) k_local3d(const __grid_constant__ Local3DArgs g,
                                                              const __grid_constant__ Source3 source) {
@@ -289,7 +290,7 @@ void front3_try(int M, Front3Kernel* k) {
 }
 // few: no more elements than three per SM: 4 warps (and one for the rows) share an element, which
 // shortens a step where a single warp's latency is what counts (24 elements, m = 4: 0.86 -> 0.48
-// ms); the same results bit for bit.
+// ms; 0.37 without the source tables' own kernel); the same results bit for bit.
 Front3Kernel front3_kernel(int M, bool few) {
     Front3Kernel k;
     if (few) {
@@ -371,9 +372,9 @@ __host__ __device__ inline Mixed3Smem mixed3_smem(int n, int R, int nb, int nsub
 //
 // Bound by issued instructions and their latencies: the FP32 sweeps take 60 % of 0.9 M warp
 // instructions per element (three passes), the FP64 pipe is 31 % busy; two elements per SM
-// (110 KB of shared memory each) hide one another's chains.  12288 elements, m = 4: 27.5 ms
+// (110 KB of shared memory each) hide one another's chains.  12288 elements, m = 4: 24.6 ms
 // (91.3 ms with a dense packed factor, 512 threads and one element per SM).  The FP64 kernel
-// takes 9.5 ms, so meshes of 512 elements or more come here only with it_max 1 or no re-solve.
+// takes 9.4 ms, so meshes of 512 elements or more come here only with it_max 1 or no re-solve.
 __global__ void __launch_bounds__(kThreads, 2) k_local3d_mixed(const __grid_constant__ Local3DArgs g,
                                                                const __grid_constant__ Source3 source) {
     extern __shared__ double sm[];
@@ -982,10 +983,12 @@ extern "C" mhm_status mhm3d_local_solve_batch(const mhm3d_mesh* m, const double*
         return cudaGetLastError();
     };
     // MIXED with room to refine and the FP64 re-solve allowed ends with FP64-quality blocks on
-    // either kernel, and the FP64 one is the faster from 512 elements on (12288 elements, m = 4:
-    // 9.9 against 27.4 ms, 1536: 1.6 against 4.1; m = 1: 6.9 against 19.2, 1.0 against 2.9; P1
-    // r = 3: 10.9 against 24.3, 1.7 against 3.7; at 192 elements the two are within 12 %).  The
-    // rule goes by the mesh and not by the call's range: a range gives the full call's bits.
+    // either kernel, and the FP64 one is the faster (12288 elements, m = 4: 9.4 against 24.6 ms,
+    // 1536: 1.5 against 3.6; m = 1: 6.6 against 17.7, 0.9 against 2.6; P1 r = 3: 10.6 against 23.3,
+    // 1.6 against 3.4; 192 elements: 0.43 against 0.65).  The line was drawn where the two met with
+    // one warp per element in FP64; with four it is the faster below 512 too, where the refinement
+    // stays for the sake of tol and iters.  The rule goes by the mesh and not by the call's range:
+    // a range gives the full call's bits.
     const bool direct = o.it_max >= 2 && !o.no_fallback && m->nK >= 512;
     const bool mixed = precision == MHM_MIXED && !direct && g.R <= kMaxMixedR && m->fslots <= FrontTilesMixed::rows;
     if (mixed)

@@ -12,7 +12,7 @@
 //
 // How.  Frontal elimination node by node in registers (front.cuh), one warp per coarse
 // triangle up to M = R + slots = 64 rows, 4 to 16 warps above.  Bound by the FP64 pipe: per
-// element of P1 r = 5, R = 19, 26.0 k FP64 warp instructions (64 clocks of a scheduler each), of
+// element of P1 r = 5, R = 19, 25.2 k FP64 warp instructions (64 clocks of a scheduler each), of
 // which 16.3 k are the algorithm's; 2048 elements in 3.30 ms with the pipe about 80 % busy (8.69 ms
 // with a window over two levels in shared memory, 128 threads per element), 4480 elements of
 // P2 r = 4 in 7.7 ms (74.3 ms), 320 elements of P1 r = 7, R = 13 in 63 ms.
@@ -45,7 +45,7 @@ struct Fp64Args {
     uint32_t* sword;          // the mesh's outcome word (mhm_sync_status)
     double src_value, src_freq;
     int64_t K0, K1;  // launch indices [K0, K1) within the level
-    double* win;     // wide window: slots of win_doubles per block (NULL: window in shared memory)
+    double* win;     // wide window: slots of win_doubles per block (NULL: frontal elimination)
     size_t win_doubles;
     double *AK, *EK, *BK, *FK;
     int32_t *status, *iters;
@@ -464,7 +464,8 @@ __global__ void __launch_bounds__(T::threads, MINB) k_local_fp64(const __grid_co
         if (g.iters) g.iters[K] = g.fallback ? -1 : 1;
         if (g.sword && (c.bad || g.fallback))
             atomicOr(g.sword, (c.bad ? 1u << MHM_ERR_INVALID_ARG : 0u) | (g.fallback ? MHM_STATUS_REFINED_IN_FP64 : 0u));
-    }    __syncthreads();   // the context and the tables serve the next element
+    }
+    __syncthreads();   // the context and the tables serve the next element
     }
 }
 
@@ -664,14 +665,14 @@ mhm_status launch_local_fp64_list_ws(const mhm_mesh* mesh, const Level& lv, cons
                                      const mhm_source& f, const int32_t* list, const int32_t* count, int64_t max_n,
                                      double* AK, double* EK, double* BK, double* FK, int32_t* status,
                                      int32_t* iters, void* ws, size_t ws_bytes, cudaStream_t stream) {
-    // re-solves of failed elements of a wide mixed level: the window may need the workspace
+    // re-solves of failed elements of a wide mixed level (ws: only for a window in global memory)
     return launch_fp64(mesh, lv, kappa, f, 0, max_n, AK, EK, BK, FK, status, iters, list, count, ws, ws_bytes, stream);
 }
 
 mhm_status launch_local_fp64_list(const mhm_mesh* mesh, const Level& lv, const double* kappa, const mhm_source& f,
                                   const int32_t* list, const int32_t* count, int64_t max_n, double* AK, double* EK,
                                   double* BK, double* FK, int32_t* status, int32_t* iters, cudaStream_t stream) {
-    // re-solves of failed mixed elements: mixed levels always have a shared-memory window
+    // re-solves of failed mixed elements: their levels have a frontal kernel, which needs no workspace
     return launch_fp64(mesh, lv, kappa, f, 0, max_n, AK, EK, BK, FK, status, iters, list, count, nullptr, 0, stream);
 }
 

@@ -207,13 +207,13 @@ struct mhm_mesh {
 
 namespace mhm {
 // Launchers (defined in the .cu files).
-// FP64 local solves of launch indices [K0, K1) of level lv; a level whose window exceeds
-// shared memory keeps it in ws (fp64_level_workspace bytes; with less, fewer blocks)
+// FP64 local solves of launch indices [K0, K1) of level lv; a level whose front is too large for
+// registers keeps a window in ws (fp64_level_workspace bytes; with less, fewer blocks)
 mhm_status launch_local_fp64(const mhm_mesh* mesh, const Level& lv, const double* kappa, const mhm_source& f,
                              int64_t K0, int64_t K1, double* AK, double* EK, double* BK, double* FK,
                              int32_t* status, int32_t* iters, void* ws, size_t ws_bytes, cudaStream_t stream);
-size_t fp64_level_workspace(const mhm_mesh* mesh, const Level& lv);   // 0: window in shared memory
-size_t fp64_slot_bytes(const mhm_mesh* mesh, const Level& lv);        // one block's window slot (0: shared memory)
+size_t fp64_level_workspace(const mhm_mesh* mesh, const Level& lv);   // 0: front in registers
+size_t fp64_slot_bytes(const mhm_mesh* mesh, const Level& lv);        // one block's window slot (0: front in registers)
 bool fp64_level_launchable(const mhm_mesh* mesh, const Level& lv);    // panel fits shared memory, R <= 64
 int fp64_window_rows(const mhm_mesh* mesh, const Level& lv);
 // workspace region of one level at the given precision, and of all levels (one after the other)

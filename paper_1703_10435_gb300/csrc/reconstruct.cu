@@ -9,7 +9,7 @@
 // collapsed 4 x 4 Gauss rule per fine triangle.
 // Levels whose front is too large (P2 r = 7) are refused.
 //
-// Bound by the FP64 pipe (81 % busy): 17.2 k FP64 warp instructions per element of P1 r = 5,
+// Bound by the FP64 pipe (85 % busy): 16.6 k FP64 warp instructions per element of P1 r = 5,
 // of which the update of the front takes 8 k, a step's fixed part (reciprocal, scaling,
 // couplings, the backward sum) the rest.  32768 elements: 32.2 ms (182.6 ms with a window
 // over two levels and a dense backward sweep).

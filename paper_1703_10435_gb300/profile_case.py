@@ -19,9 +19,10 @@ kappa field sampled at that level), e.g. the widest fronts, of r = 7:
 
 --cube nc runs the three-dimensional local solves instead (the unit cube of the paper's
 experiment, Sec. 5: 24 nc^3 tetrahedra, P2 on 64 sub-tetrahedra, m subfaces per face,
-kappa = 1, f = 12 pi^2 sin sin sin), e.g. the 1536 elements of nc = 4 in mixed precision:
+kappa = 1, f = 12 pi^2 sin sin sin), e.g. the 1536 elements of nc = 4 (mixed precision runs the
+FP64 elimination there, and the refinement kernel on nc = 1 and 2):
 
-    python -m paper_1703_10435_gb300.profile_case --cube 4 --m 4 --precision mixed
+    python -m paper_1703_10435_gb300.profile_case --cube 4 --m 16 --precision fp64
 """
 from __future__ import annotations
 
