@@ -74,13 +74,9 @@ __device__ __forceinline__ void front_element(const DeviceMesh& dm, int64_t K, c
                                    (c.X[2][0] - c.X[0][0]) * (c.X[1][1] - c.X[0][1]));
     if (tid == 0) c.area = area;
     if (tid < 8) mass[tid] = tid * (area / ((double)N * N) / 3.0);
-    element_stiffness_pair(P, N, c.X, Ke, Ke + 36, tid, nthr);
+    element_stiffness_pair(P, N, c.X, Ke, Ke + 36, tid, nthr, exp2_of(c.scale));
     source_tables(dm, src_kind, src_value, src_freq, P, N, c.X, tab, tid, nthr);
     __syncthreads();
-    if (c.scale != 0) {
-        for (int t = tid; t < 72; t += nthr) Ke[t] *= exp2_of(c.scale);
-        __syncthreads();
-    }
 }
 
 // Source loads of all nodes to src (dof order) and their sum F_K to c.FK (a constant source:

@@ -97,10 +97,10 @@ __device__ inline void element_stiffness(int P, const double X[3][2], double* S 
 }
 
 // Element matrices of the up and the down fine triangles of the coarse triangle X (N
-// segments per face) as element_stiffness, an entry per thread: Su[nb a + b], Sd[nb a + b].  (A
+// segments per face) as element_stiffness, times f, an entry per thread: Su[nb a + b], Sd[nb a + b].  (A
 // warp issues an FP64 instruction every 64 clocks: the two P2 matrices by one thread take 55 us.)
 __device__ inline void element_stiffness_pair(int P, int N, const double X[3][2], double* Su, double* Sd, int tid,
-                                              int nthr) {
+                                              int nthr, double f = 1.0) {
     const double e1[2] = {(X[1][0] - X[0][0]) / N, (X[1][1] - X[0][1]) / N};
     const double e2[2] = {(X[2][0] - X[0][0]) / N, (X[2][1] - X[0][1]) / N};
     const int nb = P == 1 ? 3 : 6;
@@ -131,7 +131,7 @@ __device__ inline void element_stiffness_pair(int P, int N, const double X[3][2]
             s += adet * (P == 1 ? 0.5 : 1.0 / 6.0) *
                  (gr[0][0] * (g00 * gr[1][0] + g01 * gr[1][1]) + gr[0][1] * (g01 * gr[1][0] + g11 * gr[1][1]));
         }
-        (dn ? Sd : Su)[ab] = s;
+        (dn ? Sd : Su)[ab] = s * f;
     }
 }
 
