@@ -370,8 +370,8 @@ __host__ __device__ inline Mixed3Smem mixed3_smem(int n, int R, int nb, int nsub
 // averaged with its transpose.  An element whose FP32 factor breaks down or that does not
 // converge gets MHM_ERR_NOT_CONVERGED (the host then re-solves it in FP64 unless asked not to).
 //
-// Bound by issued instructions and their latencies: the FP32 sweeps take 60 % of 0.9 M warp
-// instructions per element (three passes), the FP64 pipe is 31 % busy; two elements per SM
+// Bound by issued instructions and their latencies: 0.74 M warp instructions per element (two
+// passes), most of them the FP32 sweeps, 11 k of them FP64 (20 % of that pipe on 192 elements); two elements per SM
 // (110 KB of shared memory each) hide one another's chains.  12288 elements, m = 4: 24.6 ms
 // (91.3 ms with a dense packed factor, 512 threads and one element per SM).  The FP64 kernel
 // takes 9.4 ms, so meshes of 512 elements or more come here only with it_max 1 or no re-solve.
